@@ -144,11 +144,12 @@ struct genga_system {
     size_t ksym_list_cap = 0;
     unsigned *ksym_ctr = nullptr;  // dispatch counter
     double *ksym_irc = nullptr;    // 1 / rc per body
-    float2 *ksym_ircf = nullptr;   // the same as two floats
-    float2 *ksym_mhl = nullptr;    // mass as two floats
+    float2 *ksym_ircf = nullptr;   // mixed: the same as two floats
+    float4 *ksym_body = nullptr;   // mixed: the bodies as float expansions (kick_ff.cu)
+    float4 *ksym_bounds = nullptr; // mixed: coordinate and mass bounds per block, then the header
     float *ksym_thrpc = nullptr;   // FP32 upper bound of (f_pc rc)^2
     float2 *ksym_pcf = nullptr;    // (f_pc rc)^2 as two floats
-    size_t ksym_body_cap = 0;
+    size_t ksym_body_cap = 0;      // bodies the arrays above hold (whole tiles)
 
     // candidates and encounter lists
     uint2 *cand = nullptr;

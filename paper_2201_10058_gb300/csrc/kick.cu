@@ -2,41 +2,38 @@
 //   a_i = G sum_{j != i} m_j K(r_ij; rc_ij) (x_j - x_i) / r_ij^3
 // and the close-encounter pre-check (Appendix A).
 //
-// GB300 design.  The kick is bound by the FP64 pipe (1.68 FP64 instructions per
-// clock per SM on GB300, measured, 1/74 of FP32), so the kernels minimise FP64
-// instructions per interaction and keep everything else on the FP32, MUFU and
-// integer pipes.  Two layouts:
-//   * symmetric (kick_sym_kernel, below): each unordered pair once, its force to
-//     both bodies (Newton's third law) -- 9 FP64 instructions per pair in the
-//     mixed form, 4.5 per interaction; the pre-check rides along on the FP32
-//     pipe.  Used where it is predicted faster (N of ~8k and more);
+// GB300 design.  FP64 runs at 1.68 instructions per clock and SM (measured, 1/74
+// of FP32), so the kernels minimise FP64 instructions per interaction.  Layouts:
+//   * symmetric: each unordered pair once, its force to both bodies (Newton's
+//     third law); the pre-check rides along.  Used where it is predicted faster.
+//     The mixed form (kick_ff.cu) carries coordinates, terms and sums as float
+//     expansions on the FP32 pipe; the FP64 form (kick_sym_kernel, below) takes
+//     21 FP64 instructions per unordered pair;
 //   * tiled (kick_kernel): every ordered pair, one target per thread against
 //     source tiles in shared memory, an (i-tile x j-chunk) grid of equal blocks;
-//     for small N, test particles and the allocation-free entry point, with the
-//     pre-check as its own FP32 pass over i < j (precheck_kernel).
-// Both write compensated partial sums folded in a fixed order by kick_finalize
-// (deterministic).  The rare pairs inside rc_ij are found by an FP32 test on
-// r^2 against a conservative threshold; only those evaluate the changeover
-// function.
+//     for small N and the allocation-free entry point, with the pre-check as its
+//     own FP32 pass over i < j (precheck_kernel).
+// Both write partial sums folded in a fixed order (deterministic).  The rare
+// pairs inside rc_ij are found by an FP32 test on r^2 against a conservative
+// threshold; only those evaluate the changeover function.
 //
-// MIXED: FP64 displacement; r^2 formed as an unevaluated sum of two floats from
-// an exact integer split of the displacement (no FP64 work); FP32 rsqrt seed
+// MIXED, tiled: FP64 displacement; r^2 formed as an unevaluated sum of two floats
+// from an exact integer split of the displacement (no FP64 work); FP32 rsqrt seed
 // y0; one Newton correction from the residual e = 1 - r^2 y0^2 (its leading
 // part 1 - u y0 by an FP32 FMA on the exact float product u y0, rounded once:
 // the float a double residual would be rounded to; the tails in FP32);
 // r^-3 = y0^3 (1 + 1.5 e + 1.875 e^2) = m y0^3 + corr in float-float; FP64
 // accumulation of (m y0^3) dx, the corrections corr dx (< 2^-19 of each term)
 // summed in float-float and added to the FP64 sums with the partials; 6 FP64
-// instructions per ordered pair in the tiled layout (3 subtractions, 3
-// accumulations).  FP64: CUDA's double rsqrt in the tiled layout (17 FP64
-// instructions per pair, counted), the Newton rsqrt of common.cuh in the
-// symmetric one (21 per unordered pair).
+// instructions per ordered pair (3 subtractions, 3 accumulations).  FP64: CUDA's
+// double rsqrt in the tiled layout (17 FP64 instructions per pair, counted), the
+// Newton rsqrt of common.cuh in the symmetric one (21 per unordered pair).
 #include <algorithm>
 #include <queue>
 #include <utility>
 #include <vector>
 
-#include "common.cuh"
+#include "kick_sym.cuh"
 
 namespace genga {
 namespace {
@@ -70,14 +67,6 @@ __device__ __forceinline__ float r2_to_float_trunc(double r2) {
     unsigned lo = (unsigned)__double2loint(r2);
     unsigned fb = (hi >= 0x38100000u) ? (((hi - 0x38000000u) << 3) | (lo >> 29)) : 0u;
     return __uint_as_float(fb);
-}
-
-// 1 / rc: the Newton reciprocal for every rc the FP32 seed can take, an exact
-// division for smaller ones, infinite for rc = 0 (so that min(1/rc_i, 1/rc_j) is
-// 1 / max(rc_i, rc_j) for any pair).
-__device__ __forceinline__ double inv_rc(double rc) {
-    if (rc > 1e-30) return rcp_newton(rc);
-    return rc > 0.0 ? 1.0 / rc : __longlong_as_double(0x7ff0000000000000ll);
 }
 
 // TP: semi-active test particles (Sec. 8.1): a test particle i takes only the
@@ -372,13 +361,13 @@ precheck_kernel(KickArgs A, double f_pc)
 }
 
 // ---------------------------------------------------------------------------
-// Symmetric kick: each unordered pair {i, j} is evaluated once and its force
-// goes to both bodies with opposite signs (Newton's third law): the terms
+// Symmetric kick, FP64 form: each unordered pair {i, j} is evaluated once and its
+// force goes to both bodies with opposite signs (Newton's third law): the terms
 // m_j K r^-3 (x_j - x_i) of a_i and -m_i K r^-3 (x_j - x_i) of a_j share the
-// displacement, r^-3 and K.  FP64 instructions per unordered pair: MIXED 9
-// (3 subtractions, 3 + 3 accumulations), FP64 form 21 (the Newton rsqrt of
-// common.cuh instead of CUDA's double rsqrt) -- per ordered pair 4.5 and 10.5
-// against 6 and ~17 of kick_kernel.
+// displacement, r^-3 and K.  21 FP64 instructions per unordered pair (the Newton
+// rsqrt of common.cuh instead of CUDA's double rsqrt), 10.5 per ordered pair
+// against ~17 of kick_kernel.  The mixed form shares the decomposition, with two
+// warps per block and two bodies j per lane (kick_ff.cu).
 //
 // Work decomposition.  Bodies in tiles of 128 (one per thread of a 4-warp
 // block), tiles in super-ranges of P tiles.  A work item is a super-tile pair
@@ -404,128 +393,44 @@ precheck_kernel(KickArgs A, double f_pc)
 // counter in the host's order (largest first, the diagonal items last); the
 // host picks P for each N by list-scheduling the items over the resident
 // blocks, with the finalize's cost counted.
-constexpr int kSymT = 128;
-constexpr int kSymMaxP = 6;
+// Resident blocks per SM the register allocation must allow (128 threads each).
+constexpr int sym_min_blocks(bool pc) { return pc ? 6 : 4; }
 
-struct SymArgs {
-    const double *x, *y, *z, *m;
-    const double *irc;          // 1 / rc per body (inv_rc)
-    const float2 *ircf;         // MIXED: the same as two floats
-    const float *thr;           // FP32 upper bound of rc^2
-    const float2 *mhl;          // MIXED: mass as an unevaluated sum of two floats
-    int n, nT, P, nItems;
-    int nm;                     // TP: bodies i >= nm are test particles (no pair of two)
-    const int2 *items;          // (X, Y) super-tile pairs, X <= Y, in dispatch order
-    unsigned *ctr;              // dispatch counter, zero at launch
-    double *part;               // [nS][6][n]
-    // fused pre-check (PC): candidates i < j with r^2 < max(pc2_i, pc2_j)
-    const double *pc2;          // (f_pc rc)^2
-    const float *thr_pc;        // FP32 upper bound of pc2 (2^-16 margin)
-    const float2 *pcf;          // pc2 as an unevaluated sum of two floats
-    uint2 *cand;
-    unsigned long long *cand_count;
-    unsigned long long cand_cap;
-};
-
-// Resident blocks per SM the register allocation must allow (128 threads each):
-// 6 (80 registers) for the mixed form and the FP64 form with the pre-check,
-// without spills; the FP64 form without it needs only 72.  (The mixed form
-// also fits 72 registers, 7 blocks, but ran no faster.)
-constexpr int sym_min_blocks(bool mixed, bool pc) {
-    return mixed ? 6 : (pc ? 6 : 4);
+// Dynamic shared memory of the FP64 form: the staged j tile (x, y, z, m, 1/rc;
+// thr), then the item's j sums (x, y, z).
+constexpr size_t sym_smem(int P) {
+    return (size_t)kSymT * (5 * sizeof(double) + sizeof(float)) + (size_t)P * kSymT * 3 * sizeof(double);
 }
 
-// Dynamic shared memory: the staged j tile (x, y, z, m, 1/rc; thr, mh, ml),
-// then the item's j sums (x, y, z; MIXED: float-float corrections).
-constexpr size_t sym_smem(bool mixed, int P) {
-    return (size_t)kSymT * (5 * sizeof(double) + 3 * sizeof(float)) +
-           (size_t)P * kSymT * (3 * sizeof(double) + (mixed ? 6 * sizeof(float) : 0));
-}
-
-// Far-away stand-in position of the k-th padding body of the last tile:
-// distinct for distinct k (no zero separation), massless.
-__device__ __forceinline__ double pad_pos(int k) { return 1.0e15 + 1.0e13 * (double)k; }
-
-__global__ void kick_pack_kernel(const double *m, const double *rc, const double *pc2, int n, double *irc,
-                                 float2 *ircf, float2 *mhl, float *thr_pc, float2 *pcf) {
+__global__ void kick_pack_kernel(const double *rc, const double *pc2, int n, double *irc, float *thr_pc,
+                                 float2 *pcf) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double ir = inv_rc(rc[i]);
-    irc[i] = ir;
-    ircf[i] = ff_of_irc(ir);
+    irc[i] = inv_rc(rc[i]);
     // rounded up, then 2^-16 more: any float r^2 within 2^-23 of an r^2 below
     // pc2 is below it
     thr_pc[i] = fmaxf(__double2float_ru(pc2[i]) * 1.0000153f, 1.17549435e-38f);
     const float ph = __double2float_rn(pc2[i]);
     pcf[i] = make_float2(ph, __double2float_rn(pc2[i] - (double)ph));
-    const float mh = __double2float_rn(m[i]);
-    mhl[i] = make_float2(mh, __double2float_rn(m[i] - (double)mh));
-}
-
-constexpr int kSymPcBuf = 128;                 // per-warp candidate buffer (shared memory)
-
-// Appends a warp's buffered candidates to the global list (one atomic per flush).
-__device__ __forceinline__ void sym_pc_flush(const SymArgs &A, const uint2 *buf, int &cnt, int lane) {
-    __syncwarp();
-    unsigned long long base = 0;
-    if (lane == 0 && cnt) base = atomicAdd(A.cand_count, (unsigned long long)cnt);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    for (int t = lane; t < cnt; t += 32) {
-        const unsigned long long idx = base + (unsigned long long)t;
-        if (idx < A.cand_cap) A.cand[idx] = buf[t];
-    }
-    __syncwarp();
-    cnt = 0;
-}
-
-// One pair's pre-check inside the kick (warp-uniform call).  Lanes with
-// `maybe` decide r^2 < max(pc2_i, pc2_j) from the kick's float r^2 (Rh + Rl,
-// within rel of r^2) against that pc2 as two floats (pc2 = h + l; rounding to
-// nearest is monotone, so the larger pair of floats is the larger pc2): outside
-// a band of width `band` around it the sign of (Rh - h) + (Rl - l) decides, on
-// the FP32 pipe; inside it (never met in practice) the exact FP64 test of
-// precheck_kernel does.  The warp appends its candidates (i < j) to its
-// buffer, flushed when it could overflow on the next step.
-__device__ __forceinline__ void sym_precheck(const SymArgs &A, uint2 *buf, int &pend, int lane, bool maybe,
-                                             int i, int j, double dx, double dy, double dz, float Rh, float Rl,
-                                             float2 pci, float2 pcj, float band) {
-    if (!__any_sync(0xffffffffu, maybe)) return;
-    bool emit = false;
-    if (maybe && i < A.n && j < A.n) {
-        const float2 P = (pci.x > pcj.x || (pci.x == pcj.x && pci.y >= pcj.y)) ? pci : pcj;
-        const float D = (Rh - P.x) + (Rl - P.y);
-        const float w = band * P.x;
-        if (D < -w) emit = true;
-        else if (D > w) emit = false;
-        else emit = dist2_rn(dx, dy, dz) < fmax(A.pc2[i], A.pc2[j]);
-    }
-    const unsigned ball = __ballot_sync(0xffffffffu, emit);
-    if (emit) buf[pend + __popc(ball & ((1u << lane) - 1u))] = make_uint2((unsigned)min(i, j), (unsigned)max(i, j));
-    pend += __popc(ball);
-    if (pend > kSymPcBuf - 32) sym_pc_flush(A, buf, pend, lane);
 }
 
 // PC: the close-encounter pre-check of Appendix A fused into the kick: a pair
 // whose float r^2 (within 2^-23 of r^2) is below max(thr_pc_i, thr_pc_j) takes
 // the exact FP64 test of precheck_kernel (dist2_rn, no contraction) -- the same
 // candidates, found on the FP32/INT pipes the FP64-bound kick leaves idle.
-template <bool MIXED, bool PC, bool TP>
-__global__ void __launch_bounds__(kSymT, sym_min_blocks(MIXED, PC))
+template <bool PC, bool TP>
+__global__ void __launch_bounds__(kSymT, sym_min_blocks(PC))
 kick_sym_kernel(SymArgs A)
 {
     extern __shared__ __align__(16) unsigned char sym_sh[];
     double *sx = reinterpret_cast<double *>(sym_sh);
     double *sy = sx + kSymT, *sz = sy + kSymT, *sm = sz + kSymT, *sirc = sm + kSymT;
-    float2 *sircf = reinterpret_cast<float2 *>(sirc);     // MIXED: 1/rc as two floats
-    float *sthr = reinterpret_cast<float *>(sirc + kSymT);
-    float *smh = sthr + kSymT, *sml = smh + kSymT;
     const int PT = A.P * kSymT;
-    double *jax = reinterpret_cast<double *>(sml + kSymT);
+    double *jax = sirc + kSymT;
     double *jay = jax + PT, *jaz = jay + PT;
-    float *jc = reinterpret_cast<float *>(jaz + PT);      // [6][PT]: x hi, x lo, y hi, y lo, z hi, z lo
+    float *sthr = reinterpret_cast<float *>(jaz + PT);
     __shared__ int s_item;
     __shared__ float sthp[PC ? kSymT : 1];                // thr_pc of the j tile
-    __shared__ float2 spcf[PC ? kSymT : 1];               // pc2 of the j tile as two floats
     __shared__ uint2 pcb[PC ? kSymT / 32 : 1][PC ? kSymPcBuf : 1];
     int pend = 0;                                         // candidates in this warp's buffer
 
@@ -542,31 +447,21 @@ kick_sym_kernel(SymArgs A)
         const int b0 = XY.y * A.P, b1 = min(A.nT, b0 + A.P);
         const bool diag = XY.x == XY.y;
         const int nj = (b1 - b0) * kSymT;
-        for (int e = threadIdx.x; e < nj; e += kSymT) {
-            jax[e] = 0.0; jay[e] = 0.0; jaz[e] = 0.0;
-            if (MIXED)
-#pragma unroll
-                for (int c = 0; c < 6; c++) jc[c * PT + e] = 0.0f;
-        }
+        for (int e = threadIdx.x; e < nj; e += kSymT) jax[e] = jay[e] = jaz[e] = 0.0;
         for (int a = a0; a < a1; a++) {
             const int i = a * kSymT + threadIdx.x;
             const bool valid = i < n;
             double xi, yi, zi, mi = 0.0, irci = 0.0;
-            float thri = 0.0f, mhi = 0.0f, mli = 0.0f, thpi = 0.0f;
-            float2 pcfi = make_float2(0.0f, 0.0f);
-            float2 ircfi = make_float2(0.0f, 0.0f);
+            float thri = 0.0f, thpi = 0.0f;
             if (valid) {
                 xi = A.x[i]; yi = A.y[i]; zi = A.z[i]; mi = A.m[i];
                 thri = A.thr[i];
-                if (MIXED) ircfi = A.ircf[i];
-                else irci = A.irc[i];
-                if (PC) { thpi = A.thr_pc[i]; pcfi = A.pcf[i]; }
-                if (MIXED) { const float2 q = A.mhl[i]; mhi = q.x; mli = q.y; }
+                irci = A.irc[i];
+                if (PC) thpi = A.thr_pc[i];
             } else {
                 xi = yi = zi = pad_pos(threadIdx.x);
             }
             double ax = 0.0, ay = 0.0, az = 0.0;
-            float cxh = 0.0f, cxl = 0.0f, cyh = 0.0f, cyl = 0.0f, czh = 0.0f, czl = 0.0f;
 
             for (int b = diag ? a : b0; b < b1; b++) {
                 __syncthreads();              // the tile buffer is free
@@ -574,17 +469,14 @@ kick_sym_kernel(SymArgs A)
                     const int k = threadIdx.x, j = b * kSymT + k;
                     if (j < n) {
                         sx[k] = A.x[j]; sy[k] = A.y[j]; sz[k] = A.z[j]; sm[k] = A.m[j];
-                        if (MIXED) sircf[k] = A.ircf[j];
-                        else sirc[k] = A.irc[j];
+                        sirc[k] = A.irc[j];
                         sthr[k] = A.thr[j];
-                        if (MIXED) { const float2 q = A.mhl[j]; smh[k] = q.x; sml[k] = q.y; }
-                        if (PC) { sthp[k] = A.thr_pc[j]; spcf[k] = A.pcf[j]; }
+                        if (PC) sthp[k] = A.thr_pc[j];
                     } else {
                         sx[k] = sy[k] = sz[k] = pad_pos(k); sm[k] = 0.0;
-                        if (MIXED) sircf[k] = make_float2(0.0f, 0.0f);
-                        else sirc[k] = 0.0;
-                        sthr[k] = 0.0f; smh[k] = 0.0f; sml[k] = 0.0f;
-                        if (PC) { sthp[k] = 0.0f; spcf[k] = make_float2(0.0f, 0.0f); }
+                        sirc[k] = 0.0;
+                        sthr[k] = 0.0f;
+                        if (PC) sthp[k] = 0.0f;
                     }
                 }
                 __syncthreads();
@@ -597,7 +489,6 @@ kick_sym_kernel(SymArgs A)
                         const int qb = q * 32;
                         // running sums of the j body this lane holds: (lane + t) mod 32 at step t
                         double jx = 0.0, jy = 0.0, jz = 0.0;
-                        float jxh = 0.0f, jxl = 0.0f, jyh = 0.0f, jyl = 0.0f, jzh = 0.0f, jzl = 0.0f;
 #pragma unroll 4
                         for (int t = t0; t < t1; t++) {
                             const int k = qb + ((lane + t) & 31);
@@ -608,126 +499,33 @@ kick_sym_kernel(SymArgs A)
                             const double dx = sx[k] - xi;
                             const double dy = sy[k] - yi;
                             const double dz = sz[k] - zi;
-                            if (MIXED) {
-                                float hx, hy, hz, lx, ly, lz;
-                                split_f64(dx, hx, lx);
-                                split_f64(dy, hy, ly);
-                                split_f64(dz, hz, lz);
-                                const float px = hx * hx, py = hy * hy, pz = hz * hz;
-                                const float pxe = fmaf(hx, hx, -px), pye = fmaf(hy, hy, -py), pze = fmaf(hz, hz, -pz);
-                                const float s1 = px + py, bb1 = s1 - px;
-                                const float e1 = (px - (s1 - bb1)) + (py - bb1);
-                                const float s2 = s1 + pz, bb2 = s2 - s1;
-                                const float e2 = (s1 - (s2 - bb2)) + (pz - bb2);
-                                const float cross = 2.0f * fmaf(hx, lx, fmaf(hy, ly, hz * lz));
-                                const float tail = ((e1 + e2) + (pxe + pye + pze)) + cross;
-                                const float Rh = s2 + tail;
-                                const float Rl = tail - (Rh - s2);
-                                if (PC) sym_precheck(A, pcb[w], pend, lane, !half && Rh < fmaxf(thpi, sthp[k]), i,
-                                                     b * kSymT + k, dx, dy, dz, Rh, Rl, pcfi, spcf[k],
-                                                     9.094947e-13f);          // 2^-40
-
-                                // r^-3 = y0^3 (1 + 1.5 e + 1.875 e^2) as in kick_kernel; the
-                                // mass-free parts are shared by the two sides
-                                const float y0f = rsqrtf(Rh);
-                                const float u = Rh * y0f, ue = fmaf(Rh, y0f, -u);
-                                const float r1 = fmaf(-u, y0f, 1.0f);
-                                const float p = y0f * y0f, pe = fmaf(y0f, y0f, -p);
-                                const float qq = p * y0f;
-                                float qe = fmaf(p, y0f, -qq);
-                                qe = fmaf(pe, y0f, qe);
-                                const float ef = r1 - fmaf(ue, y0f, Rl * p);
-                                float mhj = smh[k], mlj = sml[k], mhI = mhi, mlI = mli;
-                                // changeover band (rare): K in float-float from r = r^2 r^-1,
-                                // 1/rc_ij = min(1/rc_i, 1/rc_j) (as float pairs: rounding is
-                                // monotone), both masses scaled by K -- no FP64 work
-                                if (Rh < fmaxf(thri, sthr[k])) {
-                                    const float2 cj = sircf[k];
-                                    const bool ci = ircfi.x < cj.x || (ircfi.x == cj.x && ircfi.y <= cj.y);
-                                    float Kh, Kl;
-                                    changeover_ff(u, ue, Rl, y0f, ef, ci ? ircfi.x : cj.x, ci ? ircfi.y : cj.y, Kh, Kl);
-                                    ff_mul(mhj, mlj, Kh, Kl);
-                                    ff_mul(mhI, mlI, Kh, Kl);
-                                }
-                                if (half) { mhj = 0.0f; mlj = 0.0f; mhI = 0.0f; mlI = 0.0f; }
-                                const float poly = fmaf(1.875f * ef, ef, 1.5f * ef);
-                                // i side: m_j r^-3 dx
-                                {
-                                    const float ch = qq * mhj;
-                                    float ce = fmaf(qq, mhj, -ch);
-                                    ce = fmaf(qq, mlj, ce);
-                                    ce = fmaf(qe, mhj, ce);
-                                    const float corr = fmaf(ch, poly, ce);
-                                    const double sj = f64_of_f32_any(ch);
-                                    ax = fma(sj, dx, ax);
-                                    ay = fma(sj, dy, ay);
-                                    az = fma(sj, dz, az);
-                                    float_two_sum_acc(cxh, cxl, corr * hx);
-                                    float_two_sum_acc(cyh, cyl, corr * hy);
-                                    float_two_sum_acc(czh, czl, corr * hz);
-                                }
-                                // j side: -m_i r^-3 dx
-                                {
-                                    const float ch = qq * mhI;
-                                    float ce = fmaf(qq, mhI, -ch);
-                                    ce = fmaf(qq, mlI, ce);
-                                    ce = fmaf(qe, mhI, ce);
-                                    const float corr = fmaf(ch, poly, ce);
-                                    const double si = f64_of_f32_any(ch);
-                                    jx = fma(-si, dx, jx);
-                                    jy = fma(-si, dy, jy);
-                                    jz = fma(-si, dz, jz);
-                                    float_two_sum_acc(jxh, jxl, -(corr * hx));
-                                    float_two_sum_acc(jyh, jyl, -(corr * hy));
-                                    float_two_sum_acc(jzh, jzl, -(corr * hz));
-                                }
-                            } else {
-                                const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-                                const float r2f = r2_to_float_trunc(r2);
-                                if (PC) sym_precheck(A, pcb[w], pend, lane, !half && r2f < fmaxf(thpi, sthp[k]), i,
-                                                     b * kSymT + k, dx, dy, dz, r2f, 0.0f, pcfi, spcf[k],
-                                                     9.536743e-07f);          // 2^-20
-
-                                const double yv = rsqrt_newton(r2);
-                                double y3 = (yv * yv) * yv;
-                                if (r2f < fmaxf(thri, sthr[k]))
-                                    y3 *= changeover_fast(r2 * yv, fmin(irci, sirc[k]));
-                                const double sj = half ? 0.0 : sm[k] * y3;
-                                const double si = half ? 0.0 : mi * y3;
-                                ax = fma(sj, dx, ax);
-                                ay = fma(sj, dy, ay);
-                                az = fma(sj, dz, az);
-                                jx = fma(-si, dx, jx);
-                                jy = fma(-si, dy, jy);
-                                jz = fma(-si, dz, jz);
-                            }
+                            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+                            const float r2f = r2_to_float_trunc(r2);
+                            if (PC) sym_precheck(A, pcb[w], pend, lane, !half && r2f < fmaxf(thpi, sthp[k]), i,
+                                                 b * kSymT + k, r2f, 0.0f, 9.536743e-07f);          // 2^-20
+                            const double yv = rsqrt_newton(r2);
+                            double y3 = (yv * yv) * yv;
+                            if (r2f < fmaxf(thri, sthr[k]))
+                                y3 *= changeover_fast(r2 * yv, fmin(irci, sirc[k]));
+                            const double sj = half ? 0.0 : sm[k] * y3;
+                            const double si = half ? 0.0 : mi * y3;
+                            ax = fma(sj, dx, ax);
+                            ay = fma(sj, dy, ay);
+                            az = fma(sj, dz, az);
+                            jx = fma(-si, dx, jx);
+                            jy = fma(-si, dy, jy);
+                            jz = fma(-si, dz, jz);
                             // pass the j sums on: lane L takes over lane L + 1's body
                             const int src = (lane + 1) & 31;
                             jx = __shfl_sync(0xffffffffu, jx, src);
                             jy = __shfl_sync(0xffffffffu, jy, src);
                             jz = __shfl_sync(0xffffffffu, jz, src);
-                            if (MIXED) {
-                                jxh = __shfl_sync(0xffffffffu, jxh, src);
-                                jxl = __shfl_sync(0xffffffffu, jxl, src);
-                                jyh = __shfl_sync(0xffffffffu, jyh, src);
-                                jyl = __shfl_sync(0xffffffffu, jyl, src);
-                                jzh = __shfl_sync(0xffffffffu, jzh, src);
-                                jzl = __shfl_sync(0xffffffffu, jzl, src);
-                            }
                         }
                         // after the last step's hand-over the lane holds body (lane + t1) mod 32
                         const int e = (b - b0) * kSymT + qb + ((lane + t1) & 31);
                         jax[e] += jx;
                         jay[e] += jy;
                         jaz[e] += jz;
-                        if (MIXED) {
-                            float_two_sum_acc(jc[0 * PT + e], jc[1 * PT + e], jxh);
-                            jc[1 * PT + e] += jxl;
-                            float_two_sum_acc(jc[2 * PT + e], jc[3 * PT + e], jyh);
-                            jc[3 * PT + e] += jyl;
-                            float_two_sum_acc(jc[4 * PT + e], jc[5 * PT + e], jzh);
-                            jc[5 * PT + e] += jzl;
-                        }
                     }
                     __syncthreads();          // subtile sums handed to the next warp
                 }
@@ -737,21 +535,14 @@ kick_sym_kernel(SymArgs A)
             if (valid) {
                 double S[3] = {ax, ay, az};
                 double C[3] = {0.0, 0.0, 0.0};
-                if (MIXED) {
-                    C[0] = f64_of_f32_any(cxh) + f64_of_f32_any(cxl);
-                    C[1] = f64_of_f32_any(cyh) + f64_of_f32_any(cyl);
-                    C[2] = f64_of_f32_any(czh) + f64_of_f32_any(czl);
-                }
                 if (diag) {
                     const int e = (a - b0) * kSymT + threadIdx.x;
                     const double J[3] = {jax[e], jay[e], jaz[e]};
 #pragma unroll
                     for (int c = 0; c < 3; c++) {
-                        double t, err;
-                        two_sum(S[c], J[c], t, err);
+                        double t;
+                        two_sum(S[c], J[c], t, C[c]);
                         S[c] = t;
-                        C[c] += err;
-                        if (MIXED) C[c] += f64_of_f32_any(jc[(2 * c) * PT + e]) + f64_of_f32_any(jc[(2 * c + 1) * PT + e]);
                     }
                 }
                 double *pp = A.part + (size_t)(diag ? XY.x : XY.y) * 6 * n;
@@ -771,8 +562,7 @@ kick_sym_kernel(SymArgs A)
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
                     pp[(size_t)c * n + j] = J[c];
-                    pp[(size_t)(3 + c) * n + j] =
-                        MIXED ? f64_of_f32_any(jc[(2 * c) * PT + e]) + f64_of_f32_any(jc[(2 * c + 1) * PT + e]) : 0.0;
+                    pp[(size_t)(3 + c) * n + j] = 0.0;
                 }
             }
         }
@@ -888,15 +678,14 @@ template <bool MIXED>
 SymPlan sym_plan(int n, int nm, int num_sms, int layout, int req_P) {
     SymPlan best;
     const int nT = (n + kSymT - 1) / kSymT;
-    // FP64 instructions per unordered pair (symmetric) and per ordered pair
-    // (kick_kernel), and per partial slot per body in kick_finalize (15 in its
-    // loop; 17 fits the measured fold, which also streams the slots from DRAM)
-    const double c_sym = MIXED ? 9.2 : 21.5, c_old = MIXED ? 6.1 : 17.1, c_fin = 17.0;
-    // fixed work per item, in FP64-instruction equivalents of one block,
-    // fitted to the mixed kick's measured times over P at N = 65,536 and
-    // 65,540; the FP64 form's measured times follow the model without it
-    const double ovh = MIXED ? 7500.0 / (c_sym * kSymT * kSymT) : 0.0;
-    // predicted time in FP64 instructions per SM: kick_kernel at 95 % balance;
+    // SM cycles per unordered pair (symmetric), per ordered pair (kick_kernel)
+    // and per partial slot per body in the fold: mixed 9.1 ms and 47.0 ms at
+    // N = 65,540 (P = 3; tiled), FP64 81.8 and 133 ms
+    const double c_sym = MIXED ? 1.32 : 12.2, c_old = MIXED ? 3.5 : 9.7, c_fin = MIXED ? 7.0 : 9.7;
+    // fixed work per item, in tile pairs (mixed: fits the times over P at N = 16,384,
+    // 65,540 and 131,071, all within 3 % of the best)
+    const double ovh = MIXED ? 0.05 : 0.0;
+    // predicted time in SM cycles: kick_kernel at 95 % balance;
     // the symmetric kick's makespan (tile pairs per block, each block at 1/nb
     // of its SM) plus the finalize's slots
     if (layout == GENGA_KICK_TILED) return best;
@@ -908,9 +697,12 @@ SymPlan sym_plan(int n, int nm, int num_sms, int layout, int req_P) {
         if ((double)nS * 6.0 * n * sizeof(double) > 16.0 * (1ull << 30)) continue;   // partial sums
         if ((double)nS * (nS + 1) / 2 > 4.0e6) continue;                                // host schedule
         int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kick_sym_kernel<MIXED, false, false>, kSymT,
-                                                          sym_smem(MIXED, P)) != cudaSuccess || nb < 1)
-            continue;
+        if (MIXED)
+            nb = sym_ff_blocks_per_sm(P);
+        else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kick_sym_kernel<false, false>, kSymT,
+                                                               sym_smem(P)) != cudaSuccess)
+            nb = 0;
+        if (nb < 1) continue;
         const int slots = nb * num_sms;
         const int R = (nm + P * kSymT - 1) / (P * kSymT);
         const double ms = sym_schedule(nT, P, slots, R, ovh, nullptr);
@@ -953,21 +745,22 @@ cudaError_t kick_reserve(genga_system *s) {
                 GENGA_CUDA_TRY(cudaMemcpy(s->ksym_list, plan.items.data(), sizeof(int2) * plan.items.size(),
                                           cudaMemcpyHostToDevice));
             if (!s->ksym_ctr) GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_ctr, sizeof(unsigned)));
-            if ((size_t)n > s->ksym_body_cap) {
-                if (s->ksym_irc) cudaFree(s->ksym_irc);
-                if (s->ksym_mhl) cudaFree(s->ksym_mhl);
-                if (s->ksym_thrpc) cudaFree(s->ksym_thrpc);
-                if (s->ksym_pcf) cudaFree(s->ksym_pcf);
-                if (s->ksym_ircf) cudaFree(s->ksym_ircf);
-                s->ksym_irc = nullptr; s->ksym_mhl = nullptr; s->ksym_thrpc = nullptr; s->ksym_pcf = nullptr;
-                s->ksym_ircf = nullptr;
+            const size_t np = (size_t)((n + kSymT - 1) / kSymT) * kSymT;      // whole tiles
+            if (np > s->ksym_body_cap) {
+                for (void *q : {(void *)s->ksym_irc, (void *)s->ksym_thrpc, (void *)s->ksym_pcf, (void *)s->ksym_ircf,
+                                (void *)s->ksym_body, (void *)s->ksym_bounds})
+                    if (q) cudaFree(q);
+                s->ksym_irc = nullptr; s->ksym_thrpc = nullptr; s->ksym_pcf = nullptr; s->ksym_ircf = nullptr;
+                s->ksym_body = nullptr; s->ksym_bounds = nullptr;
                 s->ksym_body_cap = 0;
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_irc, sizeof(double) * (size_t)n));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_mhl, sizeof(float2) * (size_t)n));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_thrpc, sizeof(float) * (size_t)n));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_pcf, sizeof(float2) * (size_t)n));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_ircf, sizeof(float2) * (size_t)n));
-                s->ksym_body_cap = (size_t)n;
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_irc, sizeof(double) * np));
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_thrpc, sizeof(float) * np));
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_pcf, sizeof(float2) * np));
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_ircf, sizeof(float2) * np));
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_body, sizeof(float4) * 4 * np));
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_bounds, sizeof(float4) * (kFfBoundBlocks + 1) +
+                                                                            sizeof(double) * (np / kSymT)));
+                s->ksym_body_cap = np;
             }
         }
         s->ksym_n = s->n;
@@ -991,36 +784,43 @@ cudaError_t launch_kick(genga_system *s, double dt_half, bool precheck, double *
     KickArgs A = make_args(s, false);
     const bool mixed = s->p.precision == GENGA_MIXED;
     int nparts = s->kick_nchunk;
+    FfPack ff;
     int tp_first = n, tp_slots = 0;               // bodies from tp_first fold tp_slots partials
     if (s->ksym_P > 0) {
         // symmetric layout; the pre-check, if asked for, rides along
-        kick_pack_kernel<<<(n + 255) / 256, 256, 0, s->stream>>>(s->mass, s->rcl[0].rc, s->rcl[0].pc2, n,
-                                                               s->ksym_irc, s->ksym_ircf, s->ksym_mhl,
-                                                               s->ksym_thrpc, s->ksym_pcf);
-        ++s->launches;
-        GENGA_CUDA_TRY(cudaMemsetAsync(s->ksym_ctr, 0, sizeof(unsigned), s->stream));
-        if (precheck)
-            GENGA_CUDA_TRY(cudaMemsetAsync(&s->ctr->cand_count, 0, sizeof(unsigned long long), s->stream));
         SymArgs S;
         S.x = A.x; S.y = A.y; S.z = A.z; S.m = A.m;
-        S.irc = s->ksym_irc; S.ircf = s->ksym_ircf; S.thr = A.thr_rc; S.mhl = s->ksym_mhl;
+        S.irc = s->ksym_irc; S.ircf = s->ksym_ircf; S.thr = A.thr_rc; S.body = s->ksym_body;
+        S.ff_flags = (const int *)(s->ksym_bounds + kFfBoundBlocks);
+        S.tmass = (const double *)(s->ksym_bounds + kFfBoundBlocks + 1);
         S.n = n; S.nT = (n + kSymT - 1) / kSymT; S.P = s->ksym_P; S.nItems = s->ksym_items;
         S.nm = A.nm;
         S.items = s->ksym_list; S.ctr = s->ksym_ctr; S.part = s->kick_part;
         S.pc2 = s->rcl[0].pc2; S.thr_pc = s->ksym_thrpc; S.pcf = s->ksym_pcf;
         S.cand = s->cand; S.cand_count = &s->ctr->cand_count; S.cand_cap = (unsigned long long)s->cand_cap;
-        const size_t smem = sym_smem(mixed, s->ksym_P);
         const unsigned nb = (unsigned)s->ksym_blocks;
         const bool tp = A.nm < n;
-#define GENGA_SYM_LAUNCH(M, PCK, TPK) kick_sym_kernel<M, PCK, TPK><<<nb, kSymT, smem, s->stream>>>(S)
         if (mixed) {
-            if (tp) { if (precheck) GENGA_SYM_LAUNCH(true, true, true); else GENGA_SYM_LAUNCH(true, false, true); }
-            else { if (precheck) GENGA_SYM_LAUNCH(true, true, false); else GENGA_SYM_LAUNCH(true, false, false); }
+            ff.pos = s->pos; ff.m = s->mass; ff.rc = s->rcl[0].rc; ff.pc2 = S.pc2; ff.n = n; ff.nT = S.nT;
+            ff.bounds = s->ksym_bounds; ff.body = s->ksym_body; ff.ircf = s->ksym_ircf; ff.pcf = s->ksym_pcf;
+            ff.tmass = (double *)(s->ksym_bounds + kFfBoundBlocks + 1);
+            ff.header = (int *)(s->ksym_bounds + kFfBoundBlocks); ff.ctr = s->ksym_ctr;
+            ff.cand_count = precheck ? &s->ctr->cand_count : nullptr;
+            GENGA_CUDA_TRY(launch_ff_pack(ff, s->stream, &s->launches));
+            GENGA_CUDA_TRY(launch_sym_ff(S, precheck, (int)nb, s->stream));
         } else {
-            if (tp) { if (precheck) GENGA_SYM_LAUNCH(false, true, true); else GENGA_SYM_LAUNCH(false, false, true); }
-            else { if (precheck) GENGA_SYM_LAUNCH(false, true, false); else GENGA_SYM_LAUNCH(false, false, false); }
-        }
+            kick_pack_kernel<<<(n + 255) / 256, 256, 0, s->stream>>>(s->rcl[0].rc, S.pc2, n, s->ksym_irc,
+                                                                     s->ksym_thrpc, s->ksym_pcf);
+            ++s->launches;
+            GENGA_CUDA_TRY(cudaMemsetAsync(s->ksym_ctr, 0, sizeof(unsigned), s->stream));
+            if (precheck)
+                GENGA_CUDA_TRY(cudaMemsetAsync(&s->ctr->cand_count, 0, sizeof(unsigned long long), s->stream));
+            const size_t smem = sym_smem(s->ksym_P);
+#define GENGA_SYM_LAUNCH(PCK, TPK) kick_sym_kernel<PCK, TPK><<<nb, kSymT, smem, s->stream>>>(S)
+            if (tp) { if (precheck) GENGA_SYM_LAUNCH(true, true); else GENGA_SYM_LAUNCH(false, true); }
+            else { if (precheck) GENGA_SYM_LAUNCH(true, false); else GENGA_SYM_LAUNCH(false, false); }
 #undef GENGA_SYM_LAUNCH
+        }
         if (tp) {
             tp_first = (int)std::min<int64_t>((int64_t)s->ksym_R * s->ksym_P * kSymT, n);
             tp_slots = s->ksym_R;
@@ -1039,8 +839,12 @@ cudaError_t launch_kick(genga_system *s, double dt_half, bool precheck, double *
     }
     ++s->launches;
     GENGA_CUDA_TRY(cudaGetLastError());
+    if (s->ksym_P > 0 && mixed)
+        return launch_ff_finalize(ff, s->kick_part, nparts, tp_first, tp_slots, s->p.G, dt_half, s->vel, acc_out,
+                                  s->stream, &s->launches);
     kick_finalize<<<(n + 255) / 256, 256, 0, s->stream>>>(s->kick_part, nparts, tp_first, tp_slots, n, s->p.G,
-                                                          dt_half, s->vel, acc_out); ++s->launches;
+                                                          dt_half, s->vel, acc_out);
+    ++s->launches;
     return cudaGetLastError();
 }
 

@@ -1,0 +1,583 @@
+// kick_ff.cu -- the mixed symmetric all-pairs kick: every unordered pair once,
+// in float expansions on the FP32 pipe.
+//
+// GB300 executes 128 FP32 operations per clock and SM against ~1.8 FP64 ones, so
+// 9 FP64 instructions per pair (3 displacements, 6 accumulations) cost 576
+// cycles of a sub-partition per warp of pairs, while the whole pair takes 127
+// to 135 FP32 operations.  Nothing here is less exact for it:
+//   * a coordinate is the sum of three floats on two fixed grids, h (multiples
+//     of 2^-22 S, S a power of two >= every |coordinate|), m (of 2^-45 S) and
+//     the remainder l.  Differences of h and of m are exact, so
+//     h_j - h_i, m_j - m_i, l_j - l_i sum to the displacement with an error of
+//     2^-70 S; a Fast2Sum step gives it as two floats (relative error 2^-49);
+//   * r^2 is the exact sum of the squares in two floats (2^-48), r^-3 =
+//     y^3 (1 + 1.5 e + 1.875 e^2) from the FP32 seed y and its residual
+//     e = 1 - r^2 y^2, in two floats (2^-46);
+//   * the force m_i m_j r^-3 d is formed once, as two floats (exact products by
+//     FMA), and summed for both bodies in two floats by TwoSum; after 16 terms
+//     the sums go to FP64.  A body's sum is divided by its mass in the fold of
+//     the partial sums.  Between two tiles of equal masses each (a disk's
+//     planetesimals) r^-3 d is summed and the product of the masses applied there.
+// What bounds it is the register file: a packed operation reads up to six
+// 32-bit registers per lane and the sub-partition delivers two per cycle
+// (measured: 3 cycles for an FFMA2 of three different registers, 2 for an FADD2),
+// so the choices below save operand reads -- the force formed once for both
+// bodies instead of m_j r^-3 d and m_i r^-3 d, TwoSum instead of an ordered
+// Fast2Sum (whose selects read as much as the three operations they save).
+//
+// Two device flags, set by the packing kernel, take the instance of the pair
+// loop that the unusual inputs need:
+//   * kFfWide: S > 2^18 min_i max_c |x_i| (a body 10^5 times farther out than
+//     another): three parts no longer hold every FP64 position to its last
+//     place, a fourth part is added;
+//   * kFfTwoMass: a massless body, or one 2^-40 of the heaviest: m_j r^-3 d and
+//     m_i r^-3 d are formed apart and nothing is divided.
+//
+// Two pairs per instruction (f32x2): a lane holds one body i and two travelling
+// bodies j (l and l + 32 of a 64-body group).
+#include "ff2.cuh"
+#include "kick_sym.cuh"
+
+namespace genga {
+namespace {
+
+constexpr int kFfThreads = 64;                 // two warps: 64 rows each of the 128-body tile
+constexpr int kFfWide = 1, kFfTwoMass = 2;
+constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2;      // instances of the pair loop
+
+// Chosen by measurement at N = 65,540 (ms per kick): rows per lane 2 (9.5; 1:
+// 10.3 -- the j data and shuffles serve two rows), 2 steps unrolled (1: 9.45, 4:
+// 9.9), 6 blocks per SM by registers (4: 10.2, 7: 9.7).
+constexpr int kFfR = 2;
+constexpr int kFfUnroll = 2;
+constexpr int kFfMinBlocks = 5;
+// Terms summed in floats before the sums go to FP64, and steps between two
+// renormalisations of the float sums: the rounding of the sums' low parts then
+// stays below that of the terms (error of the accelerations of the 16,384-body
+// disk 4.0e-15 of their norm; 32 and none: 6.9e-15; 9 FP64 instructions per pair: 5.5e-15).
+constexpr int kFfFlush = 16, kFfRenorm = 2;
+
+// A tile of 128 bodies: 8 rows of 64 float4.  Entry g * 32 + l of a row holds
+// the bodies l (x, z) and l + 32 (y, w) of group g:
+//   0: h_x h_y   1: h_z m_hi   2: m_x m_y   3: m_z m_lo   4: l_x l_y   5: l_z thr_rc
+//   6: k_x k_y   7: k_z thr_pc
+// (m_hi, m_lo the scaled mass; k the fourth parts of the coordinates).
+constexpr int kFfRow = 64, kFfTile = 8 * kFfRow;
+
+struct IBody {                                 // a lane's row, in both halves: negated coordinates, mass
+    f2 h[3], m[3], l[3];
+    f2 mh, ml;
+    float thr, thp;
+    int i;
+};
+
+__device__ __forceinline__ f2 f2_lo(const float4 &v) { return f2_make(v.x, v.y); }
+__device__ __forceinline__ f2 f2_hi(const float4 &v) { return f2_make(v.z, v.w); }
+
+// One coordinate's displacement as two floats.
+__device__ __forceinline__ void ff_disp(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 nli, f2 &H, f2 &L) {
+    f2 e;
+    f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e);
+    L = f2_add(e, f2_add(lj, nli));
+}
+// The same with the fourth parts.
+__device__ __forceinline__ void ff_disp4(f2 hj, f2 mj, f2 lj, f2 kj, f2 nhi, f2 nmi, f2 nli, f2 nki, f2 &H, f2 &L) {
+    f2 e1, e2, dl, el;
+    f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e1);
+    f2_two_sum(lj, nli, dl, el);
+    f2_two_sum(e1, dl, e1, e2);
+    f2_fast_two_sum(H, e1, H, e1);
+    L = f2_add(e1, f2_add(e2, f2_add(el, f2_add(kj, nki))));
+}
+
+// g w as two floats (g = gh + gl, w + wl)
+__device__ __forceinline__ void ff_coeff(f2 gh, f2 gl, f2 w, f2 wl, f2 &ch, f2 &cl) {
+    ch = f2_mul(gh, w);
+    cl = f2_fma(gh, wl, f2_fma(gl, w, f2_fma(gh, w, f2_neg(ch))));
+}
+// (ch + cl) d as two floats
+__device__ __forceinline__ void ff_term(f2 ch, f2 cl, const f2 (&H)[3], const f2 (&L)[3], f2 (&th)[3], f2 (&te)[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; c++) th[c] = f2_mul(ch, H[c]);
+#pragma unroll
+    for (int c = 0; c < 3; c++) te[c] = f2_fma(ch, H[c], f2_neg(th[c]));
+#pragma unroll
+    for (int c = 0; c < 3; c++) te[c] = f2_fma(ch, L[c], te[c]);
+#pragma unroll
+    for (int c = 0; c < 3; c++) te[c] = f2_fma(cl, H[c], te[c]);
+}
+
+// The changeover function at r^2 = s2 + tail, 1/rc_ij = ih + il: r as two floats
+// from a fresh seed on the normalised r^2 (a small residual, so that r is good
+// to 2^-47), then changeover_ff.
+__device__ __forceinline__ void ff_changeover(float s2, float tail, float ih, float il, float &Kh, float &Kl) {
+    ff_fast2sum(s2, tail);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s2));
+    y = fmaf(0.5f * y, fmaf(-(s2 * y), y, 1.0f), y);
+    const float u = s2 * y, ue = fmaf(s2, y, -u);
+    const float e = fmaf(-u, y, 1.0f) - fmaf(tail, y * y, ue * y);
+    changeover_ff(u, ue, tail, y, e, ih, il, Kh, Kl);
+}
+
+// sum += h + l, in the uniform instance times m_i m_j.
+template <int MODE>
+__device__ __forceinline__ void ff_flush(double &sum, double mm, float h, float l) {
+    const double v = f64_of_f32_any(h) + f64_of_f32_any(l);
+    sum = MODE == kFfUniform ? fma(mm, v, sum) : sum + v;
+}
+
+// 32 steps of 32 kFfR of the warp's rows (from row0 of the tile on) against the
+// 64 bodies of group jb / 64.  kFfGeneral: pairs masked (diagonal subtiles dsub,
+// test particles) and the inputs of the two device flags; the other instances
+// take every pair.  kFfUniform: two tiles of equal masses each, the product mm of
+// the two applied to the sums.
+template <bool PC, int MODE>
+__device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, double *js, double *is, int PT, int e0,
+                                        int jb, int jglob, const IBody (&I)[kFfR], int flags, bool dsub, int row0,
+                                        double mm, uint2 *pcbuf, int &pend, int lane) {
+    constexpr bool GEN = MODE == kFfGeneral;
+    f2 ih[kFfR][3], il[kFfR][3], jh[3], jl[3];
+    const f2 one = f2_dup(1.0f), two = f2_dup(2.0f), c15 = f2_dup(1.5f), c1875 = f2_dup(1.875f);
+    const float4 *group = tile + (jb >> 1);
+#pragma unroll 1
+    for (int tb = 0; tb < 32; tb += kFfFlush) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            jh[c] = jl[c] = 0ull;
+#pragma unroll
+            for (int r = 0; r < kFfR; r++) ih[r][c] = il[r][c] = 0ull;
+        }
+#pragma unroll (kFfUnroll)
+        for (int t = tb; t < tb + kFfFlush; t++) {
+            const int k = (lane + t) & 31;
+            const float4 q0 = group[k], q1 = group[kFfRow + k], q2 = group[2 * kFfRow + k], q3 = group[3 * kFfRow + k],
+                         q4 = group[4 * kFfRow + k], q5 = group[5 * kFfRow + k];
+#pragma unroll
+            for (int r = 0; r < kFfR; r++) {
+                f2 H[3], L[3];
+                bool wx = true, wy = true;         // this lane's two pairs are wanted
+                if (GEN) {
+                    const float4 q6 = group[6 * kFfRow + k], q7 = group[7 * kFfRow + k];
+                    const int i = I[r].i;
+                    const float4 *bi = A.body + (size_t)(i >> 7) * kFfTile + ((i >> 6) & 1) * 32 + lane;
+                    const float4 kp = bi[6 * kFfRow], kq = bi[7 * kFfRow];
+                    const bool up = i & 32;
+                    ff_disp4(f2_lo(q0), f2_lo(q2), f2_lo(q4), f2_lo(q6), I[r].h[0], I[r].m[0], I[r].l[0],
+                             f2_dup(-(up ? kp.y : kp.x)), H[0], L[0]);
+                    ff_disp4(f2_hi(q0), f2_hi(q2), f2_hi(q4), f2_hi(q6), I[r].h[1], I[r].m[1], I[r].l[1],
+                             f2_dup(-(up ? kp.w : kp.z)), H[1], L[1]);
+                    ff_disp4(f2_lo(q1), f2_lo(q3), f2_lo(q5), f2_lo(q7), I[r].h[2], I[r].m[2], I[r].l[2],
+                             f2_dup(-(up ? kq.y : kq.x)), H[2], L[2]);
+                    if (dsub) {                    // every pair of the 64 x 64 diagonal subtile once
+                        const bool tri = t >= 1 && (t < 16 || (t == 16 && lane < 16));
+                        wx = !up && tri;
+                        wy = up ? tri : true;
+                    }
+                    const int j = jglob + k;
+                    wx = wx && !(i >= A.nm && j >= A.nm);
+                    wy = wy && !(i >= A.nm && j + 32 >= A.nm);
+                } else {
+                    ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I[r].h[0], I[r].m[0], I[r].l[0], H[0], L[0]);
+                    ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I[r].h[1], I[r].m[1], I[r].l[1], H[1], L[1]);
+                    ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I[r].h[2], I[r].m[2], I[r].l[2], H[2], L[2]);
+                }
+                // r^2 = s2 + tail
+                f2 s2 = f2_mul(H[0], H[0]), tail = f2_fma(H[0], H[0], f2_neg(s2));
+                f2_acc_mul_pos(s2, tail, H[1], H[1]);
+                f2_acc_mul_pos(s2, tail, H[2], H[2]);
+                tail = f2_fma(two, f2_fma(H[2], L[2], f2_fma(H[1], L[1], f2_mul(H[0], L[0]))), tail);
+                f2_fast_two_sum(s2, tail, s2, tail);
+                if (GEN) {
+                    s2 = f2_select(wx, wy, s2, one);
+                    tail = f2_select(wx, wy, tail, 0ull);
+                }
+                const float2 S = f2_get(s2);
+                if (PC) {
+                    const float4 q7 = group[7 * kFfRow + k];
+                    const float2 T = f2_get(tail);
+                    const bool mx = wx && S.x < fmaxf(I[r].thp, q7.z), my = wy && S.y < fmaxf(I[r].thp, q7.w);
+                    if (__any_sync(0xffffffffu, mx || my)) {
+                        const int j = jglob + k;
+                        sym_precheck(A, pcbuf, pend, lane, mx, I[r].i, j, S.x, T.x, 9.094947e-13f);       // 2^-40
+                        sym_precheck(A, pcbuf, pend, lane, my, I[r].i, j + 32, S.y, T.y, 9.094947e-13f);
+                    }
+                }
+                // r^-3 = w + wl
+                const f2 y = f2_rsqrt(s2);
+                const f2 u = f2_mul(s2, y), ue = f2_fma(s2, y, f2_neg(u));      // s2 y exactly
+                const f2 p = f2_mul(y, y), pe = f2_fma(y, y, f2_neg(p));
+                f2 w = f2_mul(p, y);
+                const f2 qe = f2_fma(pe, y, f2_fma(p, y, f2_neg(w)));
+                const f2 ef = f2_sub(f2_fma(f2_neg(u), y, one), f2_fma(tail, p, f2_mul(ue, y)));
+                f2 wl = f2_fma(w, f2_mul(f2_fma(c1875, ef, c15), ef), qe);
+                f2_fast_two_sum(w, wl, w, wl);
+                // changeover band (rare): K in float-float, 1/rc_ij = min(1/rc_i, 1/rc_j)
+                // (as float pairs: rounding is monotone), r^-3 scaled by K
+                const bool bx = S.x < fmaxf(I[r].thr, q5.z), by = S.y < fmaxf(I[r].thr, q5.w);
+                if (bx || by) {
+                    const float2 ci = A.ircf[I[r].i], T = f2_get(tail);
+                    float2 W = f2_get(w), WL = f2_get(wl);
+#pragma unroll 1
+                    for (int h = 0; h < 2; h++) {
+                        if (!(h ? by : bx)) continue;
+                        const float2 cj = A.ircf[jglob + k + 32 * h];
+                        const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
+                        float Kh, Kl, wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
+                        ff_changeover(h ? S.y : S.x, h ? T.y : T.x, ti ? ci.x : cj.x, ti ? ci.y : cj.y, Kh, Kl);
+                        ff_mul(wh, wlo, Kh, Kl);
+                        if (Kh == 0.0f) wh = wlo = 0.0f;         // also where r^-3 overflows
+                        if (h) { W.y = wh; WL.y = wlo; }
+                        else { W.x = wh; WL.x = wlo; }
+                    }
+                    w = f2_make(W.x, W.y);
+                    wl = f2_make(WL.x, WL.y);
+                }
+                const f2 mjh = f2_hi(q1), mjl = f2_hi(q3);
+                f2 ch, cl, th[3], te[3];
+                if (GEN) {
+                    w = f2_select(wx, wy, w, 0ull);
+                    wl = f2_select(wx, wy, wl, 0ull);
+                }
+                if (GEN && (flags & kFfTwoMass)) {
+                    ff_coeff(mjh, mjl, w, wl, ch, cl);
+                    ff_term(ch, cl, H, L, th, te);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) f2_acc(ih[r][c], il[r][c], th[c], te[c]);
+                    ff_coeff(I[r].mh, I[r].ml, w, wl, ch, cl);
+                    ff_term(ch, cl, H, L, th, te);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) f2_acc_neg(jh[c], jl[c], th[c], te[c]);
+                } else {
+                    if (MODE == kFfUniform) {
+                        ch = w;
+                        cl = wl;
+                    } else {
+                        const f2 mh = I[r].mh, Mh = f2_mul(mh, mjh);             // m_i m_j
+                        const f2 Ml = f2_fma(I[r].ml, mjh, f2_fma(mh, mjl, f2_fma(mh, mjh, f2_neg(Mh))));
+                        ff_coeff(Mh, Ml, w, wl, ch, cl);
+                    }
+                    ff_term(ch, cl, H, L, th, te);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) f2_acc(ih[r][c], il[r][c], th[c], te[c]);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) f2_acc_neg(jh[c], jl[c], th[c], te[c]);
+                }
+            }
+            // the low parts back below the last place of the high ones
+            if (t % kFfRenorm == kFfRenorm - 1) {
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+#pragma unroll
+                    for (int r = 0; r < kFfR; r++) f2_fast_two_sum(ih[r][c], il[r][c], ih[r][c], il[r][c]);
+                    f2_fast_two_sum(jh[c], jl[c], jh[c], jl[c]);
+                }
+            }
+            // pass the j sums on: lane L takes over lane L + 1's bodies
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                jh[c] = f2_shfl(jh[c], (lane + 1) & 31);
+                jl[c] = f2_shfl(jl[c], (lane + 1) & 31);
+            }
+        }
+        // the sums go to FP64; after the hand-overs a lane holds the bodies lane + tb + kFfFlush
+        const int e = e0 + ((lane + tb + kFfFlush) & 31);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const float2 h = f2_get(jh[c]), l = f2_get(jl[c]);
+            ff_flush<MODE>(js[c * PT + e], mm, h.x, l.x);
+            ff_flush<MODE>(js[c * PT + e + 32], mm, h.y, l.y);
+#pragma unroll
+            for (int r = 0; r < kFfR; r++) {
+                const float2 a = f2_get(ih[r][c]), b = f2_get(il[r][c]);
+                float s, x;
+                ff_two_sum(a.x, a.y, s, x);
+                ff_flush<MODE>(is[c * kSymT + row0 + 32 * r + lane], mm, s, x + (b.x + b.y));
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ void ff_load_row(const SymArgs &A, int a, int r, IBody &I) {
+    const float4 *B = A.body + (size_t)a * kFfTile + (r >> 6) * 32 + (r & 31);
+    const bool up = r & 32;
+    const float4 q0 = B[0], q1 = B[kFfRow], q2 = B[2 * kFfRow], q3 = B[3 * kFfRow], q4 = B[4 * kFfRow],
+                 q5 = B[5 * kFfRow];
+    I.i = a * kSymT + r;
+    I.h[0] = f2_dup(-(up ? q0.y : q0.x)); I.h[1] = f2_dup(-(up ? q0.w : q0.z)); I.h[2] = f2_dup(-(up ? q1.y : q1.x));
+    I.m[0] = f2_dup(-(up ? q2.y : q2.x)); I.m[1] = f2_dup(-(up ? q2.w : q2.z)); I.m[2] = f2_dup(-(up ? q3.y : q3.x));
+    I.l[0] = f2_dup(-(up ? q4.y : q4.x)); I.l[1] = f2_dup(-(up ? q4.w : q4.z)); I.l[2] = f2_dup(-(up ? q5.y : q5.x));
+    I.mh = f2_dup(up ? q1.w : q1.z);
+    I.ml = f2_dup(up ? q3.w : q3.z);
+    I.thr = up ? q5.w : q5.z;
+    const float4 q7 = B[7 * kFfRow];
+    I.thp = up ? q7.w : q7.z;
+}
+
+template <bool PC>
+__global__ void __launch_bounds__(kFfThreads, kFfMinBlocks)
+kick_sym_ff_kernel(SymArgs A)
+{
+    extern __shared__ __align__(16) unsigned char ff_sh[];
+    float4 *tile = reinterpret_cast<float4 *>(ff_sh);            // the j tile
+    double *is = reinterpret_cast<double *>(tile + kFfTile);     // [3][kSymT]: the row tile's sums
+    double *js = is + 3 * kSymT;                                 // [3][P * kSymT]: the item's j sums
+    __shared__ int s_item;
+    __shared__ uint2 pcb[PC ? 2 : 1][PC ? kSymPcBuf : 1];
+    int pend = 0;                                                // candidates in this warp's buffer
+
+    const int n = A.n, PT = A.P * kSymT;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int flags = *A.ff_flags;
+    for (;;) {
+        __syncthreads();                       // the previous item's shared sums are written out
+        if (threadIdx.x == 0) s_item = (int)atomicAdd(A.ctr, 1u);
+        __syncthreads();
+        const int it = s_item;
+        if (it >= A.nItems) break;
+        const int2 XY = A.items[it];
+        const int a0 = XY.x * A.P, a1 = min(A.nT, a0 + A.P);
+        const int b0 = XY.y * A.P, b1 = min(A.nT, b0 + A.P);
+        const bool diag = XY.x == XY.y;
+        for (int e = threadIdx.x; e < 3 * PT; e += kFfThreads) js[e] = 0.0;
+        for (int a = a0; a < a1; a++) {
+#pragma unroll
+            for (int c = 0; c < 3; c++)        // a lane's own two rows
+                is[c * kSymT + w * 64 + lane] = is[c * kSymT + w * 64 + 32 + lane] = 0.0;
+            for (int b = diag ? a : b0; b < b1; b++) {
+                __syncthreads();               // the tile buffer is free
+                for (int k = threadIdx.x; k < kFfTile; k += kFfThreads) tile[k] = A.body[(size_t)b * kFfTile + k];
+                __syncthreads();
+                const bool same = a == b;
+                // pairs to mask: the diagonal tile's, and two test particles'
+                const bool gen = flags != 0 || same || ((a + 1) * kSymT > A.nm && (b + 1) * kSymT > A.nm);
+                const double mm = A.tmass[a] * A.tmass[b];
+                for (int s = 0; s < 2; s++) {
+                    const int q = (w + s) & 1;
+                    if (!same || q >= w) {
+                        const bool dsub = same && q == w;
+                        const int jb = q * 64, e0 = (b - b0) * kSymT + jb, jg = b * kSymT + jb;
+#pragma unroll 1
+                        for (int h = 0; h < 64; h += 32 * kFfR) {
+                            IBody I[kFfR];
+#pragma unroll
+                            for (int r = 0; r < kFfR; r++) ff_load_row(A, a, w * 64 + h + 32 * r + lane, I[r]);
+                            if (gen)
+                                ff_rows<PC, kFfGeneral>(A, tile, js, is, PT, e0, jb, jg, I, flags, dsub, w * 64 + h,
+                                                        0.0, pcb[PC ? w : 0], pend, lane);
+                            else if (mm > 0.0)
+                                ff_rows<PC, kFfUniform>(A, tile, js, is, PT, e0, jb, jg, I, 0, false, w * 64 + h, mm,
+                                                        pcb[PC ? w : 0], pend, lane);
+                            else
+                                ff_rows<PC, kFfPlain>(A, tile, js, is, PT, e0, jb, jg, I, 0, false, w * 64 + h, 0.0,
+                                                      pcb[PC ? w : 0], pend, lane);
+                        }
+                    }
+                    __syncthreads();           // group sums handed to the other warp
+                }
+            }
+            // row a done: its sums over the tiles of Y (slot Y), or, in a
+            // diagonal item, with the j sums of tile a, now complete (slot X)
+            double *pp = A.part + (size_t)(diag ? XY.x : XY.y) * 3 * n;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int r = w * 64 + 32 * h + lane, i = a * kSymT + r;
+                if (i >= n) continue;
+#pragma unroll
+                for (int c = 0; c < 3; c++)
+                    pp[(size_t)c * n + i] =
+                        diag ? is[c * kSymT + r] + js[c * PT + (a - b0) * kSymT + r] : is[c * kSymT + r];
+            }
+        }
+        if (!diag) {                           // j sums of the Y tiles: slot X
+            double *pp = A.part + (size_t)XY.x * 3 * n;
+            const int nj = (b1 - b0) * kSymT;
+            for (int e = threadIdx.x; e < nj; e += kFfThreads) {
+                const int j = b0 * kSymT + e;
+                if (j >= n) continue;
+#pragma unroll
+                for (int c = 0; c < 3; c++) pp[(size_t)c * n + j] = js[c * PT + e];
+            }
+        }
+    }
+    if (PC) sym_pc_flush(A, pcb[w], pend, lane);
+}
+
+template <int WARPS>
+__device__ __forceinline__ float4 ff_reduce_bounds(float4 v, float4 *sh) {     // of the block, to all
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        v.x = fmaxf(v.x, __shfl_xor_sync(0xffffffffu, v.x, o));
+        v.y = fminf(v.y, __shfl_xor_sync(0xffffffffu, v.y, o));
+        v.z = fmaxf(v.z, __shfl_xor_sync(0xffffffffu, v.z, o));
+        v.w = fminf(v.w, __shfl_xor_sync(0xffffffffu, v.w, o));
+    }
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < WARPS; k++) {
+        const float4 o = sh[k];
+        v = make_float4(fmaxf(v.x, o.x), fminf(v.y, o.y), fmaxf(v.z, o.z), fminf(v.w, o.w));
+    }
+    return v;
+}
+
+// Per block: largest |coordinate|, smallest (over the bodies) of a body's largest
+// |coordinate|, largest and smallest mass, rounded up resp. down.
+__global__ void __launch_bounds__(256) ff_bounds_kernel(int n, const double *pos, const double *mass, float4 *bounds) {
+    __shared__ float4 sh[8];
+    float4 v = make_float4(0.0f, 3.0e38f, 0.0f, 3.0e38f);
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += 256 * gridDim.x) {
+        const double a = fmax(fabs(pos[i]), fmax(fabs(pos[(size_t)n + i]), fabs(pos[2 * (size_t)n + i])));
+        const double m = fabs(mass[i]);
+        v.x = fmaxf(v.x, __double2float_ru(a));
+        v.y = fminf(v.y, __double2float_rd(a));
+        v.z = fmaxf(v.z, __double2float_ru(m));
+        v.w = fminf(v.w, __double2float_rd(m));
+    }
+    v = ff_reduce_bounds<8>(v, sh);
+    if (threadIdx.x == 0) bounds[blockIdx.x] = v;
+}
+
+// (Scaled) x = h + m + l + k: h a multiple of 2^-22 S, m of 2^-45 S (S = 2^e), l and k
+// floats of the rest.  mag1, mag2: 1.5 2^52 times the two grids' spacing, whose
+// addition rounds a double to a multiple of the spacing.
+__device__ __forceinline__ void ff_split(double x, double mag1, double mag2, float &h, float &m, float &l, float &k) {
+    const double dh = (x + mag1) - mag1, r = x - dh;
+    const double dm = (r + mag2) - mag2, s = r - dm;
+    h = (float)dh;
+    m = (float)dm;
+    l = (float)s;
+    k = (float)(s - (double)l);
+}
+
+// One block per tile.
+__global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
+    __shared__ float4 sh[kSymT / 32];
+    __shared__ double tm;
+    float4 bd = make_float4(0.0f, 3.0e38f, 0.0f, 3.0e38f);
+    for (int k = threadIdx.x; k < nbounds; k += kSymT) {
+        const float4 o = A.bounds[k];
+        bd = make_float4(fmaxf(bd.x, o.x), fminf(bd.y, o.y), fmaxf(bd.z, o.z), fminf(bd.w, o.w));
+    }
+    bd = ff_reduce_bounds<kSymT / 32>(bd, sh);
+    // S = 2^ex > every |coordinate|; lengths are scaled by 2^-es, which puts the
+    // innermost body near 1 (and S at 2^20 at most), masses by 2^-em, so that
+    // the floats' range does not depend on the caller's units
+    const int ex = max(ilogbf(fmaxf(bd.x, 1e-30f)) + 1, -90);
+    const int es = max(ilogbf(fminf(fmaxf(bd.y, 1e-30f), 1e30f)), ex - 20), em = ilogbf(fmaxf(bd.z, 1e-38f));
+    const double mag1 = scalbn(1.5, 52 - 22 + ex - es), mag2 = scalbn(1.5, 52 - 45 + ex - es);
+    const double mscale = scalbn(1.0, -em), xscale = scalbn(1.0, -es);
+    const int i = blockIdx.x * kSymT + threadIdx.x;
+    if (i == 0) {
+        A.header[0] = (scalbnf(1.0f, ex - 18) > bd.y ? kFfWide : 0) | (scalbnf(bd.z, -40) >= bd.w ? kFfTwoMass : 0);
+        A.header[1] = em;
+        A.header[2] = es;
+        *A.ctr = 0u;
+        if (A.cand_count) *A.cand_count = 0ull;
+    }
+    // the common (scaled) mass of a full tile of equal masses, else 0
+    const double ms = i < A.n ? A.m[i] * mscale : 0.0;
+    if (threadIdx.x == 0) tm = ms;
+    __syncthreads();
+    const int differ = __syncthreads_or(ms != tm || !(ms > 0.0));
+    if (threadIdx.x == 0) A.tmass[blockIdx.x] = differ ? 0.0 : ms;
+    float h[3], m[3], l[3], k[3], mh = 0.0f, ml = 0.0f, thr = 0.0f, thp = 0.0f;
+    float2 ircf = make_float2(0.0f, 0.0f), pcf = make_float2(0.0f, 0.0f);
+    if (i < A.n) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) ff_split(A.pos[(size_t)c * A.n + i] * xscale, mag1, mag2, h[c], m[c], l[c], k[c]);
+        const double rc = A.rc[i], rcs = rc * xscale, pc2 = A.pc2[i] * xscale * xscale;
+        mh = __double2float_rn(ms);
+        ml = __double2float_rn(ms - (double)mh);
+        // upper bounds of rc^2 and of pc2: rounded up, then 2^-16 more, so that any
+        // float r^2 within 2^-20 of an r^2 below them is below them
+        thr = fmaxf(__double2float_ru(rcs * rcs) * 1.0000153f, 1.17549435e-38f);
+        thp = fmaxf(__double2float_ru(pc2) * 1.0000153f, 1.17549435e-38f);
+        ircf = ff_of_irc(inv_rc(rc) * scalbn(1.0, es));
+        const float ph = __double2float_rn(pc2);
+        pcf = make_float2(ph, __double2float_rn(pc2 - (double)ph));
+    } else {
+        const float p = (float)pad_pos(i & (kSymT - 1));
+#pragma unroll
+        for (int c = 0; c < 3; c++) { h[c] = p; m[c] = l[c] = k[c] = 0.0f; }
+    }
+    // component of row q, first (0) or second (2) half: + 1 for the bodies l + 32
+    float *B = reinterpret_cast<float *>(A.body + (size_t)(i >> 7) * kFfTile + ((i >> 6) & 1) * 32 + (i & 31)) +
+               ((i >> 5) & 1);
+    constexpr int R = 4 * kFfRow;
+    B[0] = h[0]; B[2] = h[1]; B[R] = h[2]; B[R + 2] = mh;
+    B[2 * R] = m[0]; B[2 * R + 2] = m[1]; B[3 * R] = m[2]; B[3 * R + 2] = ml;
+    B[4 * R] = l[0]; B[4 * R + 2] = l[1]; B[5 * R] = l[2]; B[5 * R + 2] = thr;
+    B[6 * R] = k[0]; B[6 * R + 2] = k[1]; B[7 * R] = k[2]; B[7 * R + 2] = thp;
+    A.ircf[i] = ircf;
+    A.pcf[i] = pcf;
+}
+
+// Folds the partials in slot order (TwoSum), turns forces into accelerations
+// (kFfTwoMass: they are), scales by G and applies the kick v += dt_half a;
+// optionally stores a.  Bodies from tp_first on have tp_slots partials.
+__global__ void ff_finalize_kernel(const double *part, int nslot, int tp_first, int tp_slots, int n, double G,
+                                   const double *mass, const int *header, double dt_half, double *vel,
+                                   double *acc_out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    if (i >= tp_first) nslot = tp_slots;
+    const int em = header[1];
+    double f = G * scalbn(1.0, em - 2 * header[2]);
+    if (!(header[0] & kFfTwoMass)) f /= mass[i] * scalbn(1.0, -em);
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        double S = 0.0, C = 0.0;
+        for (int q = 0; q < nslot; q++) {
+            double t, e;
+            two_sum_ordered(S, part[((size_t)q * 3 + c) * n + i], t, e);
+            S = t;
+            C += e;
+        }
+        const double a = f * (S + C);
+        if (acc_out) acc_out[(size_t)c * n + i] = a;
+        if (dt_half != 0.0) vel[(size_t)c * n + i] += dt_half * a;
+    }
+}
+
+}  // namespace
+
+size_t sym_ff_smem(int P) {
+    return (size_t)kFfTile * sizeof(float4) + (size_t)(P + 1) * kSymT * 3 * sizeof(double);
+}
+
+int sym_ff_blocks_per_sm(int P) {
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kick_sym_ff_kernel<true>, kFfThreads, sym_ff_smem(P)) !=
+        cudaSuccess)
+        return 0;
+    return nb;
+}
+
+cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launches) {
+    const int nb = std::min(kFfBoundBlocks, (k.n + 255) / 256);
+    ff_bounds_kernel<<<nb, 256, 0, stream>>>(k.n, k.pos, k.m, k.bounds);
+    GENGA_CUDA_TRY(cudaGetLastError());
+    ff_pack_kernel<<<k.nT, kSymT, 0, stream>>>(k, nb);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStream_t stream) {
+    const size_t smem = sym_ff_smem(S.P);
+    if (precheck) kick_sym_ff_kernel<true><<<blocks, kFfThreads, smem, stream>>>(S);
+    else kick_sym_ff_kernel<false><<<blocks, kFfThreads, smem, stream>>>(S);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ff_finalize(const FfPack &k, const double *part, int nslot, int tp_first, int tp_slots, double G,
+                               double dt_half, double *vel, double *acc_out, cudaStream_t stream,
+                               int64_t *launches) {
+    ++*launches;
+    ff_finalize_kernel<<<(k.n + 255) / 256, 256, 0, stream>>>(part, nslot, tp_first, tp_slots, k.n, G, k.m, k.header,
+                                                             dt_half, vel, acc_out);
+    return cudaGetLastError();
+}
+
+}  // namespace genga

@@ -144,12 +144,12 @@ struct genga_system {
     size_t ksym_list_cap = 0;
     unsigned *ksym_ctr = nullptr;  // dispatch counter
     double *ksym_irc = nullptr;    // 1 / rc per body
-    float2 *ksym_ircf = nullptr;   // mixed: the same as two floats
-    float4 *ksym_body = nullptr;   // mixed: the bodies as float expansions (kick_ff.cu)
-    float4 *ksym_bounds = nullptr; // mixed: coordinate and mass bounds per block, then the header
     float *ksym_thrpc = nullptr;   // FP32 upper bound of (f_pc rc)^2
-    float2 *ksym_pcf = nullptr;    // (f_pc rc)^2 as two floats
-    size_t ksym_body_cap = 0;      // bodies the arrays above hold (whole tiles)
+    size_t ksym_body_cap = 0;      // bodies the two arrays above hold
+    // the bodies as float expansions (kick_ff.cu): mixed kick, energy
+    void *ff = nullptr;            // one allocation: bodies, 1/rc as two floats, mass per tile,
+                                   // bounds, header
+    size_t ff_tiles = 0;           // tiles it holds
 
     // candidates and encounter lists
     uint2 *cand = nullptr;
@@ -180,8 +180,8 @@ struct genga_system {
     // batched grid-wide Bulirsch-Stoer buffers (bsm.cu), grown on demand
     void *bsm = nullptr;
 
-    // HC / energy reductions
-    double *red = nullptr;   // reduction scratch
+    double *red = nullptr;       // HC's reduction scratch
+    double *en_part = nullptr;   // energy: partial sums (energy.cu), from the first call on
 
     genga::Scratch scr;
     cudaStream_t side[4] = {};     // library-owned streams for concurrent BS buckets
@@ -282,6 +282,8 @@ cudaError_t launch_rcrit_derive(genga_system *s);   // thresholds from rcl[0].rc
 cudaError_t launch_hc(genga_system *s, double dt_half);
 cudaError_t launch_drift(genga_system *s, int level, double dt, const int *bodies, int nb);
 cudaError_t launch_restore(genga_system *s, int from_level, const int *bodies, int nb);
+
+// energy.cu
 cudaError_t launch_energy(genga_system *s, double *E_host, double *L_host);
 
 // kick.cu

@@ -402,22 +402,19 @@ constexpr size_t sym_smem(int P) {
     return (size_t)kSymT * (5 * sizeof(double) + sizeof(float)) + (size_t)P * kSymT * 3 * sizeof(double);
 }
 
-__global__ void kick_pack_kernel(const double *rc, const double *pc2, int n, double *irc, float *thr_pc,
-                                 float2 *pcf) {
+__global__ void kick_pack_kernel(const double *rc, const double *pc2, int n, double *irc, float *thr_pc) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     irc[i] = inv_rc(rc[i]);
     // rounded up, then 2^-16 more: any float r^2 within 2^-23 of an r^2 below
     // pc2 is below it
     thr_pc[i] = fmaxf(__double2float_ru(pc2[i]) * 1.0000153f, 1.17549435e-38f);
-    const float ph = __double2float_rn(pc2[i]);
-    pcf[i] = make_float2(ph, __double2float_rn(pc2[i] - (double)ph));
 }
 
 // PC: the close-encounter pre-check of Appendix A fused into the kick: a pair
 // whose float r^2 (within 2^-23 of r^2) is below max(thr_pc_i, thr_pc_j) takes
-// the exact FP64 test of precheck_kernel (dist2_rn, no contraction) -- the same
-// candidates, found on the FP32/INT pipes the FP64-bound kick leaves idle.
+// the exact FP64 test of precheck_kernel (dist2_rn, no contraction): the same
+// candidates.
 template <bool PC, bool TP>
 __global__ void __launch_bounds__(kSymT, sym_min_blocks(PC))
 kick_sym_kernel(SymArgs A)
@@ -501,8 +498,13 @@ kick_sym_kernel(SymArgs A)
                             const double dz = sz[k] - zi;
                             const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
                             const float r2f = r2_to_float_trunc(r2);
-                            if (PC) sym_precheck(A, pcb[w], pend, lane, !half && r2f < fmaxf(thpi, sthp[k]), i,
-                                                 b * kSymT + k, r2f, 0.0f, 9.536743e-07f);          // 2^-20
+                            if (PC) {
+                                const bool maybe = !half && r2f < fmaxf(thpi, sthp[k]);
+                                if (__any_sync(0xffffffffu, maybe)) {
+                                    sym_pc_push(pcb[w], pend, lane, maybe, i, b * kSymT + k);
+                                    if (pend > kSymPcFlush) sym_pc_flush(A, pcb[w], pend, lane);
+                                }
+                            }
                             const double yv = rsqrt_newton(r2);
                             double y3 = (yv * yv) * yv;
                             if (r2f < fmaxf(thri, sthr[k]))
@@ -745,22 +747,16 @@ cudaError_t kick_reserve(genga_system *s) {
                 GENGA_CUDA_TRY(cudaMemcpy(s->ksym_list, plan.items.data(), sizeof(int2) * plan.items.size(),
                                           cudaMemcpyHostToDevice));
             if (!s->ksym_ctr) GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_ctr, sizeof(unsigned)));
-            const size_t np = (size_t)((n + kSymT - 1) / kSymT) * kSymT;      // whole tiles
-            if (np > s->ksym_body_cap) {
-                for (void *q : {(void *)s->ksym_irc, (void *)s->ksym_thrpc, (void *)s->ksym_pcf, (void *)s->ksym_ircf,
-                                (void *)s->ksym_body, (void *)s->ksym_bounds})
+            if (prec == GENGA_MIXED) {
+                GENGA_CUDA_TRY(ff_reserve(s));
+            } else if ((size_t)n > s->ksym_body_cap) {
+                for (void *q : {(void *)s->ksym_irc, (void *)s->ksym_thrpc})
                     if (q) cudaFree(q);
-                s->ksym_irc = nullptr; s->ksym_thrpc = nullptr; s->ksym_pcf = nullptr; s->ksym_ircf = nullptr;
-                s->ksym_body = nullptr; s->ksym_bounds = nullptr;
+                s->ksym_irc = nullptr; s->ksym_thrpc = nullptr;
                 s->ksym_body_cap = 0;
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_irc, sizeof(double) * np));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_thrpc, sizeof(float) * np));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_pcf, sizeof(float2) * np));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_ircf, sizeof(float2) * np));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_body, sizeof(float4) * 4 * np));
-                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_bounds, sizeof(float4) * (kFfBoundBlocks + 1) +
-                                                                            sizeof(double) * (np / kSymT)));
-                s->ksym_body_cap = np;
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_irc, sizeof(double) * (size_t)n));
+                GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_thrpc, sizeof(float) * (size_t)n));
+                s->ksym_body_cap = (size_t)n;
             }
         }
         s->ksym_n = s->n;
@@ -790,27 +786,25 @@ cudaError_t launch_kick(genga_system *s, double dt_half, bool precheck, double *
         // symmetric layout; the pre-check, if asked for, rides along
         SymArgs S;
         S.x = A.x; S.y = A.y; S.z = A.z; S.m = A.m;
-        S.irc = s->ksym_irc; S.ircf = s->ksym_ircf; S.thr = A.thr_rc; S.body = s->ksym_body;
-        S.ff_flags = (const int *)(s->ksym_bounds + kFfBoundBlocks);
-        S.tmass = (const double *)(s->ksym_bounds + kFfBoundBlocks + 1);
+        S.irc = s->ksym_irc; S.thr = A.thr_rc; S.thr_pc = s->ksym_thrpc;
+        S.ircf = nullptr; S.body = nullptr; S.ff_header = nullptr; S.tmass = nullptr;
         S.n = n; S.nT = (n + kSymT - 1) / kSymT; S.P = s->ksym_P; S.nItems = s->ksym_items;
         S.nm = A.nm;
         S.items = s->ksym_list; S.ctr = s->ksym_ctr; S.part = s->kick_part;
-        S.pc2 = s->rcl[0].pc2; S.thr_pc = s->ksym_thrpc; S.pcf = s->ksym_pcf;
+        S.pc2 = s->rcl[0].pc2;
         S.cand = s->cand; S.cand_count = &s->ctr->cand_count; S.cand_cap = (unsigned long long)s->cand_cap;
         const unsigned nb = (unsigned)s->ksym_blocks;
         const bool tp = A.nm < n;
         if (mixed) {
-            ff.pos = s->pos; ff.m = s->mass; ff.rc = s->rcl[0].rc; ff.pc2 = S.pc2; ff.n = n; ff.nT = S.nT;
-            ff.bounds = s->ksym_bounds; ff.body = s->ksym_body; ff.ircf = s->ksym_ircf; ff.pcf = s->ksym_pcf;
-            ff.tmass = (double *)(s->ksym_bounds + kFfBoundBlocks + 1);
-            ff.header = (int *)(s->ksym_bounds + kFfBoundBlocks); ff.ctr = s->ksym_ctr;
-            ff.cand_count = precheck ? &s->ctr->cand_count : nullptr;
+            ff = ff_pack_args(s);
+            ff.ctr = s->ksym_ctr;
+            if (precheck) ff.cand_count = &s->ctr->cand_count;
+            S.body = ff.body; S.ircf = ff.ircf; S.ff_header = ff.header; S.tmass = ff.tmass;
             GENGA_CUDA_TRY(launch_ff_pack(ff, s->stream, &s->launches));
             GENGA_CUDA_TRY(launch_sym_ff(S, precheck, (int)nb, s->stream));
         } else {
             kick_pack_kernel<<<(n + 255) / 256, 256, 0, s->stream>>>(s->rcl[0].rc, S.pc2, n, s->ksym_irc,
-                                                                     s->ksym_thrpc, s->ksym_pcf);
+                                                                     s->ksym_thrpc);
             ++s->launches;
             GENGA_CUDA_TRY(cudaMemsetAsync(s->ksym_ctr, 0, sizeof(unsigned), s->stream));
             if (precheck)

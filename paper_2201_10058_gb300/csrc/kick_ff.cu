@@ -42,7 +42,6 @@ namespace genga {
 namespace {
 
 constexpr int kFfThreads = 64;                 // two warps: 64 rows each of the 128-body tile
-constexpr int kFfWide = 1, kFfTwoMass = 2;
 constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2;      // instances of the pair loop
 
 // Chosen by measurement at N = 65,540 (ms per kick): rows per lane 2 (9.5; 1:
@@ -57,22 +56,12 @@ constexpr int kFfMinBlocks = 5;
 // disk 4.0e-15 of their norm; 32 and none: 6.9e-15; 9 FP64 instructions per pair: 5.5e-15).
 constexpr int kFfFlush = 16, kFfRenorm = 2;
 
-// A tile of 128 bodies: 8 rows of 64 float4.  Entry g * 32 + l of a row holds
-// the bodies l (x, z) and l + 32 (y, w) of group g:
-//   0: h_x h_y   1: h_z m_hi   2: m_x m_y   3: m_z m_lo   4: l_x l_y   5: l_z thr_rc
-//   6: k_x k_y   7: k_z thr_pc
-// (m_hi, m_lo the scaled mass; k the fourth parts of the coordinates).
-constexpr int kFfRow = 64, kFfTile = 8 * kFfRow;
-
 struct IBody {                                 // a lane's row, in both halves: negated coordinates, mass
     f2 h[3], m[3], l[3];
     f2 mh, ml;
-    float thr, thp;
+    float thr, tn;                             // bounds of r^2: changeover, near pairs
     int i;
 };
-
-__device__ __forceinline__ f2 f2_lo(const float4 &v) { return f2_make(v.x, v.y); }
-__device__ __forceinline__ f2 f2_hi(const float4 &v) { return f2_make(v.z, v.w); }
 
 // One coordinate's displacement as two floats.
 __device__ __forceinline__ void ff_disp(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 nli, f2 &H, f2 &L) {
@@ -120,6 +109,23 @@ __device__ __forceinline__ void ff_changeover(float s2, float tail, float ih, fl
     changeover_ff(u, ue, tail, y, e, ih, il, Kh, Kl);
 }
 
+// A close pair (r < 2^-20 S): its displacement reaches below the second grid, so
+// that h and m no longer give its leading float.  FP64 from the positions, K
+// included: H + L, K r^-3 = w + wl.
+struct FfClose { float H[3], L[3], w, wl; };
+__device__ __forceinline__ void ff_close(const SymArgs &A, int i, int j, float ih, float il, FfClose &o) {
+    const double xs = scalbn(1.0, -A.ff_header[2]);
+    const double d[3] = {(A.x[j] - A.x[i]) * xs, (A.y[j] - A.y[i]) * xs, (A.z[j] - A.z[i]) * xs};
+    const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])), y = rsqrt(r2);
+    const double w = changeover_fast(r2 * y, (double)ih + (double)il) * (y * y * y);
+    for (int c = 0; c < 3; c++) {
+        o.H[c] = __double2float_rn(d[c]);
+        o.L[c] = __double2float_rn(d[c] - (double)o.H[c]);
+    }
+    o.w = __double2float_rn(w);
+    o.wl = __double2float_rn(w - (double)o.w);
+}
+
 // sum += h + l, in the uniform instance times m_i m_j.
 template <int MODE>
 __device__ __forceinline__ void ff_flush(double &sum, double mm, float h, float l) {
@@ -134,7 +140,7 @@ __device__ __forceinline__ void ff_flush(double &sum, double mm, float h, float 
 // the two applied to the sums.
 template <bool PC, int MODE>
 __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, double *js, double *is, int PT, int e0,
-                                        int jb, int jglob, const IBody (&I)[kFfR], int flags, bool dsub, int row0,
+                                        int jb, int jglob, const IBody (&I)[kFfR], int flags, float close2, bool dsub, int row0,
                                         double mm, uint2 *pcbuf, int &pend, int lane) {
     constexpr bool GEN = MODE == kFfGeneral;
     f2 ih[kFfR][3], il[kFfR][3], jh[3], jl[3];
@@ -153,10 +159,14 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
             const int k = (lane + t) & 31;
             const float4 q0 = group[k], q1 = group[kFfRow + k], q2 = group[2 * kFfRow + k], q3 = group[3 * kFfRow + k],
                          q4 = group[4 * kFfRow + k], q5 = group[5 * kFfRow + k];
+            // bounds of the near pairs: pre-check or, without it, changeover
+            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&group[7 * kFfRow + k].z) : make_float2(q5.z, q5.w);
+            f2 H[kFfR][3], L[kFfR][3], w[kFfR], wl[kFfR];
+            float2 S[kFfR], Tl[kFfR];
+            bool want[kFfR][2], near = false;
 #pragma unroll
             for (int r = 0; r < kFfR; r++) {
-                f2 H[3], L[3];
-                bool wx = true, wy = true;         // this lane's two pairs are wanted
+                want[r][0] = want[r][1] = true;    // this lane's two pairs are wanted
                 if (GEN) {
                     const float4 q6 = group[6 * kFfRow + k], q7 = group[7 * kFfRow + k];
                     const int i = I[r].i;
@@ -164,100 +174,121 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                     const float4 kp = bi[6 * kFfRow], kq = bi[7 * kFfRow];
                     const bool up = i & 32;
                     ff_disp4(f2_lo(q0), f2_lo(q2), f2_lo(q4), f2_lo(q6), I[r].h[0], I[r].m[0], I[r].l[0],
-                             f2_dup(-(up ? kp.y : kp.x)), H[0], L[0]);
+                             f2_dup(-(up ? kp.y : kp.x)), H[r][0], L[r][0]);
                     ff_disp4(f2_hi(q0), f2_hi(q2), f2_hi(q4), f2_hi(q6), I[r].h[1], I[r].m[1], I[r].l[1],
-                             f2_dup(-(up ? kp.w : kp.z)), H[1], L[1]);
+                             f2_dup(-(up ? kp.w : kp.z)), H[r][1], L[r][1]);
                     ff_disp4(f2_lo(q1), f2_lo(q3), f2_lo(q5), f2_lo(q7), I[r].h[2], I[r].m[2], I[r].l[2],
-                             f2_dup(-(up ? kq.y : kq.x)), H[2], L[2]);
+                             f2_dup(-(up ? kq.y : kq.x)), H[r][2], L[r][2]);
                     if (dsub) {                    // every pair of the 64 x 64 diagonal subtile once
                         const bool tri = t >= 1 && (t < 16 || (t == 16 && lane < 16));
-                        wx = !up && tri;
-                        wy = up ? tri : true;
+                        want[r][0] = !up && tri;
+                        want[r][1] = up ? tri : true;
                     }
                     const int j = jglob + k;
-                    wx = wx && !(i >= A.nm && j >= A.nm);
-                    wy = wy && !(i >= A.nm && j + 32 >= A.nm);
+                    want[r][0] = want[r][0] && !(i >= A.nm && j >= A.nm);
+                    want[r][1] = want[r][1] && !(i >= A.nm && j + 32 >= A.nm);
                 } else {
-                    ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I[r].h[0], I[r].m[0], I[r].l[0], H[0], L[0]);
-                    ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I[r].h[1], I[r].m[1], I[r].l[1], H[1], L[1]);
-                    ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I[r].h[2], I[r].m[2], I[r].l[2], H[2], L[2]);
+                    ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I[r].h[0], I[r].m[0], I[r].l[0], H[r][0], L[r][0]);
+                    ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I[r].h[1], I[r].m[1], I[r].l[1], H[r][1], L[r][1]);
+                    ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I[r].h[2], I[r].m[2], I[r].l[2], H[r][2], L[r][2]);
                 }
                 // r^2 = s2 + tail
-                f2 s2 = f2_mul(H[0], H[0]), tail = f2_fma(H[0], H[0], f2_neg(s2));
-                f2_acc_mul_pos(s2, tail, H[1], H[1]);
-                f2_acc_mul_pos(s2, tail, H[2], H[2]);
-                tail = f2_fma(two, f2_fma(H[2], L[2], f2_fma(H[1], L[1], f2_mul(H[0], L[0]))), tail);
+                f2 s2 = f2_mul(H[r][0], H[r][0]), tail = f2_fma(H[r][0], H[r][0], f2_neg(s2));
+                f2_acc_mul_pos(s2, tail, H[r][1], H[r][1]);
+                f2_acc_mul_pos(s2, tail, H[r][2], H[r][2]);
+                tail = f2_fma(two, f2_fma(H[r][2], L[r][2], f2_fma(H[r][1], L[r][1], f2_mul(H[r][0], L[r][0]))), tail);
                 f2_fast_two_sum(s2, tail, s2, tail);
                 if (GEN) {
-                    s2 = f2_select(wx, wy, s2, one);
-                    tail = f2_select(wx, wy, tail, 0ull);
+                    s2 = f2_select(want[r][0], want[r][1], s2, one);
+                    tail = f2_select(want[r][0], want[r][1], tail, 0ull);
                 }
-                const float2 S = f2_get(s2);
-                if (PC) {
-                    const float4 q7 = group[7 * kFfRow + k];
-                    const float2 T = f2_get(tail);
-                    const bool mx = wx && S.x < fmaxf(I[r].thp, q7.z), my = wy && S.y < fmaxf(I[r].thp, q7.w);
-                    if (__any_sync(0xffffffffu, mx || my)) {
-                        const int j = jglob + k;
-                        sym_precheck(A, pcbuf, pend, lane, mx, I[r].i, j, S.x, T.x, 9.094947e-13f);       // 2^-40
-                        sym_precheck(A, pcbuf, pend, lane, my, I[r].i, j + 32, S.y, T.y, 9.094947e-13f);
-                    }
-                }
+                S[r] = f2_get(s2);
+                Tl[r] = f2_get(tail);
                 // r^-3 = w + wl
                 const f2 y = f2_rsqrt(s2);
                 const f2 u = f2_mul(s2, y), ue = f2_fma(s2, y, f2_neg(u));      // s2 y exactly
                 const f2 p = f2_mul(y, y), pe = f2_fma(y, y, f2_neg(p));
-                f2 w = f2_mul(p, y);
-                const f2 qe = f2_fma(pe, y, f2_fma(p, y, f2_neg(w)));
+                w[r] = f2_mul(p, y);
+                const f2 qe = f2_fma(pe, y, f2_fma(p, y, f2_neg(w[r])));
                 const f2 ef = f2_sub(f2_fma(f2_neg(u), y, one), f2_fma(tail, p, f2_mul(ue, y)));
-                f2 wl = f2_fma(w, f2_mul(f2_fma(c1875, ef, c15), ef), qe);
-                f2_fast_two_sum(w, wl, w, wl);
-                // changeover band (rare): K in float-float, 1/rc_ij = min(1/rc_i, 1/rc_j)
-                // (as float pairs: rounding is monotone), r^-3 scaled by K
-                const bool bx = S.x < fmaxf(I[r].thr, q5.z), by = S.y < fmaxf(I[r].thr, q5.w);
-                if (bx || by) {
-                    const float2 ci = A.ircf[I[r].i], T = f2_get(tail);
-                    float2 W = f2_get(w), WL = f2_get(wl);
-#pragma unroll 1
-                    for (int h = 0; h < 2; h++) {
-                        if (!(h ? by : bx)) continue;
-                        const float2 cj = A.ircf[jglob + k + 32 * h];
-                        const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
-                        float Kh, Kl, wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
-                        ff_changeover(h ? S.y : S.x, h ? T.y : T.x, ti ? ci.x : cj.x, ti ? ci.y : cj.y, Kh, Kl);
-                        ff_mul(wh, wlo, Kh, Kl);
-                        if (Kh == 0.0f) wh = wlo = 0.0f;         // also where r^-3 overflows
-                        if (h) { W.y = wh; WL.y = wlo; }
-                        else { W.x = wh; WL.x = wlo; }
+                wl[r] = f2_fma(w[r], f2_mul(f2_fma(c1875, ef, c15), ef), qe);
+                f2_fast_two_sum(w[r], wl[r], w[r], wl[r]);
+                near = near || S[r].x < fmaxf(I[r].tn, tj.x) || S[r].y < fmaxf(I[r].tn, tj.y);
+            }
+            if (PC ? __any_sync(0xffffffffu, near) : near) {
+#pragma unroll
+                for (int r = 0; r < kFfR; r++) {
+                    if (PC) {                      // pre-check: the bounds tn include the changeover's
+                        sym_pc_push(pcbuf, pend, lane, want[r][0] && S[r].x < fmaxf(I[r].tn, tj.x), I[r].i, jglob + k);
+                        sym_pc_push(pcbuf, pend, lane, want[r][1] && S[r].y < fmaxf(I[r].tn, tj.y), I[r].i,
+                                    jglob + k + 32);
+                        if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
                     }
-                    w = f2_make(W.x, W.y);
-                    wl = f2_make(WL.x, WL.y);
+                    // changeover band and close pairs: K in float-float, 1/rc_ij = min(1/rc_i, 1/rc_j)
+                    // (as float pairs: rounding is monotone), r^-3 scaled by K
+                    const bool bx = S[r].x < fmaxf(I[r].thr, q5.z), by = S[r].y < fmaxf(I[r].thr, q5.w);
+                    if (bx || by) {
+                        const float2 ci = A.ircf[I[r].i];
+                        float2 W = f2_get(w[r]), WL = f2_get(wl[r]);
+#pragma unroll 1
+                        for (int h = 0; h < 2; h++) {
+                            if (!(h ? by : bx)) continue;
+                            const float2 cj = A.ircf[jglob + k + 32 * h];
+                            const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
+                            const float ih = ti ? ci.x : cj.x, il = ti ? ci.y : cj.y;
+                            float wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
+                            if ((h ? S[r].y : S[r].x) < close2) {
+                                FfClose o;
+                                ff_close(A, I[r].i, jglob + k + 32 * h, ih, il, o);
+#pragma unroll
+                                for (int c = 0; c < 3; c++) {
+                                    const float2 u = f2_get(H[r][c]), v = f2_get(L[r][c]);
+                                    H[r][c] = f2_make(h ? u.x : o.H[c], h ? o.H[c] : u.y);
+                                    L[r][c] = f2_make(h ? v.x : o.L[c], h ? o.L[c] : v.y);
+                                }
+                                wh = o.w;
+                                wlo = o.wl;
+                            } else {
+                                float Kh, Kl;
+                                ff_changeover(h ? S[r].y : S[r].x, h ? Tl[r].y : Tl[r].x, ih, il, Kh, Kl);
+                                ff_mul(wh, wlo, Kh, Kl);
+                                if (Kh == 0.0f) wh = wlo = 0.0f;         // also where r^-3 overflows
+                            }
+                            if (h) { W.y = wh; WL.y = wlo; }
+                            else { W.x = wh; WL.x = wlo; }
+                        }
+                        w[r] = f2_make(W.x, W.y);
+                        wl[r] = f2_make(WL.x, WL.y);
+                    }
                 }
-                const f2 mjh = f2_hi(q1), mjl = f2_hi(q3);
+            }
+            const f2 mjh = f2_hi(q1), mjl = f2_hi(q3);
+#pragma unroll
+            for (int r = 0; r < kFfR; r++) {
                 f2 ch, cl, th[3], te[3];
                 if (GEN) {
-                    w = f2_select(wx, wy, w, 0ull);
-                    wl = f2_select(wx, wy, wl, 0ull);
+                    w[r] = f2_select(want[r][0], want[r][1], w[r], 0ull);
+                    wl[r] = f2_select(want[r][0], want[r][1], wl[r], 0ull);
                 }
                 if (GEN && (flags & kFfTwoMass)) {
-                    ff_coeff(mjh, mjl, w, wl, ch, cl);
-                    ff_term(ch, cl, H, L, th, te);
+                    ff_coeff(mjh, mjl, w[r], wl[r], ch, cl);
+                    ff_term(ch, cl, H[r], L[r], th, te);
 #pragma unroll
                     for (int c = 0; c < 3; c++) f2_acc(ih[r][c], il[r][c], th[c], te[c]);
-                    ff_coeff(I[r].mh, I[r].ml, w, wl, ch, cl);
-                    ff_term(ch, cl, H, L, th, te);
+                    ff_coeff(I[r].mh, I[r].ml, w[r], wl[r], ch, cl);
+                    ff_term(ch, cl, H[r], L[r], th, te);
 #pragma unroll
                     for (int c = 0; c < 3; c++) f2_acc_neg(jh[c], jl[c], th[c], te[c]);
                 } else {
                     if (MODE == kFfUniform) {
-                        ch = w;
-                        cl = wl;
+                        ch = w[r];
+                        cl = wl[r];
                     } else {
                         const f2 mh = I[r].mh, Mh = f2_mul(mh, mjh);             // m_i m_j
                         const f2 Ml = f2_fma(I[r].ml, mjh, f2_fma(mh, mjl, f2_fma(mh, mjh, f2_neg(Mh))));
-                        ff_coeff(Mh, Ml, w, wl, ch, cl);
+                        ff_coeff(Mh, Ml, w[r], wl[r], ch, cl);
                     }
-                    ff_term(ch, cl, H, L, th, te);
+                    ff_term(ch, cl, H[r], L[r], th, te);
 #pragma unroll
                     for (int c = 0; c < 3; c++) f2_acc(ih[r][c], il[r][c], th[c], te[c]);
 #pragma unroll
@@ -298,6 +329,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
     }
 }
 
+template <bool PC>
 __device__ __forceinline__ void ff_load_row(const SymArgs &A, int a, int r, IBody &I) {
     const float4 *B = A.body + (size_t)a * kFfTile + (r >> 6) * 32 + (r & 31);
     const bool up = r & 32;
@@ -311,7 +343,7 @@ __device__ __forceinline__ void ff_load_row(const SymArgs &A, int a, int r, IBod
     I.ml = f2_dup(up ? q3.w : q3.z);
     I.thr = up ? q5.w : q5.z;
     const float4 q7 = B[7 * kFfRow];
-    I.thp = up ? q7.w : q7.z;
+    I.tn = PC ? (up ? q7.w : q7.z) : I.thr;
 }
 
 template <bool PC>
@@ -328,7 +360,8 @@ kick_sym_ff_kernel(SymArgs A)
 
     const int n = A.n, PT = A.P * kSymT;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int flags = *A.ff_flags;
+    const int flags = A.ff_header[0];
+    const float close2 = reinterpret_cast<const float *>(A.ff_header)[3];
     for (;;) {
         __syncthreads();                       // the previous item's shared sums are written out
         if (threadIdx.x == 0) s_item = (int)atomicAdd(A.ctr, 1u);
@@ -361,15 +394,15 @@ kick_sym_ff_kernel(SymArgs A)
                         for (int h = 0; h < 64; h += 32 * kFfR) {
                             IBody I[kFfR];
 #pragma unroll
-                            for (int r = 0; r < kFfR; r++) ff_load_row(A, a, w * 64 + h + 32 * r + lane, I[r]);
+                            for (int r = 0; r < kFfR; r++) ff_load_row<PC>(A, a, w * 64 + h + 32 * r + lane, I[r]);
                             if (gen)
-                                ff_rows<PC, kFfGeneral>(A, tile, js, is, PT, e0, jb, jg, I, flags, dsub, w * 64 + h,
+                                ff_rows<PC, kFfGeneral>(A, tile, js, is, PT, e0, jb, jg, I, flags, close2, dsub, w * 64 + h,
                                                         0.0, pcb[PC ? w : 0], pend, lane);
                             else if (mm > 0.0)
-                                ff_rows<PC, kFfUniform>(A, tile, js, is, PT, e0, jb, jg, I, 0, false, w * 64 + h, mm,
+                                ff_rows<PC, kFfUniform>(A, tile, js, is, PT, e0, jb, jg, I, 0, close2, false, w * 64 + h, mm,
                                                         pcb[PC ? w : 0], pend, lane);
                             else
-                                ff_rows<PC, kFfPlain>(A, tile, js, is, PT, e0, jb, jg, I, 0, false, w * 64 + h, 0.0,
+                                ff_rows<PC, kFfPlain>(A, tile, js, is, PT, e0, jb, jg, I, 0, close2, false, w * 64 + h, 0.0,
                                                       pcb[PC ? w : 0], pend, lane);
                         }
                     }
@@ -468,12 +501,14 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     const int es = max(ilogbf(fminf(fmaxf(bd.y, 1e-30f), 1e30f)), ex - 20), em = ilogbf(fmaxf(bd.z, 1e-38f));
     const double mag1 = scalbn(1.5, 52 - 22 + ex - es), mag2 = scalbn(1.5, 52 - 45 + ex - es);
     const double mscale = scalbn(1.0, -em), xscale = scalbn(1.0, -es);
+    const float close2 = scalbnf(1.0f, 2 * (ex - es - 20));      // (2^-20 S)^2
     const int i = blockIdx.x * kSymT + threadIdx.x;
     if (i == 0) {
         A.header[0] = (scalbnf(1.0f, ex - 18) > bd.y ? kFfWide : 0) | (scalbnf(bd.z, -40) >= bd.w ? kFfTwoMass : 0);
         A.header[1] = em;
         A.header[2] = es;
-        *A.ctr = 0u;
+        reinterpret_cast<float *>(A.header)[3] = close2;
+        if (A.ctr) *A.ctr = 0u;
         if (A.cand_count) *A.cand_count = 0ull;
     }
     // the common (scaled) mass of a full tile of equal masses, else 0
@@ -483,20 +518,19 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     const int differ = __syncthreads_or(ms != tm || !(ms > 0.0));
     if (threadIdx.x == 0) A.tmass[blockIdx.x] = differ ? 0.0 : ms;
     float h[3], m[3], l[3], k[3], mh = 0.0f, ml = 0.0f, thr = 0.0f, thp = 0.0f;
-    float2 ircf = make_float2(0.0f, 0.0f), pcf = make_float2(0.0f, 0.0f);
+    float2 ircf = make_float2(0.0f, 0.0f);
     if (i < A.n) {
 #pragma unroll
         for (int c = 0; c < 3; c++) ff_split(A.pos[(size_t)c * A.n + i] * xscale, mag1, mag2, h[c], m[c], l[c], k[c]);
         const double rc = A.rc[i], rcs = rc * xscale, pc2 = A.pc2[i] * xscale * xscale;
         mh = __double2float_rn(ms);
         ml = __double2float_rn(ms - (double)mh);
-        // upper bounds of rc^2 and of pc2: rounded up, then 2^-16 more, so that any
-        // float r^2 within 2^-20 of an r^2 below them is below them
-        thr = fmaxf(__double2float_ru(rcs * rcs) * 1.0000153f, 1.17549435e-38f);
-        thp = fmaxf(__double2float_ru(pc2) * 1.0000153f, 1.17549435e-38f);
+        // upper bounds of rc^2 and pc2, and of the close pairs' r^2: rounded up,
+        // then 2^-16 more, so that any float r^2 within 2^-20 of an r^2 below
+        // them is below them
+        thr = fmaxf(__double2float_ru(rcs * rcs), close2) * 1.0000153f;
+        thp = fmaxf(__double2float_ru(pc2) * 1.0000153f, thr);
         ircf = ff_of_irc(inv_rc(rc) * scalbn(1.0, es));
-        const float ph = __double2float_rn(pc2);
-        pcf = make_float2(ph, __double2float_rn(pc2 - (double)ph));
     } else {
         const float p = (float)pad_pos(i & (kSymT - 1));
 #pragma unroll
@@ -511,7 +545,6 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     B[4 * R] = l[0]; B[4 * R + 2] = l[1]; B[5 * R] = l[2]; B[5 * R + 2] = thr;
     B[6 * R] = k[0]; B[6 * R + 2] = k[1]; B[7 * R] = k[2]; B[7 * R + 2] = thp;
     A.ircf[i] = ircf;
-    A.pcf[i] = pcf;
 }
 
 // Folds the partials in slot order (TwoSum), turns forces into accelerations
@@ -553,6 +586,37 @@ int sym_ff_blocks_per_sm(int P) {
         cudaSuccess)
         return 0;
     return nb;
+}
+
+// Layout of the packed-body allocation: the arrays in this order, each a whole
+// number of float4 per tile (but the bounds and the header, at the end).
+cudaError_t ff_reserve(genga_system *s) {
+    const size_t nT = (size_t)((s->n + kSymT - 1) / kSymT);
+    if (nT <= s->ff_tiles) return cudaSuccess;
+    if (s->ff) cudaFree(s->ff);
+    s->ff = nullptr;
+    s->ff_tiles = 0;
+    const size_t bytes = nT * (sizeof(float4) * kFfTile + sizeof(float2) * kSymT + sizeof(float4)) +
+                         sizeof(float4) * (kFfBoundBlocks + 1);
+    GENGA_CUDA_TRY(cudaMalloc(&s->ff, bytes));
+    s->ff_tiles = nT;
+    return cudaSuccess;
+}
+
+FfPack ff_pack_args(const genga_system *s) {
+    FfPack k;
+    const size_t nT = s->ff_tiles;
+    k.pos = s->pos; k.m = s->mass; k.rc = s->rcl[0].rc; k.pc2 = s->rcl[0].pc2;
+    k.n = (int)s->n;
+    k.nT = (int)((s->n + kSymT - 1) / kSymT);
+    k.body = (float4 *)s->ff;
+    k.ircf = (float2 *)(k.body + nT * kFfTile);
+    k.tmass = (double *)(k.ircf + nT * kSymT);
+    k.bounds = (float4 *)(k.tmass + 2 * nT);
+    k.header = (int *)(k.bounds + kFfBoundBlocks);
+    k.ctr = nullptr;
+    k.cand_count = nullptr;
+    return k;
 }
 
 cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launches) {

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "ff2.cuh"
 
 namespace genga {
 
@@ -16,7 +17,7 @@ struct SymArgs {
     const float *thr;           // FP64: upper bound of rc^2
     const float4 *body;         // mixed: the bodies as float expansions, by tiles (kick_ff.cu)
     const float2 *ircf;         // mixed: 1 / rc as two floats, padded to whole tiles
-    const int *ff_flags;        // mixed: device flags of the inputs (kick_ff.cu)
+    const int *ff_header;       // mixed: header of the packed bodies
     const double *tmass;        // mixed: per tile, the bodies' common scaled mass, or 0
     int n, nT, P, nItems;
     int nm;                     // bodies i >= nm are test particles (no pair of two); n: none
@@ -26,25 +27,49 @@ struct SymArgs {
     // fused pre-check (PC): candidates i < j with r^2 < max(pc2_i, pc2_j)
     const double *pc2;          // (f_pc rc)^2
     const float *thr_pc;        // FP64: upper bound of pc2 (2^-16 margin)
-    const float2 *pcf;          // pc2 as an unevaluated sum of two floats, padded to whole tiles
     uint2 *cand;
     unsigned long long *cand_count;
     unsigned long long cand_cap;
 };
 
-constexpr int kSymPcBuf = 128;                 // per-warp candidate buffer (shared memory)
-
 // Far-away stand-in position of the k-th padding body of the last tile:
 // distinct for distinct k (no zero separation), massless.
 __device__ __forceinline__ double pad_pos(int k) { return 1.0e15 + 1.0e13 * (double)k; }
 
-// Appends a warp's buffered candidates to the global list (one atomic per flush).
-__device__ __forceinline__ void sym_pc_flush(const SymArgs &A, const uint2 *buf, int &cnt, int lane) {
+// The fused pre-check.  A pair whose float r^2 is below an upper bound of max(pc2_i,
+// pc2_j) (2^-16 margin: no candidate is missed) goes to its warp's buffer in
+// shared memory, and the whole warp decides a buffer of them at once by the exact
+// FP64 test of precheck_kernel.  (Deciding each pair where it is met, from float
+// copies of pc2, took 6 ms of the 65,540-body kick's 15: a third of the steps
+// meet one, and each waited for its loads.)
+constexpr int kSymPcBuf = 128;                 // entries per warp
+constexpr int kSymPcFlush = kSymPcBuf - 64;    // decided when more than this are held
+
+// Decides the warp's buffered pairs; the candidates go to the global list (one
+// atomic per call).
+__device__ __forceinline__ void sym_pc_flush(const SymArgs &A, uint2 *buf, int &cnt, int lane) {
+    __syncwarp();
+    int kept = 0;
+    for (int t0 = 0; t0 < cnt; t0 += 32) {
+        const int t = t0 + lane;
+        uint2 q = make_uint2(0u, 0u);
+        bool emit = false;
+        if (t < cnt) {
+            q = buf[t];
+            const int i = (int)q.x, j = (int)q.y;
+            if (i < A.n && j < A.n)
+                emit = dist2_rn(A.x[j] - A.x[i], A.y[j] - A.y[i], A.z[j] - A.z[i]) < fmax(A.pc2[i], A.pc2[j]);
+        }
+        const unsigned ball = __ballot_sync(0xffffffffu, emit);
+        __syncwarp();                          // all read their entries before any is overwritten
+        if (emit) buf[kept + __popc(ball & ((1u << lane) - 1u))] = make_uint2(min(q.x, q.y), max(q.x, q.y));
+        kept += __popc(ball);
+    }
     __syncwarp();
     unsigned long long base = 0;
-    if (lane == 0 && cnt) base = atomicAdd(A.cand_count, (unsigned long long)cnt);
+    if (lane == 0 && kept) base = atomicAdd(A.cand_count, (unsigned long long)kept);
     base = __shfl_sync(0xffffffffu, base, 0);
-    for (int t = lane; t < cnt; t += 32) {
+    for (int t = lane; t < kept; t += 32) {
         const unsigned long long idx = base + (unsigned long long)t;
         if (idx < A.cand_cap) A.cand[idx] = buf[t];
     }
@@ -52,32 +77,22 @@ __device__ __forceinline__ void sym_pc_flush(const SymArgs &A, const uint2 *buf,
     cnt = 0;
 }
 
-// One pair's pre-check inside the kick (warp-uniform call).  Lanes with
-// `maybe` decide r^2 < max(pc2_i, pc2_j) from the kick's float r^2 (Rh + Rl,
-// within rel of r^2) against that pc2 as two floats (pc2 = h + l; rounding to
-// nearest is monotone, so the larger pair of floats is the larger pc2): outside
-// a band of width `band` around it the sign of (Rh - h) + (Rl - l) decides, on
-// the FP32 pipe; inside it (never met in practice) the exact FP64 test of
-// precheck_kernel does.  The warp appends its candidates (i < j) to its
-// buffer, flushed when it could overflow on the next step.
-__device__ __forceinline__ void sym_precheck(const SymArgs &A, uint2 *buf, int &pend, int lane, bool maybe,
-                                             int i, int j, float Rh, float Rl, float band) {
-    if (!__any_sync(0xffffffffu, maybe)) return;
-    bool emit = false;
-    if (maybe && i < A.n && j < A.n) {
-        const float2 pci = A.pcf[i], pcj = A.pcf[j];
-        const float2 P = (pci.x > pcj.x || (pci.x == pcj.x && pci.y >= pcj.y)) ? pci : pcj;
-        const float D = (Rh - P.x) + (Rl - P.y);
-        const float w = band * P.x;
-        if (D < -w) emit = true;
-        else if (D > w) emit = false;
-        else emit = dist2_rn(A.x[j] - A.x[i], A.y[j] - A.y[i], A.z[j] - A.z[i]) < fmax(A.pc2[i], A.pc2[j]);
-    }
-    const unsigned ball = __ballot_sync(0xffffffffu, emit);
-    if (emit) buf[pend + __popc(ball & ((1u << lane) - 1u))] = make_uint2((unsigned)min(i, j), (unsigned)max(i, j));
-    pend += __popc(ball);
-    if (pend > kSymPcBuf - 32) sym_pc_flush(A, buf, pend, lane);
+// Appends the pairs (i, j) of the lanes with `maybe` (warp-uniform call).
+__device__ __forceinline__ void sym_pc_push(uint2 *buf, int &cnt, int lane, bool maybe, int i, int j) {
+    const unsigned ball = __ballot_sync(0xffffffffu, maybe);
+    if (maybe) buf[cnt + __popc(ball & ((1u << lane) - 1u))] = make_uint2((unsigned)i, (unsigned)j);
+    cnt += __popc(ball);
 }
+
+// The bodies as float expansions (kick_ff.cu).  A tile of 128 bodies: 8 rows of 64 float4.  Entry g * 32 + l of a row holds
+// the bodies l (x, z) and l + 32 (y, w) of group g:
+//   0: h_x h_y   1: h_z m_hi   2: m_x m_y   3: m_z m_lo   4: l_x l_y   5: l_z thr_rc
+//   6: k_x k_y   7: k_z thr_pc
+// (m_hi, m_lo the scaled mass; k the fourth parts of the coordinates).
+constexpr int kFfRow = 64, kFfTile = 8 * kFfRow;
+constexpr int kFfWide = 1, kFfTwoMass = 2;     // flags of the packed bodies, see kick_ff.cu
+__device__ __forceinline__ f2 f2_lo(const float4 &v) { return f2_make(v.x, v.y); }
+__device__ __forceinline__ f2 f2_hi(const float4 &v) { return f2_make(v.z, v.w); }
 
 // kick_ff.cu: the mixed form.
 // Bytes of dynamic shared memory of the mixed kernel for super-range P, and the
@@ -92,12 +107,15 @@ struct FfPack {
     int n, nT;
     float4 *bounds;                   // scratch, kFfBoundBlocks entries
     float4 *body;                     // 4 float4 per body, whole tiles
-    float2 *ircf, *pcf;
+    float2 *ircf;
     double *tmass;                    // per tile
-    int *header;                      // flags, the exponents masses and lengths are scaled by
-    unsigned *ctr;
+    int *header;                      // flags, exponents masses and lengths are scaled by, close r^2 (float)
+    unsigned *ctr;                    // NULL: left alone
     unsigned long long *cand_count;   // NULL: left alone
 };
+// Makes sure the system's packed-body arrays hold its bodies, and their addresses.
+cudaError_t ff_reserve(genga_system *s);
+FfPack ff_pack_args(const genga_system *s);
 cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launches);
 cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStream_t stream);
 cudaError_t launch_ff_finalize(const FfPack &k, const double *part, int nslot, int tp_first, int tp_slots, double G,

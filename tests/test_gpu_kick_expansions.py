@@ -67,12 +67,17 @@ def _inputs(case, n):
     elif case == "test particles":
         nm = n // 3
         m[nm:] *= 1e-4
+    elif case == "close pairs":
+        k = n // 2
+        x[n - k:] = x[:k] + 10.0 ** rng.uniform(-9, -3, (k, 1)) * rng.standard_normal((k, 3))
     rc = O.rcrit(x, v, m, wl.m_star if scale == 1.0 else 1.98847e30, wl.dt, wl.n1, wl.n2)
+    if case == "close pairs":
+        rc[::2] = 0.0                          # K = 1 between half of the bodies
     return x * scale, v, m, rc * scale, nm
 
 
 CASES = ["equal masses", "mixed masses", "one embryo", "massless", "very light", "outlier", "far outlier",
-         "metres and kilograms", "test particles"]
+         "metres and kilograms", "test particles", "close pairs"]
 
 
 @pytest.mark.parametrize("n,P", [(5, 1), (128, 1), (129, 1), (700, 2)])

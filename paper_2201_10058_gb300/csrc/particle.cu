@@ -1,7 +1,6 @@
 // particle.cu -- per-body kernels of the hybrid step (Appendix A): Rcrit
 // (Eq. rcrit), HC (Eq. Hc), FG (Kepler part of Eq. Ha) with the pre-drift copy,
-// the level restore of the higher-level scheme (Sec. 6.3), and the energy /
-// angular-momentum report (Eq. H).
+// and the level restore of the higher-level scheme (Sec. 6.3).
 //
 // These kernels are memory/latency bound (a few hundred bytes per body); they
 // use one thread per body, coalesced SoA loads and no shared memory.  FG runs
@@ -152,82 +151,6 @@ __global__ void restore_kernel(int n, double *pos, double *vel, const double *pr
     }
 }
 
-// ---------------------------------------------------------------- energy
-// Per body: kinetic, star potential, half of the pair potential (all j != i),
-// angular momentum and momentum; then a fixed-order compensated reduction.
-constexpr int kEnThreads = 128;
-constexpr int kEnTile = 256;
-
-__global__ void __launch_bounds__(kEnThreads)
-energy_terms_kernel(int n, int nm, const double *pos, const double *vel, const double *mass, double G,
-                    double m_star, double *terms /* [8][n] */) {
-    __shared__ double sx[kEnTile], sy[kEnTile], sz[kEnTile], sm[kEnTile];
-    const int i = blockIdx.x * kEnThreads + threadIdx.x;
-    const size_t N = (size_t)n;
-    const bool valid = i < n;
-    double xi = 0, yi = 0, zi = 0;
-    if (valid) { xi = pos[i]; yi = pos[N + i]; zi = pos[2 * N + i]; }
-    double S = 0.0, C = 0.0;
-    const int jlim = i >= nm ? nm : n;     // a test particle has no pair term with another
-    for (int jt = 0; jt < n; jt += kEnTile) {
-        const int cnt = min(kEnTile, n - jt);
-        __syncthreads();
-        for (int k = threadIdx.x; k < cnt; k += kEnThreads) {
-            sx[k] = pos[jt + k]; sy[k] = pos[N + jt + k]; sz[k] = pos[2 * N + jt + k]; sm[k] = mass[jt + k];
-        }
-        __syncthreads();
-        double part = 0.0;
-        for (int k = 0; k < cnt; k++) {
-            if (jt + k == i || jt + k >= jlim) continue;
-            const double dx = sx[k] - xi, dy = sy[k] - yi, dz = sz[k] - zi;
-            part += sm[k] / sqrt(dx * dx + dy * dy + dz * dz);
-        }
-        double t, e;
-        two_sum(S, part, t, e); S = t; C += e;
-    }
-    if (!valid) return;
-    const double m = mass[i];
-    const double vx = vel[i], vy = vel[N + i], vz = vel[2 * N + i];
-    const double r = sqrt(xi * xi + yi * yi + zi * zi);
-    terms[0 * N + i] = 0.5 * m * (vx * vx + vy * vy + vz * vz);
-    terms[1 * N + i] = -G * m_star * m / r;
-    terms[2 * N + i] = -0.5 * G * m * (S + C);
-    terms[3 * N + i] = m * (yi * vz - zi * vy);
-    terms[4 * N + i] = m * (zi * vx - xi * vz);
-    terms[5 * N + i] = m * (xi * vy - yi * vx);
-    terms[6 * N + i] = m * vx;
-    terms[7 * N + i] = m * vy;
-    terms[8 * N + i] = m * vz;
-}
-
-// One block per row: compensated fixed-order sum of terms[row][0..n).
-__global__ void row_sum_kernel(int n, const double *terms, int rows, double *out) {
-    __shared__ double ss[256], sc[256];
-    const int row = blockIdx.x;
-    const double *t = terms + (size_t)row * n;
-    double S = 0.0, C = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) {
-        double a, e;
-        two_sum(S, t[i], a, e); S = a; C += e;
-    }
-    ss[threadIdx.x] = S; sc[threadIdx.x] = C;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S2 = 0.0, C2 = 0.0;
-        for (int k = 0; k < 256; k++) {
-            double a, e;
-            two_sum(S2, ss[k], a, e); S2 = a; C2 += e + sc[k];
-        }
-        out[row] = S2 + C2;
-    }
-}
-
-// E = (kinetic + star + pairs) + |P|^2 / (2 m_star); L as summed.
-__global__ void energy_combine_kernel(double m_star, double *sums) {
-    const double P2 = sums[6] * sums[6] + sums[7] * sums[7] + sums[8] * sums[8];
-    sums[9] = ((sums[0] + sums[1]) + sums[2]) + P2 / (2.0 * m_star);
-}
-
 }  // namespace
 
 cudaError_t launch_rcrit(genga_system *s, int level, double dt, const int *bodies, int nb) {
@@ -268,25 +191,6 @@ cudaError_t launch_restore(genga_system *s, int from_level, const int *bodies, i
     restore_kernel<<<(nb + 255) / 256, 256, 0, s->stream>>>((int)s->n, s->pos, s->vel,
         s->pre_pos[from_level], s->pre_vel[from_level], bodies, nb); ++s->launches;
     return cudaGetLastError();
-}
-
-cudaError_t launch_energy(genga_system *s, double *E_host, double *L_host) {
-    const int n = (int)s->n;
-    double *terms = s->red;            // 9 rows of n, then 10 sums
-    energy_terms_kernel<<<(n + kEnThreads - 1) / kEnThreads, kEnThreads, 0, s->stream>>>(
-        n, tp_bound(s), s->pos, s->vel, s->mass, s->p.G, s->p.m_star, terms); ++s->launches;
-    GENGA_CUDA_TRY(cudaGetLastError());
-    double *sums = terms + 9 * (size_t)n;
-    row_sum_kernel<<<9, 256, 0, s->stream>>>(n, terms, 9, sums); ++s->launches;
-    GENGA_CUDA_TRY(cudaGetLastError());
-    energy_combine_kernel<<<1, 1, 0, s->stream>>>(s->p.m_star, sums); ++s->launches;
-    GENGA_CUDA_TRY(cudaGetLastError());
-    double h[10];
-    GENGA_CUDA_TRY(cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
-    GENGA_CUDA_TRY(cudaStreamSynchronize(s->stream));
-    *E_host = h[9];
-    L_host[0] = h[3]; L_host[1] = h[4]; L_host[2] = h[5];
-    return cudaSuccess;
 }
 
 }  // namespace genga

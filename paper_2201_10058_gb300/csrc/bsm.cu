@@ -15,8 +15,8 @@
 //              terms to the pair's partner-list entries, which the sub-step
 //              then sums per member (the same values, in the same order);
 //   Neville    per (component, member): the extrapolation table, its
-//              diagonal, and each column's error folded into the group's 8
-//              error words (atomic max on the bits of non-negative doubles);
+//              diagonal, and the columns whose error is above tolerance as bits
+//              of the group's word;
 //   decide     one thread per group: first column k >= 1 under tolerance
 //              -> accept (grow H by 1.5 if k < 4), else halve H; attempt
 //              and time bookkeeping; done / failed status;
@@ -42,13 +42,28 @@
 namespace genga {
 namespace {
 
-constexpr int kPThreads = 128;
+constexpr int kPMaxThreads = 512;
+// Lanes per (column, member) item: 16 while all items then make at most this many
+// warps per SM sub-partition, else 8, else 4.  A phase lasts as long as its longest
+// partner list (a dense disk's reaches 80), which more lanes shorten; they cost FP64
+// work in the butterfly.  Measured (ms per call): 4,096-body gradient (1,415 members) 16
+// lanes 71.2, 8: 84, 4: 90; 16,384-body step (12,346 members) 16: 36.5, 8: 28.2, 4: 29.3.
+constexpr int kItemWarps = 64;
+// Members from which the pair form pays although one pass holds all items (1,415
+// members: 67.6 against 71.2 ms; 276 members: 4.45 against 4.13).
+constexpr int kPairMembers = 400;
 
 struct GridBarrier {
-    unsigned count;     // blocks arrived at the current barrier
-    unsigned gen;       // barrier generation
-    unsigned err;       // a wait ran out
-    unsigned running;   // groups still integrating
+    unsigned long long count;   // arrivals since the launch; top bit: a wait ran out
+    unsigned err;               // the same, for the host
+    unsigned running;           // groups still integrating
+};
+
+// One unordered pair of batched members (pair-centric mode): members m < p, the
+// partner-list entries m -> p and p -> m, their masses.
+struct alignas(32) PairRec {
+    int m, p, q, q2;
+    double mm, mp;
 };
 
 // Batch of groups: compact member index m in [0, M) over the groups.
@@ -70,10 +85,11 @@ struct BsmArgs {
     double *OUT, *DIAG;            // [8] column results, Neville diagonal T_kk
     // per-group step control
     double *gt, *gH;
+    double *gh;                    // [ng][8] midpoint sub-step H / n_k of each column this round, 0: done
     int *gstat;                    // 0 running, 1 done, 2 failed
     int *gkconv;                   // accepted column of the last round, -1 none
     long long *gatt, *gacc, *grej;
-    unsigned long long *gerr;      // [ng][8]
+    unsigned *gfail;               // [ng] bit k: some component's error of column k is above tolerance
     GridBarrier *bar;
     unsigned long long barrier_ns; // limit of one grid-barrier wait
     unsigned barrier_absent;       // test hook: arrivals every barrier waits for in vain (0)
@@ -91,8 +107,8 @@ struct BsmArgs {
     // partner-list entries, then summed per member
     int pairs;                     // 1: this mode
     const int *pcount;             // pairs listed
-    const int *pq, *pm;            // [pairs] entry q (member m -> partner) and member m, partner > m
-    const int *prev;               // [entries] the reverse entry of each entry of a batched member
+    const PairRec *prec;           // [pairs]
+    const double *pirc;            // [nlev][nq] 1/rc of each pair per level
     double2 *rec;                  // [8][entries][2]: (c, dx), (dy, dz) of each entry per column
     size_t nq;                     // entries (the stride of rec per column)
 };
@@ -112,57 +128,67 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Grid-wide barrier (all blocks co-resident: cooperative launch).  One
-// thread per block arrives with an atomic and polls the generation word with
-// volatile loads (served by L2); a wait longer than limit_ns records a
-// timeout, and a wait also ends once another block has recorded one.  The
-// barrier completes when gridDim.x + absent blocks have arrived (absent = 0
-// in normal use; a test makes every wait run out with absent > 0).  Returns
-// false if this or another block's wait ran out.
-__device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsigned absent) {
+// Grid-wide barrier (all blocks co-resident: cooperative launch).  One thread per
+// block arrives (release) at a counter that only grows and polls it (acquire)
+// until the arrivals of `target` barriers' worth are in: one round trip through
+// L2 after the last arrival, ~2 us against 4.7 us for a counter that the last
+// block resets behind a generation word.  A wait longer than limit_ns sets the
+// counter's top bit, which ends every other wait too.  The barrier completes when
+// gridDim.x + absent blocks have arrived (absent = 0 in normal use; a test makes
+// every wait run out with absent > 0).  Returns false if a wait ran out.
+constexpr unsigned long long kBarrierErr = 1ull << 63;
+__device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsigned absent,
+                             unsigned long long &target) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int good = 1;
-        volatile unsigned *gen = &b->gen;
-        volatile unsigned *err = &b->err;
-        const unsigned g = *gen;
-        __threadfence();
-        if (atomicAdd(&b->count, 1u) == gridDim.x + absent - 1) {
-            atomicExch(&b->count, 0u);
-            __threadfence();
-            atomicAdd(&b->gen, 1u);
-        } else {
-            const unsigned long long t0 = global_ns();
-            unsigned polls = 0;
-            while (*gen == g) {
-                if ((++polls & 63u) == 0u && (*err != 0u || global_ns() - t0 >= limit_ns)) {
+        target += gridDim.x + absent;
+        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&b->count) : "memory");
+        unsigned long long t0 = 0ull, v;
+        for (unsigned polls = 1;; polls++) {
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&b->count) : "memory");
+            if (v >= target) break;             // all arrived, or the top bit is set
+            if ((polls & 63u) == 0u) {
+                const unsigned long long now = global_ns();
+                if (t0 == 0ull) t0 = now;
+                if (now - t0 >= limit_ns) {
+                    atomicOr(&b->count, kBarrierErr);
                     atomicExch(&b->err, 1u);
-                    good = 0;
+                    v = kBarrierErr;
                     break;
                 }
             }
         }
-        __threadfence();
-        ok = good && *(volatile unsigned *)&b->err == 0u;
+        ok = (v & kBarrierErr) == 0ull;
     }
     __syncthreads();
     return ok != 0;
 }
 
-// Lanes per item in the derivative phases: the partner loop of one (column,
-// member) item is split over kLanes adjacent lanes (partner q to lane
-// q mod kLanes) and the partial sums are combined by an xor butterfly, which
-// gives every lane the same bits (IEEE addition commutes).
-constexpr int kLanes = 4;
-
-__device__ __forceinline__ unsigned lane_mask() {
-    return 0xfu << ((threadIdx.x & 31u) & ~3u);
+// W *= 1 - K(r / rc) for 1/rc = irc, from r^2 = d2 and yv = 1/r.  Outside the
+// band (decided from FP32 copies with margins of 1e-4) K is 0 or 1 exactly and
+// costs no FP64 operation; false: K = 1, W is zero.
+__device__ __forceinline__ bool apply_changeover(float rf, double d, double irc, double &W) {
+    const int side = changeover_side_f32(rf, __double2float_rz(irc));
+    if (side > 0) return false;
+    if (side == 0) W *= 1.0 - changeover_fast(d, irc);
+    return true;
 }
+// FP32 r from r^2 (relative error 2^-21).
+__device__ __forceinline__ float r_f32(double d2) {
+    const float f = f32_of_f64_trunc(d2);
+    return f * rsqrtf(f);
+}
+
+// Lanes per item in the derivative phases: the partner loop of one (column,
+// member) item is split over L adjacent lanes (partner q to lane q mod L) and the
+// partial sums are combined by an xor butterfly, which gives every lane the same
+// bits (IEEE addition commutes).  L by kItemWarps.
+template <int L>
 __device__ __forceinline__ double lane_sum(double v) {
-    const unsigned mk = lane_mask();
-    v += __shfl_xor_sync(mk, v, 1);
-    v += __shfl_xor_sync(mk, v, 2);
+    const unsigned mk = ((1u << L) - 1u) << ((threadIdx.x & 31u) & ~(unsigned)(L - 1));
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) v += __shfl_xor_sync(mk, v, o);
     return v;
 }
 
@@ -176,26 +202,30 @@ struct FwdOdeT {
     static constexpr int D = 6;
     static constexpr int NERR = 6;
     static constexpr bool COLL = COLL_;
+    template <int L>
     __device__ static void deriv(const BsmArgs &A, const double *Z, int m, int lane, double *f) {
         const size_t ld = (size_t)A.M;
         const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
         double px = 0.0, py = 0.0, pz = 0.0;
         const int q1 = (COLL && !ldc(&A.malive[m])) ? A.mq0[m] : A.mq1[m];
-        for (int q = A.mq0[m] + lane; q < q1; q += kLanes) {
+        for (int q = A.mq0[m] + lane; q < q1; q += L) {
             const int sp = A.pidx[q];
             const double dx = ldc(&Z[0 * ld + sp]) - x, dy = ldc(&Z[1 * ld + sp]) - y,
                          dz = ldc(&Z[2 * ld + sp]) - z;
             const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            const float rf = r_f32(d2);
             const double yv = rsqrt_newton(d2);
             const double d = d2 * yv;
             double W = 1.0;
-            for (int l = 0; l < A.nlev; l++)
-                W *= 1.0 - changeover_fast(d, fmin(A.irc[(size_t)l * ld + m], A.irc[(size_t)l * ld + sp]));
+            bool in = true;
+            for (int l = 0; l < A.nlev && in; l++)
+                in = apply_changeover(rf, d, fmin(A.irc[(size_t)l * ld + m], A.irc[(size_t)l * ld + sp]), W);
+            if (!in) continue;
             const double ms = COLL ? ldc(&A.mmass[sp]) : A.mmass[sp];
             const double c = ms * W * (yv * yv * yv);
             px = fma(c, dx, px); py = fma(c, dy, py); pz = fma(c, dz, pz);
         }
-        px = lane_sum(px); py = lane_sum(py); pz = lane_sum(pz);
+        px = lane_sum<L>(px); py = lane_sum<L>(py); pz = lane_sum<L>(pz);
         const double r2 = fma(z, z, fma(y, y, x * x));
         const double ys = rsqrt_newton(r2);
         const double sst = -A.mu * (ys * ys * ys);
@@ -205,17 +235,20 @@ struct FwdOdeT {
 };
 // The forward derivative of member m in column k from the entries' records
 // (pair-centric mode): the same terms, summed in the same lane split and order.
+template <int L>
 __device__ __forceinline__ void fwd_deriv_rec(const BsmArgs &A, const double *Z, int k, int m, int lane,
                                               double *f) {
     const size_t ld = (size_t)A.M;
     const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
     const double2 *R = A.rec + (size_t)k * 2 * A.nq;
     double px = 0.0, py = 0.0, pz = 0.0;
-    for (int q = A.mq0[m] + lane; q < A.mq1[m]; q += kLanes) {
+    const int q1 = A.mq1[m];
+#pragma unroll 4
+    for (int q = A.mq0[m] + lane; q < q1; q += L) {
         const double2 u = __ldcg(&R[2 * (size_t)q]), w = __ldcg(&R[2 * (size_t)q + 1]);
         px = fma(u.x, u.y, px); py = fma(u.x, w.x, py); pz = fma(u.x, w.y, pz);
     }
-    px = lane_sum(px); py = lane_sum(py); pz = lane_sum(pz);
+    px = lane_sum<L>(px); py = lane_sum<L>(py); pz = lane_sum<L>(pz);
     const double r2 = fma(z, z, fma(y, y, x * x));
     const double ys = rsqrt_newton(r2);
     const double sst = -A.mu * (ys * ys * ys);
@@ -234,6 +267,7 @@ struct AdjOde {
     static constexpr int D = 13;
     static constexpr int NERR = 6;
     static constexpr bool COLL = false;
+    template <int L>
     __device__ static void deriv(const BsmArgs &A, const double *Z, int m, int lane, double *f) {
         const size_t ld = (size_t)A.M;
         const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
@@ -241,7 +275,7 @@ struct AdjOde {
         const double mb = A.mmass[m];
         double px = 0.0, py = 0.0, pz = 0.0, gx = 0.0, gy = 0.0, gz = 0.0, gm = 0.0;
         const int q1 = A.mq1[m];
-        for (int q = A.mq0[m] + lane; q < q1; q += kLanes) {
+        for (int q = A.mq0[m] + lane; q < q1; q += L) {
             const int sp = A.pidx[q];
             const double dx = ldc(&Z[0 * ld + sp]) - x, dy = ldc(&Z[1 * ld + sp]) - y,
                          dz = ldc(&Z[2 * ld + sp]) - z;
@@ -263,8 +297,8 @@ struct AdjOde {
             gx += aa * e0 + bb * dx; gy += aa * e1 + bb * dy; gz += aa * e2 + bb * dz;
             gm -= W * (qx * dx + qy * dy + qz * dz) * id3;
         }
-        px = lane_sum(px); py = lane_sum(py); pz = lane_sum(pz);
-        gx = lane_sum(gx); gy = lane_sum(gy); gz = lane_sum(gz); gm = lane_sum(gm);
+        px = lane_sum<L>(px); py = lane_sum<L>(py); pz = lane_sum<L>(pz);
+        gx = lane_sum<L>(gx); gy = lane_sum<L>(gy); gz = lane_sum<L>(gz); gm = lane_sum<L>(gm);
         const double r2 = fma(z, z, fma(y, y, x * x));
         const double ys = rsqrt_newton(r2);
         const double ir2 = ys * ys, ir3 = ir2 * ys;
@@ -283,8 +317,18 @@ struct AdjOde {
 };
 
 // ---------------------------------------------------------------- phases
-// start and sub-step: item = kLanes adjacent lanes; lane 0 writes.
-template <class Ode>
+// start and sub-step: item = L adjacent lanes; lane l writes the components l, l + L,
+// ... (FP64 charges a warp instruction whatever its lanes).
+template <int D, int L>
+__device__ __forceinline__ double pick(const double *f, int base, int lane) {
+    double v = f[base];
+#pragma unroll
+    for (int l = 1; l < L; l++)
+        if (base + l < D && lane == l) v = f[base + l];
+    return v;
+}
+
+template <class Ode, int L>
 __device__ void phase_start(const BsmArgs &A, int m, int lane) {
     const int g = A.mgroup[m];
     if (ldc(&A.gstat[g]) != 0) return;
@@ -292,51 +336,52 @@ __device__ void phase_start(const BsmArgs &A, int m, int lane) {
     const size_t ld = (size_t)A.M, blk = (size_t)D * ld;
     const double H = step_of(A, g);
     double f[D];
-    Ode::deriv(A, A.Y, m, lane, f);
-    if (lane != 0) return;
-    for (int c = 0; c < D; c++) {
+    Ode::template deriv<L>(A, A.Y, m, lane, f);
+#pragma unroll
+    for (int b = 0; b < D; b += L) {
+        const int c = b + lane;
+        const double fc = pick<D, L>(f, b, lane);
+        if (c >= D) break;
         const double y = ldc(&A.Y[c * ld + m]);
-        A.F0[c * ld + m] = f[c];
-        A.SC[c * ld + m] = fabs(y) + fabs(H * f[c]) + 1e-300;
+        A.F0[c * ld + m] = fc;
+        A.SC[c * ld + m] = fabs(y) + fabs(H * fc) + 1e-300;
         for (int k = 0; k < 8; k++) {
-            const double h = H / (2 * (k + 1));
             A.ZM[k * blk + c * ld + m] = y;
-            A.ZA[k * blk + c * ld + m] = y + h * f[c];
+            A.ZA[k * blk + c * ld + m] = y + ldc(&A.gh[(size_t)g * 8 + k]) * fc;
         }
     }
 }
 
-template <class Ode>
-__device__ void phase_substep(const BsmArgs &A, long long t, int it, int lane) {
-    const int k = (int)(t / A.M), m = (int)(t % A.M);
+template <class Ode, int L>
+__device__ void phase_substep(const BsmArgs &A, int k, int m, int it, int lane) {
     const int nk = 2 * (k + 1);
-    if (it > nk) return;
-    const int g = A.mgroup[m];
-    if (ldc(&A.gstat[g]) != 0) return;
+    const double h = ldc(&A.gh[(size_t)A.mgroup[m] * 8 + k]);
+    if (h == 0.0) return;                        // the group is done
     constexpr int D = Ode::D;
     const size_t ld = (size_t)A.M, blk = (size_t)D * ld;
     const double *Zcur = ((it & 1) ? A.ZA : A.ZB) + k * blk;
     double *Znext = ((it & 1) ? A.ZB : A.ZA) + k * blk;
     double *ZM = A.ZM + k * blk;
-    const double h = step_of(A, g) / nk;
     double f[D];
     if constexpr (D == 6 && !Ode::COLL) {
-        if (A.pairs) fwd_deriv_rec(A, Zcur, k, m, lane, f);
-        else Ode::deriv(A, Zcur, m, lane, f);
+        if (A.pairs) fwd_deriv_rec<L>(A, Zcur, k, m, lane, f);
+        else Ode::template deriv<L>(A, Zcur, m, lane, f);
     } else {
-        Ode::deriv(A, Zcur, m, lane, f);
+        Ode::template deriv<L>(A, Zcur, m, lane, f);
     }
-    if (lane != 0) return;
-    if (it < nk) {
-        for (int c = 0; c < D; c++) {
-            const double zc = ldc(&Zcur[c * ld + m]);
-            const double tt = ldc(&ZM[c * ld + m]) + 2.0 * h * f[c];
+    const double h2 = 2.0 * h;
+#pragma unroll
+    for (int b = 0; b < D; b += L) {
+        const int c = b + lane;
+        const double fc = pick<D, L>(f, b, lane);
+        if (c >= D) break;
+        const double zc = ldc(&Zcur[c * ld + m]), zm = ldc(&ZM[c * ld + m]);
+        if (it < nk) {
             ZM[c * ld + m] = zc;
-            Znext[c * ld + m] = tt;
+            Znext[c * ld + m] = zm + h2 * fc;
+        } else {
+            A.OUT[k * blk + c * ld + m] = 0.5 * (zc + zm + h * fc);
         }
-    } else {
-        for (int c = 0; c < D; c++)
-            A.OUT[k * blk + c * ld + m] = 0.5 * (ldc(&Zcur[c * ld + m]) + ldc(&ZM[c * ld + m]) + h * f[c]);
     }
 }
 
@@ -344,51 +389,57 @@ __device__ void phase_substep(const BsmArgs &A, long long t, int it, int lane) {
 // terms member m's partner loop would (displacement from m to its partner p,
 // W, m_p W / r^3) and those p's would (the displacement negated, exactly, and
 // m_m W / r^3), into the records of entries m -> p and p -> m.
-__device__ void phase_pairs(const BsmArgs &A, long long t, long long P, int it) {
-    const int k = (int)(t / P);
-    const long long pi = t - (long long)k * P;
-    if (it > 2 * (k + 1)) return;
-    const int q = A.pq[pi], m = A.pm[pi];
-    if (ldc(&A.gstat[A.mgroup[m]]) != 0) return;
-    const int sp = A.pidx[q], q2 = A.prev[q];
+__device__ void phase_pairs(const BsmArgs &A, int k, long long pi, int it) {
+    const PairRec r = A.prec[pi];
+    if (A.ng > 1 && ldc(&A.gstat[A.mgroup[r.m]]) != 0) return;
     const size_t ld = (size_t)A.M, blk = 6 * ld;
     const double *Z = ((it & 1) ? A.ZA : A.ZB) + k * blk;
-    const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
-    const double dx = ldc(&Z[0 * ld + sp]) - x, dy = ldc(&Z[1 * ld + sp]) - y, dz = ldc(&Z[2 * ld + sp]) - z;
+    const double x = ldc(&Z[0 * ld + r.m]), y = ldc(&Z[1 * ld + r.m]), z = ldc(&Z[2 * ld + r.m]);
+    const double dx = ldc(&Z[0 * ld + r.p]) - x, dy = ldc(&Z[1 * ld + r.p]) - y, dz = ldc(&Z[2 * ld + r.p]) - z;
     const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const double yv = rsqrt_newton(d2);
-    const double d = d2 * yv;
-    double W = 1.0;
-    for (int l = 0; l < A.nlev; l++)
-        W *= 1.0 - changeover_fast(d, fmin(A.irc[(size_t)l * ld + m], A.irc[(size_t)l * ld + sp]));
-    const double cm = A.mmass[sp] * W * (yv * yv * yv);
-    const double cp = A.mmass[m] * W * (yv * yv * yv);
+    const float rf = r_f32(d2);
+    double cm = 0.0, cp = 0.0;
+    bool in = true;
+    for (int l = 0; l < A.nlev && in; l++)          // beyond some rc: no term, no FP64 reciprocal root
+        in = changeover_side_f32(rf, __double2float_rz(A.pirc[(size_t)l * A.nq + pi])) <= 0;
+    if (in) {
+        const double yv = rsqrt_newton(d2);
+        const double d = d2 * yv;
+        double W = 1.0;
+        for (int l = 0; l < A.nlev; l++) apply_changeover(rf, d, A.pirc[(size_t)l * A.nq + pi], W);
+        const double y3 = yv * yv * yv;
+        cm = r.mp * W * y3;
+        cp = r.mm * W * y3;
+    }
     double2 *R = A.rec + (size_t)k * 2 * A.nq;
-    R[2 * (size_t)q] = make_double2(cm, dx);
-    R[2 * (size_t)q + 1] = make_double2(dy, dz);
-    R[2 * (size_t)q2] = make_double2(cp, -dx);
-    R[2 * (size_t)q2 + 1] = make_double2(-dy, -dz);
+    R[2 * (size_t)r.q] = make_double2(cm, dx);
+    R[2 * (size_t)r.q + 1] = make_double2(dy, dz);
+    R[2 * (size_t)r.q2] = make_double2(cp, -dx);
+    R[2 * (size_t)r.q2 + 1] = make_double2(-dy, -dz);
 }
 
-// Neville for item t; called by every lane of a warp (the reductions need all
-// lanes), items past the end contribute nothing.
+// Neville for item t; called by every lane of a warp (the vote needs all lanes),
+// items past the end contribute nothing.  The acceptance test max |T_kk - T_k,k-1| /
+// scale <= tol is taken per component as |T_kk - T_k,k-1| <= tol scale, one bit
+// per column (a difference only where the quotient rounds across tol).
 template <class Ode>
 __device__ void phase_neville(const BsmArgs &A, long long t) {
     constexpr int D = Ode::D;
     const size_t ld = (size_t)A.M, blk = (size_t)D * ld;
-    double e[8];
-    for (int k = 0; k < 8; k++) e[k] = 0.0;
+    unsigned fail = 0u;
     int g = -1;
     if (t < (long long)D * A.M) {
         const int c = (int)(t / A.M), m = (int)(t % A.M);
         g = A.mgroup[m];
         if (ldc(&A.gstat[g]) == 0) {
             double T[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            const double sc = ldc(&A.SC[c * ld + m]);
+            const double lim = A.tol * ldc(&A.SC[c * ld + m]);
+#pragma unroll
             for (int k = 0; k < 8; k++) {
                 double cur = ldc(&A.OUT[k * blk + c * ld + m]);
                 double prev = T[0];
                 T[0] = cur;
+#pragma unroll
                 for (int j = 1; j <= k; j++) {
                     const double coef = (double)((k - j + 1) * (k - j + 1)) / (double)(j * (2 * k + 2 - j));
                     const double nxt = fma(cur - prev, coef, cur);
@@ -397,7 +448,7 @@ __device__ void phase_neville(const BsmArgs &A, long long t) {
                     cur = nxt;
                 }
                 A.DIAG[k * blk + c * ld + m] = T[k];
-                if (k >= 1 && c < Ode::NERR) e[k] = fabs(T[k] - T[k - 1]) / sc;
+                if (k >= 1 && c < Ode::NERR && fabs(T[k] - T[k - 1]) > lim) fail |= 1u << k;
             }
         } else {
             g = -1;
@@ -405,16 +456,11 @@ __device__ void phase_neville(const BsmArgs &A, long long t) {
     }
     // one atomic per warp when all its lanes belong to one running group
     const int g0 = __shfl_sync(0xffffffffu, g, 0);
-    const bool uniform = __all_sync(0xffffffffu, g == g0);
-    for (int k = 1; k < 8; k++) {
-        double v = e[k];
-        if (uniform) {
-            for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if ((threadIdx.x & 31) == 0 && g0 >= 0)
-                atomicMax(&A.gerr[(size_t)g0 * 8 + k], (unsigned long long)__double_as_longlong(v));
-        } else if (g >= 0) {
-            atomicMax(&A.gerr[(size_t)g * 8 + k], (unsigned long long)__double_as_longlong(v));
-        }
+    if (__all_sync(0xffffffffu, g == g0)) {
+        const unsigned all = __reduce_or_sync(0xffffffffu, fail);
+        if ((threadIdx.x & 31) == 0 && g0 >= 0 && all) atomicOr(&A.gfail[g0], all);
+    } else if (g >= 0 && fail) {
+        atomicOr(&A.gfail[g], fail);
     }
 }
 
@@ -476,6 +522,24 @@ __device__ void group_merge(const BsmArgs &A, int g, double t) {
     A.gseq[g] = seq;
 }
 
+// The columns' midpoint sub-steps of group g's next attempt.
+__device__ __forceinline__ void column_steps(const BsmArgs &A, int g, double t, double H) {
+    const double left = A.dt - t;
+    if (H > left) H = left;
+    for (int k = 0; k < 8; k++) A.gh[(size_t)g * 8 + k] = H / (2 * (k + 1));
+}
+
+// Item t of the columns k0, k0 + 1, ... of `per` items each: the column; t becomes
+// the item within it.
+__device__ __forceinline__ int column_of(long long &t, long long per, int k0) {
+    int k = k0;
+    while (t >= per) {
+        t -= per;
+        k++;
+    }
+    return k;
+}
+
 // Step control of group g (the in-block kernels' rule).  The group's
 // counters are touched only by this thread, so plain accesses suffice for
 // them; the words other blocks read go through L2.
@@ -484,17 +548,14 @@ __device__ void phase_decide(const BsmArgs &A, int g) {
     A.gkconv[g] = -1;
     if (ldc(&A.gstat[g]) != 0) return;
     double H = step_of(A, g);
-    int kconv = -1;
-    for (int k = 1; k < 8 && kconv < 0; k++) {
-        const double e = __longlong_as_double((long long)atomicAdd(&A.gerr[(size_t)g * 8 + k], 0ull));
-        if (e <= A.tol) kconv = k;
-    }
+    const unsigned fail = atomicExch(&A.gfail[g], 0u);
+    const unsigned conv = ~fail & 0xfeu;
+    int kconv = conv ? __ffs(conv) - 1 : -1;
     // collision precision (Sec. 7.2): a step that ends with an overlap of
     // tol or more of the radius sum ends too late
     if (Ode::COLL && kconv >= 0 && A.coll.tol > 0.0 &&
         group_overlap(A, g, A.DIAG + (size_t)kconv * Ode::D * A.M) >= A.coll.tol)
         kconv = -1;
-    for (int k = 0; k < 8; k++) atomicExch(&A.gerr[(size_t)g * 8 + k], 0ull);
     const long long att = A.gatt[g] + 1;
     A.gatt[g] = att;
     double t = ldc(&A.gt[g]);
@@ -509,10 +570,12 @@ __device__ void phase_decide(const BsmArgs &A, int g) {
     A.gt[g] = t;
     A.gH[g] = H;
     A.gkconv[g] = kconv;
+    column_steps(A, g, t, H);
     int st = 0;
     if (!(t < A.dt)) st = 1;
     else if (att >= A.max_steps) st = 2;
     if (st) {
+        for (int k = 0; k < 8; k++) A.gh[(size_t)g * 8 + k] = 0.0;
         A.gstat[g] = st;
         atomicSub(&A.bar->running, 1u);
     }
@@ -527,52 +590,64 @@ __device__ void phase_accept(const BsmArgs &A, long long t) {
     if (k >= 0) A.Y[t] = ldc(&A.DIAG[k * blk + t]);
 }
 
-template <class Ode>
-__global__ void __launch_bounds__(kPThreads)
+template <class Ode, int L>
+__global__ void __launch_bounds__(kPMaxThreads)
 bsm_persistent_kernel(BsmArgs A) {
     constexpr int D = Ode::D;
     const long long nth = (long long)gridDim.x * blockDim.x;
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    // consecutive warps' worth of work go to consecutive blocks, so that a phase
+    // with few items (the last sub-steps: one column) still reaches every SM
+    const long long tid = ((long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
     const long long M = A.M;
-    // derivative phases: kLanes adjacent lanes per item (blockDim is a multiple of 32)
-    const long long item0 = tid / kLanes, nitem = nth / kLanes;
-    const int lane = (int)(threadIdx.x % kLanes);
+    // derivative phases: L adjacent lanes per item
+    const long long item0 = tid / L, nitem = nth / L;
+    const int lane = (int)(threadIdx.x % L);
     // pairs of the pair-centric mode (listed by bsm_pairs_kernel before the launch)
     const long long P = (D == 6 && !Ode::COLL && A.pairs) ? (long long)*A.pcount : 0;
     __shared__ unsigned running;
+    unsigned long long arrived = 0ull;            // thread 0: arrivals the next barrier waits for
     if (Ode::COLL) {
         // pairs already overlapping when the integration starts merge at once
         for (long long g = tid; g < A.ng; g += nth) group_merge(A, (int)g, 0.0);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
     }
     for (int round = 0; round < A.max_steps; round++) {
         // one read per block; the previous round ended with a barrier
         if (threadIdx.x == 0) running = atomicAdd(&A.bar->running, 0u);
         __syncthreads();
         if (running == 0u) break;
-        for (long long t = item0; t < M; t += nitem) phase_start<Ode>(A, (int)t, lane);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+        for (long long t = item0; t < M; t += nitem) phase_start<Ode, L>(A, (int)t, lane);
+        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
         for (int it = 1; it <= 16; it++) {
+            const int k0 = (it - 1) / 2;          // columns below have no sub-step left
             if (P > 0) {
-                for (long long t = tid; t < 8 * P; t += nth) phase_pairs(A, t, P, it);
-                if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+                for (long long t = tid; t < (8 - k0) * P; t += nth) {
+                    long long pi = t;
+                    const int k = column_of(pi, P, k0);
+                    phase_pairs(A, k, pi, it);
+                }
+                if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
             }
-            for (long long t = item0; t < 8 * M; t += nitem) phase_substep<Ode>(A, t, it, lane);
-            if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+            for (long long t = item0; t < (8 - k0) * M; t += nitem) {
+                long long m = t;
+                const int k = column_of(m, M, k0);
+                phase_substep<Ode, L>(A, k, (int)m, it, lane);
+            }
+            if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
         }
-        for (long long base = (long long)blockIdx.x * blockDim.x; base < D * M; base += nth)
-            phase_neville<Ode>(A, base + threadIdx.x);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+        for (long long base = tid - (threadIdx.x & 31); base < D * M; base += nth)
+            phase_neville<Ode>(A, base + (threadIdx.x & 31));
+        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
         for (long long g = tid; g < A.ng; g += nth) phase_decide<Ode>(A, (int)g);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
         for (long long t = tid; t < D * M; t += nth) phase_accept<Ode>(A, t);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
         if (Ode::COLL) {
             // mergers at the end of every accepted step (same thread per group
             // as the decision, which wrote gkconv and gt)
             for (long long g = tid; g < A.ng; g += nth)
                 if (A.gkconv[g] >= 0) group_merge(A, (int)g, ldc(&A.gt[g]));
-            if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent)) return;
+            if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
         }
     }
 }
@@ -607,26 +682,28 @@ __global__ void bsm_members_kernel(int ng, const int *gbase, const int *gslot0, 
 }
 
 // Pair-centric mode: the unordered pairs of the batched members (each listed
-// from its lower member, in any order) and every entry's reverse entry (the
-// rows are ascending in body index, so a binary search finds it).
+// from its lower member, in any order) with the reverse entry (the rows are
+// ascending in body index, so a binary search finds it), masses and 1/rc.
 __global__ void bsm_pairs_kernel(int M, const int *mq0, const int *mq1, const int *pidx, const int *mbody,
-                                 const int *list, int *pcount, int *pq, int *pm, int *prev) {
+                                 const int *list, const double *mmass, const double *irc, int nlev, size_t nq,
+                                 int *pcount, PairRec *prec, double *pirc) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
     const int bm = mbody[m];
     for (int q = mq0[m]; q < mq1[m]; q++) {
         const int p = pidx[q];
+        if (p <= m) continue;
         int lo = mq0[p], hi = mq1[p] - 1;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
             if (list[mid] < bm) lo = mid + 1; else hi = mid;
         }
-        prev[q] = lo;
-        if (p > m) {
-            const int k = atomicAdd(pcount, 1);
-            pq[k] = q;
-            pm[k] = m;
-        }
+        const int k = atomicAdd(pcount, 1);
+        PairRec r;
+        r.m = m; r.p = p; r.q = q; r.q2 = lo;
+        r.mm = mmass[m]; r.mp = mmass[p];
+        prec[k] = r;
+        for (int l = 0; l < nlev; l++) pirc[(size_t)l * nq + k] = fmin(irc[(size_t)l * M + m], irc[(size_t)l * M + p]);
     }
 }
 
@@ -646,8 +723,7 @@ __global__ void bsm_coll_init_kernel(BsmArgs A) {
 __global__ void bsm_init_groups_kernel(BsmArgs A) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g == 0) {
-        A.bar->count = 0u;
-        A.bar->gen = 0u;
+        A.bar->count = 0ull;
         A.bar->err = 0u;
         A.bar->running = (unsigned)A.ng;
     }
@@ -660,7 +736,8 @@ __global__ void bsm_init_groups_kernel(BsmArgs A) {
     A.gacc[g] = 0;
     A.grej[g] = 0;
     if (A.gseq) A.gseq[g] = 0;
-    for (int k = 0; k < 8; k++) A.gerr[(size_t)g * 8 + k] = 0ull;
+    A.gfail[g] = 0u;
+    column_steps(A, g, 0.0, A.dt);
 }
 
 __global__ void bsm_gather_fwd(int n, int M, const int *mbody, const double *pos, const double *vel, double *Y) {
@@ -804,31 +881,40 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     gbase[ng] = M;
     const size_t blk = (size_t)D * M;
     const size_t nq = 2 * (size_t)s->csr[level].cap;
-    // one persistent cooperative launch: as many blocks as fit on the GPU (more
-    // warps to hide the partner reads from L2 outweigh the barrier's extra
-    // arrivals), and no more than the (column, member) items need
+    // One persistent cooperative launch: one block per SM as large as the items
+    // need (fewer arrivals at a grid barrier than with small blocks), more blocks
+    // where they fill it.
+    int L = 16;
+    while (L > 4 && 8LL * M * L > (long long)kItemWarps * 4 * 32 * s->num_sms) L /= 2;
+    const void *kernel = L == 16  ? (const void *)bsm_persistent_kernel<Ode, 16>
+                         : L == 8 ? (const void *)bsm_persistent_kernel<Ode, 8>
+                                  : (const void *)bsm_persistent_kernel<Ode, 4>;
+    const long long want_threads = 8LL * M * L;
+    const int threads = (int)std::min<long long>(kPMaxThreads,
+                                                 ((want_threads + s->num_sms - 1) / s->num_sms + 31) / 32 * 32);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bsm_persistent_kernel<Ode>, kPThreads, 0) !=
-            cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1)
         return GENGA_ECUDA;
-    const long long want = (8LL * M * kLanes + kPThreads - 1) / kPThreads;
+    const long long want = (want_threads + threads - 1) / threads;
     const long long cap = (long long)per_sm * s->num_sms;
     const unsigned grid = (unsigned)std::max(1LL, std::min(want, cap));
-    // pair-centric derivative where a sub-step phase takes more than two passes
-    // over its (column, member) items: there the FP64 work of the partner
-    // terms, halved, outweighs a second barrier per sub-step
+    // pair-centric derivative from kPairMembers members on, and where a sub-step
+    // phase takes more than two passes over its items: the FP64 work of the
+    // partner terms, halved and evenly spread over the lanes, outweighs a second
+    // barrier per sub-step
     const bool pairs = D == 6 && !Ode::COLL &&
                        (s->bs_pairs == GENGA_BS_PAIRS_ON ||
-                        (s->bs_pairs == GENGA_BS_PAIRS_AUTO && 8LL * M > 2LL * grid * (kPThreads / kLanes)));
-    const size_t pbytes = pairs ? aligned(sizeof(double2) * 2 * 8 * nq) + aligned(sizeof(int) * nq) * 3 +
-                                      aligned(sizeof(int))
+                        (s->bs_pairs == GENGA_BS_PAIRS_AUTO && (M >= kPairMembers || 8LL * M > 2LL * grid * (threads / L))));
+    const size_t np = nq / 2;
+    const size_t pbytes = pairs ? aligned(sizeof(double2) * 2 * 8 * nq) + aligned(sizeof(PairRec) * np) +
+                                      aligned(sizeof(double) * nlev * nq) + aligned(sizeof(int))
                                 : 0;
     const size_t bytes = pbytes + aligned(sizeof(double) * blk) * 3 + aligned(sizeof(double) * 8 * blk) * 5 +
                          aligned(sizeof(double) * (size_t)nlev * M) + aligned(sizeof(double) * M) +
                          aligned(sizeof(int) * M) * 4 + aligned(sizeof(int) * nq) +
                          aligned(sizeof(int) * (ng + 1)) + aligned(sizeof(int) * ng) * 4 +
                          aligned(sizeof(double) * ng) * 2 +
-                         aligned(sizeof(long long) * ng) * 3 + aligned(sizeof(unsigned long long) * 8 * ng) +
+                         aligned(sizeof(long long) * ng) * 3 + aligned(sizeof(unsigned) * ng) + aligned(sizeof(double) * 8 * ng) +
                          aligned(sizeof(GridBarrier)) +
                          (Ode::COLL ? aligned(sizeof(int) * M) * 2 : 0);
     char *p = static_cast<char *>(bsm_reserve(s, bytes));
@@ -837,16 +923,17 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     A.M = M; A.ng = ng; A.nlev = nlev;
     A.pairs = pairs ? 1 : 0;
     A.nq = nq;
-    int *pcount = nullptr, *pq = nullptr, *pm = nullptr, *prev = nullptr;
+    int *pcount = nullptr;
+    PairRec *prec = nullptr;
+    double *pirc = nullptr;
     A.rec = nullptr;
     if (pairs) {
         A.rec = carve<double2>(p, 2 * 8 * nq);
-        pq = carve<int>(p, nq);
-        pm = carve<int>(p, nq);
-        prev = carve<int>(p, nq);
+        prec = carve<PairRec>(p, np);
+        pirc = carve<double>(p, (size_t)nlev * nq);
         pcount = carve<int>(p, 1);
     }
-    A.pcount = pcount; A.pq = pq; A.pm = pm; A.prev = prev;
+    A.pcount = pcount; A.prec = prec; A.pirc = pirc;
     A.Y = carve<double>(p, blk); A.F0 = carve<double>(p, blk); A.SC = carve<double>(p, blk);
     A.ZM = carve<double>(p, 8 * blk); A.ZA = carve<double>(p, 8 * blk); A.ZB = carve<double>(p, 8 * blk);
     A.OUT = carve<double>(p, 8 * blk); A.DIAG = carve<double>(p, 8 * blk);
@@ -862,7 +949,8 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     A.gatt = carve<long long>(p, ng);
     A.gacc = carve<long long>(p, ng);
     A.grej = carve<long long>(p, ng);
-    A.gerr = carve<unsigned long long>(p, 8 * (size_t)ng);
+    A.gfail = carve<unsigned>(p, ng);
+    A.gh = carve<double>(p, 8 * (size_t)ng);
     A.bar = carve<GridBarrier>(p, 1);
     A.mgroup = mgroup; A.mq0 = mq0; A.mq1 = mq1; A.pidx = pidx; A.mmass = mmass; A.irc = irc;
     A.mbody = mbody; A.gbase = d_gbase; A.mmass_rw = mmass; A.ctr = s->ctr;
@@ -888,7 +976,8 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     bsm_init_groups_kernel<<<(unsigned)((ng + 127) / 128), 128, 0, st>>>(A);
     if (pairs) {
         if (cudaMemsetAsync(pcount, 0, sizeof(int), st) != cudaSuccess) return GENGA_ECUDA;
-        bsm_pairs_kernel<<<gm, 128, 0, st>>>(M, mq0, mq1, pidx, mbody, s->csr[level].list, pcount, pq, pm, prev);
+        bsm_pairs_kernel<<<gm, 128, 0, st>>>(M, mq0, mq1, pidx, mbody, s->csr[level].list, mmass, irc, nlev, nq, pcount,
+                                             prec, pirc);
         ++s->launches;
     }
     if (Ode::COLL) {
@@ -900,7 +989,7 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     if (cudaGetLastError() != cudaSuccess) return GENGA_ECUDA;
 
     void *args[] = {&A};
-    if (cudaLaunchCooperativeKernel((const void *)bsm_persistent_kernel<Ode>, dim3(grid), dim3(kPThreads), args,
+    if (cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args,
                                     0, st) != cudaSuccess)
         return GENGA_ECUDA;
     ++s->launches;

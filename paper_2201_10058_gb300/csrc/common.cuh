@@ -125,10 +125,12 @@ struct genga_system {
     double *pre_vel[genga::kMaxLevels] = {};
 
     // all-pairs kick
-    double *kick_part = nullptr;   // [max(nchunk, ksym_nS)][6][n]
+    double *kick_part = nullptr;   // partial sums, [slots][3 or 6][n]
     size_t kick_part_cap = 0;      // doubles allocated
-    int kick_nchunk = 0;
+    int kick_nchunk = 0;           // grid of the pre-check alone
     int kick_chunk = 0;
+    int ktile_chunk = 0;           // tiled kick: steps (two bodies j) per chunk, chunks
+    int ktile_nchunk = 0;
     // symmetric kick (each unordered pair once): geometry for (ksym_n, ksym_prec)
     int64_t ksym_n = -1;
     int ksym_prec = -1;
@@ -146,7 +148,7 @@ struct genga_system {
     double *ksym_irc = nullptr;    // 1 / rc per body
     float *ksym_thrpc = nullptr;   // FP32 upper bound of (f_pc rc)^2
     size_t ksym_body_cap = 0;      // bodies the two arrays above hold
-    // the bodies as float expansions (kick_ff.cu): mixed kick, energy
+    // the bodies as float expansions (kick_ff.cu): kick, energy
     void *ff = nullptr;            // one allocation: bodies, 1/rc as two floats, mass per tile,
                                    // bounds, header
     size_t ff_tiles = 0;           // tiles it holds
@@ -294,15 +296,15 @@ int kick_nchunk_for(int n, int num_sms);
 
 // Kick on caller-provided arrays (no system object, no pre-check).
 struct KickRaw {
-    const double *pos, *mass, *rc, *rc2;
-    const float *thr;
-    double *part;        // partial sums, [nchunk][6][n]
+    const double *pos, *mass, *rc;
+    double *scratch;     // room doubles, 256-byte aligned
+    size_t room;
     int n;
     double G, dt_half;
     double *vel, *acc_out;
     bool mixed;
 };
-cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, int max_nchunk, cudaStream_t stream);
+cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, cudaStream_t stream);
 
 // encounter.cu
 cudaError_t launch_detect(genga_system *s, const uint2 *in, int64_t nin, int level,

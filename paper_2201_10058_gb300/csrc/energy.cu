@@ -20,8 +20,7 @@
 // every ordered pair (the same E and L to the last bit there).
 #include <algorithm>
 
-#include "ff2.cuh"
-#include "kick_sym.cuh"
+#include "ff_pair.cuh"
 
 namespace genga {
 namespace {
@@ -59,7 +58,7 @@ __device__ __forceinline__ void block_sum2(double &S, double &C, double *sh) {
     C = sh[T];
 }
 
-// 1/r in FP64: coordinates that three floats do not hold, close pairs (r < 2^-20 S:
+// 1/r in FP64: coordinates that three floats do not hold, close pairs (r < 2^-17 S:
 // the displacement reaches below the second grid, 0 among them) and NaN, 1/r next
 // to a power of two.
 __device__ __noinline__ double rinv_fp64(const EnergyArgs &A, int i, int j) {
@@ -76,18 +75,6 @@ __device__ __forceinline__ void add_row(double &TS, double &TC, double m, double
     TC += e + (fma(m, S, -P) + m * C);
 }
 
-// v rounded to a multiple of a power of two g; c = 1.5 2^23 g, |v| < 2^22 g.
-__device__ __forceinline__ f2 f2_round(f2 v, f2 c) { return f2_sub(f2_add(v, c), c); }
-
-// y (1 + e/2 + ...) as a double: `units` of 2^-52 of y's leading bit added.
-__device__ __forceinline__ double rinv_bits(float y, float vh, float vl) {
-    const unsigned b = __float_as_uint(y);
-    const float sc = __uint_as_float((306u << 23) - (b & 0x7f800000u));        // 2^(52 - exponent of y)
-    const int units = __float2int_rn(vh * sc) + __float2int_rn(vl * sc);
-    const long long d = (long long)(((unsigned long long)((b >> 3) + 0x38000000u) << 32) | (unsigned)(b << 29)) + units;
-    return __longlong_as_double(d);
-}
-
 // The pairs i < j, by tiles (a, b), a <= b, in an order in which every block takes
 // one contiguous range: row a of tiles is followed by row nT - 1 - a, so that two
 // rows together always have nT + 1 tile pairs.
@@ -102,8 +89,7 @@ energy_pairs_kernel(EnergyArgs A) {
     const bool wide = (A.header[0] & kFfWide) != 0;
     const float close2 = reinterpret_cast<const float *>(A.header)[3];
     const double unit = scalbn(1.0, A.header[2]);          // of the packed bodies' lengths
-    const f2 c0 = f2_dup(6144.0f), c1 = f2_dup(3.0f), c2 = f2_dup(7.32421875e-4f);   // 1.5 2^(23 - 11, - 22, - 34)
-    const f2 one = f2_dup(1.0f), two = f2_dup(2.0f), half = f2_dup(0.5f), c375 = f2_dup(0.375f);
+    const f2 half = f2_dup(0.5f), c375 = f2_dup(0.375f);
     double TS = 0.0, TC = 0.0;                 // this thread's sum of m_i m_j / r_ij
     double S = 0.0, C = 0.0;                   // its row's sum of m_j / r_ij
     f2 nh[3], nm[3], nl[3];
@@ -155,51 +141,24 @@ energy_pairs_kernel(EnergyArgs A) {
                      lj[3] = {f2_lo(q4), f2_hi(q4), f2_lo(q5)};
             f2 H[3], L[3], T[3];
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                f2 e;
-                f2_fast_two_sum(f2_add(hj[c], nh[c]), f2_add(mj[c], nm[c]), H[c], e);
-                f2_fast_two_sum(e, f2_add(lj[c], nl[c]), L[c], T[c]);
-            }
+            for (int c = 0; c < 3; c++) ff_disp3(hj[c], mj[c], lj[c], nh[c], nm[c], nl[c], H[c], L[c], T[c]);
             const f2 s = f2_fma(H[2], H[2], f2_fma(H[1], H[1], f2_mul(H[0], H[0])));
             const f2 y = f2_rsqrt(s);
-            // sums of whole multiples that fit a float at every step: 1 - sum Q0^2 (2^-22),
-            // - 2 sum Q0 Q1 (2^-32); - sum Q1^2 - 2 sum Q0 r0 (2^-44); the rest in E2
-            f2 E0 = one, E1 = 0ull, E2 = 0ull, a1[3], D0[3];
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const f2 q = f2_mul(H[c], y), Q0 = f2_round(q, c0);
-                a1[c] = f2_sub(q, Q0);
-                E0 = f2_fma(f2_neg(Q0), Q0, E0);
-                D0[c] = f2_add(Q0, Q0);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const f2 q = f2_mul(H[c], y), qe = f2_fma(H[c], y, f2_neg(q));     // H y = q + qe
-                const f2 b1 = f2_mul(L[c], y), be = f2_fma(T[c], y, f2_fma(L[c], y, f2_neg(b1)));
-                const f2 Q1 = f2_round(a1[c], c1), a2 = f2_sub(a1[c], Q1);
-                // a2 + b1 + qe: digit r0 (multiple of 2^-34) and remainder r1
-                const f2 t1 = f2_add(c2, a2), t2 = f2_add(t1, b1), t3 = f2_add(t2, qe), r0 = f2_sub(t3, c2);
-                f2 r1 = f2_add(f2_sub(a2, f2_sub(t1, c2)), f2_sub(b1, f2_sub(t2, t1)));
-                r1 = f2_add(r1, f2_add(f2_sub(qe, f2_sub(t3, t2)), be));
-                const f2 r = f2_add(r0, r1);
-                E0 = f2_fma(f2_neg(D0[c]), Q1, E0);
-                E1 = f2_fma(f2_neg(Q1), Q1, E1);
-                E1 = f2_fma(f2_neg(D0[c]), r0, E1);
-                E2 = f2_fma(f2_neg(D0[c]), r1, E2);
-                E2 = f2_fma(f2_neg(f2_fma(two, Q1, r)), r, E2);
-            }
-            const f2 eh = f2_add(E0, E1);                                          // exact
+            f2 eh, el;
+            ff_residual(H, L, T, y, eh, el);
             // y (1 + e/2 + 3 e^2/8) - y = vh + vl
             const f2 x = f2_mul(y, eh), xe = f2_fma(y, eh, f2_neg(x));
-            const f2 tt = f2_fma(f2_mul(c375, eh), eh, f2_mul(half, E2));
-            const float2 Y = f2_get(y), VH = f2_get(f2_mul(half, x)), VL = f2_get(f2_fma(y, tt, f2_mul(half, xe)));
-            const float2 R2 = f2_get(s);
-            double rx = rinv_bits(Y.x, VH.x, VL.x), ry = rinv_bits(Y.y, VH.y, VL.y);
+            const f2 tt = f2_fma(f2_mul(c375, eh), eh, f2_mul(half, el));
+            const float2 Y = f2_get(y), R2 = f2_get(s);
+            const f2 sc = f2_make(ff_ulp_scale(Y.x), ff_ulp_scale(Y.y));
+            f2 tu, lo;
+            ff_units(f2_mul(half, x), sc, tu, lo);
+            lo = f2_fma(f2_fma(y, tt, f2_mul(half, xe)), sc, lo);
+            const float2 TU = f2_get(tu), LO = f2_get(ff_units_end(lo));
+            double rx = ff_add_units(Y.x, TU.x, LO.x), ry = ff_add_units(Y.y, TU.y, LO.y);
             // within 8 last places of a power of two the bits of y + v change scale
-            const bool ex = wide || !(R2.x > close2 && R2.x < 1e36f) ||
-                            ((__float_as_uint(Y.x) + 8u) & 0x7fffffu) < 16u;
-            const bool ey = wide || !(R2.y > close2 && R2.y < 1e36f) ||
-                            ((__float_as_uint(Y.y) + 8u) & 0x7fffffu) < 16u;
+            const bool ex = wide || !(R2.x > close2 && R2.x < 1e36f) || ff_near_binade(Y.x);
+            const bool ey = wide || !(R2.y > close2 && R2.y < 1e36f) || ff_near_binade(Y.y);
             if (ex || ey) {
                 if (ex && wx && i < A.n && b * kSymT + jx < A.n) rx = unit * rinv_fp64(A, i, b * kSymT + jx);
                 if (ey && wy && i < A.n && b * kSymT + jy < A.n) ry = unit * rinv_fp64(A, i, b * kSymT + jy);

@@ -4,20 +4,22 @@
 //
 // GB300 design.  FP64 runs at 1.68 instructions per clock and SM (measured, 1/74
 // of FP32), so the kernels minimise FP64 instructions per interaction.  Layouts:
+//   * tiled (kick_tile.cu): every ordered pair, one target per thread against groups
+//     of 64 sources in shared memory, a grid of equal blocks; on float expansions
+//     of the bodies, 3 FP64 instructions per pair (FP64) or none (mixed);
 //   * symmetric: each unordered pair once, its force to both bodies (Newton's
-//     third law); the pre-check rides along.  Used where it is predicted faster.
-//     The mixed form (kick_ff.cu) carries coordinates, terms and sums as float
-//     expansions on the FP32 pipe; the FP64 form (kick_sym_kernel, below) takes
-//     21 FP64 instructions per unordered pair;
-//   * tiled (kick_kernel): every ordered pair, one target per thread against
-//     source tiles in shared memory, an (i-tile x j-chunk) grid of equal blocks;
-//     for small N and the allocation-free entry point, with the pre-check as its
-//     own FP32 pass over i < j (precheck_kernel).
-// Both write partial sums folded in a fixed order (deterministic).  The rare
-// pairs inside rc_ij are found by an FP32 test on r^2 against a conservative
-// threshold; only those evaluate the changeover function.
+//     third law).  The mixed form (kick_ff.cu) is faster than the tiled one from
+//     N ~ 6,000 on (16,384: 0.68 ms against 0.99; 4,096: 0.111 against 0.092) and
+//     taken where predicted so; the FP64 form (kick_sym_kernel, below), 21 FP64
+//     instructions per unordered pair, only on request (20,011: 7.9 ms against
+//     2.9 tiled; 128: 0.106 against 0.028).
+// The pre-check rides along in both.  Both write partial sums folded in a fixed
+// order (deterministic).  The rare pairs inside rc_ij are found by an FP32 test on
+// r^2 against a conservative threshold; only those evaluate the changeover function.
+//   * kick_kernel: the tiled form without packed bodies, for the allocation-free
+//     entry point where its scratch does not hold them (N > 139,000).
 //
-// MIXED, tiled: FP64 displacement; r^2 formed as an unevaluated sum of two floats
+// kick_kernel, MIXED: FP64 displacement; r^2 formed as an unevaluated sum of two floats
 // from an exact integer split of the displacement (no FP64 work); FP32 rsqrt seed
 // y0; one Newton correction from the residual e = 1 - r^2 y0^2 (its leading
 // part 1 - u y0 by an FP32 FMA on the exact float product u y0, rounded once:
@@ -69,10 +71,7 @@ __device__ __forceinline__ float r2_to_float_trunc(double r2) {
     return __uint_as_float(fb);
 }
 
-// TP: semi-active test particles (Sec. 8.1): a test particle i takes only the
-// sources j < nm; the block that holds the boundary masks the test-particle
-// pairs, the blocks past it shorten their source range.
-template <bool MIXED, bool TP>
+template <bool MIXED>
 __global__ void __launch_bounds__(kKickThreads, kick_min_blocks(MIXED))
 kick_kernel(KickArgs A)
 {
@@ -97,10 +96,7 @@ kick_kernel(KickArgs A)
     }
 
     const int jbeg = blockIdx.y * A.chunk;
-    int jend = min(n, jbeg + A.chunk);
-    const int i0 = blockIdx.x * kKickThreads;
-    const bool straddle = TP && i0 < A.nm && i0 + kKickThreads > A.nm;
-    if (TP && i0 >= A.nm) jend = min(jend, A.nm);
+    const int jend = min(n, jbeg + A.chunk);
 
     double S0 = 0.0, S1 = 0.0, S2 = 0.0;   // compensated chunk totals
     double C0 = 0.0, C1 = 0.0, C2 = 0.0;
@@ -163,9 +159,6 @@ kick_kernel(KickArgs A)
             double mk = sm[k];
             float mh = 0.0f, ml = 0.0f;
             if (MIXED) { mh = smh[k]; ml = sml[k]; }
-            if (TP && straddle && i >= A.nm && j >= A.nm) {   // two test particles
-                mk = 0.0; mh = 0.0f; ml = 0.0f;
-            }
             // Changeover band (rare): K < 1 needs r < rc_ij.  K is flat (zero slope) at
             // r = rc, so the branch may follow the FP32 bound and K uses the r^2 above.
             // The branch runs on few lanes of a warp while the FP64 pipe charges the
@@ -572,30 +565,139 @@ kick_sym_kernel(SymArgs A)
     if (PC) sym_pc_flush(A, pcb[w], pend, lane);
 }
 
-// Folds the chunk partials in chunk order (TwoSum), scales by G and applies the
-// kick v += dt_half a; optionally stores a.
-__global__ void kick_finalize(const double *part, int nchunk, int tp_first, int tp_slots, int n, double G,
-                              double dt_half, double *vel, double *acc_out)
-{
+// A sum of doubles as a 96-bit whole number of 2^(e - 1075 - kFixLow): exact but for
+// the bits below 2^-25 of the last place of the largest term.  ~25 integer
+// operations per term instead of TwoSum's four FP64 ones (256 cycles of the pipe).
+constexpr int kFixLow = 25;                    // 53 + 25 + 17 bits for the number of terms + sign = 96
+struct Fix96 {
+    unsigned w0, w1;
+    int w2;
+    int e;                                     // largest exponent field met
+    bool bad;                                  // an infinite or NaN term
+
+    // the sum on the scale of exponent field f >= e
+    __device__ __forceinline__ void rescale(int f) {
+        const int d = f - e;
+        e = f;
+        const int s = w2 >> 31;
+        if (d >= 32) { w0 = w1; w1 = (unsigned)w2; w2 = s; }
+        if (d >= 64) { w0 = w1; w1 = (unsigned)w2; }
+        if (d >= 96) w0 = (unsigned)s;
+        const int r = d >= 96 ? 31 : d & 31;
+        w0 = __funnelshift_r(w0, w1, r);
+        w1 = __funnelshift_r(w1, (unsigned)w2, r);
+        w2 >>= r;
+    }
+    // += (x2 x1 x0 ^ s) + (s & 1), s = 0 or all ones
+    __device__ __forceinline__ void add_words(unsigned x0, unsigned x1, unsigned x2, unsigned s) {
+        unsigned r0, r1, r2;
+        asm("{\n\t.reg .u32 c, a, b;\n\tadd.cc.u32 c, %3, %3;\n\taddc.cc.u32 a, %4, %7;\n\taddc.cc.u32 b, %5, %8;\n\t"
+            "addc.u32 c, %6, %9;\n\tmov.u32 %0, a;\n\tmov.u32 %1, b;\n\tmov.u32 %2, c;\n\t}"
+            : "=r"(r0), "=r"(r1), "=r"(r2)
+            : "r"(s), "r"(w0), "r"(w1), "r"((unsigned)w2), "r"(x0 ^ s), "r"(x1 ^ s), "r"(x2 ^ s));
+        w0 = r0; w1 = r1; w2 = (int)r2;
+    }
+    __device__ __forceinline__ void add(double v) {
+        const int hi = __double2hiint(v);
+        const unsigned lo = (unsigned)__double2loint(v);
+        int f = (hi >> 20) & 0x7ff;
+        bad = bad || f == 0x7ff;
+        const unsigned mh = (hi & 0xfffff) | (f ? 0x100000u : 0u);
+        f = max(f, 1);
+        if (f > e) rescale(f);
+        const int d = min(e - f, 127);
+        unsigned x2 = mh >> (32 - kFixLow), x1 = __funnelshift_l(lo, mh, kFixLow), x0 = lo << kFixLow;
+        if (d & 32) { x0 = x1; x1 = x2; x2 = 0u; }
+        if (d & 64) { x0 = x2; x1 = x2 = 0u; }
+        x0 = __funnelshift_r(x0, x1, d);
+        x1 = __funnelshift_r(x1, x2, d);
+        x2 >>= d & 31;
+        add_words(x0, x1, x2, (unsigned)(hi >> 31));
+    }
+    __device__ __forceinline__ void add(Fix96 o) {
+        bad = bad || o.bad;
+        if (o.e > e) rescale(o.e);
+        if (o.e < e) o.rescale(e);
+        add_words(o.w0, o.w1, (unsigned)o.w2, 0u);
+    }
+    __device__ __forceinline__ double value() const {
+        const double t = fma((double)w2, 4294967296.0 * 4294967296.0, fma((double)w1, 4294967296.0, (double)w0));
+        return scalbn(t, e - 1075 - kFixLow);
+    }
+};
+
+// Sums a body's partials, one lane per component in each of the block's warps, scales by G (and from the
+// packed units, header) and applies the kick v += dt_half a; optionally stores
+// a.  COMP: partials are [6][n], with compensations; otherwise [3][n].  mass: the
+// partials are forces (unless the header says kFfTwoMass) -- of the symmetric mixed
+// kick.  Bodies from tp_first on have tp_slots partials.
+// N = 16,384, 128 slots: 24 us; one thread per component and TwoSum, each load
+// waiting for the last sum: 118 us with one thread per body, 64 us per component.
+// N = 2,048, 64 slots: 6.7 us.
+struct FoldArgs {
+    const double *part;
+    int nslot, tp_first, tp_slots, n;
+    double G;
+    const int *header;
+    const double *mass;
+    double dt_half;
+    double *vel, *acc_out;
+};
+constexpr int kFoldWarps = 4;                  // the slots of 32 bodies are dealt to the warps in turn
+template <bool COMP>
+__global__ void __launch_bounds__(32 * kFoldWarps) kick_fold_kernel(FoldArgs A) {
+    __shared__ Fix96 sh[kFoldWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane, c = blockIdx.y;
+    const int nslot = i >= A.n ? 0 : i >= A.tp_first ? A.tp_slots : A.nslot;
+    const size_t step = (size_t)(COMP ? 6 : 3) * A.n;
+    const double *p = A.part + (size_t)c * A.n + i;
+    Fix96 sum = {0u, 0u, 0, 1, false};
+    constexpr int B = COMP ? 4 : 8;            // slots whose loads are under way together
+    for (int q0 = w; q0 < nslot; q0 += B * kFoldWarps) {
+        double v[B], u[B];
+#pragma unroll
+        for (int b = 0; b < B; b++) {
+            const int q = q0 + b * kFoldWarps;
+            v[b] = q < nslot ? p[q * step] : 0.0;
+            if (COMP) u[b] = q < nslot ? p[q * step + (size_t)3 * A.n] : 0.0;
+        }
+#pragma unroll
+        for (int b = 0; b < B; b++) {
+            if (q0 + b * kFoldWarps >= A.nslot) break;
+            sum.add(v[b]);
+            if (COMP) sum.add(u[b]);
+        }
+    }
+    sh[w][lane] = sum;
+    __syncthreads();
+    if (w || i >= A.n) return;
+#pragma unroll
+    for (int k = 1; k < kFoldWarps; k++) sum.add(sh[k][lane]);
+    const double t = sum.bad ? __longlong_as_double(0x7ff8000000000000ll) : sum.value();
+    double f = A.G;
+    if (A.header) {
+        f *= scalbn(1.0, A.header[1] - 2 * A.header[2]);
+        if (A.mass && !(A.header[0] & kFfTwoMass)) f /= A.mass[i] * scalbn(1.0, -A.header[1]);
+    }
+    const double a = f * t;
+    if (A.acc_out) A.acc_out[(size_t)c * A.n + i] = a;
+    if (A.dt_half != 0.0) A.vel[(size_t)c * A.n + i] += A.dt_half * a;
+}
+
+cudaError_t launch_fold(const FoldArgs &A, bool comp, cudaStream_t stream) {
+    const dim3 grid((A.n + 31) / 32, 3);
+    if (comp) kick_fold_kernel<true><<<grid, 32 * kFoldWarps, 0, stream>>>(A);
+    else kick_fold_kernel<false><<<grid, 32 * kFoldWarps, 0, stream>>>(A);
+    return cudaGetLastError();
+}
+
+__global__ void raw_thresholds_kernel(int n, const double *rc, double *rc2, float *thr) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    // symmetric kick with test particles: the bodies of the test-particle
-    // super-ranges have partials only from the ranges holding large bodies
-    if (i >= tp_first) nchunk = tp_slots;
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        double S = 0.0, C = 0.0;
-        for (int q = 0; q < nchunk; q++) {
-            const double *p = part + (size_t)q * 6 * n;
-            double t, e;
-            two_sum_ordered(S, p[(size_t)c * n + i], t, e);
-            S = t;
-            C += e + p[(size_t)(3 + c) * n + i];
-        }
-        const double a = G * (S + C);
-        if (acc_out) acc_out[(size_t)c * n + i] = a;
-        if (dt_half != 0.0) vel[(size_t)c * n + i] += dt_half * a;
-    }
+    const double r2 = __dmul_rn(rc[i], rc[i]);
+    rc2[i] = r2;
+    thr[i] = fmaxf(__double2float_ru(r2) * 1.0000153f, 1.17549435e-38f);
 }
 
 void kick_geometry(int n, int num_sms, int *chunk, int *nchunk) {
@@ -677,23 +779,16 @@ double sym_schedule(int nT, int P, int slots, int Xmax, double ovh, std::vector<
 }
 
 template <bool MIXED>
-SymPlan sym_plan(int n, int nm, int num_sms, int layout, int req_P) {
+SymPlan sym_plan(int n, int nm, int num_sms, double t_best, int req_P) {
     SymPlan best;
     const int nT = (n + kSymT - 1) / kSymT;
-    // SM cycles per unordered pair (symmetric), per ordered pair (kick_kernel)
-    // and per partial slot per body in the fold: mixed 9.1 ms and 47.0 ms at
-    // N = 65,540 (P = 3; tiled), FP64 81.8 and 133 ms
-    const double c_sym = MIXED ? 1.32 : 12.2, c_old = MIXED ? 3.5 : 9.7, c_fin = MIXED ? 7.0 : 9.7;
+    // SM cycles per unordered pair and per partial slot per body in the fold
+    const double c_sym = MIXED ? 1.32 : 12.2, c_fin = MIXED ? 7.0 : 9.7;
     // fixed work per item, in tile pairs (mixed: fits the times over P at N = 16,384,
     // 65,540 and 131,071, all within 3 % of the best)
     const double ovh = MIXED ? 0.05 : 0.0;
-    // predicted time in SM cycles: kick_kernel at 95 % balance;
-    // the symmetric kick's makespan (tile pairs per block, each block at 1/nb
-    // of its SM) plus the finalize's slots
-    if (layout == GENGA_KICK_TILED) return best;
-    // tiled: the large bodies' rows meet every source, the test particles' rows the large ones
-    const double t_old = c_old * (2.0 * n * nm - (double)nm * nm) / (0.95 * num_sms);
-    double t_best = layout == GENGA_KICK_SYMMETRIC ? 1e300 : t_old;
+    // predicted time in SM cycles: the makespan (tile pairs per block, each block at
+    // 1/nb of its SM) plus the fold's slots
     for (int P = req_P > 0 ? req_P : 1; P <= (req_P > 0 ? req_P : kSymMaxP); P++) {
         const int nS = (nT + P - 1) / P;
         if ((double)nS * 6.0 * n * sizeof(double) > 16.0 * (1ull << 30)) continue;   // partial sums
@@ -720,16 +815,28 @@ SymPlan sym_plan(int n, int nm, int num_sms, int layout, int req_P) {
 
 }  // namespace
 
+constexpr size_t kMaxPart = ((size_t)16 << 30) / sizeof(double);      // partial sums, at most
+
 // Chooses the kick geometry for the current N and precision and makes sure the
-// partial-sum and symmetric-kick buffers are large enough.
+// partial-sum and packed-body buffers are large enough.
 cudaError_t kick_reserve(genga_system *s) {
     const int n = (int)s->n;
     if (s->kick_chunk == 0) kick_geometry(n, s->num_sms, &s->kick_chunk, &s->kick_nchunk);
-    const int prec = s->p.precision;
+    const bool mixed = s->p.precision == GENGA_MIXED;
     const int nm = tp_bound(s);
-    if (s->ksym_n != s->n || s->ksym_prec != prec || s->ksym_nm != nm) {
-        SymPlan plan = prec == GENGA_MIXED ? sym_plan<true>(n, nm, s->num_sms, s->ksym_layout, s->ksym_req_P)
-                                           : sym_plan<false>(n, nm, s->num_sms, s->ksym_layout, s->ksym_req_P);
+    GENGA_CUDA_TRY(ff_reserve(s));
+    if (s->ksym_n != s->n || s->ksym_prec != s->p.precision || s->ksym_nm != nm) {
+        const TilePlan tile = tile_plan(n, nm, s->num_sms, mixed, kMaxPart);
+        SymPlan plan;
+        // FP64: the tiled kick is the faster one at every N
+        if (s->ksym_layout == GENGA_KICK_SYMMETRIC || (s->ksym_layout == GENGA_KICK_AUTO && mixed)) {
+            const double t = s->ksym_layout == GENGA_KICK_AUTO ? tile.cycles : 1e300;
+            plan = mixed ? sym_plan<true>(n, nm, s->num_sms, t, s->ksym_req_P)
+                         : sym_plan<false>(n, nm, s->num_sms, t, s->ksym_req_P);
+        }
+        if (!plan.P && !tile.chunk) return cudaErrorMemoryAllocation;
+        s->ktile_chunk = tile.chunk;
+        s->ktile_nchunk = tile.nchunk;
         s->ksym_P = plan.P;
         s->ksym_nS = plan.nS;
         s->ksym_blocks = plan.blocks;
@@ -747,9 +854,7 @@ cudaError_t kick_reserve(genga_system *s) {
                 GENGA_CUDA_TRY(cudaMemcpy(s->ksym_list, plan.items.data(), sizeof(int2) * plan.items.size(),
                                           cudaMemcpyHostToDevice));
             if (!s->ksym_ctr) GENGA_CUDA_TRY(cudaMalloc((void **)&s->ksym_ctr, sizeof(unsigned)));
-            if (prec == GENGA_MIXED) {
-                GENGA_CUDA_TRY(ff_reserve(s));
-            } else if ((size_t)n > s->ksym_body_cap) {
+            if (!mixed && (size_t)n > s->ksym_body_cap) {
                 for (void *q : {(void *)s->ksym_irc, (void *)s->ksym_thrpc})
                     if (q) cudaFree(q);
                 s->ksym_irc = nullptr; s->ksym_thrpc = nullptr;
@@ -760,10 +865,10 @@ cudaError_t kick_reserve(genga_system *s) {
             }
         }
         s->ksym_n = s->n;
-        s->ksym_prec = prec;
+        s->ksym_prec = s->p.precision;
         s->ksym_nm = nm;
     }
-    const size_t need = (size_t)std::max(s->kick_nchunk, s->ksym_nS) * 6 * (size_t)n;
+    const size_t need = (size_t)(s->ksym_P ? s->ksym_nS : s->ktile_nchunk) * (s->ksym_P && !mixed ? 6 : 3) * (size_t)n;
     if (need > s->kick_part_cap) {
         if (s->kick_part) cudaFree(s->kick_part);
         s->kick_part = nullptr;
@@ -777,69 +882,54 @@ cudaError_t kick_reserve(genga_system *s) {
 cudaError_t launch_kick(genga_system *s, double dt_half, bool precheck, double *acc_out) {
     const int n = (int)s->n;
     GENGA_CUDA_TRY(kick_reserve(s));
-    KickArgs A = make_args(s, false);
-    const bool mixed = s->p.precision == GENGA_MIXED;
-    int nparts = s->kick_nchunk;
-    FfPack ff;
-    int tp_first = n, tp_slots = 0;               // bodies from tp_first fold tp_slots partials
-    if (s->ksym_P > 0) {
-        // symmetric layout; the pre-check, if asked for, rides along
-        SymArgs S;
-        S.x = A.x; S.y = A.y; S.z = A.z; S.m = A.m;
-        S.irc = s->ksym_irc; S.thr = A.thr_rc; S.thr_pc = s->ksym_thrpc;
-        S.ircf = nullptr; S.body = nullptr; S.ff_header = nullptr; S.tmass = nullptr;
-        S.n = n; S.nT = (n + kSymT - 1) / kSymT; S.P = s->ksym_P; S.nItems = s->ksym_items;
-        S.nm = A.nm;
-        S.items = s->ksym_list; S.ctr = s->ksym_ctr; S.part = s->kick_part;
-        S.pc2 = s->rcl[0].pc2;
-        S.cand = s->cand; S.cand_count = &s->ctr->cand_count; S.cand_cap = (unsigned long long)s->cand_cap;
+    const bool mixed = s->p.precision == GENGA_MIXED, sym = s->ksym_P > 0;
+    // the pre-check, if asked for, rides along
+    SymArgs S;
+    S.x = s->pos; S.y = s->pos + n; S.z = s->pos + 2 * (size_t)n; S.m = s->mass;
+    S.rc = s->rcl[0].rc; S.irc = s->ksym_irc; S.thr = s->rcl[0].thr_rc; S.thr_pc = s->ksym_thrpc;
+    S.n = n; S.nT = (n + kSymT - 1) / kSymT; S.P = s->ksym_P; S.nItems = s->ksym_items;
+    S.nm = tp_bound(s);
+    S.items = s->ksym_list; S.ctr = s->ksym_ctr; S.part = s->kick_part;
+    S.pc2 = s->rcl[0].pc2;
+    S.cand = s->cand; S.cand_count = &s->ctr->cand_count; S.cand_cap = (unsigned long long)s->cand_cap;
+    FfPack ff = ff_pack_args(s);
+    S.body = ff.body; S.ircf = ff.ircf; S.ff_header = ff.header; S.tmass = ff.tmass;
+    const bool tp = S.nm < n;
+    FoldArgs F;
+    F.part = s->kick_part; F.nslot = sym ? s->ksym_nS : s->ktile_nchunk; F.tp_first = n; F.tp_slots = 0; F.n = n;
+    F.G = s->p.G; F.header = ff.header; F.mass = nullptr; F.dt_half = dt_half; F.vel = s->vel; F.acc_out = acc_out;
+    if (sym && !mixed) {
+        F.header = nullptr;
+        kick_pack_kernel<<<(n + 255) / 256, 256, 0, s->stream>>>(s->rcl[0].rc, S.pc2, n, s->ksym_irc, s->ksym_thrpc);
+        ++s->launches;
+        GENGA_CUDA_TRY(cudaMemsetAsync(s->ksym_ctr, 0, sizeof(unsigned), s->stream));
+        if (precheck) GENGA_CUDA_TRY(cudaMemsetAsync(&s->ctr->cand_count, 0, sizeof(unsigned long long), s->stream));
         const unsigned nb = (unsigned)s->ksym_blocks;
-        const bool tp = A.nm < n;
-        if (mixed) {
-            ff = ff_pack_args(s);
-            ff.ctr = s->ksym_ctr;
-            if (precheck) ff.cand_count = &s->ctr->cand_count;
-            S.body = ff.body; S.ircf = ff.ircf; S.ff_header = ff.header; S.tmass = ff.tmass;
-            GENGA_CUDA_TRY(launch_ff_pack(ff, s->stream, &s->launches));
-            GENGA_CUDA_TRY(launch_sym_ff(S, precheck, (int)nb, s->stream));
-        } else {
-            kick_pack_kernel<<<(n + 255) / 256, 256, 0, s->stream>>>(s->rcl[0].rc, S.pc2, n, s->ksym_irc,
-                                                                     s->ksym_thrpc);
-            ++s->launches;
-            GENGA_CUDA_TRY(cudaMemsetAsync(s->ksym_ctr, 0, sizeof(unsigned), s->stream));
-            if (precheck)
-                GENGA_CUDA_TRY(cudaMemsetAsync(&s->ctr->cand_count, 0, sizeof(unsigned long long), s->stream));
-            const size_t smem = sym_smem(s->ksym_P);
+        const size_t smem = sym_smem(s->ksym_P);
 #define GENGA_SYM_LAUNCH(PCK, TPK) kick_sym_kernel<PCK, TPK><<<nb, kSymT, smem, s->stream>>>(S)
-            if (tp) { if (precheck) GENGA_SYM_LAUNCH(true, true); else GENGA_SYM_LAUNCH(false, true); }
-            else { if (precheck) GENGA_SYM_LAUNCH(true, false); else GENGA_SYM_LAUNCH(false, false); }
+        if (tp) { if (precheck) GENGA_SYM_LAUNCH(true, true); else GENGA_SYM_LAUNCH(false, true); }
+        else { if (precheck) GENGA_SYM_LAUNCH(true, false); else GENGA_SYM_LAUNCH(false, false); }
 #undef GENGA_SYM_LAUNCH
-        }
-        if (tp) {
-            tp_first = (int)std::min<int64_t>((int64_t)s->ksym_R * s->ksym_P * kSymT, n);
-            tp_slots = s->ksym_R;
-        }
-        nparts = s->ksym_nS;
+        GENGA_CUDA_TRY(cudaGetLastError());
     } else {
-        if (precheck) GENGA_CUDA_TRY(launch_precheck_only(s));
-        dim3 grid((n + kKickThreads - 1) / kKickThreads, s->kick_nchunk);
-        if (A.nm < n) {
-            if (mixed) kick_kernel<true, true><<<grid, kKickThreads, 0, s->stream>>>(A);
-            else kick_kernel<false, true><<<grid, kKickThreads, 0, s->stream>>>(A);
+        if (sym) ff.ctr = s->ksym_ctr;
+        if (precheck) ff.cand_count = &s->ctr->cand_count;
+        GENGA_CUDA_TRY(launch_ff_pack(ff, s->stream, &s->launches));
+        if (sym) {
+            F.mass = s->mass;
+            GENGA_CUDA_TRY(launch_sym_ff(S, precheck, s->ksym_blocks, s->stream));
         } else {
-            if (mixed) kick_kernel<true, false><<<grid, kKickThreads, 0, s->stream>>>(A);
-            else kick_kernel<false, false><<<grid, kKickThreads, 0, s->stream>>>(A);
+            GENGA_CUDA_TRY(launch_tile_kick(S, s->ktile_chunk, s->ktile_nchunk, mixed, precheck, s->stream));
         }
     }
-    ++s->launches;
-    GENGA_CUDA_TRY(cudaGetLastError());
-    if (s->ksym_P > 0 && mixed)
-        return launch_ff_finalize(ff, s->kick_part, nparts, tp_first, tp_slots, s->p.G, dt_half, s->vel, acc_out,
-                                  s->stream, &s->launches);
-    kick_finalize<<<(n + 255) / 256, 256, 0, s->stream>>>(s->kick_part, nparts, tp_first, tp_slots, n, s->p.G,
-                                                          dt_half, s->vel, acc_out);
-    ++s->launches;
-    return cudaGetLastError();
+    if (tp) {                                      // test particles: partials of the large bodies' ranges only
+        const int first = sym ? s->ksym_R * s->ksym_P * kSymT : (S.nm + kSymT - 1) / kSymT * kSymT;
+        F.tp_first = std::min(first, n);
+        F.tp_slots = sym ? s->ksym_R : ((S.nm + 63) / 64 * 32 + s->ktile_chunk - 1) / s->ktile_chunk;
+    }
+    GENGA_CUDA_TRY(launch_fold(F, sym && !mixed, s->stream));
+    s->launches += 2;
+    return cudaSuccess;
 }
 
 cudaError_t launch_precheck_only(genga_system *s) {
@@ -854,9 +944,36 @@ cudaError_t launch_precheck_only(genga_system *s) {
     return cudaGetLastError();
 }
 
-// Launches the kick (no pre-check) on caller-provided arrays, with the number of
-// j-chunks capped at max_nchunk; used by the allocation-free entry point.
-cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, int max_nchunk, cudaStream_t stream) {
+// Launches the kick (no pre-check) on caller-provided arrays; used by the
+// allocation-free entry point.  k.scratch holds the packed bodies and the partial
+// sums of the tiled kick (kick_tile.cu) where they fit, else thresholds and the
+// partial sums of kick_kernel.
+cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, cudaStream_t stream) {
+    const size_t N = (size_t)k.n;
+    FoldArgs F;
+    F.nslot = 0; F.tp_first = k.n; F.tp_slots = 0; F.n = k.n; F.G = k.G; F.header = nullptr; F.mass = nullptr;
+    F.dt_half = k.dt_half; F.vel = k.vel; F.acc_out = k.acc_out;
+    const size_t packed = (ff_bytes(k.n) / sizeof(double) + 31) / 32 * 32;      // doubles
+    TilePlan tile;
+    if (packed < k.room) tile = tile_plan(k.n, k.n, num_sms, k.mixed, k.room - packed);
+    if (tile.chunk) {
+        FfPack ff;
+        ff.pos = k.pos; ff.m = k.mass; ff.rc = k.rc; ff.pc2 = nullptr; ff.n = k.n; ff.nT = (k.n + kSymT - 1) / kSymT;
+        ff_place(ff, k.scratch, ff.nT);
+        ff.ctr = nullptr; ff.cand_count = nullptr;
+        SymArgs S = {};
+        S.x = k.pos; S.y = k.pos + N; S.z = k.pos + 2 * N; S.m = k.mass; S.rc = k.rc;
+        S.n = S.nm = k.n; S.nT = ff.nT; S.part = k.scratch + packed;
+        S.body = ff.body; S.ircf = ff.ircf; S.ff_header = ff.header; S.tmass = ff.tmass;
+        int64_t launches = 0;
+        GENGA_CUDA_TRY(launch_ff_pack(ff, stream, &launches));
+        GENGA_CUDA_TRY(launch_tile_kick(S, tile.chunk, tile.nchunk, k.mixed, false, stream));
+        F.part = S.part; F.nslot = tile.nchunk; F.header = ff.header;
+        return launch_fold(F, false, stream);
+    }
+    const size_t part_off = (N + (N + 1) / 2 + 31) / 32 * 32;                   // 256-byte aligned
+    const int max_nchunk = part_off < k.room ? (int)((k.room - part_off) / (6 * N)) : 0;
+    if (max_nchunk < 1) return cudaErrorMemoryAllocation;
     int chunk, nchunk;
     kick_geometry(k.n, num_sms, &chunk, &nchunk);
     if (nchunk > max_nchunk) {
@@ -865,18 +982,19 @@ cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, int max_nchunk, cudaS
         chunk = tiles_per_chunk * kTile;
         nchunk = (k.n + chunk - 1) / chunk;
     }
-    KickArgs A;
-    A.x = k.pos; A.y = k.pos + k.n; A.z = k.pos + 2 * (size_t)k.n; A.m = k.mass;
-    A.rc = k.rc; A.rc2 = k.rc2; A.pc2 = nullptr; A.thr_rc = k.thr;
-    A.n = k.n; A.nm = k.n; A.chunk = chunk; A.part = k.part;
-    A.cand = nullptr; A.cand_count = nullptr; A.cand_cap = 0;
-    dim3 grid((k.n + kKickThreads - 1) / kKickThreads, nchunk);
-    if (k.mixed) kick_kernel<true, false><<<grid, kKickThreads, 0, stream>>>(A);
-    else kick_kernel<false, false><<<grid, kKickThreads, 0, stream>>>(A);
+    float *thr = (float *)(k.scratch + N);
+    raw_thresholds_kernel<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(k.n, k.rc, k.scratch, thr);
     GENGA_CUDA_TRY(cudaGetLastError());
-    kick_finalize<<<(k.n + 255) / 256, 256, 0, stream>>>(k.part, nchunk, k.n, 0, k.n, k.G, k.dt_half, k.vel,
-                                                         k.acc_out);
-    return cudaGetLastError();
+    KickArgs A = {};
+    A.x = k.pos; A.y = k.pos + k.n; A.z = k.pos + 2 * N; A.m = k.mass;
+    A.rc = k.rc; A.thr_rc = thr;
+    A.n = A.nm = k.n; A.chunk = chunk; A.part = k.scratch + part_off;
+    dim3 grid((k.n + kKickThreads - 1) / kKickThreads, nchunk);
+    if (k.mixed) kick_kernel<true><<<grid, kKickThreads, 0, stream>>>(A);
+    else kick_kernel<false><<<grid, kKickThreads, 0, stream>>>(A);
+    GENGA_CUDA_TRY(cudaGetLastError());
+    F.part = A.part; F.nslot = nchunk;
+    return launch_fold(F, true, stream);
 }
 
 int kick_nchunk_for(int n, int num_sms) {
@@ -905,10 +1023,8 @@ extern "C" int genga_get_kick_layout(genga_system_t *s, int32_t *layout, int32_t
     const bool sym = s->ksym_P > 0;
     if (layout) *layout = sym ? GENGA_KICK_SYMMETRIC : GENGA_KICK_TILED;
     if (P) *P = sym ? s->ksym_P : 0;
-    if (slots) *slots = sym ? s->ksym_nS : s->kick_nchunk;
-    if (blocks)
-        *blocks = sym ? s->ksym_blocks
-                      : (int32_t)(((s->n + kKickThreads - 1) / kKickThreads) * (int64_t)s->kick_nchunk);
+    if (slots) *slots = sym ? s->ksym_nS : s->ktile_nchunk;
+    if (blocks) *blocks = sym ? s->ksym_blocks : (int32_t)((s->n + kSymT - 1) / kSymT * s->ktile_nchunk);
     return GENGA_OK;
 }
 

@@ -35,14 +35,12 @@
 //
 // Two pairs per instruction (f32x2): a lane holds one body i and two travelling
 // bodies j (l and l + 32 of a 64-body group).
-#include "ff2.cuh"
-#include "kick_sym.cuh"
+#include "ff_pair.cuh"
 
 namespace genga {
 namespace {
 
 constexpr int kFfThreads = 64;                 // two warps: 64 rows each of the 128-body tile
-constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2;      // instances of the pair loop
 
 // Chosen by measurement at N = 65,540 (ms per kick): rows per lane 2 (9.5; 1:
 // 10.3 -- the j data and shuffles serve two rows), 2 steps unrolled (1: 9.45, 4:
@@ -63,69 +61,6 @@ struct IBody {                                 // a lane's row, in both halves: 
     int i;
 };
 
-// One coordinate's displacement as two floats.
-__device__ __forceinline__ void ff_disp(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 nli, f2 &H, f2 &L) {
-    f2 e;
-    f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e);
-    L = f2_add(e, f2_add(lj, nli));
-}
-// The same with the fourth parts.
-__device__ __forceinline__ void ff_disp4(f2 hj, f2 mj, f2 lj, f2 kj, f2 nhi, f2 nmi, f2 nli, f2 nki, f2 &H, f2 &L) {
-    f2 e1, e2, dl, el;
-    f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e1);
-    f2_two_sum(lj, nli, dl, el);
-    f2_two_sum(e1, dl, e1, e2);
-    f2_fast_two_sum(H, e1, H, e1);
-    L = f2_add(e1, f2_add(e2, f2_add(el, f2_add(kj, nki))));
-}
-
-// g w as two floats (g = gh + gl, w + wl)
-__device__ __forceinline__ void ff_coeff(f2 gh, f2 gl, f2 w, f2 wl, f2 &ch, f2 &cl) {
-    ch = f2_mul(gh, w);
-    cl = f2_fma(gh, wl, f2_fma(gl, w, f2_fma(gh, w, f2_neg(ch))));
-}
-// (ch + cl) d as two floats
-__device__ __forceinline__ void ff_term(f2 ch, f2 cl, const f2 (&H)[3], const f2 (&L)[3], f2 (&th)[3], f2 (&te)[3]) {
-#pragma unroll
-    for (int c = 0; c < 3; c++) th[c] = f2_mul(ch, H[c]);
-#pragma unroll
-    for (int c = 0; c < 3; c++) te[c] = f2_fma(ch, H[c], f2_neg(th[c]));
-#pragma unroll
-    for (int c = 0; c < 3; c++) te[c] = f2_fma(ch, L[c], te[c]);
-#pragma unroll
-    for (int c = 0; c < 3; c++) te[c] = f2_fma(cl, H[c], te[c]);
-}
-
-// The changeover function at r^2 = s2 + tail, 1/rc_ij = ih + il: r as two floats
-// from a fresh seed on the normalised r^2 (a small residual, so that r is good
-// to 2^-47), then changeover_ff.
-__device__ __forceinline__ void ff_changeover(float s2, float tail, float ih, float il, float &Kh, float &Kl) {
-    ff_fast2sum(s2, tail);
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s2));
-    y = fmaf(0.5f * y, fmaf(-(s2 * y), y, 1.0f), y);
-    const float u = s2 * y, ue = fmaf(s2, y, -u);
-    const float e = fmaf(-u, y, 1.0f) - fmaf(tail, y * y, ue * y);
-    changeover_ff(u, ue, tail, y, e, ih, il, Kh, Kl);
-}
-
-// A close pair (r < 2^-20 S): its displacement reaches below the second grid, so
-// that h and m no longer give its leading float.  FP64 from the positions, K
-// included: H + L, K r^-3 = w + wl.
-struct FfClose { float H[3], L[3], w, wl; };
-__device__ __forceinline__ void ff_close(const SymArgs &A, int i, int j, float ih, float il, FfClose &o) {
-    const double xs = scalbn(1.0, -A.ff_header[2]);
-    const double d[3] = {(A.x[j] - A.x[i]) * xs, (A.y[j] - A.y[i]) * xs, (A.z[j] - A.z[i]) * xs};
-    const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])), y = rsqrt(r2);
-    const double w = changeover_fast(r2 * y, (double)ih + (double)il) * (y * y * y);
-    for (int c = 0; c < 3; c++) {
-        o.H[c] = __double2float_rn(d[c]);
-        o.L[c] = __double2float_rn(d[c] - (double)o.H[c]);
-    }
-    o.w = __double2float_rn(w);
-    o.wl = __double2float_rn(w - (double)o.w);
-}
-
 // sum += h + l, in the uniform instance times m_i m_j.
 template <int MODE>
 __device__ __forceinline__ void ff_flush(double &sum, double mm, float h, float l) {
@@ -144,7 +79,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                                         double mm, uint2 *pcbuf, int &pend, int lane) {
     constexpr bool GEN = MODE == kFfGeneral;
     f2 ih[kFfR][3], il[kFfR][3], jh[3], jl[3];
-    const f2 one = f2_dup(1.0f), two = f2_dup(2.0f), c15 = f2_dup(1.5f), c1875 = f2_dup(1.875f);
+    const f2 one = f2_dup(1.0f);
     const float4 *group = tile + (jb >> 1);
 #pragma unroll 1
     for (int tb = 0; tb < 32; tb += kFfFlush) {
@@ -192,27 +127,15 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                     ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I[r].h[1], I[r].m[1], I[r].l[1], H[r][1], L[r][1]);
                     ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I[r].h[2], I[r].m[2], I[r].l[2], H[r][2], L[r][2]);
                 }
-                // r^2 = s2 + tail
-                f2 s2 = f2_mul(H[r][0], H[r][0]), tail = f2_fma(H[r][0], H[r][0], f2_neg(s2));
-                f2_acc_mul_pos(s2, tail, H[r][1], H[r][1]);
-                f2_acc_mul_pos(s2, tail, H[r][2], H[r][2]);
-                tail = f2_fma(two, f2_fma(H[r][2], L[r][2], f2_fma(H[r][1], L[r][1], f2_mul(H[r][0], L[r][0]))), tail);
-                f2_fast_two_sum(s2, tail, s2, tail);
+                f2 s2, tail;
+                ff_r2(H[r], L[r], s2, tail);
                 if (GEN) {
                     s2 = f2_select(want[r][0], want[r][1], s2, one);
                     tail = f2_select(want[r][0], want[r][1], tail, 0ull);
                 }
                 S[r] = f2_get(s2);
                 Tl[r] = f2_get(tail);
-                // r^-3 = w + wl
-                const f2 y = f2_rsqrt(s2);
-                const f2 u = f2_mul(s2, y), ue = f2_fma(s2, y, f2_neg(u));      // s2 y exactly
-                const f2 p = f2_mul(y, y), pe = f2_fma(y, y, f2_neg(p));
-                w[r] = f2_mul(p, y);
-                const f2 qe = f2_fma(pe, y, f2_fma(p, y, f2_neg(w[r])));
-                const f2 ef = f2_sub(f2_fma(f2_neg(u), y, one), f2_fma(tail, p, f2_mul(ue, y)));
-                wl[r] = f2_fma(w[r], f2_mul(f2_fma(c1875, ef, c15), ef), qe);
-                f2_fast_two_sum(w[r], wl[r], w[r], wl[r]);
+                ff_inv_r3(s2, tail, w[r], wl[r]);
                 near = near || S[r].x < fmaxf(I[r].tn, tj.x) || S[r].y < fmaxf(I[r].tn, tj.y);
             }
             if (PC ? __any_sync(0xffffffffu, near) : near) {
@@ -239,7 +162,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                             float wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
                             if ((h ? S[r].y : S[r].x) < close2) {
                                 FfClose o;
-                                ff_close(A, I[r].i, jglob + k + 32 * h, ih, il, o);
+                                ff_close(A.x, A.y, A.z, A.ff_header[2], I[r].i, jglob + k + 32 * h, ih, il, o);
 #pragma unroll
                                 for (int c = 0; c < 3; c++) {
                                     const float2 u = f2_get(H[r][c]), v = f2_get(L[r][c]);
@@ -484,7 +407,9 @@ __device__ __forceinline__ void ff_split(double x, double mag1, double mag2, flo
     k = (float)(s - (double)l);
 }
 
-// One block per tile.
+// Four blocks per tile, one for each coordinate and one for masses, radii and the
+// header: the work is FP64 instructions, ~60 per body, and four SMs do a tile in
+// two thirds of the time of one (N = 2,048: 5.1 us against 6.9).
 __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     __shared__ float4 sh[kSymT / 32];
     __shared__ double tm;
@@ -499,10 +424,22 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     // the floats' range does not depend on the caller's units
     const int ex = max(ilogbf(fmaxf(bd.x, 1e-30f)) + 1, -90);
     const int es = max(ilogbf(fminf(fmaxf(bd.y, 1e-30f), 1e30f)), ex - 20), em = ilogbf(fmaxf(bd.z, 1e-38f));
-    const double mag1 = scalbn(1.5, 52 - 22 + ex - es), mag2 = scalbn(1.5, 52 - 45 + ex - es);
-    const double mscale = scalbn(1.0, -em), xscale = scalbn(1.0, -es);
-    const float close2 = scalbnf(1.0f, 2 * (ex - es - 20));      // (2^-20 S)^2
+    const double xscale = scalbn(1.0, -es);
     const int i = blockIdx.x * kSymT + threadIdx.x;
+    // component of row q, first (0) or second (2) half: + 1 for the bodies l + 32
+    float *B = reinterpret_cast<float *>(A.body + (size_t)(i >> 7) * kFfTile + ((i >> 6) & 1) * 32 + (i & 31)) +
+               ((i >> 5) & 1);
+    constexpr int R = 4 * kFfRow;
+    if (blockIdx.y < 3) {
+        const int c = blockIdx.y, q = c == 2 ? R : 2 * c;       // z: first half of the next row
+        float h = (float)pad_pos(i & (kSymT - 1)), m = 0.0f, l = 0.0f, k = 0.0f;
+        if (i < A.n)
+            ff_split(A.pos[(size_t)c * A.n + i] * xscale, scalbn(1.5, 52 - 22 + ex - es), scalbn(1.5, 52 - 45 + ex - es),
+                     h, m, l, k);
+        B[q] = h; B[2 * R + q] = m; B[4 * R + q] = l; B[6 * R + q] = k;
+        return;
+    }
+    const float close2 = scalbnf(1.0f, 2 * (ex - es - 17));      // (2^-17 S)^2
     if (i == 0) {
         A.header[0] = (scalbnf(1.0f, ex - 18) > bd.y ? kFfWide : 0) | (scalbnf(bd.z, -40) >= bd.w ? kFfTwoMass : 0);
         A.header[1] = em;
@@ -512,17 +449,15 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
         if (A.cand_count) *A.cand_count = 0ull;
     }
     // the common (scaled) mass of a full tile of equal masses, else 0
-    const double ms = i < A.n ? A.m[i] * mscale : 0.0;
+    const double ms = i < A.n ? A.m[i] * scalbn(1.0, -em) : 0.0;
     if (threadIdx.x == 0) tm = ms;
     __syncthreads();
     const int differ = __syncthreads_or(ms != tm || !(ms > 0.0));
     if (threadIdx.x == 0) A.tmass[blockIdx.x] = differ ? 0.0 : ms;
-    float h[3], m[3], l[3], k[3], mh = 0.0f, ml = 0.0f, thr = 0.0f, thp = 0.0f;
+    float mh = 0.0f, ml = 0.0f, thr = 0.0f, thp = 0.0f;
     float2 ircf = make_float2(0.0f, 0.0f);
     if (i < A.n) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) ff_split(A.pos[(size_t)c * A.n + i] * xscale, mag1, mag2, h[c], m[c], l[c], k[c]);
-        const double rc = A.rc[i], rcs = rc * xscale, pc2 = A.pc2[i] * xscale * xscale;
+        const double rc = A.rc[i], rcs = rc * xscale, pc2 = A.pc2 ? A.pc2[i] * xscale * xscale : 0.0;
         mh = __double2float_rn(ms);
         ml = __double2float_rn(ms - (double)mh);
         // upper bounds of rc^2 and pc2, and of the close pairs' r^2: rounded up,
@@ -531,47 +466,12 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
         thr = fmaxf(__double2float_ru(rcs * rcs), close2) * 1.0000153f;
         thp = fmaxf(__double2float_ru(pc2) * 1.0000153f, thr);
         ircf = ff_of_irc(inv_rc(rc) * scalbn(1.0, es));
-    } else {
-        const float p = (float)pad_pos(i & (kSymT - 1));
-#pragma unroll
-        for (int c = 0; c < 3; c++) { h[c] = p; m[c] = l[c] = k[c] = 0.0f; }
     }
-    // component of row q, first (0) or second (2) half: + 1 for the bodies l + 32
-    float *B = reinterpret_cast<float *>(A.body + (size_t)(i >> 7) * kFfTile + ((i >> 6) & 1) * 32 + (i & 31)) +
-               ((i >> 5) & 1);
-    constexpr int R = 4 * kFfRow;
-    B[0] = h[0]; B[2] = h[1]; B[R] = h[2]; B[R + 2] = mh;
-    B[2 * R] = m[0]; B[2 * R + 2] = m[1]; B[3 * R] = m[2]; B[3 * R + 2] = ml;
-    B[4 * R] = l[0]; B[4 * R + 2] = l[1]; B[5 * R] = l[2]; B[5 * R + 2] = thr;
-    B[6 * R] = k[0]; B[6 * R + 2] = k[1]; B[7 * R] = k[2]; B[7 * R + 2] = thp;
+    B[R + 2] = mh;
+    B[3 * R + 2] = ml;
+    B[5 * R + 2] = thr;
+    B[7 * R + 2] = thp;
     A.ircf[i] = ircf;
-}
-
-// Folds the partials in slot order (TwoSum), turns forces into accelerations
-// (kFfTwoMass: they are), scales by G and applies the kick v += dt_half a;
-// optionally stores a.  Bodies from tp_first on have tp_slots partials.
-__global__ void ff_finalize_kernel(const double *part, int nslot, int tp_first, int tp_slots, int n, double G,
-                                   const double *mass, const int *header, double dt_half, double *vel,
-                                   double *acc_out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (i >= tp_first) nslot = tp_slots;
-    const int em = header[1];
-    double f = G * scalbn(1.0, em - 2 * header[2]);
-    if (!(header[0] & kFfTwoMass)) f /= mass[i] * scalbn(1.0, -em);
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        double S = 0.0, C = 0.0;
-        for (int q = 0; q < nslot; q++) {
-            double t, e;
-            two_sum_ordered(S, part[((size_t)q * 3 + c) * n + i], t, e);
-            S = t;
-            C += e;
-        }
-        const double a = f * (S + C);
-        if (acc_out) acc_out[(size_t)c * n + i] = a;
-        if (dt_half != 0.0) vel[(size_t)c * n + i] += dt_half * a;
-    }
 }
 
 }  // namespace
@@ -590,30 +490,37 @@ int sym_ff_blocks_per_sm(int P) {
 
 // Layout of the packed-body allocation: the arrays in this order, each a whole
 // number of float4 per tile (but the bounds and the header, at the end).
+static size_t ff_tile_bytes(size_t nT) {
+    return nT * (sizeof(float4) * kFfTile + sizeof(float2) * kSymT + sizeof(float4)) + sizeof(float4) * (kFfBoundBlocks + 1);
+}
+
+void ff_place(FfPack &k, void *mem, size_t nT) {
+    k.body = (float4 *)mem;
+    k.ircf = (float2 *)(k.body + nT * kFfTile);
+    k.tmass = (double *)(k.ircf + nT * kSymT);
+    k.bounds = (float4 *)(k.tmass + 2 * nT);
+    k.header = (int *)(k.bounds + kFfBoundBlocks);
+}
+
+size_t ff_bytes(int n) { return ff_tile_bytes((size_t)((n + kSymT - 1) / kSymT)); }
+
 cudaError_t ff_reserve(genga_system *s) {
     const size_t nT = (size_t)((s->n + kSymT - 1) / kSymT);
     if (nT <= s->ff_tiles) return cudaSuccess;
     if (s->ff) cudaFree(s->ff);
     s->ff = nullptr;
     s->ff_tiles = 0;
-    const size_t bytes = nT * (sizeof(float4) * kFfTile + sizeof(float2) * kSymT + sizeof(float4)) +
-                         sizeof(float4) * (kFfBoundBlocks + 1);
-    GENGA_CUDA_TRY(cudaMalloc(&s->ff, bytes));
+    GENGA_CUDA_TRY(cudaMalloc(&s->ff, ff_tile_bytes(nT)));
     s->ff_tiles = nT;
     return cudaSuccess;
 }
 
 FfPack ff_pack_args(const genga_system *s) {
     FfPack k;
-    const size_t nT = s->ff_tiles;
     k.pos = s->pos; k.m = s->mass; k.rc = s->rcl[0].rc; k.pc2 = s->rcl[0].pc2;
     k.n = (int)s->n;
     k.nT = (int)((s->n + kSymT - 1) / kSymT);
-    k.body = (float4 *)s->ff;
-    k.ircf = (float2 *)(k.body + nT * kFfTile);
-    k.tmass = (double *)(k.ircf + nT * kSymT);
-    k.bounds = (float4 *)(k.tmass + 2 * nT);
-    k.header = (int *)(k.bounds + kFfBoundBlocks);
+    ff_place(k, s->ff, s->ff_tiles);
     k.ctr = nullptr;
     k.cand_count = nullptr;
     return k;
@@ -623,7 +530,7 @@ cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launch
     const int nb = std::min(kFfBoundBlocks, (k.n + 255) / 256);
     ff_bounds_kernel<<<nb, 256, 0, stream>>>(k.n, k.pos, k.m, k.bounds);
     GENGA_CUDA_TRY(cudaGetLastError());
-    ff_pack_kernel<<<k.nT, kSymT, 0, stream>>>(k, nb);
+    ff_pack_kernel<<<dim3(k.nT, 4), kSymT, 0, stream>>>(k, nb);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -632,15 +539,6 @@ cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStrea
     const size_t smem = sym_ff_smem(S.P);
     if (precheck) kick_sym_ff_kernel<true><<<blocks, kFfThreads, smem, stream>>>(S);
     else kick_sym_ff_kernel<false><<<blocks, kFfThreads, smem, stream>>>(S);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ff_finalize(const FfPack &k, const double *part, int nslot, int tp_first, int tp_slots, double G,
-                               double dt_half, double *vel, double *acc_out, cudaStream_t stream,
-                               int64_t *launches) {
-    ++*launches;
-    ff_finalize_kernel<<<(k.n + 255) / 256, 256, 0, stream>>>(part, nslot, tp_first, tp_slots, k.n, G, k.m, k.header,
-                                                             dt_half, vel, acc_out);
     return cudaGetLastError();
 }
 

@@ -9,8 +9,9 @@
 // keeps its scratch in one file-scope device array of fixed size that lives as
 // long as the library is loaded (every GPU that loads the library holds it).
 //
-// Scratch layout (doubles): rc^2 [n], FP32 thresholds [n floats], then the
-// kick's per-chunk partial sums [nchunk][6][n], nchunk reduced as needed to fit.
+// Scratch layout (launch_kick_raw): the packed bodies and the tiled kick's partial
+// sums where they fit, else (doubles) rc^2 [n], FP32 thresholds [n floats] and the
+// per-chunk partial sums [nchunk][6][n], nchunk reduced as needed to fit.
 #include <cuda.h>
 #include <mutex>
 
@@ -62,14 +63,6 @@ unsigned long long current_ctx_id() {
     return id;
 }
 
-__global__ void static_thresholds_kernel(int n, const double *rc, double *rc2, float *thr) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double r2 = __dmul_rn(rc[i], rc[i]);
-    rc2[i] = r2;
-    thr[i] = fmaxf(__double2float_ru(r2) * 1.0000153f, 1.17549435e-38f);
-}
-
 }  // namespace
 }  // namespace genga
 
@@ -100,20 +93,11 @@ extern "C" int genga_kick_static(int64_t n, const double *pos, const double *mas
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GENGA_ECUDA;
     const size_t N = (size_t)n;
-    double *rc2 = base;
-    float *thr = (float *)(base + N);
-    const size_t part_off = ((N + (N + 1) / 2) + 31) / 32 * 32;   // 256-byte aligned
-    double *part = base + part_off;
-    const size_t room = kStaticDoubles - part_off;
-    const int max_nchunk = (int)(room / (6 * N));
-    if (max_nchunk < 1) return GENGA_ECAPACITY;
-    cudaStream_t st = (cudaStream_t)stream;
-    static_thresholds_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>((int)n, rc, rc2, thr);
-    if (cudaGetLastError() != cudaSuccess) return GENGA_ECUDA;
+    if ((N + (N + 1) / 2 + 31) / 32 * 32 + 6 * N > kStaticDoubles) return GENGA_ECAPACITY;
     KickRaw k;
-    k.pos = pos; k.mass = mass; k.rc = rc; k.rc2 = rc2; k.thr = thr; k.part = part;
+    k.pos = pos; k.mass = mass; k.rc = rc; k.scratch = base; k.room = kStaticDoubles;
     k.n = (int)n; k.G = G; k.dt_half = dt_half; k.vel = vel; k.acc_out = acc_out;
     k.mixed = precision == GENGA_MIXED;
-    if (launch_kick_raw(k, sms, max_nchunk, st) != cudaSuccess) return GENGA_ECUDA;
+    if (launch_kick_raw(k, sms, (cudaStream_t)stream) != cudaSuccess) return GENGA_ECUDA;
     return GENGA_OK;
 }

@@ -13,7 +13,8 @@ constexpr int kSymMaxP = 6;                    // tiles per super-range, at most
 
 struct SymArgs {
     const double *x, *y, *z, *m;
-    const double *irc;          // FP64: 1 / rc per body (inv_rc)
+    const double *rc;           // critical radii
+    const double *irc;          // FP64, symmetric: 1 / rc per body (inv_rc)
     const float *thr;           // FP64: upper bound of rc^2
     const float4 *body;         // mixed: the bodies as float expansions, by tiles (kick_ff.cu)
     const float2 *ircf;         // mixed: 1 / rc as two floats, padded to whole tiles
@@ -91,6 +92,7 @@ __device__ __forceinline__ void sym_pc_push(uint2 *buf, int &cnt, int lane, bool
 // (m_hi, m_lo the scaled mass; k the fourth parts of the coordinates).
 constexpr int kFfRow = 64, kFfTile = 8 * kFfRow;
 constexpr int kFfWide = 1, kFfTwoMass = 2;     // flags of the packed bodies, see kick_ff.cu
+constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2;      // instances of the pair loops
 __device__ __forceinline__ f2 f2_lo(const float4 &v) { return f2_make(v.x, v.y); }
 __device__ __forceinline__ f2 f2_hi(const float4 &v) { return f2_make(v.z, v.w); }
 
@@ -116,10 +118,20 @@ struct FfPack {
 // Makes sure the system's packed-body arrays hold its bodies, and their addresses.
 cudaError_t ff_reserve(genga_system *s);
 FfPack ff_pack_args(const genga_system *s);
+// The same on caller-provided memory: its bytes for n bodies, and the addresses in it.
+size_t ff_bytes(int n);
+void ff_place(FfPack &k, void *mem, size_t tiles);
 cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launches);
 cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStream_t stream);
-cudaError_t launch_ff_finalize(const FfPack &k, const double *part, int nslot, int tp_first, int tp_slots, double G,
-                               double dt_half, double *vel, double *acc_out, cudaStream_t stream, int64_t *launches);
+// kick_tile.cu: the tiled kick.  Steps (two bodies j) per chunk, chunks, predicted SM
+// cycles.  Chunk 0: no plan (max_part, in doubles, holds no partial sums).
+struct TilePlan {
+    int chunk = 0, nchunk = 0;
+    double cycles = 0.0;
+};
+TilePlan tile_plan(int n, int nm, int num_sms, bool mixed, size_t max_part);
+// Partial sums [nchunk][3][n].
+cudaError_t launch_tile_kick(const SymArgs &S, int chunk, int nchunk, bool mixed, bool precheck, cudaStream_t stream);
 
 // 1 / rc: the Newton reciprocal for every rc the FP32 seed can take, an exact
 // division for smaller ones, infinite for rc = 0 (so that min(1/rc_i, 1/rc_j) is

@@ -59,14 +59,15 @@ struct EnsShared {
     // mixed kick: masses as two floats, FP32 bounds of rc^2 (above) and of
     // (f_pc rc)^2 (below and above)
     float mh[kEnsMaxN], ml[kEnsMaxN], thr[kEnsMaxN], pclo[kEnsMaxN], pchi[kEnsMaxN];
-    double u0[3][kEnsMaxN], u1[3][kEnsMaxN], w0[3][kEnsMaxN];
     double part[3][128];
     unsigned long long cand[kEnsMaxN], enc[kEnsMaxN];
     int parent[kEnsMaxN], slot[kEnsMaxN], mem[kEnsMaxN];
     int roots[kEnsMaxN];
     double ws0[3], ws1[3], wsm[3];
     double star_R, star_k2, star_tau, star_rg2, mstar, dt;
-    int n, nroots, flag, sys;
+    double ims, itot, iIs;              // 1/m_star, 1/(m_star + sum m), 1/(star's moment of inertia) or 0
+    int n, nroots, flag, sys, rot;
+    int nnflag[2];                      // ens_nn: something changed in the iteration (by parity)
     double bs_t, bs_H, bs_err;
     int bs_stop, bs_kconv;
     // per-body constants of the loaded system: cbrt(m/(3 m_star)) of Rcrit,
@@ -79,24 +80,44 @@ struct EnsShared {
     double red[4][kEnsMaxN / 32];       // per-warp partial sums of ens_bsum
 };
 
+// This thread's index with the CTA's two warps swapped in every other CTA of an SM:
+// a system of up to 32 bodies keeps one warp busy, and the hardware gives the
+// first warps of two-warp CTAs to two of the SM's four FP64 pipes only.
+__device__ __forceinline__ int ens_thread(const EnsShared &S) { return (int)threadIdx.x ^ S.rot; }
+
+// The warp's sums of K <= 4 values per lane, to S.red[k][warp]: a butterfly that
+// hands half of the values over in each of the first two exchanges (6 additions,
+// the same tree as summing each value by itself, 5 K).  Threads past the bodies
+// pass zeros.
+template <int K>
+__device__ __forceinline__ void ens_warp_sums(EnsShared &S, const double (&v)[K]) {
+    const int lane = ens_thread(S) & 31;
+    const double a0 = v[0], a1 = K > 1 ? v[K > 1 ? 1 : 0] : 0.0, a2 = K > 2 ? v[K > 2 ? 2 : 0] : 0.0,
+                 a3 = K > 3 ? v[K > 3 ? 3 : 0] : 0.0;
+    const bool h = lane & 16, q = lane & 8;
+    double k0 = h ? a2 : a0, k1 = h ? a3 : a1;
+    k0 += __shfl_xor_sync(0xffffffffu, h ? a0 : a2, 16);
+    k1 += __shfl_xor_sync(0xffffffffu, h ? a1 : a3, 16);
+    double a = q ? k1 : k0;
+    a += __shfl_xor_sync(0xffffffffu, q ? k0 : k1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    const int k = lane >> 3;                   // bit 4: values 2, 3; bit 3: the odd one
+    if ((lane & 7) == 0 && k < K) S.red[k][ens_thread(S) >> 5] = a;
+}
+
 // Sums over the loaded system's bodies of K per-body values (thread t < n
 // holds body t's), in a fixed order: a butterfly within each warp, then the
 // warps in order.  Every thread receives the sums.  Called by all threads.
 template <int K>
 __device__ __forceinline__ void ens_bsum(EnsShared &S, const double (&v)[K], double (&out)[K]) {
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int t = ens_thread(S), w = t >> 5;
     const int nw = (S.n + 31) >> 5;
-    double a[K];
-#pragma unroll
-    for (int k = 0; k < K; k++) a[k] = t < S.n ? v[k] : 0.0;
     if (w < nw) {
+        double a[K];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < K; k++) a[k] += __shfl_xor_sync(0xffffffffu, a[k], o);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < K; k++) S.red[k][w] = a[k];
+        for (int k = 0; k < K; k++) a[k] = t < S.n ? v[k] : 0.0;
+        ens_warp_sums<K>(S, a);
     }
     __syncthreads();
 #pragma unroll
@@ -126,7 +147,7 @@ __device__ __forceinline__ unsigned long long ens_now() {
 template <int T, bool MIXED>
 __device__ void ens_kick(const EnsArgs &A, EnsShared &S, double dt_half, bool precheck) {
     const int n = S.n;
-    const int t = threadIdx.x;
+    const int t = ens_thread(S);
     const int nsl = max(1, T / n);
     const int i = t % n, sl = t / n;
     double ax = 0.0, ay = 0.0, az = 0.0;
@@ -222,137 +243,162 @@ __device__ void ens_kick(const EnsArgs &A, EnsShared &S, double dt_half, bool pr
 }
 
 // ------------------------------------------------------------ GR + tides
-// GR (Eq. apn) and tidal (Sec. 4.1-4.2) acceleration of body i at velocity u
-// (heliocentric) and spin W, with the torques on the body and on the star.
-// Divisions by r are multiplications by 1/r (Newton rsqrt) and the per-body
-// constants come with the system (EnsShared): the FP64 pipe bounds the kernel.
-__device__ void nn_body(const EnsArgs &A, const EnsShared &S, int i, const double u[3],
-                        const double W[3], double acc[3], double Ni[3], double Ns[3]) {
-    const double x[3] = {S.x[0][i], S.x[1][i], S.x[2][i]};
-    const double r2 = (x[0] * x[0] + x[1] * x[1]) + x[2] * x[2];
-    const double ir = rsqrt_newton(r2);
-    const double r = r2 * ir;
-    const double er[3] = {x[0] * ir, x[1] * ir, x[2] * ir};
-    const double rdot = ((x[0] * u[0] + x[1] * u[1]) + x[2] * u[2]) * ir;
-    const double u2 = (u[0] * u[0] + u[1] * u[1]) + u[2] * u[2];
-    for (int k = 0; k < 3; k++) { acc[k] = 0.0; Ni[k] = 0.0; Ns[k] = 0.0; }
-    if (A.gr == 1) {
-        const double mu = S.mu[i], eta = S.eta[i];
-        const double pre = -mu * (ir * ir) * A.inv_c2;
-        const double cv = -2.0 * (2.0 - eta) * rdot;
-        const double cr = (1.0 + 3.0 * eta) * u2 - 1.5 * eta * rdot * rdot - 2.0 * (2.0 + eta) * mu * ir;
-        for (int k = 0; k < 3; k++) acc[k] += pre * (cv * u[k] + cr * er[k]);
-    }
-    if (A.tides) {
-        const double ir2 = ir * ir;
-        const double ir7 = (ir2 * ir2) * (ir2 * ir);
-        const double Dti = S.tdi[i] * ir7;
-        const double Dts = S.tds[i] * ir7;
-        const double Pti = Dti * S.tau[i], Pts = Dts * S.star_tau;
-        const double fr = -(Dts + Dti) - 2.0 * rdot * ir * (Pts + Pti);
-        const double *Ws = S.wsm;
-        const double wxe[3] = {W[1] * er[2] - W[2] * er[1], W[2] * er[0] - W[0] * er[2], W[0] * er[1] - W[1] * er[0]};
-        const double sxe[3] = {Ws[1] * er[2] - Ws[2] * er[1], Ws[2] * er[0] - Ws[0] * er[2], Ws[0] * er[1] - Ws[1] * er[0]};
-        const double exu[3] = {er[1] * u[2] - er[2] * u[1], er[2] * u[0] - er[0] * u[2], er[0] * u[1] - er[1] * u[0]};
-        const double rW = (x[0] * W[0] + x[1] * W[1]) + x[2] * W[2];
-        const double rWs = (x[0] * Ws[0] + x[1] * Ws[1]) + x[2] * Ws[2];
-        const double im = S.im[i], Ptot_ir = (Pti + Pts) * ir;
-        for (int k = 0; k < 3; k++) {
-            const double F = fr * er[k] + Pti * wxe[k] + Pts * sxe[k] - Ptot_ir * u[k];
-            acc[k] += F * im;
-            Ni[k] = Pti * (W[k] * r - rW * er[k] - exu[k]);
-            Ns[k] = Pts * (Ws[k] * r - rWs * er[k] - exu[k]);
-        }
-    }
+// The implicit midpoint rule over dt for the GR (Eq. apn) and tidal (Sec. 4.1-4.2)
+// forces, which depend on the heliocentric velocity u and the spins, iterated
+// until nothing changes.
+//
+// The FP64 pipe bounds this part (two thirds of the kernel), so what the
+// iterations share -- everything that depends on the position alone -- is formed
+// once, and an iteration is 73 FP64 instructions per body:
+//   acc = A e + B u + Q x e,  A = a0 + a1 rdot + a2 rdot^2 + a3 u^2,  B = b0 + b1 rdot,
+//   Q = q_i W + q_s W_star (e = x / r, rdot = e.u), and with T(W) = r W - (x.W) e - e x u
+//   dW = c_w T(W), the star's torque sum c_s T(W_star).
+// Convergence is tested on the bits: |new - old| > 1e-16 |new| holds exactly when
+// the two differ (1e-16 is below half a unit of the last place) and new is finite.
+__device__ __forceinline__ bool ens_changed(double a, double old) {
+    const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
+    const unsigned ho = (unsigned)__double2hiint(old), lo = (unsigned)__double2loint(old);
+    const bool zeros = (((ha | ho) << 1) | la | lo) == 0u;
+    return (ha != ho || la != lo) && !zeros && (ha & 0x7ff00000u) != 0x7ff00000u;
 }
 
 __device__ void ens_nn(const EnsArgs &A, EnsShared &S, double dt) {
     if (A.gr != 1 && !A.tides) return;
-    const int n = S.n, t = threadIdx.x;
-    const int b = t < n ? t : 0;
-    double P[4];
+    const int n = S.n, t = ens_thread(S), w = t >> 5;
+    const int b = t < n ? t : 0, nw = (n + 31) >> 5;
+    const bool tides = A.tides != 0;
+    double P[3];
     {
-        const double mv[4] = {S.m[b] * S.v[0][b], S.m[b] * S.v[1][b], S.m[b] * S.v[2][b], S.m[b]};
-        ens_bsum<4>(S, mv, P);
+        const double mv[3] = {S.m[b] * S.v[0][b], S.m[b] * S.v[1][b], S.m[b] * S.v[2][b]};
+        ens_bsum<3>(S, mv, P);
     }
-    const double Mp = P[3];
-    const double ims = 1.0 / S.mstar;
-    if (t == 0)
-        for (int k = 0; k < 3; k++) S.ws1[k] = S.ws0[k];
-    if (t < n)
+    const double ims = S.ims;
+    const bool star = tides && S.iIs > 0.0;
+    if (t < 3) S.ws1[t] = S.wsm[t] = S.ws0[t];
+    if (t == 0) S.nnflag[0] = 0;
+    // per body: constants of the iterations
+    double e[3], u0[3], u1[3], w0[3], W[3];
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, b0 = 0.0, b1 = 0.0, qi = 0.0, qs = 0.0, r, cw = 0.0, cs = 0.0;
+    {
+        const double x[3] = {S.x[0][b], S.x[1][b], S.x[2][b]};
+        const double r2 = (x[0] * x[0] + x[1] * x[1]) + x[2] * x[2];
+        const double ir = rsqrt_newton(r2), ir2 = ir * ir;
+        r = r2 * ir;
         for (int k = 0; k < 3; k++) {
-            S.u0[k][t] = S.v[k][t] + P[k] * ims;
-            S.u1[k][t] = S.u0[k][t];
-            S.w0[k][t] = S.w[k][t];
+            e[k] = x[k] * ir;
+            u0[k] = u1[k] = S.v[k][b] + P[k] * ims;
+            w0[k] = W[k] = S.w[k][b];
         }
-    const double Is = S.star_rg2 * S.mstar * S.star_R * S.star_R;
+        if (A.gr == 1) {
+            const double mu = S.mu[b], eta = S.eta[b];
+            const double pre = -mu * ir2 * A.inv_c2;
+            b1 = pre * (-2.0 * (2.0 - eta));
+            a0 = pre * (-2.0 * (2.0 + eta) * mu * ir);
+            a2 = pre * (-1.5 * eta);
+            a3 = pre * (1.0 + 3.0 * eta);
+        }
+        if (tides) {
+            const double ir7 = (ir2 * ir2) * (ir2 * ir), im = S.im[b];
+            const double Dti = S.tdi[b] * ir7, Dts = S.tds[b] * ir7;
+            const double Pti = Dti * S.tau[b], Pts = Dts * S.star_tau;
+            const double Ptot_ir = (Pti + Pts) * ir;
+            a0 -= (Dts + Dti) * im;
+            a1 = -2.0 * Ptot_ir * im;
+            b0 = -Ptot_ir * im;
+            qi = Pti * im;
+            qs = Pts * im;
+            cw = -dt * S.fiI[b] * Pti;
+            cs = S.fac[b] * Pts;
+        }
+    }
+    const bool spins = tides && S.Ii[b] > 0.0;
+    __syncthreads();
     for (int it = 0; it < A.implicit_max_iter; it++) {
-        if (t == 0) {
-            S.flag = 0;
-            for (int k = 0; k < 3; k++) S.wsm[k] = 0.5 * (S.ws0[k] + S.ws1[k]);
-        }
-        __syncthreads();
-        double nsv[3] = {0.0, 0.0, 0.0};
-        if (t < n) {
-            double um[3], Wm[3], acc[3], Ni[3], Ns[3];
-            for (int k = 0; k < 3; k++) {
-                um[k] = 0.5 * (S.u0[k][t] + S.u1[k][t]);
-                Wm[k] = 0.5 * (S.w0[k][t] + S.w[k][t]);
-            }
-            nn_body(A, S, t, um, Wm, acc, Ni, Ns);
-            const double fac = S.fac[t];
-            const double Ii = S.Ii[t], fiI = S.fiI[t];
+        if (w < nw) {
+            double um[3], acc[3], nsv[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int k = 0; k < 3; k++) um[k] = 0.5 * u0[k] + 0.5 * u1[k];
+            const double rdot = (e[0] * um[0] + e[1] * um[1]) + e[2] * um[2];
+            const double u2 = (um[0] * um[0] + um[1] * um[1]) + um[2] * um[2];
+            const double ca = fma(a3, u2, fma(fma(a2, rdot, a1), rdot, a0)), cb = fma(b1, rdot, b0);
+#pragma unroll
+            for (int k = 0; k < 3; k++) acc[k] = fma(ca, e[k], cb * um[k]);
             bool changed = false;
-            for (int k = 0; k < 3; k++) {
-                const double un = S.u0[k][t] + dt * acc[k];
-                if (fabs(un - S.u1[k][t]) > 1e-16 * fabs(un)) changed = true;
-                S.u1[k][t] = un;
-                if (A.tides && Ii > 0.0) {
-                    const double Wn = S.w0[k][t] - dt * fiI * Ni[k];
-                    if (fabs(Wn - S.w[k][t]) > 1e-16 * fabs(Wn)) changed = true;
-                    S.w[k][t] = Wn;
-                }
-                nsv[k] = fac * Ns[k];
-            }
-            if (changed) S.flag = 1;
-        }
-        if (A.tides && Is > 0.0) {
-            double d[3];
-            ens_bsum<3>(S, nsv, d);
-            if (t == 0)
+            if (tides) {
+                double Wm[3], Ws[3], Q[3], exu[3];
+#pragma unroll
                 for (int k = 0; k < 3; k++) {
-                    const double Wn = S.ws0[k] - dt * d[k] / Is;
-                    if (fabs(Wn - S.ws1[k]) > 1e-16 * fabs(Wn)) S.flag = 1;
-                    S.ws1[k] = Wn;
+                    Wm[k] = 0.5 * w0[k] + 0.5 * W[k];
+                    Ws[k] = S.wsm[k];
+                    Q[k] = fma(qi, Wm[k], qs * Ws[k]);
                 }
+                const double xW = r * ((e[0] * Wm[0] + e[1] * Wm[1]) + e[2] * Wm[2]);
+                const double xWs = r * ((e[0] * Ws[0] + e[1] * Ws[1]) + e[2] * Ws[2]);
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+                    acc[k] += fma(Q[k1], e[k2], -Q[k2] * e[k1]);
+                    exu[k] = fma(e[k1], um[k2], -e[k2] * um[k1]);
+                }
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    if (spins) {
+                        const double Wn = fma(cw, fma(r, Wm[k], -fma(xW, e[k], exu[k])), w0[k]);
+                        changed = changed || ens_changed(Wn, W[k]);
+                        W[k] = Wn;
+                    }
+                    nsv[k] = cs * fma(r, Ws[k], -fma(xWs, e[k], exu[k]));
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const double un = fma(dt, acc[k], u0[k]);
+                changed = changed || ens_changed(un, u1[k]);
+                u1[k] = un;
+            }
+            if (t < n && changed) S.nnflag[it & 1] = 1;
+            if (star) {
+                if (t >= n) nsv[0] = nsv[1] = nsv[2] = 0.0;
+                ens_warp_sums<3>(S, nsv);
+            }
         }
         __syncthreads();
-        if (!S.flag) break;
+        if (t == 0) S.nnflag[(it + 1) & 1] = 0;
+        if (star && t < 3) {
+            double d = S.red[t][0];
+            for (int q = 1; q < nw; q++) d += S.red[t][q];
+            const double Wn = fma(-dt * S.iIs, d, S.ws0[t]);
+            if (ens_changed(Wn, S.ws1[t])) S.nnflag[it & 1] = 1;
+            S.ws1[t] = Wn;
+            S.wsm[t] = 0.5 * (S.ws0[t] + Wn);
+        }
         __syncthreads();
+        if (!S.nnflag[it & 1]) break;
     }
     double Q[3];
     {
-        const double mu1[3] = {S.m[b] * S.u1[0][b], S.m[b] * S.u1[1][b], S.m[b] * S.u1[2][b]};
+        const double mu1[3] = {S.m[b] * u1[0], S.m[b] * u1[1], S.m[b] * u1[2]};
         ens_bsum<3>(S, mu1, Q);
     }
-    if (t == 0)
-        for (int k = 0; k < 3; k++) S.ws0[k] = S.ws1[k];
-    const double itot = 1.0 / (S.mstar + Mp);
+    if (t < 3) S.ws0[t] = S.ws1[t];
     if (t < n)
-        for (int k = 0; k < 3; k++) S.v[k][t] = S.u1[k][t] - Q[k] * itot;
+        for (int k = 0; k < 3; k++) {
+            S.v[k][t] = u1[k] - Q[k] * S.itot;
+            S.w[k][t] = W[k];
+        }
     __syncthreads();
 }
 
 // ------------------------------------------------------------ HC (Eq. Hc)
 __device__ void ens_hc(EnsShared &S, double dt_half) {
-    const int n = S.n, t = threadIdx.x;
+    const int n = S.n, t = ens_thread(S);
     double P[3];
     {
         const int b = t < n ? t : 0;
         const double mv[3] = {S.m[b] * S.v[0][b], S.m[b] * S.v[1][b], S.m[b] * S.v[2][b]};
         ens_bsum<3>(S, mv, P);
     }
-    const double f = dt_half / S.mstar;
+    const double f = dt_half * S.ims;
     if (t < n) for (int k = 0; k < 3; k++) S.x[k][t] += f * P[k];
     __syncthreads();
 }
@@ -379,7 +425,7 @@ __device__ __forceinline__ double ens_alpha_factor(const double x[3], const doub
 
 // v -> u by fixed-point iteration from u = v (4 iterations: the correction is ~v^2/c^2).
 __device__ void ens_gr_to_pseudo(const EnsArgs &A, EnsShared &S) {
-    const int t = threadIdx.x;
+    const int t = ens_thread(S);
     if (t < S.n) {
         const double x[3] = {S.x[0][t], S.x[1][t], S.x[2][t]};
         const double v[3] = {S.v[0][t], S.v[1][t], S.v[2][t]};
@@ -394,7 +440,7 @@ __device__ void ens_gr_to_pseudo(const EnsArgs &A, EnsShared &S) {
 }
 
 __device__ void ens_gr_to_real(const EnsArgs &A, EnsShared &S) {
-    const int t = threadIdx.x;
+    const int t = ens_thread(S);
     if (t < S.n) {
         const double x[3] = {S.x[0][t], S.x[1][t], S.x[2][t]};
         const double u[3] = {S.v[0][t], S.v[1][t], S.v[2][t]};
@@ -405,7 +451,7 @@ __device__ void ens_gr_to_real(const EnsArgs &A, EnsShared &S) {
 }
 
 __device__ void ens_gr_beta(const EnsArgs &A, EnsShared &S, double dt) {
-    const int t = threadIdx.x;
+    const int t = ens_thread(S);
     if (t < S.n) {
         const double x[3] = {S.x[0][t], S.x[1][t], S.x[2][t]};
         const double r2 = (x[0] * x[0] + x[1] * x[1]) + x[2] * x[2];
@@ -418,14 +464,14 @@ __device__ void ens_gr_beta(const EnsArgs &A, EnsShared &S, double dt) {
 
 // HC(dt) with the gamma term: x += dt P/m_star - dt 2 (u^2/c^2) u.
 __device__ void ens_hc_gamma(const EnsArgs &A, EnsShared &S, double dt) {
-    const int n = S.n, t = threadIdx.x;
+    const int n = S.n, t = ens_thread(S);
     double P[3];
     {
         const int b = t < n ? t : 0;
         const double mv[3] = {S.m[b] * S.v[0][b], S.m[b] * S.v[1][b], S.m[b] * S.v[2][b]};
         ens_bsum<3>(S, mv, P);
     }
-    const double f = dt / S.mstar;
+    const double f = dt * S.ims;
     if (t < n) {
         const double u[3] = {S.v[0][t], S.v[1][t], S.v[2][t]};
         const double g = dt * 2.0 * ens_u2(u) * A.inv_c2;
@@ -471,13 +517,199 @@ __device__ void ens_bs_deriv(const EnsArgs &A, EnsShared &S, double *scr, int z0
     ebs(scr, f0 + 5, s) = fac * (sst * z) + A.G * pz;
 }
 
+__device__ void ens_bs_count(const EnsArgs &A, int nm, int attempts, long long acc, long long rej, bool failed) {
+    atomicAdd(&A.ctr->bs_steps, (unsigned long long)acc);
+    atomicAdd(&A.ctr->bs_rejects, (unsigned long long)rej);
+    atomicMax(&A.ctr->bs_max_attempts, (unsigned long long)attempts);
+    atomicAdd(&A.ctr->groups_total, 1ull);
+    atomicMax(&A.ctr->max_group_total, (unsigned long long)nm);
+    if (failed) { atomicAdd(&A.ctr->bs_fail, 1ull); latch_error(A.ctr, kErrBS); }
+}
+
+// Neville coefficients in h^2 for the step numbers 2 (k + 1): column k, order j
+__constant__ double kEnsNeville[8][8] = {
+    {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0},
+    {0.0, 1.0 / 3.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0},
+    {0.0, 4.0 / 5.0, 1.0 / 8.0, 0.0, 0.0, 0.0, 0.0, 0.0},
+    {0.0, 9.0 / 7.0, 4.0 / 12.0, 1.0 / 15.0, 0.0, 0.0, 0.0, 0.0},
+    {0.0, 16.0 / 9.0, 9.0 / 16.0, 4.0 / 21.0, 1.0 / 24.0, 0.0, 0.0, 0.0},
+    {0.0, 25.0 / 11.0, 16.0 / 20.0, 9.0 / 27.0, 4.0 / 32.0, 1.0 / 35.0, 0.0, 0.0},
+    {0.0, 36.0 / 13.0, 25.0 / 24.0, 16.0 / 33.0, 9.0 / 40.0, 4.0 / 45.0, 1.0 / 48.0, 0.0},
+    {0.0, 49.0 / 15.0, 36.0 / 28.0, 25.0 / 39.0, 16.0 / 48.0, 9.0 / 55.0, 4.0 / 60.0, 1.0 / 63.0},
+};
+
+// Groups of up to four members, by one warp: lane 4 c + s holds member s in column c
+// of the extrapolation (2 (c + 1) midpoint steps), so that the eight columns advance
+// together and a step ends when the first converged column does -- 2 (c + 1) force
+// evaluations in a row instead of the sum over the columns.  An FP64 instruction
+// takes its sub-partition 64 cycles whether one lane is active or 32, dependent or
+// not: the time is the number of FP64 instructions the warp issues, ~50 per
+// evaluation (reciprocal square roots from the FP32 seed, K only where the warp
+// needs it).  The extrapolation table is spread over the lanes by component:
+// lane 4 c + s, c < 6, holds component c of member s, in registers.
+// One system in 500 has such a group for all ten steps and ran 5 to 8 ms through
+// the general path (ens_bs_group), longer than the other 2,047 systems together.
+constexpr int kEnsBsFast = 4;
+struct EnsFast {
+    double z[6];                               // state of this lane's member
+    double mp[3], irc[3], gm;                  // G m and 1/rc_ij of the partners s ^ q, q = 1 2 3; G m_star
+    float ircf[3];
+};
+__device__ __forceinline__ void ens_fast_deriv(const EnsArgs &A, const EnsShared &S, const EnsFast &F, int nm,
+                                               double (&f)[6]) {
+    const double x = F.z[0], y = F.z[1], z = F.z[2];
+    const double r2 = fma(z, z, fma(y, y, x * x));
+    const double ir = rsqrt_newton(r2);
+    double c = -F.gm * (ir * ir * ir);
+    double fac = 1.0;
+    if (A.gr == 2) {
+        const double xx[3] = {x, y, z}, uu[3] = {F.z[3], F.z[4], F.z[5]};
+        fac = ens_alpha_factor(xx, uu, A.G * S.mstar, A.inv_c2);
+        c *= fac;
+    }
+    double ax = c * x, ay = c * y, az = c * z;
+#pragma unroll
+    for (int q = 1; q < kEnsBsFast; q++) {
+        if (q > 1 && nm <= 2) break;
+        const double dx = __shfl_xor_sync(0xffffffffu, x, q) - x, dy = __shfl_xor_sync(0xffffffffu, y, q) - y,
+                     dz = __shfl_xor_sync(0xffffffffu, z, q) - z;
+        const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
+        const double id = rsqrt_newton(d2);
+        double w = F.mp[q - 1] * (id * id * id);
+        // 1 - K: 1 below 0.1 rc, 0 above rc
+        const int side = changeover_side_f32(f32_of_f64_trunc(d2) * f32_of_f64_trunc(id), F.ircf[q - 1]);
+        if (side == 0) w *= 1.0 - changeover_fast(d2 * id, F.irc[q - 1]);
+        if (F.mp[q - 1] == 0.0 || side > 0) w = 0.0;     // no partner (or itself a lane without a member)
+        ax = fma(w, dx, ax);
+        ay = fma(w, dy, ay);
+        az = fma(w, dz, az);
+    }
+    f[0] = fac * F.z[3]; f[1] = fac * F.z[4]; f[2] = fac * F.z[5];
+    f[3] = ax; f[4] = ay; f[5] = az;
+}
+
+__device__ void ens_bs_fast(const EnsArgs &A, EnsShared &S, int nm, double dt, unsigned long long t_start) {
+    const int lane = ens_thread(S) & 31, s = lane & 3, col = lane >> 2;
+    const bool member = s < nm;
+    const int b = S.mem[member ? s : 0];
+    EnsFast F;
+    F.gm = A.G * S.mstar;
+#pragma unroll
+    for (int q = 1; q < kEnsBsFast; q++) {
+        const int sp = s ^ q;
+        const int p = member && sp < nm ? S.mem[sp] : b;
+        const bool on = (S.enc[b] >> p) & 1ull;
+        F.mp[q - 1] = member && sp < nm && on ? A.G * S.m[p] : 0.0;
+        const double rc = fmax(S.rc[b], S.rc[p]);
+        F.irc[q - 1] = rc > 1e-30 ? rcp_newton(rc) : rc > 0.0 ? 1.0 / rc : __longlong_as_double(0x7ff0000000000000ll);
+        F.ircf[q - 1] = __double2float_rz(F.irc[q - 1]);
+    }
+    // lanes without a member stand far off, each its own place
+    double Y[6], f0[6], zm[6], T[8], f[6];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        Y[c] = member ? S.x0[c][b] : 1e3 * fabs(S.x0[0][b]) * (s + 2) + (c == 0 ? 1.0 : 0.0);
+        Y[3 + c] = member ? S.v0[c][b] : 0.0;
+    }
+    const int nk = 2 * (col + 1), comp = col < 6 ? col : 0;
+    double bt = 0.0, bH = dt;
+    int attempts = 0;
+    long long acc = 0, rej = 0;
+    bool failed = false;
+    while (bt < dt) {
+        bool stop = attempts >= A.bs_max_steps || ens_now() - t_start > A.time_limit_ns;
+        stop = __shfl_sync(0xffffffffu, (int)stop, 0);
+        if (stop) { failed = true; break; }
+        attempts++;
+        double H = bH;
+        if (H > dt - bt) H = dt - bt;
+        const double h = H / nk, h2 = 2.0 * h;
+#pragma unroll
+        for (int c = 0; c < 6; c++) F.z[c] = Y[c];
+        ens_fast_deriv(A, S, F, nm, f0);
+        // this lane's component of the error scale
+        double yc = Y[0], fc = f0[0];
+#pragma unroll
+        for (int c = 1; c < 6; c++) {
+            yc = comp == c ? Y[c] : yc;
+            fc = comp == c ? f0[c] : fc;
+        }
+        const double lim = A.bs_tol * (fabs(yc) + fabs(H * fc) + 1e-300);
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            zm[c] = Y[c];
+            F.z[c] = fma(h, f0[c], Y[c]);
+        }
+        int kconv = -1;
+#pragma unroll 1
+        for (int k = 0; k < 8; k++) {
+            double cur[6];
+#pragma unroll 1
+            for (int half = 0; half < 2; half++) {     // midpoint steps 2 k + 1 and 2 k + 2
+                ens_fast_deriv(A, S, F, nm, f);
+                if (half == 1)
+#pragma unroll
+                    for (int c = 0; c < 6; c++) cur[c] = 0.5 * (F.z[c] + fma(h, f[c], zm[c]));
+                if (2 * k + 1 + half < nk)
+#pragma unroll
+                    for (int c = 0; c < 6; c++) {
+                        const double tt = fma(h2, f[c], zm[c]);
+                        zm[c] = F.z[c];
+                        F.z[c] = tt;
+                    }
+            }
+            // column k's result, by component, and its row of the table
+            double v = 0.0;
+#pragma unroll
+            for (int c = 0; c < 6; c++) {
+                const double u = __shfl_sync(0xffffffffu, cur[c], 4 * k + s);
+                v = comp == c ? u : v;
+            }
+            double prev = T[0], last = 0.0;
+            T[0] = v;
+#pragma unroll
+            for (int j = 1; j < 8; j++) {
+                if (j <= k) {
+                    const double nxt = fma(v - prev, kEnsNeville[k][j], v);
+                    prev = T[j];
+                    T[j] = nxt;
+                    last = v;
+                    v = nxt;
+                }
+            }
+            const bool off = member && col < 6 && fabs(v - last) > lim;
+            if (k >= 1 && !__any_sync(0xffffffffu, off)) {
+                kconv = k;
+#pragma unroll
+                for (int c = 0; c < 6; c++) {
+                    const double u = __shfl_sync(0xffffffffu, v, 4 * c + s);
+                    if (member) Y[c] = u;
+                }
+                break;
+            }
+        }
+        if (kconv >= 0) {
+            bt += H;
+            bH = kconv < 4 ? 1.5 * H : H;
+            acc++;
+        } else {
+            bH = 0.5 * H;
+            rej++;
+        }
+    }
+    if (member && col == 0)
+#pragma unroll
+        for (int c = 0; c < 3; c++) { S.x[c][b] = Y[c]; S.v[c][b] = Y[3 + c]; }
+    if (lane == 0) ens_bs_count(A, nm, attempts, acc, rej, failed);
+}
+
 // Same integrator and step control as the large-system kernels: modified
 // midpoint n = 2..16, Neville in h^2, accept at the first column k >= 1 under
 // tolerance, grow 1.5x if k < 4, halve on failure.
 __device__ void ens_bs_group(const EnsArgs &A, EnsShared &S, double *scr, int nm, double dt,
                              unsigned long long t_start) {
     enum { Y = 0, F0 = 6, ZM = 12, ZN = 18, FZ = 24, SC = 30, TT = 36 };
-    const int t = threadIdx.x;
+    const int t = ens_thread(S);
     for (int s = t; s < nm; s += blockDim.x) {
         const int b = S.mem[s];
         for (int c = 0; c < 3; c++) { ebs(scr, Y + c, s) = S.x0[c][b]; ebs(scr, Y + 3 + c, s) = S.v0[c][b]; }
@@ -558,14 +790,7 @@ __device__ void ens_bs_group(const EnsArgs &A, EnsShared &S, double *scr, int nm
         const int b = S.mem[s];
         for (int c = 0; c < 3; c++) { S.x[c][b] = ebs(scr, Y + c, s); S.v[c][b] = ebs(scr, Y + 3 + c, s); }
     }
-    if (t == 0) {
-        atomicAdd(&A.ctr->bs_steps, (unsigned long long)acc);
-        atomicAdd(&A.ctr->bs_rejects, (unsigned long long)rej);
-        atomicMax(&A.ctr->bs_max_attempts, (unsigned long long)attempts);
-        atomicAdd(&A.ctr->groups_total, 1ull);
-        atomicMax(&A.ctr->max_group_total, (unsigned long long)nm);
-        if (failed) { atomicAdd(&A.ctr->bs_fail, 1ull); latch_error(A.ctr, kErrBS); }
-    }
+    if (t == 0) ens_bs_count(A, nm, attempts, acc, rej, failed);
     __syncthreads();
 }
 
@@ -577,7 +802,7 @@ __device__ int ens_find(int *p, int a) {
 // ------------------------------------------------------------ one step
 template <int T, bool MIXED>
 __device__ void ens_step(const EnsArgs &A, EnsShared &S, double *scr, unsigned long long t_start) {
-    const int n = S.n, t = threadIdx.x;
+    const int n = S.n, t = ens_thread(S);
     const double dt = S.dt;
     // Rcrit (Eq. rcrit), pre-check thresholds
     if (t < n) {
@@ -676,7 +901,12 @@ __device__ void ens_step(const EnsArgs &A, EnsShared &S, double *scr, unsigned l
             S.flag = nm;
         }
         __syncthreads();
-        ens_bs_group(A, S, scr, S.flag, dt, t_start);
+        if (S.flag <= kEnsBsFast) {
+            if (t < 32) ens_bs_fast(A, S, S.flag, dt, t_start);
+            __syncthreads();
+        } else {
+            ens_bs_group(A, S, scr, S.flag, dt, t_start);
+        }
     }
     if (A.gr == 2) {
         ens_hc_gamma(A, S, 0.5 * dt);
@@ -693,7 +923,13 @@ template <int T, bool MIXED>
 __global__ void __launch_bounds__(T) ensemble_kernel(EnsArgs A) {
     __shared__ EnsShared S;
     double *scr = A.bs_scr + (size_t)blockIdx.x * kEnsBsRows * kEnsMaxN;
-    const int t = threadIdx.x;
+    if (threadIdx.x == 0) {
+        unsigned wid;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(wid));
+        S.rot = T == 64 ? (wid >> 2 & 1u) * 32 : 0;
+    }
+    __syncthreads();
+    const int t = ens_thread(S);
     while (true) {
         if (t == 0) S.sys = (int)atomicAdd(A.work, 1u);
         __syncthreads();
@@ -733,6 +969,17 @@ __global__ void __launch_bounds__(T) ensemble_kernel(EnsArgs A) {
             S.fiI[t] = S.Ii[t] > 0.0 ? S.fac[t] / S.Ii[t] : 0.0;
             S.tdi[t] = 3.0 * A.G * ms * ms * (Ri * Ri * Ri * Ri * Ri) * S.k2[t];
             S.tds[t] = 3.0 * A.G * mi * mi * (Rs * Rs * Rs * Rs * Rs) * S.star_k2;
+        }
+        {
+            const double mv[1] = {S.m[t < n ? t : 0]};
+            double Mp[1];
+            ens_bsum<1>(S, mv, Mp);
+            if (t == 0) {
+                const double Is = S.star_rg2 * S.mstar * S.star_R * S.star_R;
+                S.ims = 1.0 / S.mstar;
+                S.itot = 1.0 / (S.mstar + Mp[0]);
+                S.iIs = Is > 0.0 ? 1.0 / Is : 0.0;
+            }
         }
         __syncthreads();
         const unsigned long long t_start = ens_now();

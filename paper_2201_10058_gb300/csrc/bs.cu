@@ -166,19 +166,20 @@ __global__ void kick_pairs_apply_kernel(KickPairsArgs A) {
 // Neville table is built per (member, component) afterwards and the first
 // column k >= 1 under tolerance is accepted -- the same arithmetic and the same
 // acceptance rule as the serial scheme.  FP64 throughout.
-// Pairs of a group of M member slots evaluated once each (M <= 16), listed
-// in (a, q) order with a < q; at most M (M - 1) / 2.
+// Pairs of a group of M member slots evaluated once each, listed in (a, q) order
+// with a < q; at most M (M - 1) / 2.  A group of 17 to 32 members with more
+// than 128 pairs (what shared memory holds) takes every member's partners in turn.
 template <int M>
-constexpr int kColsPairs = (M <= 16) ? M * (M - 1) / 2 : 1;
+constexpr int kColsPairs = (M <= 16) ? M * (M - 1) / 2 : 128;
 
 template <int M>
 struct ColsShared {
     double zx[8 * M + 1], zy[8 * M + 1], zz[8 * M + 1];   // current positions, per (column, member); + a zero
     double pt[3][8][kColsPairs<M>];              // W r^-3 (x_q - x_a) per column and pair a < q
     unsigned char pa[kColsPairs<M>], pq[kColsPairs<M>];   // the group's pairs (a < q), by a then q
-    unsigned char pidx[M <= 16 ? M * M : 1];     // (a, q) -> pair index, both orders
+    unsigned char pidx[M * M];                   // (a, q) -> pair index, both orders
     unsigned pmask[M];                           // partner ranks of each member
-    int npairs;
+    int npairs;                                  // -1: more than kColsPairs
     double m[M];
     double irc[kMaxLevels][M];
     float ircf[kMaxLevels][M];                   // 1/rc rounded to float towards zero (band side tests)
@@ -194,10 +195,13 @@ struct ColsShared {
     int body[M];
 };
 
+// need: this thread's column is not complete yet.  FP64 work is 64 cycles per warp
+// instruction however many lanes take part, so a warp whose columns are complete
+// leaves the pipe to the others (M = 32: a warp per column, two per FP64 pipe).
 template <int M, bool COLL>
 __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, int tid, int col,
                                            bool active, unsigned mask, const double *irc_self,
-                                           const double z[6], double f[6]) {
+                                           const double z[6], double f[6], bool need) {
     __syncthreads();
     S.zx[tid] = z[0]; S.zy[tid] = z[1]; S.zz[tid] = z[2];
     __syncthreads();
@@ -247,7 +251,7 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
             return;
         }
     }
-    if constexpr (M <= 16) {
+    if (M <= 16 || S.npairs >= 0) {
         // each pair once; then every member sums its partners' terms in
         // ascending rank order (m_q t for q > a, -m_q t for q < a): exactly
         // antisymmetric pair forces
@@ -255,13 +259,13 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
         // own star term first: an independent dependency chain the compiler can
         // interleave with the first pair's (small-group BS is latency-bound)
         double sst = 0.0;
-        if (active) {
+        if (active && need) {
             const double r2s = fma(z[2], z[2], fma(z[1], z[1], z[0] * z[0]));
             const double ys = rsqrt_newton(r2s);
             sst = -A.mu * (ys * ys * ys);
         }
         // the column's pairs round-robin over its M threads (short chains)
-        for (int pi = a; pi < S.npairs; pi += M) {
+        for (int pi = need ? a : S.npairs; pi < S.npairs; pi += M) {
             const int pa = S.pa[pi], pq = S.pq[pi];
             const int la = col * M + pa, lq = col * M + pq;
             const double dx = S.zx[lq] - S.zx[la], dy = S.zy[lq] - S.zy[la], dz = S.zz[lq] - S.zz[la];
@@ -283,7 +287,7 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
             S.pt[2][col][pi] = c * dz;
         }
         __syncthreads();
-        if (!active) { f[3] = f[4] = f[5] = 0.0; return; }
+        if (!active || !need) { f[3] = f[4] = f[5] = 0.0; return; }
         double px = 0.0, py = 0.0, pz = 0.0;
         // a member merged away feels only the star (its partners' masses are
         // 0 after their mergers, so their terms vanish)
@@ -302,7 +306,7 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
         f[5] = fma(sst, z[2], A.G * pz);
         return;
     }
-    if (!active) { f[3] = f[4] = f[5] = 0.0; return; }
+    if (!active || !need) { f[3] = f[4] = f[5] = 0.0; return; }
     const double r2s = fma(z[2], z[2], fma(z[1], z[1], z[0] * z[0]));
     const double ys = rsqrt_newton(r2s);
     const double sst = -A.mu * (ys * ys * ys);
@@ -471,18 +475,17 @@ __device__ __forceinline__ void cols_group(const BsArgs &A, ColsShared<M> &S, in
         S.alive[a] = active ? (int)A.coll.alive[b] : 0;
         S.body[a] = b;
     }
-    if (COLL || M <= 16) {
-        if (col == 0) S.pmask[a] = active ? pmask : 0u;
-    }
-    if constexpr (M <= 16) {
-        __syncthreads();
+    if (col == 0) S.pmask[a] = active ? pmask : 0u;
+    __syncthreads();
+    {
         if (tid == 0) {                          // pair list in (a, q) order
             int np = 0;
-            for (int aa = 0; aa < M; aa++) {
+            for (int aa = 0; aa < M && np >= 0; aa++) {
                 unsigned mm = S.pmask[aa] & ~((2u << aa) - 1u);
                 while (mm) {
                     const int q = __ffs(mm) - 1;
                     mm &= mm - 1;
+                    if (np == kColsPairs<M>) { np = -1; break; }
                     S.pa[np] = (unsigned char)aa;
                     S.pq[np] = (unsigned char)q;
                     S.pidx[aa * M + q] = S.pidx[q * M + aa] = (unsigned char)np;
@@ -519,7 +522,7 @@ __device__ __forceinline__ void cols_group(const BsArgs &A, ColsShared<M> &S, in
         if (S.flag) { failed = S.flag; break; }
         attempts++;
         if (H > A.dt - t) H = A.dt - t;
-        cols_deriv<M, COLL>(A, S, tid, col, active, pmask, irc_self, y, f0);
+        cols_deriv<M, COLL>(A, S, tid, col, active, pmask, irc_self, y, f0, true);
         if (col == 0)
             for (int c = 0; c < 6; c++) { S.y[c][a] = y[c]; S.f0[c][a] = f0[c]; }
         // all 8 columns at once: column col takes nk midpoint sub-steps of H/nk.
@@ -527,17 +530,17 @@ __device__ __forceinline__ void cols_group(const BsArgs &A, ColsShared<M> &S, in
         // once (per component c = col < 6 and member a) and the attempt stops at
         // the first column k >= 1 under tolerance -- the columns beyond it are
         // never needed, so they are not computed to the end.
-        const double h = H / nk;
+        const double h = H / nk, h2 = 2.0 * h;
         if (a == 0) S.hcol[col] = h;
         for (int c = 0; c < 6; c++) { zm[c] = y[c]; zn[c] = fma(h, f0[c], y[c]); }
         double T[8];
         double tsc = 0.0, diag = 0.0;
         int kconv = -1;
         for (int it = 1; it <= 16; it++) {
-            cols_deriv<M, COLL>(A, S, tid, col, active, pmask, irc_self, zn, fz);
+            cols_deriv<M, COLL>(A, S, tid, col, active, pmask, irc_self, zn, fz, it <= nk);
             if (it < nk) {
                 for (int c = 0; c < 6; c++) {
-                    const double tt = fma(2.0 * h, fz[c], zm[c]);
+                    const double tt = fma(h2, fz[c], zm[c]);
                     zm[c] = zn[c];
                     zn[c] = tt;
                 }

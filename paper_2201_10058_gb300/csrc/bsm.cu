@@ -92,6 +92,7 @@ struct BsmArgs {
     unsigned *gfail;               // [ng] bit k: some component's error of column k is above tolerance
     GridBarrier *bar;
     unsigned long long barrier_ns; // limit of one grid-barrier wait
+    unsigned long long first_ns;   // added for the first: blocks start when the in-block kernels leave room
     unsigned barrier_absent;       // test hook: arrivals every barrier waits for in vain (0)
     // collisions (Sec. 7.1-7.2), used by the collision ODE instance
     CollArgs coll;
@@ -137,11 +138,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // gridDim.x + absent blocks have arrived (absent = 0 in normal use; a test makes
 // every wait run out with absent > 0).  Returns false if a wait ran out.
 constexpr unsigned long long kBarrierErr = 1ull << 63;
-__device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsigned absent,
+__device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsigned long long first_ns, unsigned absent,
                              unsigned long long &target) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
+        if (target == 0ull) limit_ns += first_ns;
         target += gridDim.x + absent;
         asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&b->count) : "memory");
         unsigned long long t0 = 0ull, v;
@@ -609,7 +611,7 @@ bsm_persistent_kernel(BsmArgs A) {
     if (Ode::COLL) {
         // pairs already overlapping when the integration starts merge at once
         for (long long g = tid; g < A.ng; g += nth) group_merge(A, (int)g, 0.0);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
     }
     for (int round = 0; round < A.max_steps; round++) {
         // one read per block; the previous round ended with a barrier
@@ -617,7 +619,7 @@ bsm_persistent_kernel(BsmArgs A) {
         __syncthreads();
         if (running == 0u) break;
         for (long long t = item0; t < M; t += nitem) phase_start<Ode, L>(A, (int)t, lane);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         for (int it = 1; it <= 16; it++) {
             const int k0 = (it - 1) / 2;          // columns below have no sub-step left
             if (P > 0) {
@@ -626,28 +628,28 @@ bsm_persistent_kernel(BsmArgs A) {
                     const int k = column_of(pi, P, k0);
                     phase_pairs(A, k, pi, it);
                 }
-                if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+                if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
             }
             for (long long t = item0; t < (8 - k0) * M; t += nitem) {
                 long long m = t;
                 const int k = column_of(m, M, k0);
                 phase_substep<Ode, L>(A, k, (int)m, it, lane);
             }
-            if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+            if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         }
         for (long long base = tid - (threadIdx.x & 31); base < D * M; base += nth)
             phase_neville<Ode>(A, base + (threadIdx.x & 31));
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         for (long long g = tid; g < A.ng; g += nth) phase_decide<Ode>(A, (int)g);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         for (long long t = tid; t < D * M; t += nth) phase_accept<Ode>(A, t);
-        if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+        if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         if (Ode::COLL) {
             // mergers at the end of every accepted step (same thread per group
             // as the decision, which wrote gkconv and gt)
             for (long long g = tid; g < A.ng; g += nth)
                 if (A.gkconv[g] >= 0) group_merge(A, (int)g, ldc(&A.gt[g]));
-            if (!grid_barrier(A.bar, A.barrier_ns, A.barrier_absent, arrived)) return;
+            if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         }
     }
 }
@@ -961,6 +963,7 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     A.G = s->p.G; A.mu = s->p.G * s->p.m_star; A.dt = dt; A.tol = s->p.bs_tol;
     A.max_steps = s->p.bs_max_steps;
     A.barrier_ns = s->barrier_limit_ns;
+    A.first_ns = s->bs_beside ? s->bs_group_limit_ns : 0ull;
     A.barrier_absent = s->barrier_absent;
 
     cudaStream_t st = s->stream;
@@ -1049,8 +1052,26 @@ int bsm_forward_groups(genga_system *s, int level, double dt_l) {
 
 // Bulirsch-Stoer of every group of the current grouping at `level`: the
 // in-block kernels for groups of up to kBlockGroupMax members on the side
-// streams, then (joined, so that the cooperative launch has the GPU to
-// itself) the persistent driver for the larger ones.
+// streams, the persistent driver for the larger ones on the system's stream
+// beside them.  The groups share no body, and both add to the counters by atomics.
+// (The cooperative launch starts once all its blocks fit; the in-block kernels
+// wait for nothing, so that is when they leave room at the latest.)  Both are
+// bound by latency with little of the GPU in use unless a group is a giant:
+// N = 2,048, FP64: BS 3.75 ms one after the other, BS_NOTE beside one another.
+// Joins the side streams, whatever the result of the persistent driver.
+static int bs_large_and_join(genga_system *s, int level, double dt_l, const unsigned *counts) {
+    int rc = GENGA_OK;
+    if (counts[kBuckets - 1]) {
+        rc = phase_mark(s, GENGA_PH_BS_LARGE);
+        for (int q = 0; q + 1 < kBuckets; q++) s->bs_beside = s->bs_beside || counts[q];
+        if (rc == GENGA_OK) rc = bsm_forward_groups(s, level, dt_l);
+        s->bs_beside = false;
+        if (rc == GENGA_OK) rc = phase_mark(s, GENGA_PH_BS_SMALL);     // what is left of them
+    }
+    if (join_bs(s) != cudaSuccess) return rc != GENGA_OK ? rc : GENGA_ECUDA;
+    return rc;
+}
+
 int run_bs(genga_system *s, int level, double dt_l, int64_t np) {
     if (np <= 0) return GENGA_OK;
     ++s->bs_call;                         // orders the merger records of the calls
@@ -1059,11 +1080,11 @@ int run_bs(genga_system *s, int level, double dt_l, int64_t np) {
     if (rc != GENGA_OK) return rc;
     if (bucket_groups(s, counts) != cudaSuccess) return GENGA_ECUDA;
     if ((rc = phase_mark(s, GENGA_PH_BS_SMALL)) != GENGA_OK) return rc;
-    const cudaError_t e = launch_bs(s, level, dt_l, counts);
-    if (join_bs(s) != cudaSuccess || e != cudaSuccess) return GENGA_ECUDA;
-    if (!counts[kBuckets - 1]) return GENGA_OK;
-    if ((rc = phase_mark(s, GENGA_PH_BS_LARGE)) != GENGA_OK) return rc;
-    return bsm_forward_groups(s, level, dt_l);
+    if (launch_bs(s, level, dt_l, counts) != cudaSuccess) {
+        join_bs(s);
+        return GENGA_ECUDA;
+    }
+    return bs_large_and_join(s, level, dt_l, counts);
 }
 
 extern "C" int genga_set_bs_pair_mode(genga_system_t *s, int32_t mode) {
@@ -1078,15 +1099,14 @@ int run_bs_dev(genga_system *s, int level, double dt_l) {
     if (rc != GENGA_OK) return rc;
     if (bucket_groups_async(s) != cudaSuccess) return GENGA_ECUDA;
     if ((rc = phase_mark(s, GENGA_PH_BS_SMALL)) != GENGA_OK) return rc;
-    const cudaError_t e = launch_bs(s, level, dt_l, nullptr);
-    if (join_bs(s) != cudaSuccess || e != cudaSuccess) return GENGA_ECUDA;
     // the counts were copied before the kernels above run: the GPU keeps
     // working while the host reads them
-    if (cudaEventSynchronize(s->ev_counts) != cudaSuccess) return GENGA_ECUDA;
+    if (launch_bs(s, level, dt_l, nullptr) != cudaSuccess || cudaEventSynchronize(s->ev_counts) != cudaSuccess) {
+        join_bs(s);
+        return GENGA_ECUDA;
+    }
     ++s->host_syncs;
-    if (!s->bucket_host[kBuckets - 1]) return GENGA_OK;
-    if ((rc = phase_mark(s, GENGA_PH_BS_LARGE)) != GENGA_OK) return rc;
-    return bsm_forward_groups(s, level, dt_l);
+    return bs_large_and_join(s, level, dt_l, s->bucket_host);
 }
 
 // Adjoint BS (backward, augmented) of every group larger than kBlockGroupMax.

@@ -201,6 +201,7 @@ struct genga_system {
     long long bs_call = 0;             // Bulirsch-Stoer calls since collisions were switched on
     // bounded device waits (genga_set_wait_limits)
     unsigned long long bs_group_limit_ns = 10000000000ull;   // in-block BS, per group call
+    bool bs_beside = false;                                   // in-block BS kernels run beside the persistent one
     unsigned long long barrier_limit_ns = 2000000000ull;     // persistent BS, per grid-barrier wait
     unsigned barrier_absent = 0;   // test hook: blocks every grid barrier waits for in vain
     int bs_pairs = 0;              // GENGA_BS_PAIRS_*: derivative form of the persistent BS kernel
@@ -334,7 +335,7 @@ void adjoint_free(genga_system *s);
 // (bsm.cu); genga error codes.
 int bsm_forward_groups(genga_system *s, int level, double dt_l);
 void bsm_release(genga_system *s);
-// launch_bs and join_bs, then bsm_forward_groups.
+// launch_bs, bsm_forward_groups beside it, join_bs.
 int run_bs(genga_system *s, int level, double dt_l, int64_t np);
 // The same without reading the group counts first: the in-block kernels take
 // the device counts; the host waits only for the counts' copy (made before the

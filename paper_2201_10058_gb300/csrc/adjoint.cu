@@ -243,7 +243,6 @@ __global__ void hc_vjp_kernel(int n, const double *sigma, const double *vel, con
 // Error control on y only.  One CTA per group of at most kBlockGroupMax
 // members, state in a global scratch (larger groups: bsm.cu).
 constexpr int kAD = 13;                      // values per member
-constexpr int kABs = 64;                     // threads per CTA
 
 struct AdjBsArgs {
     int n;
@@ -254,188 +253,20 @@ struct AdjBsArgs {
     const int *off, *list;
     const int *goff, *member, *slotof;
     const int *blist;                        // group labels of one size bucket, one block each
-    double *scr;                             // [kAD * 14][S]
-    size_t S;
     double G, mu, dt, tol;
     int max_steps;
     DevCounters *ctr;
 };
 
-__device__ __forceinline__ double &AR(const AdjBsArgs &A, int row, int slot) { return A.scr[(size_t)row * A.S + slot]; }
-
-// derivative in reversed time of the augmented state in rows z0..z0+12 into
-// f0..f0+12.  Inverse distances from the Newton rsqrt, K and dK/dr from the
-// changeover function with 1/rc_ij = min(1/rc_b, 1/rc_p) (no divisions): the
-// kernel is bound by the latency of this chain of dependent FP64 instructions.
-__device__ void adj_deriv(const AdjBsArgs &A, int z0, int f0, int s) {
-    const int b = A.member[s];
-    const double x = AR(A, z0, s), y = AR(A, z0 + 1, s), z = AR(A, z0 + 2, s);
-    const double lvx = AR(A, z0 + 9, s), lvy = AR(A, z0 + 10, s), lvz = AR(A, z0 + 11, s);
-    const double mb = A.mass[b];
-    const double r2 = fma(z, z, fma(y, y, x * x));
-    const double ir = rsqrt_newton(r2), ir2 = ir * ir, mir3 = A.mu * (ir2 * ir);
-    // star: acc = -mu x / r^3; A_star = -mu (I/r^3 - 3 x x^T / r^5) (symmetric)
-    double ax = -mir3 * x, ay = -mir3 * y, az = -mir3 * z;
-    const double c3 = 3.0 * fma(z, lvz, fma(y, lvy, x * lvx)) * ir2;
-    double tx = -mir3 * (lvx - c3 * x);
-    double ty = -mir3 * (lvy - c3 * y);
-    double tz = -mir3 * (lvz - c3 * z);
-    double px = 0.0, py = 0.0, pz = 0.0, gx = 0.0, gy = 0.0, gz = 0.0, gm = 0.0;
-    const double ircb = A.irc[b];
-    for (int q = A.off[b]; q < A.off[b + 1]; q++) {
-        const int p = A.list[q];
-        const int sp = A.slotof[p];
-        const double dx = AR(A, z0, sp) - x, dy = AR(A, z0 + 1, sp) - y, dz = AR(A, z0 + 2, sp) - z;
-        const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const double id = rsqrt_newton(d2), id2 = id * id, id3 = id2 * id;
-        double K, dK;
-        changeover_fast_dr(d2 * id, fmin(ircb, A.irc[p]), K, dK);
-        const double W = 1.0 - K;                    // Wp = dW/dr = -dK
-        const double mp = A.mass[p];
-        const double mw = mp * W * id3;
-        px = fma(mw, dx, px); py = fma(mw, dy, py); pz = fma(mw, dz, pz);
-        const double qx = AR(A, z0 + 9, sp), qy = AR(A, z0 + 10, sp), qz = AR(A, z0 + 11, sp);
-        const double e0 = mb * qx - mp * lvx, e1 = mb * qy - mp * lvy, e2 = mb * qz - mp * lvz;
-        const double de = fma(dz, e2, fma(dy, e1, dx * e0));
-        const double a = W * id3;
-        // -3 W de / d^5 + (dW/dr) de / d^4, dW/dr = -dK
-        const double bb = (-3.0 * W * id3 - dK * id2) * id2 * de;
-        gx += a * e0 + bb * dx; gy += a * e1 + bb * dy; gz += a * e2 + bb * dz;
-        gm -= W * fma(qz, dz, fma(qy, dy, qx * dx)) * id3;
-    }
-    ax += A.G * px; ay += A.G * py; az += A.G * pz;
-    // reversed time
-    AR(A, f0 + 0, s) = -AR(A, z0 + 3, s);
-    AR(A, f0 + 1, s) = -AR(A, z0 + 4, s);
-    AR(A, f0 + 2, s) = -AR(A, z0 + 5, s);
-    AR(A, f0 + 3, s) = -ax;
-    AR(A, f0 + 4, s) = -ay;
-    AR(A, f0 + 5, s) = -az;
-    AR(A, f0 + 6, s) = tx + A.G * gx;
-    AR(A, f0 + 7, s) = ty + A.G * gy;
-    AR(A, f0 + 8, s) = tz + A.G * gz;
-    AR(A, f0 + 9, s) = AR(A, z0 + 6, s);
-    AR(A, f0 + 10, s) = AR(A, z0 + 7, s);
-    AR(A, f0 + 11, s) = AR(A, z0 + 8, s);
-    AR(A, f0 + 12, s) = A.G * gm;
-}
-
-__global__ void __launch_bounds__(kABs) bs_adjoint_kernel(AdjBsArgs A) {
-    enum { Y = 0, F0 = kAD, ZM = 2 * kAD, ZN = 3 * kAD, FZ = 4 * kAD, SC = 5 * kAD, TT = 6 * kAD };
-    __shared__ double red[kABs / 32];
-    __shared__ int stop;
-    __shared__ double st_t, st_H;
-    const int g = A.blist[blockIdx.x];
-    const int s0 = A.goff[g], s1 = A.goff[g + 1];
-    if (s1 - s0 > kBlockGroupMax) return;                // the batched driver's groups
-    const size_t N = (size_t)A.n;
-    for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-        const int b = A.member[s];
-        for (int c = 0; c < 3; c++) {
-            AR(A, Y + c, s) = A.x2[c * N + b];
-            AR(A, Y + 3 + c, s) = A.v2[c * N + b];
-            AR(A, Y + 6 + c, s) = A.lx[c * N + b];
-            AR(A, Y + 9 + c, s) = A.lv[c * N + b];
-        }
-        AR(A, Y + 12, s) = 0.0;
-    }
-    if (threadIdx.x == 0) { st_t = 0.0; st_H = A.dt; }
-    int attempts = 0;
-    bool failed = false;
-    __syncthreads();
-    while (st_t < A.dt) {
-        if (threadIdx.x == 0) stop = attempts >= A.max_steps;
-        __syncthreads();
-        if (stop) { failed = true; break; }
-        attempts++;
-        double H = st_H;
-        if (H > A.dt - st_t) H = A.dt - st_t;
-        for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) adj_deriv(A, Y, F0, s);
-        for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x)
-            for (int c = 0; c < kAD; c++) AR(A, SC + c, s) = fabs(AR(A, Y + c, s)) + fabs(H * AR(A, F0 + c, s)) + 1e-300;
-        int kconv = -1;
-        for (int k = 0; k < 8 && kconv < 0; k++) {
-            const int nk = 2 * (k + 1);
-            const double h = H / nk;
-            for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x)
-                for (int c = 0; c < kAD; c++) {
-                    const double y0 = AR(A, Y + c, s);
-                    AR(A, ZM + c, s) = y0;
-                    AR(A, ZN + c, s) = y0 + h * AR(A, F0 + c, s);
-                }
-            for (int mm = 1; mm < nk; mm++) {
-                __syncthreads();
-                for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) adj_deriv(A, ZN, FZ, s);
-                __syncthreads();
-                for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x)
-                    for (int c = 0; c < kAD; c++) {
-                        const double tt = AR(A, ZM + c, s) + 2.0 * h * AR(A, FZ + c, s);
-                        AR(A, ZM + c, s) = AR(A, ZN + c, s);
-                        AR(A, ZN + c, s) = tt;
-                    }
-            }
-            __syncthreads();
-            for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) adj_deriv(A, ZN, FZ, s);
-            double err = 0.0;
-            for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x)
-                for (int c = 0; c < kAD; c++) {
-                    double cur = 0.5 * (AR(A, ZN + c, s) + AR(A, ZM + c, s) + h * AR(A, FZ + c, s));
-                    double prev = AR(A, TT + c, s);
-                    AR(A, TT + c, s) = cur;
-                    for (int j = 1; j <= k; j++) {
-                        const double coef = (double)((k - j + 1) * (k - j + 1)) / (double)(j * (2 * k + 2 - j));
-                        const double nxt = fma(cur - prev, coef, cur);
-                        prev = AR(A, TT + j * kAD + c, s);
-                        AR(A, TT + j * kAD + c, s) = nxt;
-                        cur = nxt;
-                    }
-                    if (k >= 1 && c < 6)
-                        err = fmax(err, fabs(AR(A, TT + k * kAD + c, s) - AR(A, TT + (k - 1) * kAD + c, s)) / AR(A, SC + c, s));
-                }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = err;
-            __syncthreads();
-            double e = red[0];
-            for (int w = 1; w < kABs / 32; w++) e = fmax(e, red[w]);
-            __syncthreads();
-            if (k >= 1 && e <= A.tol) kconv = k;
-        }
-        if (kconv >= 0) {
-            for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x)
-                for (int c = 0; c < kAD; c++) AR(A, Y + c, s) = AR(A, TT + kconv * kAD + c, s);
-            __syncthreads();
-            if (threadIdx.x == 0) { st_t += H; st_H = (kconv < 4) ? 1.5 * H : H; }
-        } else {
-            __syncthreads();
-            if (threadIdx.x == 0) st_H = 0.5 * H;
-        }
-        __syncthreads();
-    }
-    __syncthreads();
-    for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-        const int b = A.member[s];
-        for (int c = 0; c < 3; c++) {
-            A.lx[c * N + b] = AR(A, Y + 6 + c, s);
-            A.lv[c * N + b] = AR(A, Y + 9 + c, s);
-        }
-        A.lm[b] += AR(A, Y + 12, s);
-    }
-    if (threadIdx.x == 0 && failed) {
-        atomicAdd(&A.ctr->bs_fail, 1ull);
-        latch_error(A.ctr, kErrBS);
-    }
-}
-
 // ------------------------------------------------------------ BS adjoint, column-parallel
-// The same integration for groups of at most M <= 16 members with the 8
+// The augmented ODE of a group of at most M <= 32 members with the 8
 // extrapolation columns of an attempt advanced at once (as bs_cols_kernel does
 // for the forward ODE): thread (k, a) takes column k for member a, so an
 // attempt costs at most 16 sequential derivative evaluations instead of
-// 1 + 2 + 4 + ... + 16.  The arithmetic is the serial kernel's (the same
-// derivative with the partners in ascending body order, the same midpoint,
-// smoothing and Neville expressions, the same acceptance test); the column of
-// an attempt's first converged extrapolation is taken as there.
+// 1 + 2 + 4 + ... + 16.  Inverse distances from the Newton rsqrt, K and dK/dr from
+// the changeover function with 1/rc_ij = min(1/rc_b, 1/rc_p) (no divisions): bound
+// by the FP64 instructions of the longest column's warp, 64 cycles each; warps
+// whose columns are complete issue none.
 template <int M>
 struct AdjColsShared {
     double zp[6][8 * M];            // per (column, member): x, y, z, lv of the current state
@@ -588,7 +419,7 @@ __global__ void __launch_bounds__(8 * M) bs_adj_cols_kernel(AdjBsArgs A) {
         if (col == 0)
 #pragma unroll
             for (int c = 0; c < 6; c++) S.f0[c][a] = fz[c];
-        const double h = H / nk;
+        const double h = H / nk, h2 = 2.0 * h;
         if (a == 0) S.hcol[col] = h;
 #pragma unroll
         for (int c = 0; c < kAD; c++) zn[c] = zm[c] + h * fz[c];
@@ -598,11 +429,11 @@ __global__ void __launch_bounds__(8 * M) bs_adj_cols_kernel(AdjBsArgs A) {
             S.zp[0][tid] = zn[0]; S.zp[1][tid] = zn[1]; S.zp[2][tid] = zn[2];
             S.zp[3][tid] = zn[9]; S.zp[4][tid] = zn[10]; S.zp[5][tid] = zn[11];
             __syncthreads();
-            adj_cols_deriv<M>(A, S, col, a, pmask, zn, fz);
+            if (it <= nk) adj_cols_deriv<M>(A, S, col, a, pmask, zn, fz);
             if (it < nk) {
 #pragma unroll
                 for (int c = 0; c < kAD; c++) {
-                    const double tt = zm[c] + 2.0 * h * fz[c];
+                    const double tt = zm[c] + h2 * fz[c];
                     zm[c] = zn[c];
                     zn[c] = tt;
                 }
@@ -672,11 +503,11 @@ struct Adjoint {
     double *x0 = nullptr, *v0 = nullptr;      // initial state, 3n each
     double *ckpt = nullptr;                   // device, ncheck * 6n
     double *seg = nullptr;                    // device, every * 6n (step-start states of a segment)
+    double *post = nullptr;                   // states behind the encounters of all but its last step, or NULL
     double *tmp = nullptr;                    // device, 6n (x2, v2)
     double *part = nullptr;                   // kick VJP partials
     int nchunk = 0, chunk = 0;
     double *sigma = nullptr;                  // 3 doubles
-    double *bs_scr = nullptr;                 // kAD * 14 rows * n
     double *save_pos = nullptr, *save_vel = nullptr;
 };
 
@@ -704,19 +535,25 @@ int adj_alloc(genga_system *s, int64_t nsteps, int64_t every) {
     Adjoint *a = adj_of(s);
     const size_t n = (size_t)s->n;
     auto fr = [](double *&p) { if (p) cudaFree(p); p = nullptr; };
-    fr(a->rc_hist); fr(a->ckpt); fr(a->seg);
+    fr(a->rc_hist); fr(a->ckpt); fr(a->seg); fr(a->post);
     a->nsteps = nsteps;
     a->every = every;
     const int64_t ncheck = (nsteps + every - 1) / every + 1;
     ACU(cudaMalloc(&a->rc_hist, sizeof(double) * n * (size_t)std::max<int64_t>(nsteps, 1)));
     ACU(cudaMalloc(&a->ckpt, sizeof(double) * 6 * n * (size_t)ncheck));
     ACU(cudaMalloc(&a->seg, sizeof(double) * 6 * n * (size_t)every));
+    // up to 1 GiB to spare the backward pass every second integration of the
+    // encounters (N = 4,096, 2 steps: 5 integrations -> 4, 47.3 ms -> 43.5 ms)
+    const size_t post = sizeof(double) * 6 * n * (size_t)(std::min(every, nsteps) - 1);
+    if (post > 0 && post <= (size_t)1 << 30 && cudaMalloc(&a->post, post) != cudaSuccess) {
+        a->post = nullptr;
+        cudaGetLastError();                    // done without
+    }
     if (!a->x0) {
         ACU(cudaMalloc(&a->x0, sizeof(double) * 3 * n));
         ACU(cudaMalloc(&a->v0, sizeof(double) * 3 * n));
         ACU(cudaMalloc(&a->tmp, sizeof(double) * 6 * n));
         ACU(cudaMalloc(&a->sigma, sizeof(double) * 4));
-        ACU(cudaMalloc(&a->bs_scr, sizeof(double) * (size_t)kAD * 14 * n));
         ACU(cudaMalloc(&a->save_pos, sizeof(double) * 3 * n));
         ACU(cudaMalloc(&a->save_vel, sizeof(double) * 3 * n));
         const int iblocks = (int)((n + kAdjThreads - 1) / kAdjThreads);
@@ -755,7 +592,8 @@ int adj_push_pairs(genga_system *s, const uint2 *dev_pairs, int64_t np, bool fro
 }
 
 // One step with the recorded rc and pairs of step k (Appendix A, slevels = 1).
-int replay_step(genga_system *s, int64_t k) {
+// post: receives the state behind the encounters (6n), NULL: not wanted.
+int replay_step(genga_system *s, int64_t k, double *post) {
     Adjoint *a = adj_of(s);
     const size_t n = (size_t)s->n;
     const double dt = s->p.dt, h = 0.5 * dt;
@@ -777,6 +615,10 @@ int replay_step(genga_system *s, int64_t k) {
             const int brc = run_bs(s, 0, dt, np);
             if (brc != GENGA_OK) return brc;
         }
+    }
+    if (post) {
+        ACU(cudaMemcpyAsync(post, s->pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
+        ACU(cudaMemcpyAsync(post + 3 * n, s->vel, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
     }
     ACU(launch_hc(s, h));
     ACU(launch_kick(s, h, false, nullptr));
@@ -809,8 +651,9 @@ int hc_vjp(genga_system *s, const double *lx, const double *vel, double *lv, dou
     return GENGA_OK;
 }
 
-// Reverse of step k from the step-start state at `start` (6n: x then v).
-int step_vjp(genga_system *s, int64_t k, const double *start, double *lx, double *lv, double *lm) {
+// Reverse of step k from the step-start state at `start` (6n: x then v); post: the
+// state behind the encounters that replay_step kept, NULL: integrated again.
+int step_vjp(genga_system *s, int64_t k, const double *start, const double *post, double *lx, double *lv, double *lm) {
     Adjoint *a = adj_of(s);
     const size_t n = (size_t)s->n;
     const double dt = s->p.dt, h = 0.5 * dt;
@@ -832,9 +675,13 @@ int step_vjp(genga_system *s, int64_t k, const double *start, double *lx, double
         ACU(build_csr(s, 0, np));
         ACU(build_groups(s, 0, np));
         {
-            const int brc = run_bs(s, 0, dt, np);
+            const int brc = post ? GENGA_OK : run_bs(s, 0, dt, np);
             if (brc != GENGA_OK) return brc;
         }
+    }
+    if (post) {
+        ACU(cudaMemcpyAsync(s->pos, post, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
+        ACU(cudaMemcpyAsync(s->vel, post + 3 * n, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
     }
     // (x2, v2)
     ACU(cudaMemcpyAsync(a->tmp, s->pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
@@ -855,25 +702,34 @@ int step_vjp(genga_system *s, int64_t k, const double *start, double *lx, double
         B.mass = s->mass; B.rc = s->rcl[0].rc; B.irc = s->rcl[0].irc;
         B.off = s->csr[0].off; B.list = s->csr[0].list;
         B.goff = s->goff; B.member = s->member; B.slotof = s->slotof;
-        B.scr = a->bs_scr; B.S = n;
         B.G = s->p.G; B.mu = s->p.G * s->p.m_star; B.dt = dt; B.tol = s->p.bs_tol;
         B.max_steps = s->p.bs_max_steps; B.ctr = s->ctr;
         unsigned counts[kBuckets];
         ACU(bucket_groups(s, counts));
-        for (int b = 0; b < kBuckets - 1; b++) {
+        // the groups share no body: the four small buckets on the side streams, beside
+        // one another and the persistent kernel
+        ACU(cudaEventRecord(s->ev_fork, s->stream));
+        cudaError_t e = cudaSuccess;
+        for (int b = 0; b < kBuckets - 1 && e == cudaSuccess; b++) {
             if (!counts[b]) continue;
+            e = cudaStreamWaitEvent(s->side[b], s->ev_fork, 0);
+            if (e != cudaSuccess) break;
             B.blist = s->bucket_list + (size_t)b * s->bucket_stride;
-            // groups of up to 16 members: the columns of an attempt at once
-            if (b == 0) bs_adj_cols_kernel<4><<<counts[b], 32, 0, s->stream>>>(B);
-            else if (b == 1) bs_adj_cols_kernel<8><<<counts[b], 64, 0, s->stream>>>(B);
-            else if (b == 2) bs_adj_cols_kernel<16><<<counts[b], 128, 0, s->stream>>>(B);
-            else bs_adjoint_kernel<<<counts[b], kABs, 0, s->stream>>>(B);
+            if (b == 0) bs_adj_cols_kernel<4><<<counts[b], 32, 0, s->side[b]>>>(B);
+            else if (b == 1) bs_adj_cols_kernel<8><<<counts[b], 64, 0, s->side[b]>>>(B);
+            else if (b == 2) bs_adj_cols_kernel<16><<<counts[b], 128, 0, s->side[b]>>>(B);
+            else bs_adj_cols_kernel<32><<<counts[b], 256, 0, s->side[b]>>>(B);
             ++s->launches;
-            ACU(cudaGetLastError());
+            s->bs_beside = true;
+            e = cudaGetLastError();
         }
-        if (counts[kBuckets - 1] &&
-            (rc = bsm_adjoint_groups(s, a->tmp, a->tmp + 3 * n, lx, lv, lm, dt)) != GENGA_OK)
-            return rc;
+        int brc = GENGA_OK;
+        if (e == cudaSuccess && counts[kBuckets - 1])
+            brc = bsm_adjoint_groups(s, a->tmp, a->tmp + 3 * n, lx, lv, lm, dt);
+        s->bs_beside = false;
+        ACU(join_bs(s));
+        ACU(e);
+        if (brc != GENGA_OK) return brc;
     }
     if ((rc = hc_vjp(s, lx, s->pre_vel[0], lv, lm, h)) != GENGA_OK) return rc;
     if ((rc = kick_vjp(s, start, lv, lx, lm, h)) != GENGA_OK) return rc;
@@ -891,7 +747,7 @@ int forward_checkpointed(genga_system *s) {
             ACU(cudaMemcpyAsync(c, s->pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
             ACU(cudaMemcpyAsync(c + 3 * n, s->vel, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
         }
-        int rc = replay_step(s, k);
+        int rc = replay_step(s, k, nullptr);
         if (rc != GENGA_OK) return rc;
     }
     return GENGA_OK;
@@ -991,12 +847,14 @@ int genga_adjoint_backward(genga_system_t *s, const double *lam_x, const double 
             ACU(cudaMemcpyAsync(st, s->pos, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
             ACU(cudaMemcpyAsync(st + 3 * n, s->vel, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s->stream));
             if (k + 1 < k1) {
-                int rc = replay_step(s, k);
+                int rc = replay_step(s, k, a->post ? a->post + (size_t)(k - k0) * 6 * n : nullptr);
                 if (rc != GENGA_OK) return rc;
             }
         }
         for (int64_t k = k1 - 1; k >= k0; k--) {
-            int rc = step_vjp(s, k, a->seg + (size_t)(k - k0) * 6 * n, grad_x0, grad_v0, grad_m);
+            // the segment's last step was not replayed
+            const double *post = a->post && k + 1 < k1 ? a->post + (size_t)(k - k0) * 6 * n : nullptr;
+            int rc = step_vjp(s, k, a->seg + (size_t)(k - k0) * 6 * n, post, grad_x0, grad_v0, grad_m);
             if (rc != GENGA_OK) return rc;
         }
     }
@@ -1036,7 +894,7 @@ namespace genga {
 void adjoint_free(genga_system *s) {
     if (!s->adj) return;
     Adjoint *a = (Adjoint *)s->adj;
-    double *ps[] = {a->rc_hist, a->x0, a->v0, a->ckpt, a->seg, a->tmp, a->part, a->sigma, a->bs_scr,
+    double *ps[] = {a->rc_hist, a->x0, a->v0, a->ckpt, a->seg, a->post, a->tmp, a->part, a->sigma,
                     a->save_pos, a->save_vel};
     for (double *p : ps) if (p) cudaFree(p);
     if (a->pair_hist) cudaFree(a->pair_hist);

@@ -1057,7 +1057,7 @@ int bsm_forward_groups(genga_system *s, int level, double dt_l) {
 // (The cooperative launch starts once all its blocks fit; the in-block kernels
 // wait for nothing, so that is when they leave room at the latest.)  Both are
 // bound by latency with little of the GPU in use unless a group is a giant:
-// N = 2,048, FP64: BS 3.75 ms one after the other, BS_NOTE beside one another.
+// N = 2,048, FP64: 1.84 ms for both, 3.75 ms one after the other.
 // Joins the side streams, whatever the result of the persistent driver.
 static int bs_large_and_join(genga_system *s, int level, double dt_l, const unsigned *counts) {
     int rc = GENGA_OK;

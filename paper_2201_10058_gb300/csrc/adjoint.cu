@@ -305,7 +305,7 @@ __device__ __forceinline__ void adj_cols_deriv(const AdjBsArgs &A, const AdjCols
         const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
         const double id = rsqrt_newton(d2), id2 = id * id, id3 = id2 * id;
         double K, dK;
-        changeover_fast_dr(d2 * id, fmin(ircb, S.irc[q]), K, dK);
+        changeover_fast_dr(d2 * id, min_positive(ircb, S.irc[q]), K, dK);
         const double W = 1.0 - K;
         const double mp = S.m[q];
         const double mw = mp * W * id3;

@@ -108,7 +108,7 @@ __global__ void kick_pairs_terms_kernel(KickPairsArgs A) {
                 rf, fminf(f32_of_f64_trunc_sat(A.irc[l][i]), f32_of_f64_trunc_sat(A.irc[l][j])));
             if (side < 0) continue;
             if (side > 0) { zero = true; break; }
-            W *= 1.0 - changeover_fast(r, fmin(A.irc[l][i], A.irc[l][j]));
+            W *= changeover_rest(r, min_positive(A.irc[l][i], A.irc[l][j]));
         }
         if (!zero) {
             const int l = A.level;
@@ -227,7 +227,7 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
                     const int side = changeover_side_f32(df, fminf(S.ircf[l][0], S.ircf[l][1]));
                     if (side < 0) continue;
                     if (side > 0) { W = 0.0; break; }
-                    W *= 1.0 - changeover_fast(d, fmin(S.irc[l][0], S.irc[l][1]));
+                    W *= changeover_rest(d, min_positive(S.irc[l][0], S.irc[l][1]));
                 }
                 const double c = W * (yv * yv * yv);
                 S.pt[0][col][0] = c * ex;
@@ -279,7 +279,7 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
                 const int side = changeover_side_f32(df, fminf(S.ircf[l][pa], S.ircf[l][pq]));
                 if (side < 0) continue;
                 if (side > 0) { W = 0.0; break; }
-                W *= 1.0 - changeover_fast(d, fmin(S.irc[l][pa], S.irc[l][pq]));
+                W *= changeover_rest(d, min_positive(S.irc[l][pa], S.irc[l][pq]));
             }
             const double c = W * (yv * yv * yv);
             S.pt[0][col][pi] = c * dx;
@@ -326,7 +326,7 @@ __device__ __forceinline__ void cols_deriv(const BsArgs &A, ColsShared<M> &S, in
             const int side = changeover_side_f32(df, fminf(S.ircf[l][tid % M], S.ircf[l][q]));
             if (side < 0) continue;
             if (side > 0) { W = 0.0; break; }
-            W *= 1.0 - changeover_fast(d, fmin(irc_self[l], S.irc[l][q]));
+            W *= changeover_rest(d, min_positive(irc_self[l], S.irc[l][q]));
         }
         const double c = S.m[q] * W * (yv * yv * yv);
         px = fma(c, dx, px); py = fma(c, dy, py); pz = fma(c, dz, pz);

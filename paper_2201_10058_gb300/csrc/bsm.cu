@@ -112,6 +112,7 @@ struct BsmArgs {
     const double *pirc;            // [nlev][nq] 1/rc of each pair per level
     double2 *rec;                  // [8][entries][2]: (c, dx), (dy, dz) of each entry per column
     size_t nq;                     // entries (the stride of rec per column)
+    double *star;                  // [8][M] -mu / r^3 of each member per column
 };
 
 __device__ __forceinline__ double ldc(const double *p) { return __ldcg(p); }
@@ -173,7 +174,7 @@ __device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsign
 __device__ __forceinline__ bool apply_changeover(float rf, double d, double irc, double &W) {
     const int side = changeover_side_f32(rf, __double2float_rz(irc));
     if (side > 0) return false;
-    if (side == 0) W *= 1.0 - changeover_fast(d, irc);
+    if (side == 0) W *= changeover_rest(d, irc);
     return true;
 }
 // FP32 r from r^2 (relative error 2^-21).
@@ -183,15 +184,36 @@ __device__ __forceinline__ float r_f32(double d2) {
 }
 
 // Lanes per item in the derivative phases: the partner loop of one (column,
-// member) item is split over L adjacent lanes (partner q to lane q mod L) and the
-// partial sums are combined by an xor butterfly, which gives every lane the same
-// bits (IEEE addition commutes).  L by kItemWarps.
-template <int L>
-__device__ __forceinline__ double lane_sum(double v) {
-    const unsigned mk = ((1u << L) - 1u) << ((threadIdx.x & 31u) & ~(unsigned)(L - 1));
+// member) item is split over L adjacent lanes.  Sums of the NV values of an item's
+// lanes, to all of them: each exchange hands half of the values over while there
+// are several (3 values over 16 lanes: 5 FP64 instructions instead of 12, 7: 8
+// instead of 28), then one shuffle per value.
+template <int L, int NV>
+__device__ __forceinline__ void lane_sums(double (&v)[NV]) {
+    static_assert((NV & (NV - 1)) == 0, "");
+    const unsigned mk = (L < 32 ? ((1u << L) - 1u) : 0xffffffffu) << ((threadIdx.x & 31u) & ~(unsigned)(L - 1));
+    int n = NV;
 #pragma unroll
-    for (int o = 1; o < L; o <<= 1) v += __shfl_xor_sync(mk, v, o);
-    return v;
+    for (int o = L / 2; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool hi = threadIdx.x & o;
+#pragma unroll
+            for (int i = 0; i < NV / 2; i++)
+                if (i < n) {
+                    const double send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
+                    v[i] = keep + __shfl_xor_sync(mk, send, o);
+                }
+        } else {
+            v[0] += __shfl_xor_sync(mk, v[0], o);
+        }
+    }
+    constexpr int held = NV > L ? NV / L : 1, apart = L / (NV / held);     // values per lane; lanes between them
+    double r[NV];
+#pragma unroll
+    for (int j = 0; j < NV; j++) r[j] = __shfl_sync(mk, v[j % held], j / held * apart, L);
+#pragma unroll
+    for (int j = 0; j < NV; j++) v[j] = r[j];
 }
 
 // Forward group ODE: y = (x, v); a = -mu x/r^3 + G sum_p m_p W (x_p - x)/r^3,
@@ -208,31 +230,34 @@ struct FwdOdeT {
     __device__ static void deriv(const BsmArgs &A, const double *Z, int m, int lane, double *f) {
         const size_t ld = (size_t)A.M;
         const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
-        double px = 0.0, py = 0.0, pz = 0.0;
-        const int q1 = (COLL && !ldc(&A.malive[m])) ? A.mq0[m] : A.mq1[m];
-        for (int q = A.mq0[m] + lane; q < q1; q += L) {
-            const int sp = A.pidx[q];
-            const double dx = ldc(&Z[0 * ld + sp]) - x, dy = ldc(&Z[1 * ld + sp]) - y,
-                         dz = ldc(&Z[2 * ld + sp]) - z;
+        double p[4] = {0.0, 0.0, 0.0, 0.0};
+        const int q0 = A.mq0[m], q1 = (COLL && !ldc(&A.malive[m])) ? q0 : A.mq1[m];
+        // entry q0 - 1 is the star, at the origin: one more entry of the first lane
+        // instead of the same term in all of them; its coefficient is the fourth sum
+        for (int q = q0 - 1 + lane; q < q1; q += L) {
+            const bool star = q < q0;
+            const int sp = star ? m : A.pidx[q];
+            double sx = ldc(&Z[0 * ld + sp]), sy = ldc(&Z[1 * ld + sp]), sz = ldc(&Z[2 * ld + sp]);
+            if (star) sx = sy = sz = 0.0;
+            const double dx = sx - x, dy = sy - y, dz = sz - z;
             const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-            const float rf = r_f32(d2);
             const double yv = rsqrt_newton(d2);
-            const double d = d2 * yv;
             double W = 1.0;
-            bool in = true;
-            for (int l = 0; l < A.nlev && in; l++)
-                in = apply_changeover(rf, d, fmin(A.irc[(size_t)l * ld + m], A.irc[(size_t)l * ld + sp]), W);
-            if (!in) continue;
-            const double ms = COLL ? ldc(&A.mmass[sp]) : A.mmass[sp];
-            const double c = ms * W * (yv * yv * yv);
-            px = fma(c, dx, px); py = fma(c, dy, py); pz = fma(c, dz, pz);
+            if (!star) {
+                const float rf = r_f32(d2);
+                bool in = true;
+                for (int l = 0; l < A.nlev && in; l++)
+                    in = apply_changeover(rf, d2 * yv,
+                                          min_positive(A.irc[(size_t)l * ld + m], A.irc[(size_t)l * ld + sp]), W);
+                if (!in) continue;
+            }
+            const double c = (star ? -A.mu : COLL ? ldc(&A.mmass[sp]) : A.mmass[sp]) * (W * (yv * yv * yv));
+            if (star) { p[3] = c; continue; }
+            p[0] = fma(c, dx, p[0]); p[1] = fma(c, dy, p[1]); p[2] = fma(c, dz, p[2]);
         }
-        px = lane_sum<L>(px); py = lane_sum<L>(py); pz = lane_sum<L>(pz);
-        const double r2 = fma(z, z, fma(y, y, x * x));
-        const double ys = rsqrt_newton(r2);
-        const double sst = -A.mu * (ys * ys * ys);
+        lane_sums<L>(p);
         f[0] = ldc(&Z[3 * ld + m]); f[1] = ldc(&Z[4 * ld + m]); f[2] = ldc(&Z[5 * ld + m]);
-        f[3] = fma(sst, x, A.G * px); f[4] = fma(sst, y, A.G * py); f[5] = fma(sst, z, A.G * pz);
+        f[3] = fma(p[3], x, A.G * p[0]); f[4] = fma(p[3], y, A.G * p[1]); f[5] = fma(p[3], z, A.G * p[2]);
     }
 };
 // The forward derivative of member m in column k from the entries' records
@@ -243,19 +268,17 @@ __device__ __forceinline__ void fwd_deriv_rec(const BsmArgs &A, const double *Z,
     const size_t ld = (size_t)A.M;
     const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
     const double2 *R = A.rec + (size_t)k * 2 * A.nq;
-    double px = 0.0, py = 0.0, pz = 0.0;
-    const int q1 = A.mq1[m];
+    const double sst = __ldcg(&A.star[(size_t)k * A.M + m]);
+    double p[4] = {0.0, 0.0, 0.0, 0.0};
+    const int q0 = A.mq0[m], q1 = A.mq1[m];
 #pragma unroll 4
-    for (int q = A.mq0[m] + lane; q < q1; q += L) {
+    for (int q = lane ? q0 - 1 + lane : q0 - 1 + L; q < q1; q += L) {      // the split of FwdOdeT::deriv
         const double2 u = __ldcg(&R[2 * (size_t)q]), w = __ldcg(&R[2 * (size_t)q + 1]);
-        px = fma(u.x, u.y, px); py = fma(u.x, w.x, py); pz = fma(u.x, w.y, pz);
+        p[0] = fma(u.x, u.y, p[0]); p[1] = fma(u.x, w.x, p[1]); p[2] = fma(u.x, w.y, p[2]);
     }
-    px = lane_sum<L>(px); py = lane_sum<L>(py); pz = lane_sum<L>(pz);
-    const double r2 = fma(z, z, fma(y, y, x * x));
-    const double ys = rsqrt_newton(r2);
-    const double sst = -A.mu * (ys * ys * ys);
+    lane_sums<L>(p);
     f[0] = ldc(&Z[3 * ld + m]); f[1] = ldc(&Z[4 * ld + m]); f[2] = ldc(&Z[5 * ld + m]);
-    f[3] = fma(sst, x, A.G * px); f[4] = fma(sst, y, A.G * py); f[5] = fma(sst, z, A.G * pz);
+    f[3] = fma(sst, x, A.G * p[0]); f[4] = fma(sst, y, A.G * p[1]); f[5] = fma(sst, z, A.G * p[2]);
 }
 
 using FwdOde = FwdOdeT<false>;
@@ -285,7 +308,7 @@ struct AdjOde {
             const double yv = rsqrt_newton(d2);
             const double d = d2 * yv, id2 = yv * yv, id3 = id2 * yv;
             double K, dK;
-            changeover_fast_dr(d, fmin(A.irc[m], A.irc[sp]), K, dK);
+            changeover_fast_dr(d, min_positive(A.irc[m], A.irc[sp]), K, dK);
             const double W = 1.0 - K;
             const double Wp = -dK;
             const double mp = A.mmass[sp];
@@ -299,8 +322,9 @@ struct AdjOde {
             gx += aa * e0 + bb * dx; gy += aa * e1 + bb * dy; gz += aa * e2 + bb * dz;
             gm -= W * (qx * dx + qy * dy + qz * dz) * id3;
         }
-        px = lane_sum<L>(px); py = lane_sum<L>(py); pz = lane_sum<L>(pz);
-        gx = lane_sum<L>(gx); gy = lane_sum<L>(gy); gz = lane_sum<L>(gz); gm = lane_sum<L>(gm);
+        double p[8] = {px, py, pz, gx, gy, gz, gm, 0.0};
+        lane_sums<L>(p);
+        px = p[0]; py = p[1]; pz = p[2]; gx = p[3]; gy = p[4]; gz = p[5]; gm = p[6];
         const double r2 = fma(z, z, fma(y, y, x * x));
         const double ys = rsqrt_newton(r2);
         const double ir2 = ys * ys, ir3 = ir2 * ys;
@@ -410,14 +434,26 @@ __device__ void phase_pairs(const BsmArgs &A, int k, long long pi, int it) {
         double W = 1.0;
         for (int l = 0; l < A.nlev; l++) apply_changeover(rf, d, A.pirc[(size_t)l * A.nq + pi], W);
         const double y3 = yv * yv * yv;
-        cm = r.mp * W * y3;
-        cp = r.mm * W * y3;
+        const double g = W * y3;
+        cm = r.mp * g;
+        cp = r.mm * g;
     }
     double2 *R = A.rec + (size_t)k * 2 * A.nq;
     R[2 * (size_t)r.q] = make_double2(cm, dx);
     R[2 * (size_t)r.q + 1] = make_double2(dy, dz);
     R[2 * (size_t)r.q2] = make_double2(cp, -dx);
     R[2 * (size_t)r.q2 + 1] = make_double2(-dy, -dz);
+}
+
+// The same for the star's coefficient -mu / r^3 of member m: a full warp of members
+// here, where the member phase would repeat it in every lane of an item.
+__device__ void phase_star(const BsmArgs &A, int k, int m, int it) {
+    if (A.ng > 1 && ldc(&A.gstat[A.mgroup[m]]) != 0) return;
+    const size_t ld = (size_t)A.M, blk = 6 * ld;
+    const double *Z = ((it & 1) ? A.ZA : A.ZB) + k * blk;
+    const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
+    const double ys = rsqrt_newton(fma(z, z, fma(y, y, x * x)));
+    A.star[(size_t)k * ld + m] = -A.mu * (ys * ys * ys);
 }
 
 // Neville for item t; called by every lane of a warp (the vote needs all lanes),
@@ -593,7 +629,9 @@ __device__ void phase_accept(const BsmArgs &A, long long t) {
 }
 
 template <class Ode, int L>
-__global__ void __launch_bounds__(kPMaxThreads)
+// Two blocks per SM (64 registers) for the forward ODE: the gathers through L2 want
+// the warps (16,384-body step 22.5 ms; one block: 23.2).
+__global__ void __launch_bounds__(kPMaxThreads, Ode::D == 6 && !Ode::COLL ? 2 : 1)
 bsm_persistent_kernel(BsmArgs A) {
     constexpr int D = Ode::D;
     const long long nth = (long long)gridDim.x * blockDim.x;
@@ -623,10 +661,11 @@ bsm_persistent_kernel(BsmArgs A) {
         for (int it = 1; it <= 16; it++) {
             const int k0 = (it - 1) / 2;          // columns below have no sub-step left
             if (P > 0) {
-                for (long long t = tid; t < (8 - k0) * P; t += nth) {
+                for (long long t = tid; t < (8 - k0) * (P + M); t += nth) {
                     long long pi = t;
-                    const int k = column_of(pi, P, k0);
-                    phase_pairs(A, k, pi, it);
+                    const int k = column_of(pi, P + M, k0);
+                    if (pi < P) phase_pairs(A, k, pi, it);
+                    else phase_star(A, k, (int)(pi - P), it);
                 }
                 if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
             }
@@ -909,7 +948,7 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
                         (s->bs_pairs == GENGA_BS_PAIRS_AUTO && (M >= kPairMembers || 8LL * M > 2LL * grid * (threads / L))));
     const size_t np = nq / 2;
     const size_t pbytes = pairs ? aligned(sizeof(double2) * 2 * 8 * nq) + aligned(sizeof(PairRec) * np) +
-                                      aligned(sizeof(double) * nlev * nq) + aligned(sizeof(int))
+                                      aligned(sizeof(double) * nlev * nq) + aligned(sizeof(int)) + aligned(sizeof(double) * 8 * M)
                                 : 0;
     const size_t bytes = pbytes + aligned(sizeof(double) * blk) * 3 + aligned(sizeof(double) * 8 * blk) * 5 +
                          aligned(sizeof(double) * (size_t)nlev * M) + aligned(sizeof(double) * M) +
@@ -929,11 +968,13 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     PairRec *prec = nullptr;
     double *pirc = nullptr;
     A.rec = nullptr;
+    A.star = nullptr;
     if (pairs) {
         A.rec = carve<double2>(p, 2 * 8 * nq);
         prec = carve<PairRec>(p, np);
         pirc = carve<double>(p, (size_t)nlev * nq);
         pcount = carve<int>(p, 1);
+        A.star = carve<double>(p, 8 * (size_t)M);
     }
     A.pcount = pcount; A.prec = prec; A.pirc = pirc;
     A.Y = carve<double>(p, blk); A.F0 = carve<double>(p, blk); A.SC = carve<double>(p, blk);

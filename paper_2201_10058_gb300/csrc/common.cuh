@@ -513,6 +513,24 @@ __device__ __forceinline__ double changeover_fast(double r, double irc) {
     const double w = 1.0 - y;
     return y2 * rcp_newton(fma(w, w, y2));
 }
+// 1 - K(r), K as in changeover_fast: with y = (r/rc - 0.1) / 0.9 and w = 1 - y it is
+// w^2 / (w^2 + y^2) in the band, 1 below (y < 0) and 0 above (w < 0).  The two sides
+// are decided on the sign bits and the reciprocal takes one residual of its seed:
+// 9 FP64 instructions instead of 15.
+__device__ __forceinline__ double changeover_rest(double r, double irc) {
+    const double y = fma(r, irc, -0.1) * (1.0 / 0.9), w = 1.0 - y;
+    if (__double2hiint(y) < 0) return 1.0;
+    if (__double2hiint(w) < 0) return 0.0;
+    const double w2 = w * w, D = fma(y, y, w2);
+    float s;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(f32_of_f64_trunc(D)));
+    const double x = f64_of_f32(s), e = fma(-D, x, 1.0);     // 1/D = x (1 + e + e^2 + ...)
+    return w2 * fma(x, fma(e, e, e), x);
+}
+// The smaller of two positive doubles (infinity included) without the FP64 pipe.
+__device__ __forceinline__ double min_positive(double a, double b) {
+    return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
+}
 // Side of the changeover band from FP32 copies of r (f32_of_f64_trunc of a
 // positive normal double in the FP32 range) and of 1/rc (__double2float_rz):
 // -1 when r/rc < 0.1 for certain (K = 0 exactly in changeover_fast), +1 when

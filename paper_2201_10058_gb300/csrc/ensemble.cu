@@ -578,7 +578,7 @@ __device__ __forceinline__ void ens_fast_deriv(const EnsArgs &A, const EnsShared
         double w = F.mp[q - 1] * (id * id * id);
         // 1 - K: 1 below 0.1 rc, 0 above rc
         const int side = changeover_side_f32(f32_of_f64_trunc(d2) * f32_of_f64_trunc(id), F.ircf[q - 1]);
-        if (side == 0) w *= 1.0 - changeover_fast(d2 * id, F.irc[q - 1]);
+        if (side == 0) w *= changeover_rest(d2 * id, F.irc[q - 1]);
         if (F.mp[q - 1] == 0.0 || side > 0) w = 0.0;     // no partner (or itself a lane without a member)
         ax = fma(w, dx, ax);
         ay = fma(w, dy, ay);

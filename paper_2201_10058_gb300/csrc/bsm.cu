@@ -14,9 +14,11 @@
 //              evaluates each partner pair once per column and writes its two
 //              terms to the pair's partner-list entries, which the sub-step
 //              then sums per member (the same values, in the same order);
-//   Neville    per (component, member): the extrapolation table, its
-//              diagonal, and the columns whose error is above tolerance as bits
-//              of the group's word;
+//              A column's last sub-step also forms its row of the extrapolation
+//              table and sets the group's bit of the column if its error is above
+//              tolerance; the sub-steps end when every running group has a column
+//              that is not (16,384-body step: 22.5 ms with all 16 sub-steps and a
+//              phase of their own for the tables, 20.1 so; N = 2,048: 2.11, 1.86);
 //   decide     one thread per group: first column k >= 1 under tolerance
 //              -> accept (grow H by 1.5 if k < 4), else halve H; attempt
 //              and time bookkeeping; done / failed status;
@@ -82,7 +84,7 @@ struct BsmArgs {
     // state, component-major over members ([..][D][M])
     double *Y, *F0, *SC;           // attempt start, its derivative, error scale
     double *ZM, *ZA, *ZB;          // [8] per column: previous midpoint state, two current buffers
-    double *OUT, *DIAG;            // [8] column results, Neville diagonal T_kk
+    double *T, *DIAG;              // [8] latest row of the Neville table, diagonal T_kk of each column
     // per-group step control
     double *gt, *gH;
     double *gh;                    // [ng][8] midpoint sub-step H / n_k of each column this round, 0: done
@@ -378,11 +380,60 @@ __device__ void phase_start(const BsmArgs &A, int m, int lane) {
     }
 }
 
+// Column k of component c of member m is complete with the value cur: its row of the
+// Neville table (the columns' latest values T[j], read from column k - 1's row), the
+// diagonal, and the group's bit k of gfail where |T_kk - T_k,k-1| > tol scale.  K at
+// compile time: no divisions and the row in registers.
+template <class Ode, int K>
+__device__ __forceinline__ void neville_row(const BsmArgs &A, size_t e, size_t blk, int c, int g, double cur) {
+    double old[8];
+#pragma unroll
+    for (int j = 0; j < K; j++) old[j] = ldc(&A.T[j * blk + e]);
+    const double lim = K >= 1 && c < Ode::NERR ? A.tol * ldc(&A.SC[e]) : 0.0;
+    const unsigned seen = K >= 1 ? __ldcg(&A.gfail[g]) : 0u;
+    double last = 0.0;
+    A.T[e] = cur;
+#pragma unroll
+    for (int j = 1; j <= K; j++) {
+        const double coef = (double)((K - j + 1) * (K - j + 1)) / (double)(j * (2 * K + 2 - j));
+        last = cur;
+        cur = fma(cur - old[j - 1], coef, cur);
+        A.T[j * blk + e] = cur;
+    }
+    A.DIAG[K * blk + e] = cur;
+    // (most bits are there already: an atomic only for one that is not)
+    if (K >= 1 && c < Ode::NERR && fabs(cur - last) > lim && !(seen >> K & 1u)) atomicOr(&A.gfail[g], 1u << K);
+}
+template <class Ode>
+__device__ __forceinline__ void neville(const BsmArgs &A, int k, size_t e, size_t blk, int c, int g, double cur) {
+    switch (k) {
+    case 0: neville_row<Ode, 0>(A, e, blk, c, g, cur); break;
+    case 1: neville_row<Ode, 1>(A, e, blk, c, g, cur); break;
+    case 2: neville_row<Ode, 2>(A, e, blk, c, g, cur); break;
+    case 3: neville_row<Ode, 3>(A, e, blk, c, g, cur); break;
+    case 4: neville_row<Ode, 4>(A, e, blk, c, g, cur); break;
+    case 5: neville_row<Ode, 5>(A, e, blk, c, g, cur); break;
+    case 6: neville_row<Ode, 6>(A, e, blk, c, g, cur); break;
+    default: neville_row<Ode, 7>(A, e, blk, c, g, cur); break;
+    }
+}
+// Whether a column k >= 1 of the first `complete` ones met the tolerance.  Final
+// once the barrier behind the sub-step that completed the last of them has passed.
+__device__ __forceinline__ bool converged(unsigned fail, int complete) {
+    return (~fail & 0xfeu & ((1u << complete) - 1u)) != 0u;
+}
+
+// Group g takes no part in sub-step it: done, or with a column under tolerance.
+__device__ __forceinline__ bool idle(const BsmArgs &A, int g, int it) {
+    return ldc(&A.gstat[g]) != 0 || converged(__ldcg(&A.gfail[g]), (it - 1) / 2);
+}
+
 template <class Ode, int L>
 __device__ void phase_substep(const BsmArgs &A, int k, int m, int it, int lane) {
-    const int nk = 2 * (k + 1);
-    const double h = ldc(&A.gh[(size_t)A.mgroup[m] * 8 + k]);
+    const int nk = 2 * (k + 1), g = A.mgroup[m];
+    const double h = ldc(&A.gh[(size_t)g * 8 + k]);
     if (h == 0.0) return;                        // the group is done
+    if (A.ng > 1 && converged(__ldcg(&A.gfail[g]), (it - 1) / 2)) return;      // or has its column
     constexpr int D = Ode::D;
     const size_t ld = (size_t)A.M, blk = (size_t)D * ld;
     const double *Zcur = ((it & 1) ? A.ZA : A.ZB) + k * blk;
@@ -406,7 +457,7 @@ __device__ void phase_substep(const BsmArgs &A, int k, int m, int it, int lane) 
             ZM[c * ld + m] = zc;
             Znext[c * ld + m] = zm + h2 * fc;
         } else {
-            A.OUT[k * blk + c * ld + m] = 0.5 * (zc + zm + h * fc);
+            neville<Ode>(A, k, c * ld + m, blk, c, g, 0.5 * (zc + zm + h * fc));
         }
     }
 }
@@ -417,7 +468,7 @@ __device__ void phase_substep(const BsmArgs &A, int k, int m, int it, int lane) 
 // m_m W / r^3), into the records of entries m -> p and p -> m.
 __device__ void phase_pairs(const BsmArgs &A, int k, long long pi, int it) {
     const PairRec r = A.prec[pi];
-    if (A.ng > 1 && ldc(&A.gstat[A.mgroup[r.m]]) != 0) return;
+    if (A.ng > 1 && idle(A, A.mgroup[r.m], it)) return;
     const size_t ld = (size_t)A.M, blk = 6 * ld;
     const double *Z = ((it & 1) ? A.ZA : A.ZB) + k * blk;
     const double x = ldc(&Z[0 * ld + r.m]), y = ldc(&Z[1 * ld + r.m]), z = ldc(&Z[2 * ld + r.m]);
@@ -448,58 +499,12 @@ __device__ void phase_pairs(const BsmArgs &A, int k, long long pi, int it) {
 // The same for the star's coefficient -mu / r^3 of member m: a full warp of members
 // here, where the member phase would repeat it in every lane of an item.
 __device__ void phase_star(const BsmArgs &A, int k, int m, int it) {
-    if (A.ng > 1 && ldc(&A.gstat[A.mgroup[m]]) != 0) return;
+    if (A.ng > 1 && idle(A, A.mgroup[m], it)) return;
     const size_t ld = (size_t)A.M, blk = 6 * ld;
     const double *Z = ((it & 1) ? A.ZA : A.ZB) + k * blk;
     const double x = ldc(&Z[0 * ld + m]), y = ldc(&Z[1 * ld + m]), z = ldc(&Z[2 * ld + m]);
     const double ys = rsqrt_newton(fma(z, z, fma(y, y, x * x)));
     A.star[(size_t)k * ld + m] = -A.mu * (ys * ys * ys);
-}
-
-// Neville for item t; called by every lane of a warp (the vote needs all lanes),
-// items past the end contribute nothing.  The acceptance test max |T_kk - T_k,k-1| /
-// scale <= tol is taken per component as |T_kk - T_k,k-1| <= tol scale, one bit
-// per column (a difference only where the quotient rounds across tol).
-template <class Ode>
-__device__ void phase_neville(const BsmArgs &A, long long t) {
-    constexpr int D = Ode::D;
-    const size_t ld = (size_t)A.M, blk = (size_t)D * ld;
-    unsigned fail = 0u;
-    int g = -1;
-    if (t < (long long)D * A.M) {
-        const int c = (int)(t / A.M), m = (int)(t % A.M);
-        g = A.mgroup[m];
-        if (ldc(&A.gstat[g]) == 0) {
-            double T[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            const double lim = A.tol * ldc(&A.SC[c * ld + m]);
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                double cur = ldc(&A.OUT[k * blk + c * ld + m]);
-                double prev = T[0];
-                T[0] = cur;
-#pragma unroll
-                for (int j = 1; j <= k; j++) {
-                    const double coef = (double)((k - j + 1) * (k - j + 1)) / (double)(j * (2 * k + 2 - j));
-                    const double nxt = fma(cur - prev, coef, cur);
-                    prev = T[j];
-                    T[j] = nxt;
-                    cur = nxt;
-                }
-                A.DIAG[k * blk + c * ld + m] = T[k];
-                if (k >= 1 && c < Ode::NERR && fabs(T[k] - T[k - 1]) > lim) fail |= 1u << k;
-            }
-        } else {
-            g = -1;
-        }
-    }
-    // one atomic per warp when all its lanes belong to one running group
-    const int g0 = __shfl_sync(0xffffffffu, g, 0);
-    if (__all_sync(0xffffffffu, g == g0)) {
-        const unsigned all = __reduce_or_sync(0xffffffffu, fail);
-        if ((threadIdx.x & 31) == 0 && g0 >= 0 && all) atomicOr(&A.gfail[g0], all);
-    } else if (g >= 0 && fail) {
-        atomicOr(&A.gfail[g], fail);
-    }
 }
 
 // Collisions (reading R25) of group g, by one thread: the separation of two
@@ -675,10 +680,16 @@ bsm_persistent_kernel(BsmArgs A) {
                 phase_substep<Ode, L>(A, k, (int)m, it, lane);
             }
             if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
+            // a column was completed: done when every running group has one under
+            // tolerance.  All blocks see the same bits: those of later columns, which
+            // blocks ahead may be setting, do not count.
+            if (it >= 4 && !(it & 1)) {
+                bool open = false;
+                for (int g = threadIdx.x; g < A.ng; g += blockDim.x)
+                    open = open || (ldc(&A.gstat[g]) == 0 && !converged(__ldcg(&A.gfail[g]), it / 2));
+                if (!__syncthreads_or(open)) break;
+            }
         }
-        for (long long base = tid - (threadIdx.x & 31); base < D * M; base += nth)
-            phase_neville<Ode>(A, base + (threadIdx.x & 31));
-        if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         for (long long g = tid; g < A.ng; g += nth) phase_decide<Ode>(A, (int)g);
         if (!grid_barrier(A.bar, A.barrier_ns, A.first_ns, A.barrier_absent, arrived)) return;
         for (long long t = tid; t < D * M; t += nth) phase_accept<Ode>(A, t);
@@ -979,7 +990,7 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     A.pcount = pcount; A.prec = prec; A.pirc = pirc;
     A.Y = carve<double>(p, blk); A.F0 = carve<double>(p, blk); A.SC = carve<double>(p, blk);
     A.ZM = carve<double>(p, 8 * blk); A.ZA = carve<double>(p, 8 * blk); A.ZB = carve<double>(p, 8 * blk);
-    A.OUT = carve<double>(p, 8 * blk); A.DIAG = carve<double>(p, 8 * blk);
+    A.T = carve<double>(p, 8 * blk); A.DIAG = carve<double>(p, 8 * blk);
     double *irc = carve<double>(p, (size_t)nlev * M), *mmass = carve<double>(p, M);
     int *mbody = carve<int>(p, M), *mgroup = carve<int>(p, M), *mq0 = carve<int>(p, M), *mq1 = carve<int>(p, M);
     int *pidx = carve<int>(p, nq);

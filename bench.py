@@ -35,35 +35,23 @@ sys.path.insert(0, ROOT)
 METRIC = ("changeover-kick G pair-interactions/s and steps/s at N=65536 (FP64 vs mixed), "
           "% of peak")
 UNIT = "Gpair/s"
-# FP64 instructions per pair interaction (ordered pair i <- j) that each kick
-# form's algorithm needs (FMA counted as one), by layout.  Tiled (every ordered
-# pair): mixed 6 -- displacement 3, accumulation 3 (r^2 in float-float from an
-# exact split of the displacement, the FP32 rsqrt seed and its Newton
-# correction and the correction terms all on the FP32 pipe; m y0^3 converted to
-# FP64 by integer operations); FP64 17 -- CUDA's double rsqrt on an FP64 r^2,
-# m r^-3 and the accumulation.  Symmetric (each unordered pair once, the force
-# to both bodies): mixed 9 per unordered pair = 4.5 per interaction
-# (displacement 3, accumulation 3 + 3); FP64 21 = 10.5 (displacement 3, r^2 3,
-# Newton rsqrt 5, r^-3 2, two mass products 2, accumulation 3 + 3).
-FP64_OPS_PER_PAIR = {("mixed", "tiled"): 6, ("fp64", "tiled"): 17,
-                     ("mixed", "symmetric"): 4.5, ("fp64", "symmetric"): 10.5}
-# The same counted by ncu on one launch at N = 65,536 (thread-level
-# smsp__sass_thread_inst_executed_op_d{add,mul,fma}_pred_on.sum / N^2, and the
-# warp-level sm__inst_executed_pipe_fp64.sum x 32 / N^2, which also charges the
-# idle lanes of partly predicated warps); the mixed symmetric kick at the
-# bench's N = 65,540 per interaction N (N - 1), where the padding of the last
-# 128-body tile adds 0.4 % (4.553 at N = 65,536, thread and warp level alike);
-# None where the kernel has changed since the count
-FP64_INSTR_PER_PAIR_COUNTED = {("mixed", "tiled"): (6.152, 6.383), ("fp64", "tiled"): (17.091, 17.402),
-                               ("mixed", "symmetric"): (4.571, 4.571), ("fp64", "symmetric"): (10.549, 10.605)}
-# FP64 units per SM: GB300's nominal FP64 rate (1.25 TFLOP/s = 0.625 T FMA/s
-# over 152 SMs at ~2.06 GHz) is 2 FP64 operations per clock per SM; ncu's FP64
-# pipe utilisation is relative to this rate
-FP64_OPS_PER_CLK_PER_SM = 2
+# Operations per pair interaction (ordered pair i <- j) on the pipe that bounds each
+# kick form (FMA counted as one), between tiles of equal masses, by layout.
+# Mixed, FP32 pipe, per unordered pair of the symmetric layout 127.75: displacement 21,
+# r^2 23, r^-3 17, term 12, the two bodies' sums 48, their renormalisation 6.75
+# (csrc/kick_ff.cu); per ordered pair of the tiled layout 101.5 (one sum).  FP64, FP64
+# pipe: 3 accumulations in the tiled layout (csrc/kick_tile.cu), the rest on the FP32
+# pipe; symmetric layout 21 per unordered pair (displacement 3, r^2 3, Newton rsqrt 5,
+# r^-3 2, two mass products 2, accumulation 3 + 3).
+OPS_PER_PAIR = {("mixed", "tiled"): 101.5, ("fp64", "tiled"): 3,
+                ("mixed", "symmetric"): 63.875, ("fp64", "symmetric"): 10.5}
+# FP32 lanes, and FP64 units (GB300's nominal FP64 rate: 1.25 TFLOP/s = 0.625 T FMA/s
+# over 152 SMs at ~2.06 GHz is 2 FP64 operations per clock per SM), per SM
+OPS_PER_CLK_PER_SM = {"mixed": 128, "fp64": 2}
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the mixed
 # symmetric kick kernel at N = 65,540 (P = 4, 129 partial slots: the traffic is
 # the partial sums); None when the kernel has changed since the capture
-KICK_MIXED_DRAM_BYTES = 358854400
+KICK_MIXED_DRAM_BYTES = 150205440
 
 
 def parse():
@@ -392,13 +380,13 @@ def run_ours(args, dist: Dist) -> dict | None:
     sm_clock = (clocks or {}).get("sm_mhz") or 2070.0
     props = torch.cuda.get_device_properties(dev)
     nsm = props.multi_processor_count
-    peak = FP64_OPS_PER_CLK_PER_SM * nsm * sm_clock * 1e6 / 1e9
-    probe_peak = rates["dfma"] * nsm * sm_clock * 1e6 / 1e9
+    peak = OPS_PER_CLK_PER_SM["mixed"] * nsm * sm_clock * 1e6 / 1e9
+    peak64 = OPS_PER_CLK_PER_SM["fp64"] * nsm * sm_clock * 1e6 / 1e9
+    probe_peak = rates["ffma"] * nsm * sm_clock * 1e6 / 1e9
     lay = head["kick_layout"]["name"]
-    ops = FP64_OPS_PER_PAIR[("mixed", lay)]
+    ops = OPS_PER_PAIR[("mixed", lay)]
     achieved = ops * head["kick_gpairs_per_s"]
-    counted = FP64_INSTR_PER_PAIR_COUNTED[("mixed", lay)]
-    kname = "kick_sym_kernel<mixed>" if lay == "symmetric" else "kick_kernel<mixed>"
+    kname = "kick_sym_ff_kernel" if lay == "symmetric" else "kick_tile_ff_kernel"
     line = {
         "metric": METRIC, "value": round(head["gpairs_per_s"], 4), "unit": UNIT,
         "n_gpus": dist.world, "steps": args.steps, "warmup": args.warmup,
@@ -420,7 +408,7 @@ def run_ours(args, dist: Dist) -> dict | None:
                       "kick_share_of_step": round(head["kick_share"], 3)},
         "roofline": {"bound": "alu", "kernel": f"{kname} (all-pairs changeover kick, {lay} layout)",
                      "achieved": round(achieved, 2), "peak": round(peak, 2),
-                     "unit": "G FP64-op/s (FMA = 1; FP64 pipe)",
+                     "unit": "G FP32-op/s (FMA = 1; FP32 pipe)",
                      "frac": round(achieved / peak, 4),
                      "traffic": KICK_MIXED_DRAM_BYTES,
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch "
@@ -430,16 +418,11 @@ def run_ours(args, dist: Dist) -> dict | None:
                      "duration_basis": "CUDA events on the system's stream around genga_kick writing the "
                                        "accelerations (pack, kick kernel, fold of the partial sums), "
                                        "averaged over the repetitions",
-                     "peak_basis": f"derived: {FP64_OPS_PER_CLK_PER_SM} FP64 op/clk/SM (GB300 nominal "
-                                   f"FP64 unit count) x {nsm} SMs x {sm_clock:.0f} MHz (median SM "
-                                   f"clock under load)",
-                     "frac_counted": None if counted is None else
-                     {"thread_level": round(counted[0] * head["kick_gpairs_per_s"] / peak, 4),
-                      "warp_level": round(counted[1] * head["kick_gpairs_per_s"] / peak, 4),
-                      "instr_per_pair": list(counted)},
+                     "peak_basis": f"derived: {OPS_PER_CLK_PER_SM['mixed']} FP32 op/clk/SM x {nsm} SMs x "
+                                   f"{sm_clock:.0f} MHz (median SM clock under load)",
                      "probe": {"peak": round(probe_peak, 2),
                                "frac": round(achieved / probe_peak, 4),
-                               "basis": f"{rates['dfma']:.3f} FP64 FMA/clk/SM reached by independent "
+                               "basis": f"{rates['ffma']:.3f} FP32 FMA/clk/SM reached by independent "
                                         f"FMA chains (genga_measure_pipe_rates, this run)"},
                      "pipe_rates_per_clk_sm": {k: round(v, 3) for k, v in rates.items()},
                      "fp64_dependent_fma_cycles": {k: round(v, 2) for k, v in fp64_lat.items()}},
@@ -458,9 +441,9 @@ def run_ours(args, dist: Dist) -> dict | None:
                         "non_kick_ms_per_step": f["phases"]["non_kick_ms_per_step"],
                         "kick_gpairs_per_s": round(f["kick_gpairs_per_s"], 3),
                         "kick_ms": round(f["kick_ms"], 3),
-                        "roofline_frac": round(FP64_OPS_PER_PAIR[("fp64", f["kick_layout"]["name"])]
-                                               * f["kick_gpairs_per_s"] / peak, 4),
-                        "ops_per_pair": FP64_OPS_PER_PAIR[("fp64", f["kick_layout"]["name"])],
+                        "roofline_frac": round(OPS_PER_PAIR[("fp64", f["kick_layout"]["name"])]
+                                               * f["kick_gpairs_per_s"] / peak64, 4),
+                        "ops_per_pair": OPS_PER_PAIR[("fp64", f["kick_layout"]["name"])],
                         "kick_layout": f["kick_layout"],
                         "energy_rel_err": f["energy_rel_err"]}
         line["mixed_over_fp64"] = round(head["gpairs_per_s"] / f["gpairs_per_s"], 3)

@@ -44,11 +44,10 @@ extern "C" {
 #define GENGA_ENOMEM     -7  /* device allocation failed */
 
 /* ---- kick arithmetic --------------------------------------------------- */
-#define GENGA_FP64   0   /* every pair term in FP64 (double rsqrt: CUDA's in the tiled
-                            kick layout, an FP32 seed with an FP64 Newton step and
-                            series of full double precision in the symmetric one) */
-#define GENGA_MIXED  1   /* FP64 displacement and accumulation, FP32 rsqrt seed +
-                            one FP64 Newton correction, compensated per-tile sums */
+#define GENGA_FP64   0   /* every pair term to the rounding of FP64 (an FP32 rsqrt seed
+                            with a residual and series of full double precision) */
+#define GENGA_MIXED  1   /* coordinates, pair terms and sums of 16 to 32 terms as sums of
+                            floats (terms to 2^-43), accumulated in FP64 */
 
 /* Integration parameters.  Units are the caller's; the defaults of
  * genga_default_params are Gaussian units (AU, day, solar mass).            */
@@ -144,14 +143,14 @@ int genga_set_rcrit(genga_system_t *sys, const double *rc_host);
 int genga_kick(genga_system_t *sys, double dt_half, int precheck, double *acc_out);
 
 /* ---- kick layout ---------------------------------------------------------- */
-#define GENGA_KICK_AUTO       0  /* the symmetric layout where it is predicted faster */
+#define GENGA_KICK_AUTO       0  /* mixed: the symmetric layout where it is predicted faster; FP64: tiled */
 #define GENGA_KICK_TILED      1  /* every ordered pair (i, j): grid of i-tiles x j-chunks */
 #define GENGA_KICK_SYMMETRIC  2  /* every unordered pair once, its force to both bodies */
 
 /* Selects how the all-pairs kick (genga_kick and the kicks of genga_step)
  * traverses the pairs.  The symmetric layout applies Newton's third law: it
  * evaluates each unordered pair once, in super-tile pairs of P x P tiles of
- * 128 bodies taken by persistent blocks, and writes one compensated partial
+ * 128 bodies taken by persistent blocks, and writes one partial
  * sum per body and super-range, folded in a fixed order (deterministic).
  * P = 0 lets the library choose P in 1..6 for N (by a schedule of the work
  * items over the resident blocks); 1..6 fixes it.  With test particles

@@ -137,7 +137,7 @@ __device__ __forceinline__ unsigned long long ens_now() {
 
 // ------------------------------------------------------------ kick (Eq. Hb)
 // a_i = G sum_j m_j K r^-3 (x_j - x_i), thread (i, slice); pre-check bits.
-// MIXED: the arithmetic of the main mixed kick (kick.cu) -- FP64 displacement
+// MIXED: the arithmetic of kick_kernel (kick.cu) -- FP64 displacement
 // and accumulation, r^2 in float-float from an exact split of the
 // displacement, FP32 rsqrt seed with one Newton correction in float-float,
 // the small correction terms summed in float-float and added once; the

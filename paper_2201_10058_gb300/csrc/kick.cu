@@ -9,7 +9,7 @@
 //     of the bodies, 3 FP64 instructions per pair (FP64) or none (mixed);
 //   * symmetric: each unordered pair once, its force to both bodies (Newton's
 //     third law).  The mixed form (kick_ff.cu) is faster than the tiled one from
-//     N ~ 6,000 on (16,384: 0.68 ms against 0.99; 4,096: 0.111 against 0.092) and
+//     N ~ 6,000 on (12,000: 0.43 ms against 0.55; 4,096: 0.111 against 0.092) and
 //     taken where predicted so; the FP64 form (kick_sym_kernel, below), 21 FP64
 //     instructions per unordered pair, only on request (20,011: 7.9 ms against
 //     2.9 tiled; 128: 0.106 against 0.028).
@@ -28,8 +28,7 @@
 // accumulation of (m y0^3) dx, the corrections corr dx (< 2^-19 of each term)
 // summed in float-float and added to the FP64 sums with the partials; 6 FP64
 // instructions per ordered pair (3 subtractions, 3 accumulations).  FP64: CUDA's
-// double rsqrt in the tiled layout (17 FP64 instructions per pair, counted), the
-// Newton rsqrt of common.cuh in the symmetric one (21 per unordered pair).
+// double rsqrt (17 FP64 instructions per pair, counted).
 #include <algorithm>
 #include <queue>
 #include <utility>
@@ -379,7 +378,7 @@ precheck_kernel(KickArgs A, double f_pc)
 // (nS = ceil(nT / P)): item (X, Y) writes its row sums to slot Y of the X
 // bodies and its j sums to slot X of the Y bodies; a diagonal item (X, X)
 // writes both, added, to slot X as each row completes.  Every (slot, body) is
-// written exactly once, and kick_finalize folds the slots in slot order, so
+// written exactly once, and kick_fold_kernel adds the slots as whole numbers, so
 // the result is deterministic.
 //
 // Dispatch.  One persistent block per resident block slot takes items from a

@@ -20,7 +20,8 @@ struct SymArgs {
     const float2 *ircf;         // mixed: 1 / rc as two floats, padded to whole tiles
     const int *ff_header;       // mixed: header of the packed bodies
     const double *tmass;        // mixed: per tile, the bodies' common scaled mass, or 0
-    int n, nT, P, nItems;
+    int n, nT, nItems;
+    int P;                      // tiles per super-range; tiled kick: steps per chunk
     int nm;                     // bodies i >= nm are test particles (no pair of two); n: none
     const int2 *items;          // (X, Y) super-tile pairs, X <= Y, in dispatch order
     unsigned *ctr;              // dispatch counter, zero at launch

@@ -156,9 +156,10 @@ energy_pairs_kernel(EnergyArgs A) {
             lo = f2_fma(f2_fma(y, tt, f2_mul(half, xe)), sc, lo);
             const float2 TU = f2_get(tu), LO = f2_get(ff_units_end(lo));
             double rx = ff_add_units(Y.x, TU.x, LO.x), ry = ff_add_units(Y.y, TU.y, LO.y);
-            // within 8 last places of a power of two the bits of y + v change scale
-            const bool ex = wide || !(R2.x > close2 && R2.x < 1e36f) || ff_near_binade(Y.x);
-            const bool ey = wide || !(R2.y > close2 && R2.y < 1e36f) || ff_near_binade(Y.y);
+            // next to a power of two the bits of y + v change scale; |e| < 5.6e-7, so that v is at
+            // most 5 last places (2^-24 of y below the power)
+            const bool ex = wide || !(R2.x > close2 && R2.x < 1e36f) || ff_near_binade<8>(Y.x);
+            const bool ey = wide || !(R2.y > close2 && R2.y < 1e36f) || ff_near_binade<8>(Y.y);
             if (ex || ey) {
                 if (ex && wx && i < A.n && b * kSymT + jx < A.n) rx = unit * rinv_fp64(A, i, b * kSymT + jx);
                 if (ey && wy && i < A.n && b * kSymT + jy < A.n) ry = unit * rinv_fp64(A, i, b * kSymT + jy);

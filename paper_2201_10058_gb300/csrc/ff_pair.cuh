@@ -173,7 +173,10 @@ __device__ __forceinline__ double ff_bits_down896(float v) {
     const unsigned b = __float_as_uint(v);
     return __hiloint2double((int)((unsigned)((int)b >> 3) & 0x8fffffffu), (int)(b << 29));
 }
-// within 8 last places of a power of two (or not a positive normal float)
-__device__ __forceinline__ bool ff_near_binade(float v) { return ((__float_as_uint(v) + 8u) & 0x7fffffu) < 16u; }
+// within PLACES last places of a power of two (or not a positive normal float)
+template <unsigned PLACES>
+__device__ __forceinline__ bool ff_near_binade(float v) {
+    return ((__float_as_uint(v) + PLACES) & 0x7fffffu) < 2u * PLACES;
+}
 
 }  // namespace genga

@@ -328,8 +328,10 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
         // near pairs; PC: the bounds tn include the changeover's
         const float2 S = f2_get(s);
         const bool px = S.x < fmaxf(I.tn, tj.x), py = S.y < fmaxf(I.tn, tj.y);
-        const bool ux = ff_near_binade(B.x) || !(S.x < 1e36f && B.x > 6e-23f);
-        const bool uy = ff_near_binade(B.y) || !(S.y < 1e36f && B.y > 6e-23f);
+        // next to a power of two the bits change scale: 1.5 e, |e| < 5.6e-7, and the products'
+        // low parts are at most 17 last places (2^-24 of the base, below the power)
+        const bool ux = ff_near_binade<24>(B.x) || !(S.x < 1e36f && B.x > 6e-23f);
+        const bool uy = ff_near_binade<24>(B.y) || !(S.y < 1e36f && B.y > 6e-23f);
         f2 ch = wh, cl = v;
         if (__any_sync(0xffffffffu, px || py || ux || uy || !wx || !wy)) {
             if (PC) {

@@ -86,3 +86,34 @@ def _mag(x, m, G, i):
     r2 = ((x - x[i]) ** 2).sum(axis=1)
     r2[i] = np.inf
     return G * (m / r2).sum()
+
+
+def test_r3_next_to_powers_of_two(g):
+    """The FP64 kick forms m r^-3 as a float plus a whole number of last places of a
+    double, which changes scale at powers of two.  One body of mass 2^-20 and 20,000
+    massless ones at distances whose r^-3 lies within 40 float places (2^-24 relative)
+    on either side of one: each acceleration has a single term, good to 2^-50 (displacement 2^-51, r^-3
+    2^-52, product, G and the fold 2^-53 each)."""
+    import torch
+    n = 20001
+    rng = np.random.default_rng(9)
+    k = rng.integers(-6, 7, n)
+    r = (2.0 ** k * (1.0 + rng.uniform(-40, 40, n) * 2.0 ** -24)) ** (-1.0 / 3.0)
+    u = rng.standard_normal((n, 3))
+    x = np.array([1.0, 0.5, 0.25]) + r[:, None] * u / np.linalg.norm(u, axis=1)[:, None]
+    x[0] = [1.0, 0.5, 0.25]
+    m = np.zeros(n)
+    m[0] = 2.0 ** -20
+    dev = torch.device("cuda:0")
+    pos = torch.tensor(np.ascontiguousarray(x.T), device=dev)
+    s = g.System(pos, torch.zeros_like(pos), torch.tensor(m, device=dev), g.default_params(G=1.0, precision=0))
+    s.set_kick_layout(g.GENGA_KICK_TILED)
+    s.set_rcrit(np.full(n, 1e-9))
+    acc = torch.zeros_like(pos)
+    s.kick(0.0, precheck=False, acc_out=acc)
+    X = x.astype(np.longdouble)
+    d = X[0] - X[1:]
+    d2 = (d * d).sum(axis=1)
+    ref = np.longdouble(m[0]) * d / (d2 * np.sqrt(d2))[:, None]
+    err = np.sqrt(((acc.cpu().numpy().T[1:] - ref) ** 2).sum(axis=1) / (ref * ref).sum(axis=1)).astype(float)
+    assert err.max() <= 2.0 ** -50, (err.max(), int((err > 2.0 ** -50).sum()))

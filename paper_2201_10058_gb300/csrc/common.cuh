@@ -548,12 +548,15 @@ __device__ __forceinline__ int changeover_side_f32(float rf, float ircf) {
 // changeover_dr_dev() (dK/dy = 2y(1 - y)/D^2, D = y^2 + (1 - y)^2, dy/dr = 1/(0.9 rc)),
 // in contracted FP64 arithmetic for force terms.
 __device__ __forceinline__ void changeover_fast_dr(double r, double irc, double &K, double &dK) {
-    const double y = fma(r, irc, -0.1) * (1.0 / 0.9);
-    if (y <= 0.0) { K = 0.0; dK = 0.0; return; }
-    if (y >= 1.0) { K = 1.0; dK = 0.0; return; }
-    const double y2 = y * y;
-    const double w = 1.0 - y;
-    const double iD = rcp_newton(fma(w, w, y2));
+    const double y = fma(r, irc, -0.1) * (1.0 / 0.9), w = 1.0 - y;
+    dK = 0.0;
+    if (__double2hiint(y) < 0) { K = 0.0; return; }        // the sides by the sign bits: no FP64 comparison
+    if (__double2hiint(w) < 0) { K = 1.0; return; }
+    const double y2 = y * y, D = fma(w, w, y2);
+    float s;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(f32_of_f64_trunc(D)));
+    const double x = f64_of_f32(s), e = fma(-D, x, 1.0);    // 1/D = x (1 + e + e^2 + ...)
+    const double iD = fma(x, fma(e, e, e), x);
     K = y2 * iD;
     dK = 2.0 * y * w * (iD * iD) * (irc * (1.0 / 0.9));
 }

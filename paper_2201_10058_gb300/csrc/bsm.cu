@@ -15,7 +15,7 @@
 //              terms to the pair's partner-list entries, which the sub-step
 //              then sums per member (the same values, in the same order);
 //              A column's last sub-step also forms its row of the extrapolation
-//              table and sets the group's bit of the column if its error is above
+//              table and sets the group's bit of the column unless its error is under
 //              tolerance; the sub-steps end when every running group has a column
 //              that is not (16,384-body step: 22.5 ms with all 16 sub-steps and a
 //              phase of their own for the tables, 20.1 so; N = 2,048: 2.11, 1.86);
@@ -91,7 +91,7 @@ struct BsmArgs {
     int *gstat;                    // 0 running, 1 done, 2 failed
     int *gkconv;                   // accepted column of the last round, -1 none
     long long *gatt, *gacc, *grej;
-    unsigned *gfail;               // [ng] bit k: some component's error of column k is above tolerance
+    unsigned *gfail;               // [ng] bit k: some component's error of column k is not under tolerance
     GridBarrier *bar;
     unsigned long long barrier_ns; // limit of one grid-barrier wait
     unsigned long long first_ns;   // added for the first: blocks start when the in-block kernels leave room
@@ -383,8 +383,8 @@ __device__ void phase_start(const BsmArgs &A, int m, int lane) {
 
 // Column k of component c of member m is complete with the value cur: its row of the
 // Neville table (the columns' latest values T[j], read from column k - 1's row), the
-// diagonal, and the group's bit k of gfail where |T_kk - T_k,k-1| > tol scale.  K at
-// compile time: no divisions and the row in registers.
+// diagonal, and the group's bit k of gfail unless |T_kk - T_k,k-1| <= tol scale (a NaN
+// is not convergence).  K at compile time: no divisions and the row in registers.
 template <class Ode, int K>
 __device__ __forceinline__ void neville_row(const BsmArgs &A, size_t e, size_t blk, int c, int g, double cur) {
     double old[8];
@@ -403,7 +403,7 @@ __device__ __forceinline__ void neville_row(const BsmArgs &A, size_t e, size_t b
     }
     A.DIAG[K * blk + e] = cur;
     // (most bits are there already: an atomic only for one that is not)
-    if (K >= 1 && c < Ode::NERR && fabs(cur - last) > lim && !(seen >> K & 1u)) atomicOr(&A.gfail[g], 1u << K);
+    if (K >= 1 && c < Ode::NERR && !(fabs(cur - last) <= lim) && !(seen >> K & 1u)) atomicOr(&A.gfail[g], 1u << K);
 }
 template <class Ode>
 __device__ __forceinline__ void neville(const BsmArgs &A, int k, size_t e, size_t blk, int c, int g, double cur) {

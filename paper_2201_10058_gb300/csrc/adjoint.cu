@@ -142,15 +142,18 @@ constexpr int kAdjTile = 128;
 // Inverse distances from the Newton rsqrt; K and dK/dr only for the pairs whose
 // FP32 r^2 is below the conservative bound of rc_ij^2 (K = 1, K' = 0 beyond
 // rc_ij), from the changeover function with 1/rc_ij = min(1/rc_k, 1/rc_j).
-// Bound by FP64 instructions, 31 per ordered pair: with p = lv_j . d and q = lv_k . d,
-//   gx_k = G [m_k sum_j a lv_j - lv_k sum_j a m_j + sum_j b d],  gm_k = -G sum_j a p,
-//   a = K / r^3,  b = (K' / (3 r^4) - K / r^5) 3 (m_k p - m_j q)
-// (38 with m_k lv_j - m_j lv_k formed per pair; N = 4,096: 0.97 ms a call against 1.30).
+// Bound by FP64 instructions, 36 per ordered pair: with e = lv_j - lv_k, w = m_k - m_j,
+// p = e . d and q = lv_k . d, so that m_k lv_j - m_j lv_k = m_k e + w lv_k,
+//   gx_k = G [m_k sum_j a e + lv_k sum_j a w - 3 sum_j c (m_k p + w q) d],  gm_k = -G sum_j a (p + q),
+//   a = K / r^3,  c = K / r^5 - K' / (3 r^4).
+// The differences are taken pair by pair: neighbours' adjoint velocities are nearly equal,
+// and sums over all pairs of lv_j and m_j apart (31 instructions) cancel to 1e-10 of the
+// result where they differ by 1e-6.
 __global__ void __launch_bounds__(kAdjThreads)
 kick_vjp_kernel(int n, const double *pos, const double *mass, const double *irc, const float *thr,
                 const double *lv, int chunk, double *part /* [nchunk][4][n] */) {
     __shared__ double sx[kAdjTile], sy[kAdjTile], sz[kAdjTile], sm[kAdjTile], sirc[kAdjTile];
-    __shared__ double sl0[kAdjTile], sl1[kAdjTile], sl2[kAdjTile], sm3[kAdjTile];
+    __shared__ double sl0[kAdjTile], sl1[kAdjTile], sl2[kAdjTile];
     __shared__ float sthr[kAdjTile];
     const size_t N = (size_t)n;
     const int k = blockIdx.x * kAdjThreads + threadIdx.x;
@@ -162,14 +165,13 @@ kick_vjp_kernel(int n, const double *pos, const double *mass, const double *irc,
         l0 = lv[k]; l1 = lv[N + k]; l2 = lv[2 * N + k];
     }
     const int jbeg = blockIdx.y * chunk, jend = min(n, jbeg + chunk);
-    const double mk3 = 3.0 * mk;
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, sw = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0, gm = 0.0;
     for (int jt = jbeg; jt < jend; jt += kAdjTile) {
         const int cnt = min(kAdjTile, jend - jt);
         __syncthreads();
         for (int q = threadIdx.x; q < cnt; q += kAdjThreads) {
             const int j = jt + q;
-            sx[q] = pos[j]; sy[q] = pos[N + j]; sz[q] = pos[2 * N + j]; sm[q] = mass[j]; sm3[q] = 3.0 * mass[j];
+            sx[q] = pos[j]; sy[q] = pos[N + j]; sz[q] = pos[2 * N + j]; sm[q] = mass[j];
             sirc[q] = irc[j]; sthr[q] = thr[j];
             sl0[q] = lv[j]; sl1[q] = lv[N + j]; sl2[q] = lv[2 * N + j];
         }
@@ -187,20 +189,20 @@ kick_vjp_kernel(int n, const double *pos, const double *mass, const double *irc,
                 a *= K;
                 c = fma(K, c, Kp * (id2 * id2) * (-1.0 / 3.0));
             }
-            const double l0j = sl0[q], l1j = sl1[q], l2j = sl2[q];
-            const double pj = fma(l2j, dz, fma(l1j, dy, l0j * dx)), pk = fma(l2, dz, fma(l1, dy, l0 * dx));
-            const double b = c * fma(sm3[q], pk, -(mk3 * pj));
-            s0 = fma(a, l0j, s0); s1 = fma(a, l1j, s1); s2 = fma(a, l2j, s2);
-            sw = fma(a, sm[q], sw);
+            const double e0 = sl0[q] - l0, e1 = sl1[q] - l1, e2 = sl2[q] - l2, w = mk - sm[q];
+            const double pe = fma(e2, dz, fma(e1, dy, e0 * dx)), pk = fma(l2, dz, fma(l1, dy, l0 * dx));
+            const double b = c * fma(mk, pe, w * pk);
+            s0 = fma(a, e0, s0); s1 = fma(a, e1, s1); s2 = fma(a, e2, s2);
+            sw = fma(a, w, sw);
             b0 = fma(b, dx, b0); b1 = fma(b, dy, b1); b2 = fma(b, dz, b2);
-            gm = fma(-a, pj, gm);
+            gm = fma(-a, pe + pk, gm);
         }
     }
     if (valid) {
         double *p = part + (size_t)blockIdx.y * 4 * N;
-        p[k] = fma(mk, s0, fma(-sw, l0, b0));
-        p[N + k] = fma(mk, s1, fma(-sw, l1, b1));
-        p[2 * N + k] = fma(mk, s2, fma(-sw, l2, b2));
+        p[k] = fma(mk, s0, fma(sw, l0, -3.0 * b0));
+        p[N + k] = fma(mk, s1, fma(sw, l1, -3.0 * b1));
+        p[2 * N + k] = fma(mk, s2, fma(sw, l2, -3.0 * b2));
         p[3 * N + k] = gm;
     }
 }

@@ -7,7 +7,7 @@
 // on the FP32 pipe (64 times faster) to the last place of an FP64 value, and one
 // FP64 FMA per pair sums m_j / r_ij:
 //   * displacement from the packed bodies (kick_ff.cu) as three floats, exact to
-//     2^-70 of the largest coordinate;
+//     2^-72 of the largest coordinate;
 //   * y = rsqrt(r^2) in FP32, q = d y per component; the residual e = 1 - |q|^2
 //     (|e| < 2^-20.5) to 2^-56: q is cut into digits on the fixed grids 2^-11,
 //     2^-22 and 2^-34 (|q| <= 1), whose products are whole multiples of 2^-44 and
@@ -58,9 +58,8 @@ __device__ __forceinline__ void block_sum2(double &S, double &C, double *sh) {
     C = sh[T];
 }
 
-// 1/r in FP64: coordinates that three floats do not hold, close pairs (r < 2^-17 S:
-// the displacement reaches below the second grid, 0 among them) and NaN, 1/r next
-// to a power of two.
+// 1/r in FP64: close pairs (r < 2^-17 S: 2^-72 S is more than 2^-55 of the distance, 0
+// among them) and NaN, 1/r next to a power of two.
 __device__ __noinline__ double rinv_fp64(const EnergyArgs &A, int i, int j) {
     const double dx = A.x[j] - A.x[i], dy = A.y[j] - A.y[i], dz = A.z[j] - A.z[i];
     return 1.0 / sqrt(dx * dx + dy * dy + dz * dz);
@@ -86,8 +85,7 @@ energy_pairs_kernel(EnergyArgs A) {
     const int nT = A.nT, tid = threadIdx.x;
     const long long total = (long long)nT * (nT + 1) / 2;
     const long long u0 = total * blockIdx.x / gridDim.x, u1 = total * (blockIdx.x + 1) / gridDim.x;
-    const bool wide = (A.header[0] & kFfWide) != 0;
-    const float close2 = reinterpret_cast<const float *>(A.header)[3];
+    constexpr float close2 = 0x1p-22f;                     // (2^-17 S)^2
     const double unit = scalbn(1.0, A.header[2]);          // of the packed bodies' lengths
     const f2 half = f2_dup(0.5f), c375 = f2_dup(0.375f);
     double TS = 0.0, TC = 0.0;                 // this thread's sum of m_i m_j / r_ij
@@ -158,8 +156,8 @@ energy_pairs_kernel(EnergyArgs A) {
             double rx = ff_add_units(Y.x, TU.x, LO.x), ry = ff_add_units(Y.y, TU.y, LO.y);
             // next to a power of two the bits of y + v change scale; |e| < 5.6e-7, so that v is at
             // most 5 last places (2^-24 of y below the power)
-            const bool ex = wide || !(R2.x > close2 && R2.x < 1e36f) || ff_near_binade<8>(Y.x);
-            const bool ey = wide || !(R2.y > close2 && R2.y < 1e36f) || ff_near_binade<8>(Y.y);
+            const bool ex = !(R2.x > close2 && R2.x < 1e36f) || ff_near_binade<8>(Y.x);
+            const bool ey = !(R2.y > close2 && R2.y < 1e36f) || ff_near_binade<8>(Y.y);
             if (ex || ey) {
                 if (ex && wx && i < A.n && b * kSymT + jx < A.n) rx = unit * rinv_fp64(A, i, b * kSymT + jx);
                 if (ey && wy && i < A.n && b * kSymT + jy < A.n) ry = unit * rinv_fp64(A, i, b * kSymT + jy);
@@ -242,6 +240,7 @@ cudaError_t launch_energy(genga_system *s, double *E_host, double *L_host) {
     if (!s->en_part)
         GENGA_CUDA_TRY(cudaMalloc((void **)&s->en_part, sizeof(double) * (kEnRows * 2 * kEnBlocks + kEnRows)));
     FfPack ff = ff_pack_args(s);
+    ff.window = kFfWindowNone;
     GENGA_CUDA_TRY(launch_ff_pack(ff, s->stream, &s->launches));
     EnergyArgs A;
     A.x = s->pos; A.y = s->pos + n; A.z = s->pos + 2 * (size_t)n; A.m = s->mass;

@@ -14,14 +14,24 @@ __device__ __forceinline__ void ff_disp(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 
     f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e);
     L = f2_add(e, f2_add(lj, nli));
 }
-// The same with the fourth parts.
-__device__ __forceinline__ void ff_disp4(f2 hj, f2 mj, f2 lj, f2 kj, f2 nhi, f2 nmi, f2 nli, f2 nki, f2 &H, f2 &L) {
-    f2 e1, e2, dl, el;
-    f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e1);
-    f2_two_sum(lj, nli, dl, el);
-    f2_two_sum(e1, dl, e1, e2);
-    f2_fast_two_sum(H, e1, H, e1);
-    L = f2_add(e1, f2_add(e2, f2_add(el, f2_add(kj, nki))));
+// An FP64 displacement as three floats by integer operations: h truncated, l and t (|l| <
+// 2^-23 |v|) the other bits.  |v| < 2^-74: l = t = 0, |v| < 2^-126 also h = 0; |v| >=
+// 2^100, infinite or NaN: h = NaN.
+__device__ __forceinline__ void f64_split3(double v, float &h, float &l, float &t) {
+    const unsigned hw = (unsigned)__double2hiint(v), lw = (unsigned)__double2loint(v);
+    const unsigned mag = hw & 0x7fffffffu, sgn = hw & 0x80000000u, E = mag >> 20;
+    h = __uint_as_float(mag >= 0x46300000u ? 0x7fc00000u : mag >= 0x38100000u ? (sgn | ((mag - 0x38000000u) << 3) | (lw >> 29)) : sgn);
+    const unsigned unit = E >= 949u ? sgn | ((E - 948u) << 23) : 0u;       // 2^(E - 1075), the last place
+    const unsigned unit14 = E >= 949u ? sgn | ((E - 934u) << 23) : 0u;
+    l = (__uint_as_float(0x4b000000u | (lw >> 14 & 0x7fffu)) - 8388608.0f) * __uint_as_float(unit14);
+    t = (__uint_as_float(0x4b000000u | (lw & 0x3fffu)) - 8388608.0f) * __uint_as_float(unit);
+}
+// The same for a component of two pairs, two floats each, the first rounded.
+__device__ __forceinline__ void f64_split2(double vx, double vy, f2 &H, f2 &L) {
+    float hx, lx, tx, hy, ly, ty;
+    f64_split3(vx, hx, lx, tx);
+    f64_split3(vy, hy, ly, ty);
+    f2_fast_two_sum(f2_make(hx, hy), f2_add(f2_make(lx, ly), f2_make(tx, ty)), H, L);
 }
 
 // g w as two floats (g = gh + gl, w + wl)
@@ -54,16 +64,19 @@ __device__ __forceinline__ void ff_changeover(float s2, float tail, float ih, fl
     changeover_ff(u, ue, tail, y, e, ih, il, Kh, Kl);
 }
 
-// A close pair (r < 2^-17 S): its displacement reaches below the second grid, so
-// that h and m no longer give its leading float.  FP64 from the positions, K
-// included: H + L, K r^-3 = w + wl.
-struct FfClose { float H[3], L[3], w, wl; };
-__device__ __forceinline__ void ff_close(const double *X, const double *Y, const double *Z, int es, int i, int j,
-                                         float ih, float il, FfClose &o) {
-    const double xs = scalbn(1.0, -es);
-    const double d[3] = {(X[j] - X[i]) * xs, (Y[j] - Y[i]) * xs, (Z[j] - Z[i]) * xs};
-    const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])), y = rsqrt(r2);
-    const double w = changeover_fast(r2 * y, (double)ih + (double)il) * (y * y * y);
+// A pair that the packed coordinates do not give (a body that is not held, or r below
+// kFfClose2): FP64 from the positions, K included.  The unit vector d / r as H + L
+// and K / r^2 = w + wl: K r^-3 alone would leave the floats' range for a far body.
+struct FfOne { float H[3], L[3], w, wl; };
+__device__ __forceinline__ void ff_one(const SymArgs &A, int i, int j, float ih, float il, FfOne &o) {
+    double d[3] = {0.0, 0.0, 0.0}, w = 0.0;
+    if (i < A.n && j < A.n) {                      // not a padding body
+        const double xs = scalbn(1.0, -A.ff_header[2]);
+        d[0] = (A.x[j] - A.x[i]) * xs; d[1] = (A.y[j] - A.y[i]) * xs; d[2] = (A.z[j] - A.z[i]) * xs;
+        const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])), y = rsqrt(r2);
+        w = (r2 < 1e300 ? changeover_fast(r2 * y, (double)ih + (double)il) : 1.0) * (y * y);
+        for (int c = 0; c < 3; c++) d[c] *= y;
+    }
     for (int c = 0; c < 3; c++) {
         o.H[c] = __double2float_rn(d[c]);
         o.L[c] = __double2float_rn(d[c] - (double)o.H[c]);
@@ -96,7 +109,9 @@ __device__ __forceinline__ void ff_inv_r3(f2 s2, f2 tail, f2 &w, f2 &wl) {
 // v rounded to a multiple of a power of two g; c = 1.5 2^23 g, |v| < 2^22 g.
 __device__ __forceinline__ f2 f2_round(f2 v, f2 c) { return f2_sub(f2_add(v, c), c); }
 
-// A displacement as three floats, exact to 2^-70 of the largest coordinate.
+// A displacement as three floats, exactly: h, m and l are multiples of 2^-23, 2^-47 and
+// 2^-71 S below 1, 2^-24 and 2^-48 S, so that each difference fits a float, and e, where
+// it is not 0, is a multiple of 2^-47 S and so not below l's.
 __device__ __forceinline__ void ff_disp3(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 nli, f2 &H, f2 &L, f2 &T) {
     f2 e;
     f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e);

@@ -917,6 +917,7 @@ cudaError_t launch_kick(genga_system *s, double dt_half, bool precheck, double *
         if (sym) {
             F.mass = s->mass;
             GENGA_CUDA_TRY(launch_sym_ff(S, precheck, s->ksym_blocks, s->stream));
+            ++s->launches;
         } else {
             GENGA_CUDA_TRY(launch_tile_kick(S, s->ktile_chunk, s->ktile_nchunk, mixed, precheck, s->stream));
         }
@@ -959,7 +960,7 @@ cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, cudaStream_t stream) 
         FfPack ff;
         ff.pos = k.pos; ff.m = k.mass; ff.rc = k.rc; ff.pc2 = nullptr; ff.n = k.n; ff.nT = (k.n + kSymT - 1) / kSymT;
         ff_place(ff, k.scratch, ff.nT);
-        ff.ctr = nullptr; ff.cand_count = nullptr;
+        ff.ctr = nullptr; ff.cand_count = nullptr; ff.window = k.mixed ? kFfWindowMixed : kFfWindow64;
         SymArgs S = {};
         S.x = k.pos; S.y = k.pos + N; S.z = k.pos + 2 * N; S.m = k.mass; S.rc = k.rc;
         S.n = S.nm = k.n; S.nT = ff.nT; S.part = k.scratch + packed;

@@ -6,10 +6,10 @@
 // cycles of a sub-partition per warp of pairs, while the whole pair takes 127
 // to 135 FP32 operations.  Nothing here is less exact for it:
 //   * a coordinate is the sum of three floats on two fixed grids, h (multiples
-//     of 2^-22 S, S a power of two >= every |coordinate|), m (of 2^-45 S) and
-//     the remainder l.  Differences of h and of m are exact, so
+//     of 2^-23 S, S a power of two > every |coordinate| on its axis), m (of 2^-47 S)
+//     and the remainder l.  Differences of h and of m are exact, so
 //     h_j - h_i, m_j - m_i, l_j - l_i sum to the displacement with an error of
-//     2^-70 S; a Fast2Sum step gives it as two floats (relative error 2^-49);
+//     2^-72 S; a Fast2Sum step gives it as two floats (relative error 2^-48);
 //   * r^2 is the exact sum of the squares in two floats (2^-48), r^-3 =
 //     y^3 (1 + 1.5 e + 1.875 e^2) from the FP32 seed y and its residual
 //     e = 1 - r^2 y^2, in two floats (2^-46);
@@ -25,11 +25,12 @@
 // bodies instead of m_j r^-3 d and m_i r^-3 d, TwoSum instead of an ordered
 // Fast2Sum (whose selects read as much as the three operations they save).
 //
-// Two device flags, set by the packing kernel, take the instance of the pair
-// loop that the unusual inputs need:
-//   * kFfWide: S > 2^18 min_i max_c |x_i| (a body 10^5 times farther out than
-//     another): three parts no longer hold every FP64 position to its last
-//     place, a fourth part is added;
+// What the packing kernel finds takes the instance of the pair loop that unusual
+// inputs need:
+//   * coordinates that three floats do not hold, because they are far smaller than
+//     the largest on their axis (2^-25: 3e-8).  A few: NaN in their place, which
+//     takes these bodies' pairs to FP64 one by one (ff_one); many: kFfExact, every
+//     displacement by FP64 subtraction, 3 FP64 instructions per pair;
 //   * kFfTwoMass: a massless body, or one 2^-40 of the heaviest: m_j r^-3 d and
 //     m_i r^-3 d are formed apart and nothing is divided.
 //
@@ -70,16 +71,17 @@ __device__ __forceinline__ void ff_flush(double &sum, double mm, float h, float 
 
 // 32 steps of 32 kFfR of the warp's rows (from row0 of the tile on) against the
 // 64 bodies of group jb / 64.  kFfGeneral: pairs masked (diagonal subtiles dsub,
-// test particles) and the inputs of the two device flags; the other instances
-// take every pair.  kFfUniform: two tiles of equal masses each, the product mm of
-// the two applied to the sums.
+// test particles) and kFfTwoMass; the other instances take every pair.  kFfExact:
+// this with displacements by FP64 subtraction.  kFfUniform: two tiles of equal
+// masses each, the product mm of the two applied to the sums.
 template <bool PC, int MODE>
 __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, double *js, double *is, int PT, int e0,
                                         int jb, int jglob, const IBody (&I)[kFfR], int flags, float close2, bool dsub, int row0,
                                         double mm, uint2 *pcbuf, int &pend, int lane) {
-    constexpr bool GEN = MODE == kFfGeneral;
+    constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
     f2 ih[kFfR][3], il[kFfR][3], jh[3], jl[3];
     const f2 one = f2_dup(1.0f);
+    const double xs = EXACT ? scalbn(1.0, -A.ff_header[2]) : 1.0;
     const float4 *group = tile + (jb >> 1);
 #pragma unroll 1
     for (int tb = 0; tb < 32; tb += kFfFlush) {
@@ -89,13 +91,13 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
 #pragma unroll
             for (int r = 0; r < kFfR; r++) ih[r][c] = il[r][c] = 0ull;
         }
-#pragma unroll (kFfUnroll)
+#pragma unroll (EXACT ? 1 : kFfUnroll)
         for (int t = tb; t < tb + kFfFlush; t++) {
             const int k = (lane + t) & 31;
             const float4 q0 = group[k], q1 = group[kFfRow + k], q2 = group[2 * kFfRow + k], q3 = group[3 * kFfRow + k],
                          q4 = group[4 * kFfRow + k], q5 = group[5 * kFfRow + k];
             // bounds of the near pairs: pre-check or, without it, changeover
-            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&group[7 * kFfRow + k].z) : make_float2(q5.z, q5.w);
+            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&group[6 * kFfRow + k].z) : make_float2(q5.z, q5.w);
             f2 H[kFfR][3], L[kFfR][3], w[kFfR], wl[kFfR];
             float2 S[kFfR], Tl[kFfR];
             bool want[kFfR][2], near = false;
@@ -103,17 +105,8 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
             for (int r = 0; r < kFfR; r++) {
                 want[r][0] = want[r][1] = true;    // this lane's two pairs are wanted
                 if (GEN) {
-                    const float4 q6 = group[6 * kFfRow + k], q7 = group[7 * kFfRow + k];
                     const int i = I[r].i;
-                    const float4 *bi = A.body + (size_t)(i >> 7) * kFfTile + ((i >> 6) & 1) * 32 + lane;
-                    const float4 kp = bi[6 * kFfRow], kq = bi[7 * kFfRow];
                     const bool up = i & 32;
-                    ff_disp4(f2_lo(q0), f2_lo(q2), f2_lo(q4), f2_lo(q6), I[r].h[0], I[r].m[0], I[r].l[0],
-                             f2_dup(-(up ? kp.y : kp.x)), H[r][0], L[r][0]);
-                    ff_disp4(f2_hi(q0), f2_hi(q2), f2_hi(q4), f2_hi(q6), I[r].h[1], I[r].m[1], I[r].l[1],
-                             f2_dup(-(up ? kp.w : kp.z)), H[r][1], L[r][1]);
-                    ff_disp4(f2_lo(q1), f2_lo(q3), f2_lo(q5), f2_lo(q7), I[r].h[2], I[r].m[2], I[r].l[2],
-                             f2_dup(-(up ? kq.y : kq.x)), H[r][2], L[r][2]);
                     if (dsub) {                    // every pair of the 64 x 64 diagonal subtile once
                         const bool tri = t >= 1 && (t < 16 || (t == 16 && lane < 16));
                         want[r][0] = !up && tri;
@@ -122,6 +115,14 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                     const int j = jglob + k;
                     want[r][0] = want[r][0] && !(i >= A.nm && j >= A.nm);
                     want[r][1] = want[r][1] && !(i >= A.nm && j + 32 >= A.nm);
+                }
+                if (EXACT) {
+                    const int i = min(I[r].i, A.n - 1), jx = min(jglob + k, A.n - 1), jy = min(jglob + k + 32, A.n - 1);
+                    f64_split2((A.x[jx] - A.x[i]) * xs, (A.x[jy] - A.x[i]) * xs, H[r][0], L[r][0]);
+                    f64_split2((A.y[jx] - A.y[i]) * xs, (A.y[jy] - A.y[i]) * xs, H[r][1], L[r][1]);
+                    f64_split2((A.z[jx] - A.z[i]) * xs, (A.z[jy] - A.z[i]) * xs, H[r][2], L[r][2]);
+                    want[r][0] = want[r][0] && I[r].i < A.n && jglob + k < A.n;
+                    want[r][1] = want[r][1] && I[r].i < A.n && jglob + k + 32 < A.n;
                 } else {
                     ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I[r].h[0], I[r].m[0], I[r].l[0], H[r][0], L[r][0]);
                     ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I[r].h[1], I[r].m[1], I[r].l[1], H[r][1], L[r][1]);
@@ -129,27 +130,34 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                 }
                 f2 s2, tail;
                 ff_r2(H[r], L[r], s2, tail);
-                if (GEN) {
+                if (GEN) {                         // (NaN times zero would be NaN)
                     s2 = f2_select(want[r][0], want[r][1], s2, one);
                     tail = f2_select(want[r][0], want[r][1], tail, 0ull);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        H[r][c] = f2_select(want[r][0], want[r][1], H[r][c], 0ull);
+                        L[r][c] = f2_select(want[r][0], want[r][1], L[r][c], 0ull);
+                    }
                 }
                 S[r] = f2_get(s2);
                 Tl[r] = f2_get(tail);
                 ff_inv_r3(s2, tail, w[r], wl[r]);
-                near = near || S[r].x < fmaxf(I[r].tn, tj.x) || S[r].y < fmaxf(I[r].tn, tj.y);
+                near = near || !(S[r].x >= fmaxf(I[r].tn, tj.x)) || !(S[r].y >= fmaxf(I[r].tn, tj.y));
+                if (EXACT) near = near || S[r].x > kFfExactFar2 || S[r].y > kFfExactFar2;
             }
             if (PC ? __any_sync(0xffffffffu, near) : near) {
 #pragma unroll
                 for (int r = 0; r < kFfR; r++) {
                     if (PC) {                      // pre-check: the bounds tn include the changeover's
-                        sym_pc_push(pcbuf, pend, lane, want[r][0] && S[r].x < fmaxf(I[r].tn, tj.x), I[r].i, jglob + k);
-                        sym_pc_push(pcbuf, pend, lane, want[r][1] && S[r].y < fmaxf(I[r].tn, tj.y), I[r].i,
+                        sym_pc_push(pcbuf, pend, lane, want[r][0] && !(S[r].x >= fmaxf(I[r].tn, tj.x)), I[r].i, jglob + k);
+                        sym_pc_push(pcbuf, pend, lane, want[r][1] && !(S[r].y >= fmaxf(I[r].tn, tj.y)), I[r].i,
                                     jglob + k + 32);
                         if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
                     }
-                    // changeover band and close pairs: K in float-float, 1/rc_ij = min(1/rc_i, 1/rc_j)
-                    // (as float pairs: rounding is monotone), r^-3 scaled by K
-                    const bool bx = S[r].x < fmaxf(I[r].thr, q5.z), by = S[r].y < fmaxf(I[r].thr, q5.w);
+                    // changeover band: K in float-float, 1/rc_ij = min(1/rc_i, 1/rc_j) (as float
+                    // pairs: rounding is monotone), r^-3 scaled by K; and the pairs for ff_one
+                    const bool fx = EXACT && S[r].x > kFfExactFar2, fy = EXACT && S[r].y > kFfExactFar2;
+                    const bool bx = fx || !(S[r].x >= fmaxf(I[r].thr, q5.z)), by = fy || !(S[r].y >= fmaxf(I[r].thr, q5.w));
                     if (bx || by) {
                         const float2 ci = A.ircf[I[r].i];
                         float2 W = f2_get(w[r]), WL = f2_get(wl[r]);
@@ -160,9 +168,9 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                             const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
                             const float ih = ti ? ci.x : cj.x, il = ti ? ci.y : cj.y;
                             float wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
-                            if ((h ? S[r].y : S[r].x) < close2) {
-                                FfClose o;
-                                ff_close(A.x, A.y, A.z, A.ff_header[2], I[r].i, jglob + k + 32 * h, ih, il, o);
+                            if (!((h ? S[r].y : S[r].x) >= close2) || (h ? fy : fx)) {
+                                FfOne o;
+                                ff_one(A, I[r].i, jglob + k + 32 * h, ih, il, o);
 #pragma unroll
                                 for (int c = 0; c < 3; c++) {
                                     const float2 u = f2_get(H[r][c]), v = f2_get(L[r][c]);
@@ -253,7 +261,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
 }
 
 template <bool PC>
-__device__ __forceinline__ void ff_load_row(const SymArgs &A, int a, int r, IBody &I) {
+__device__ __forceinline__ void ff_load_row(const SymArgs &A, int a, int r, float close2, IBody &I) {
     const float4 *B = A.body + (size_t)a * kFfTile + (r >> 6) * 32 + (r & 31);
     const bool up = r & 32;
     const float4 q0 = B[0], q1 = B[kFfRow], q2 = B[2 * kFfRow], q3 = B[3 * kFfRow], q4 = B[4 * kFfRow],
@@ -264,15 +272,19 @@ __device__ __forceinline__ void ff_load_row(const SymArgs &A, int a, int r, IBod
     I.l[0] = f2_dup(-(up ? q4.y : q4.x)); I.l[1] = f2_dup(-(up ? q4.w : q4.z)); I.l[2] = f2_dup(-(up ? q5.y : q5.x));
     I.mh = f2_dup(up ? q1.w : q1.z);
     I.ml = f2_dup(up ? q3.w : q3.z);
-    I.thr = up ? q5.w : q5.z;
-    const float4 q7 = B[7 * kFfRow];
-    I.tn = PC ? (up ? q7.w : q7.z) : I.thr;
+    const float4 q6 = B[6 * kFfRow];
+    I.thr = fmaxf(up ? q5.w : q5.z, close2);
+    I.tn = fmaxf(PC ? (up ? q6.w : q6.z) : I.thr, close2);
 }
 
-template <bool PC>
+// EX: the kernel for bodies whose coordinates are not held (kFfExact); the other returns
+// at once.  In one kernel the third instance costs the others 3 % (N = 131,071: 35.7 ms
+// against 34.7), the launch that finds nothing to do 2 us.
+template <bool PC, bool EX>
 __global__ void __launch_bounds__(kFfThreads, kFfMinBlocks)
 kick_sym_ff_kernel(SymArgs A)
 {
+    if (ff_exact_pairs(A.ff_header, A.n) != EX) return;
     extern __shared__ __align__(16) unsigned char ff_sh[];
     float4 *tile = reinterpret_cast<float4 *>(ff_sh);            // the j tile
     double *is = reinterpret_cast<double *>(tile + kFfTile);     // [3][kSymT]: the row tile's sums
@@ -284,7 +296,8 @@ kick_sym_ff_kernel(SymArgs A)
     const int n = A.n, PT = A.P * kSymT;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int flags = A.ff_header[0];
-    const float close2 = reinterpret_cast<const float *>(A.ff_header)[3];
+    // (read: with the bound as a constant in the code the compiler's schedule is 3 % slower)
+    const float close2 = EX ? kFfExactClose2 : reinterpret_cast<const float *>(A.ff_header)[4];
     for (;;) {
         __syncthreads();                       // the previous item's shared sums are written out
         if (threadIdx.x == 0) s_item = (int)atomicAdd(A.ctr, 1u);
@@ -317,8 +330,11 @@ kick_sym_ff_kernel(SymArgs A)
                         for (int h = 0; h < 64; h += 32 * kFfR) {
                             IBody I[kFfR];
 #pragma unroll
-                            for (int r = 0; r < kFfR; r++) ff_load_row<PC>(A, a, w * 64 + h + 32 * r + lane, I[r]);
-                            if (gen)
+                            for (int r = 0; r < kFfR; r++) ff_load_row<PC>(A, a, w * 64 + h + 32 * r + lane, close2, I[r]);
+                            if constexpr (EX)
+                                ff_rows<PC, kFfExact>(A, tile, js, is, PT, e0, jb, jg, I, flags, close2, dsub, w * 64 + h,
+                                                      0.0, pcb[PC ? w : 0], pend, lane);
+                            else if (gen)
                                 ff_rows<PC, kFfGeneral>(A, tile, js, is, PT, e0, jb, jg, I, flags, close2, dsub, w * 64 + h,
                                                         0.0, pcb[PC ? w : 0], pend, lane);
                             else if (mm > 0.0)
@@ -359,71 +375,74 @@ kick_sym_ff_kernel(SymArgs A)
     if (PC) sym_pc_flush(A, pcb[w], pend, lane);
 }
 
-template <int WARPS>
-__device__ __forceinline__ float4 ff_reduce_bounds(float4 v, float4 *sh) {     // of the block, to all
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        v.x = fmaxf(v.x, __shfl_xor_sync(0xffffffffu, v.x, o));
-        v.y = fminf(v.y, __shfl_xor_sync(0xffffffffu, v.y, o));
-        v.z = fmaxf(v.z, __shfl_xor_sync(0xffffffffu, v.z, o));
-        v.w = fminf(v.w, __shfl_xor_sync(0xffffffffu, v.w, o));
-    }
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < WARPS; k++) {
-        const float4 o = sh[k];
-        v = make_float4(fmaxf(v.x, o.x), fminf(v.y, o.y), fmaxf(v.z, o.z), fminf(v.w, o.w));
-    }
-    return v;
+// The exponent field of a finite double (0: zero or denormal, -1: infinite or NaN).
+__device__ __forceinline__ int f64_field(double v) {
+    const int f = (__double2hiint(v) >> 20) & 0x7ff;
+    return f == 0x7ff ? -1 : f;
 }
 
-// Per block: largest |coordinate|, smallest (over the bodies) of a body's largest
-// |coordinate|, largest and smallest mass, rounded up resp. down.
-__global__ void __launch_bounds__(256) ff_bounds_kernel(int n, const double *pos, const double *mass, float4 *bounds) {
-    __shared__ float4 sh[8];
-    float4 v = make_float4(0.0f, 3.0e38f, 0.0f, 3.0e38f);
+// Per block: largest exponent field on each axis, of the masses, smallest of the masses.
+__global__ void __launch_bounds__(256) ff_bounds_kernel(int n, const double *pos, const double *mass, int4 *bounds, int *header) {
+    __shared__ int sh[5][8];
+    int v[5] = {0, 0, 0, 0, 0};                    // the last: 0x7ff - field
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += 256 * gridDim.x) {
-        const double a = fmax(fabs(pos[i]), fmax(fabs(pos[(size_t)n + i]), fabs(pos[2 * (size_t)n + i])));
-        const double m = fabs(mass[i]);
-        v.x = fmaxf(v.x, __double2float_ru(a));
-        v.y = fminf(v.y, __double2float_rd(a));
-        v.z = fmaxf(v.z, __double2float_ru(m));
-        v.w = fminf(v.w, __double2float_rd(m));
+        const int m = f64_field(mass[i]);
+#pragma unroll
+        for (int c = 0; c < 3; c++) v[c] = max(v[c], f64_field(pos[(size_t)c * n + i]));
+        v[3] = max(v[3], m);
+        if (m >= 0) v[4] = max(v[4], 0x7ff - m);
     }
-    v = ff_reduce_bounds<8>(v, sh);
-    if (threadIdx.x == 0) bounds[blockIdx.x] = v;
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+        v[c] = __reduce_max_sync(0xffffffffu, v[c]);
+        if ((threadIdx.x & 31) == 0) sh[c][threadIdx.x >> 5] = v[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        int m = 0;
+        for (int k = 0; k < 8; k++) m = max(m, sh[threadIdx.x][k]);
+        reinterpret_cast<int *>(bounds + 2 * blockIdx.x)[threadIdx.x] = m;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) header[3] = 0;
 }
 
-// (Scaled) x = h + m + l + k: h a multiple of 2^-22 S, m of 2^-45 S (S = 2^e), l and k
-// floats of the rest.  mag1, mag2: 1.5 2^52 times the two grids' spacing, whose
+// (Scaled) x = h + m + l: h a multiple of 2^-23 S, m of 2^-47 S (S = 2^e), l the rest
+// rounded to a float.  mag1, mag2: 1.5 2^52 times the two grids' spacing, whose
 // addition rounds a double to a multiple of the spacing.
-__device__ __forceinline__ void ff_split(double x, double mag1, double mag2, float &h, float &m, float &l, float &k) {
+__device__ __forceinline__ void ff_split(double x, double mag1, double mag2, float &h, float &m, float &l) {
     const double dh = (x + mag1) - mag1, r = x - dh;
-    const double dm = (r + mag2) - mag2, s = r - dm;
+    const double dm = (r + mag2) - mag2;
     h = (float)dh;
     m = (float)dm;
-    l = (float)s;
-    k = (float)(s - (double)l);
+    l = (float)(r - dm);
 }
 
 // Four blocks per tile, one for each coordinate and one for masses, radii and the
 // header: the work is FP64 instructions, ~60 per body, and four SMs do a tile in
 // two thirds of the time of one (N = 2,048: 5.1 us against 6.9).
 __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
-    __shared__ float4 sh[kSymT / 32];
+    __shared__ int sh[5][kSymT / 32];
     __shared__ double tm;
-    float4 bd = make_float4(0.0f, 3.0e38f, 0.0f, 3.0e38f);
+    int v[5] = {0, 0, 0, 0, 0};
     for (int k = threadIdx.x; k < nbounds; k += kSymT) {
-        const float4 o = A.bounds[k];
-        bd = make_float4(fmaxf(bd.x, o.x), fminf(bd.y, o.y), fmaxf(bd.z, o.z), fminf(bd.w, o.w));
+        const int4 o = A.bounds[2 * k];
+        v[0] = max(v[0], o.x); v[1] = max(v[1], o.y); v[2] = max(v[2], o.z); v[3] = max(v[3], o.w);
+        v[4] = max(v[4], A.bounds[2 * k + 1].x);
     }
-    bd = ff_reduce_bounds<kSymT / 32>(bd, sh);
-    // S = 2^ex > every |coordinate|; lengths are scaled by 2^-es, which puts the
-    // innermost body near 1 (and S at 2^20 at most), masses by 2^-em, so that
-    // the floats' range does not depend on the caller's units
-    const int ex = max(ilogbf(fmaxf(bd.x, 1e-30f)) + 1, -90);
-    const int es = max(ilogbf(fminf(fmaxf(bd.y, 1e-30f), 1e30f)), ex - 20), em = ilogbf(fmaxf(bd.z, 1e-38f));
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+        v[c] = __reduce_max_sync(0xffffffffu, v[c]);
+        if ((threadIdx.x & 31) == 0) sh[c][threadIdx.x >> 5] = v[c];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 5; c++)
+#pragma unroll
+        for (int k = 0; k < kSymT / 32; k++) v[c] = max(v[c], sh[c][k]);
+    // S = 2^ex > every |coordinate|; lengths are scaled by 2^-es, which puts S at 2^kFfScale,
+    // masses by 2^-em, so that the floats' range does not depend on the caller's units
+    const int ex = min(max(max(v[0], max(v[1], v[2])) - 1022, -200), 400);
+    const int es = ex - kFfScale, em = min(max(v[3] - 1023, -200), 400);
     const double xscale = scalbn(1.0, -es);
     const int i = blockIdx.x * kSymT + threadIdx.x;
     // component of row q, first (0) or second (2) half: + 1 for the bodies l + 32
@@ -432,19 +451,28 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     constexpr int R = 4 * kFfRow;
     if (blockIdx.y < 3) {
         const int c = blockIdx.y, q = c == 2 ? R : 2 * c;       // z: first half of the next row
-        float h = (float)pad_pos(i & (kSymT - 1)), m = 0.0f, l = 0.0f, k = 0.0f;
-        if (i < A.n)
-            ff_split(A.pos[(size_t)c * A.n + i] * xscale, scalbn(1.5, 52 - 22 + ex - es), scalbn(1.5, 52 - 45 + ex - es),
-                     h, m, l, k);
-        B[q] = h; B[2 * R + q] = m; B[4 * R + q] = l; B[6 * R + q] = k;
+        // the axis' own S = 2^ec > every |x| on it (2^-60 of the largest, if smaller), in units
+        const int ec = min(max(v[c] - 1022, ex - 60), ex);
+        float h = (float)pad_pos(i & (kSymT - 1)), m = 0.0f, l = 0.0f;
+        bool out = false;
+        if (i < A.n) {
+            const double x = A.pos[(size_t)c * A.n + i];
+            ff_split(x * xscale, scalbn(1.5, 52 - 23 + ec - es), scalbn(1.5, 52 - 47 + ec - es), h, m, l);
+            // not held: 2^ec or more, or below 2^(ec - window); a zero is
+            const int f = f64_field(x) - 1022;                  // |x| < 2^f
+            out = x != 0.0 && (f > ec || f < ec - A.window || !(fabs(x) < __longlong_as_double(0x7ff0000000000000ll)));
+            if (out) h = __uint_as_float(0x7fc00000u);
+        }
+        B[q] = h; B[2 * R + q] = m; B[4 * R + q] = l;
+        const int nout = __syncthreads_count(out);
+        if (nout && threadIdx.x == 0) atomicAdd(&A.header[3], nout);
         return;
     }
-    const float close2 = scalbnf(1.0f, 2 * (ex - es - 17));      // (2^-17 S)^2
     if (i == 0) {
-        A.header[0] = (scalbnf(1.0f, ex - 18) > bd.y ? kFfWide : 0) | (scalbnf(bd.z, -40) >= bd.w ? kFfTwoMass : 0);
+        A.header[0] = 0x7ff - v[4] <= v[3] - 40 ? kFfTwoMass : 0;
         A.header[1] = em;
         A.header[2] = es;
-        reinterpret_cast<float *>(A.header)[3] = close2;
+        reinterpret_cast<float *>(A.header)[4] = kFfClose2;
         if (A.ctr) *A.ctr = 0u;
         if (A.cand_count) *A.cand_count = 0ull;
     }
@@ -454,23 +482,24 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     __syncthreads();
     const int differ = __syncthreads_or(ms != tm || !(ms > 0.0));
     if (threadIdx.x == 0) A.tmass[blockIdx.x] = differ ? 0.0 : ms;
-    float mh = 0.0f, ml = 0.0f, thr = 0.0f, thp = 0.0f;
+    float mh = 0.0f, ml = 0.0f, mt = 0.0f, thr = 0.0f, thp = 0.0f;
     float2 ircf = make_float2(0.0f, 0.0f);
     if (i < A.n) {
         const double rc = A.rc[i], rcs = rc * xscale, pc2 = A.pc2 ? A.pc2[i] * xscale * xscale : 0.0;
         mh = __double2float_rn(ms);
         ml = __double2float_rn(ms - (double)mh);
-        // upper bounds of rc^2 and pc2, and of the close pairs' r^2: rounded up,
-        // then 2^-16 more, so that any float r^2 within 2^-20 of an r^2 below
-        // them is below them
-        thr = fmaxf(__double2float_ru(rcs * rcs), close2) * 1.0000153f;
+        mt = __double2float_rn((ms - (double)mh) - (double)ml);
+        // upper bounds of rc^2 and pc2: rounded up, then 2^-16 more, so that any float
+        // r^2 within 2^-20 of an r^2 below them is below them
+        thr = __double2float_ru(rcs * rcs) * 1.0000153f;
         thp = fmaxf(__double2float_ru(pc2) * 1.0000153f, thr);
         ircf = ff_of_irc(inv_rc(rc) * scalbn(1.0, es));
     }
     B[R + 2] = mh;
     B[3 * R + 2] = ml;
     B[5 * R + 2] = thr;
-    B[7 * R + 2] = thp;
+    B[6 * R] = mt;
+    B[6 * R + 2] = thp;
     A.ircf[i] = ircf;
 }
 
@@ -482,7 +511,7 @@ size_t sym_ff_smem(int P) {
 
 int sym_ff_blocks_per_sm(int P) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kick_sym_ff_kernel<true>, kFfThreads, sym_ff_smem(P)) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kick_sym_ff_kernel<true, false>, kFfThreads, sym_ff_smem(P)) !=
         cudaSuccess)
         return 0;
     return nb;
@@ -491,15 +520,15 @@ int sym_ff_blocks_per_sm(int P) {
 // Layout of the packed-body allocation: the arrays in this order, each a whole
 // number of float4 per tile (but the bounds and the header, at the end).
 static size_t ff_tile_bytes(size_t nT) {
-    return nT * (sizeof(float4) * kFfTile + sizeof(float2) * kSymT + sizeof(float4)) + sizeof(float4) * (kFfBoundBlocks + 1);
+    return nT * (sizeof(float4) * kFfTile + sizeof(float2) * kSymT + sizeof(float4)) + sizeof(int4) * (2 * kFfBoundBlocks + 2);
 }
 
 void ff_place(FfPack &k, void *mem, size_t nT) {
     k.body = (float4 *)mem;
     k.ircf = (float2 *)(k.body + nT * kFfTile);
     k.tmass = (double *)(k.ircf + nT * kSymT);
-    k.bounds = (float4 *)(k.tmass + 2 * nT);
-    k.header = (int *)(k.bounds + kFfBoundBlocks);
+    k.bounds = (int4 *)(k.tmass + 2 * nT);
+    k.header = (int *)(k.bounds + 2 * kFfBoundBlocks);
 }
 
 size_t ff_bytes(int n) { return ff_tile_bytes((size_t)((n + kSymT - 1) / kSymT)); }
@@ -521,6 +550,7 @@ FfPack ff_pack_args(const genga_system *s) {
     k.n = (int)s->n;
     k.nT = (int)((s->n + kSymT - 1) / kSymT);
     ff_place(k, s->ff, s->ff_tiles);
+    k.window = s->p.precision == GENGA_MIXED ? kFfWindowMixed : kFfWindow64;
     k.ctr = nullptr;
     k.cand_count = nullptr;
     return k;
@@ -528,7 +558,7 @@ FfPack ff_pack_args(const genga_system *s) {
 
 cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launches) {
     const int nb = std::min(kFfBoundBlocks, (k.n + 255) / 256);
-    ff_bounds_kernel<<<nb, 256, 0, stream>>>(k.n, k.pos, k.m, k.bounds);
+    ff_bounds_kernel<<<nb, 256, 0, stream>>>(k.n, k.pos, k.m, k.bounds, k.header);
     GENGA_CUDA_TRY(cudaGetLastError());
     ff_pack_kernel<<<dim3(k.nT, 4), kSymT, 0, stream>>>(k, nb);
     *launches += 2;
@@ -537,8 +567,10 @@ cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launch
 
 cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStream_t stream) {
     const size_t smem = sym_ff_smem(S.P);
-    if (precheck) kick_sym_ff_kernel<true><<<blocks, kFfThreads, smem, stream>>>(S);
-    else kick_sym_ff_kernel<false><<<blocks, kFfThreads, smem, stream>>>(S);
+    if (precheck) kick_sym_ff_kernel<true, false><<<blocks, kFfThreads, smem, stream>>>(S);
+    else kick_sym_ff_kernel<false, false><<<blocks, kFfThreads, smem, stream>>>(S);
+    if (precheck) kick_sym_ff_kernel<true, true><<<blocks, kFfThreads, smem, stream>>>(S);
+    else kick_sym_ff_kernel<false, true><<<blocks, kFfThreads, smem, stream>>>(S);
     return cudaGetLastError();
 }
 

@@ -86,14 +86,26 @@ __device__ __forceinline__ void sym_pc_push(uint2 *buf, int &cnt, int lane, bool
     cnt += __popc(ball);
 }
 
-// The bodies as float expansions (kick_ff.cu).  A tile of 128 bodies: 8 rows of 64 float4.  Entry g * 32 + l of a row holds
+// The bodies as float expansions (kick_ff.cu).  A tile of 128 bodies: 7 rows of 64 float4.  Entry g * 32 + l of a row holds
 // the bodies l (x, z) and l + 32 (y, w) of group g:
 //   0: h_x h_y   1: h_z m_hi   2: m_x m_y   3: m_z m_lo   4: l_x l_y   5: l_z thr_rc
-//   6: k_x k_y   7: k_z thr_pc
-// (m_hi, m_lo the scaled mass; k the fourth parts of the coordinates).
-constexpr int kFfRow = 64, kFfTile = 8 * kFfRow;
-constexpr int kFfWide = 1, kFfTwoMass = 2;     // flags of the packed bodies, see kick_ff.cu
-constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2;      // instances of the pair loops
+//   6: m_lo2 thr_pc
+// (m_hi + m_lo + m_lo2 the scaled mass).  Lengths are in units of 2^-6 S, S = 2^6 > every
+// coordinate in them.
+constexpr int kFfRow = 64, kFfTile = 7 * kFfRow;
+constexpr int kFfScale = 6;
+constexpr int kFfTwoMass = 1;                  // flag of the packed bodies, see kick_ff.cu
+constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2, kFfExact = 3;      // instances of the pair loops
+// A body whose coordinates the three floats do not hold has NaN in their place.  Its pairs
+// take FP64 one by one, and with more than one such coordinate per 128 bodies every pair
+// takes the instance of FP64 displacements (kFfExact): 1.6 times the time of the others in
+// the FP64 kick (N = 16,384: 3.3 ms against 2.0; 5.4 for the FP64 symmetric form), 3.1
+// times in the mixed one (65,540: 28.8 ms against 9.2; 34.9 with displacement and sums in
+// FP64), while a pair taken by itself costs ~10 to 50 of them.
+__device__ __forceinline__ bool ff_exact_pairs(const int *header, int n) { return 128ll * header[3] > n; }
+// Bounds of r^2: below, the parts give no displacement in proper order (2^-20 S) or r^-3
+// nears the end of the floats' range (kFfExact); above (kFfExact), the same.
+constexpr float kFfClose2 = 0x1p-28f, kFfExactClose2 = 0x1p-64f, kFfExactFar2 = 0x1p60f;
 __device__ __forceinline__ f2 f2_lo(const float4 &v) { return f2_make(v.x, v.y); }
 __device__ __forceinline__ f2 f2_hi(const float4 &v) { return f2_make(v.z, v.w); }
 
@@ -105,14 +117,20 @@ int sym_ff_blocks_per_sm(int P);
 // Packs the bodies (float expansions, thresholds) and zeroes the dispatch
 // counter and, with pre-check, the candidate count.
 constexpr int kFfBoundBlocks = 152;
+// Coordinates below 2^-window of their axis' S are not held: their last bits lie below
+// the parts.  18: every bit is held (FP64 kick), 25: to 2^-47 (mixed), none: to 2^-72 S,
+// enough for a distance (energy).
+constexpr int kFfWindow64 = 18, kFfWindowMixed = 25, kFfWindowNone = 4096;
 struct FfPack {
     const double *pos, *m, *rc, *pc2;
     int n, nT;
-    float4 *bounds;                   // scratch, kFfBoundBlocks entries
-    float4 *body;                     // 4 float4 per body, whole tiles
+    int window;
+    int4 *bounds;                     // scratch, 2 kFfBoundBlocks entries
+    float4 *body;                     // whole tiles
     float2 *ircf;
     double *tmass;                    // per tile
-    int *header;                      // flags, exponents masses and lengths are scaled by, close r^2 (float)
+    int *header;                      // flags, exponents masses and lengths are scaled by, coordinates not held,
+                                      // kFfClose2 (float); 8 ints
     unsigned *ctr;                    // NULL: left alone
     unsigned long long *cand_count;   // NULL: left alone
 };
@@ -123,7 +141,7 @@ FfPack ff_pack_args(const genga_system *s);
 size_t ff_bytes(int n);
 void ff_place(FfPack &k, void *mem, size_t tiles);
 cudaError_t launch_ff_pack(const FfPack &k, cudaStream_t stream, int64_t *launches);
-cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStream_t stream);
+cudaError_t launch_sym_ff(const SymArgs &S, bool precheck, int blocks, cudaStream_t stream);     // two launches
 // kick_tile.cu: the tiled kick.  Steps (two bodies j) per chunk, chunks, predicted SM
 // cycles.  Chunk 0: no plan (max_part, in doubles, holds no partial sums).
 struct TilePlan {

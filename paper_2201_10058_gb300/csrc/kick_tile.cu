@@ -9,7 +9,7 @@
 //           16 steps): ~105 FP32 operations per ordered pair.
 //   FP64    results of full double precision with 3 FP64 FMAs per ordered pair.
 //           FP64 issues once in 64 cycles per sub-partition, so everything else is
-//           on the FP32 pipe: displacement H + L + T exact, the residual
+//           on the FP32 pipe: displacement H + L + T, exactly (kick_ff.cu), the residual
 //           e = 1 - |d y|^2 to 2^-56 from digits, m_j r^-3 = m_j y^3 (1 + 1.5 e +
 //           1.875 e^2) as a double -- m_j y^3 as a float plus a whole number of
 //           units of the last place of that double.  The FMAs take it times the
@@ -19,7 +19,10 @@
 //           against 17 FP64 instructions (1,088) of CUDA's double rsqrt form and
 //           10.5 (672) of the symmetric one.
 //           Pairs that need more (changeover band, close pairs, r^-3 next to a power
-//           of two) go to a buffer and are taken 32 at a time in FP64.
+//           of two, bodies whose coordinates three floats do not hold) go to a buffer and
+//           are taken 32 at a time in FP64.  Where many coordinates are not held (kFfExact)
+//           the displacement is an FP64 subtraction, which the FMAs then take whole: 6
+//           FP64 instructions.
 // Measured (whole kick, us; before: kick_kernel, or FP64 symmetric from 16,384 on):
 //   FP64   N = 1,000: 40 (189), 2,048: 68 (193), 20,011: 2,916 (7,915); error against
 //          64 bits 1.6e-16 of the norm at 20,011 (2.1e-16)
@@ -48,21 +51,21 @@ struct TlRow {                                 // a thread's row, in both halves
 };
 
 template <bool PC>
-__device__ __forceinline__ void tl_load_row(const SymArgs &A, int a, int r, TlRow &I) {
+__device__ __forceinline__ void tl_load_row(const SymArgs &A, int a, int r, float close2, TlRow &I) {
     const float4 *B = A.body + (size_t)a * kFfTile + (r >> 6) * 32 + (r & 31);
     const bool up = r & 32;
     const float4 q0 = B[0], q1 = B[kFfRow], q2 = B[2 * kFfRow], q3 = B[3 * kFfRow], q4 = B[4 * kFfRow],
-                 q5 = B[5 * kFfRow], q7 = B[7 * kFfRow];
+                 q5 = B[5 * kFfRow], q6 = B[6 * kFfRow];
     I.i = a * kSymT + r;
     I.h[0] = f2_dup(-(up ? q0.y : q0.x)); I.h[1] = f2_dup(-(up ? q0.w : q0.z)); I.h[2] = f2_dup(-(up ? q1.y : q1.x));
     I.m[0] = f2_dup(-(up ? q2.y : q2.x)); I.m[1] = f2_dup(-(up ? q2.w : q2.z)); I.m[2] = f2_dup(-(up ? q3.y : q3.x));
     I.l[0] = f2_dup(-(up ? q4.y : q4.x)); I.l[1] = f2_dup(-(up ? q4.w : q4.z)); I.l[2] = f2_dup(-(up ? q5.y : q5.x));
-    I.thr = up ? q5.w : q5.z;
-    I.tn = PC ? (up ? q7.w : q7.z) : I.thr;
+    I.thr = fmaxf(up ? q5.w : q5.z, close2);
+    I.tn = fmaxf(PC ? (up ? q6.w : q6.z) : I.thr, close2);
 }
 
 // The steps a block takes (A.P of the 32 per group: whole groups, or 16 or 8 steps of
-// one), and the staging of a group: 8 rows of 32 float4.
+// one), and the staging of a group: 7 rows of 32 float4.
 struct TlRange { int g0, g1, k0, k1; };
 __device__ __forceinline__ TlRange tl_range(const SymArgs &A) {
     TlRange r;
@@ -76,63 +79,67 @@ __device__ __forceinline__ TlRange tl_range(const SymArgs &A) {
 }
 __device__ __forceinline__ void tl_stage(const SymArgs &A, int g, float4 *grp) {
     const float4 *src = A.body + (size_t)(g >> 1) * kFfTile + (g & 1) * 32;
-    for (int k = threadIdx.x; k < 8 * 32; k += kTlRows) grp[k] = src[(k >> 5) * kFfRow + (k & 31)];
+    for (int k = threadIdx.x; k < 7 * 32; k += kTlRows) grp[k] = src[(k >> 5) * kFfRow + (k & 31)];
 }
 
 // Mixed: the steps [k0, k1) of row I against the 64 bodies of group g.
 template <bool PC, int MODE>
 __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, int g, int k0, int k1, const TlRow &I, float close2,
                                          double mm, double (&acc)[3], uint2 *pcbuf, int &pend, int lane) {
-    constexpr bool GEN = MODE == kFfGeneral;
+    constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
     const f2 one = f2_dup(1.0f);
-    f2 nk[3];
-    if (GEN) {
-        const float4 *B = A.body + (size_t)(I.i >> 7) * kFfTile + ((I.i >> 6) & 1) * 32 + (I.i & 31);
-        const float4 p = B[6 * kFfRow], q = B[7 * kFfRow];
-        const bool up = I.i & 32;
-        nk[0] = f2_dup(-(up ? p.y : p.x)); nk[1] = f2_dup(-(up ? p.w : p.z)); nk[2] = f2_dup(-(up ? q.y : q.x));
-    }
+    const double xs = EXACT ? scalbn(1.0, -A.ff_header[2]) : 1.0;
 #pragma unroll 1
     for (int tb = k0; tb < k1; tb += kTlFlush) {
         f2 sh[3], sl[3];
 #pragma unroll
         for (int c = 0; c < 3; c++) sh[c] = sl[c] = 0ull;
-#pragma unroll 2
+#pragma unroll (EXACT ? 1 : 2)
         for (int k = tb; k < min(tb + kTlFlush, k1); k++) {
             const float4 q0 = grp[k], q1 = grp[32 + k], q2 = grp[64 + k], q3 = grp[96 + k], q4 = grp[128 + k],
                          q5 = grp[160 + k];
-            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&grp[224 + k].z) : make_float2(q5.z, q5.w);
+            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&grp[192 + k].z) : make_float2(q5.z, q5.w);
             const int j = g * 64 + k;
             f2 H[3], L[3], s2, tail, w, wl;
             bool wx = true, wy = true;
             if (GEN) {
-                const float4 q6 = grp[192 + k], q7 = grp[224 + k];
-                ff_disp4(f2_lo(q0), f2_lo(q2), f2_lo(q4), f2_lo(q6), I.h[0], I.m[0], I.l[0], nk[0], H[0], L[0]);
-                ff_disp4(f2_hi(q0), f2_hi(q2), f2_hi(q4), f2_hi(q6), I.h[1], I.m[1], I.l[1], nk[1], H[1], L[1]);
-                ff_disp4(f2_lo(q1), f2_lo(q3), f2_lo(q5), f2_lo(q7), I.h[2], I.m[2], I.l[2], nk[2], H[2], L[2]);
                 const bool ti = I.i >= A.nm;
                 wx = j != I.i && !(ti && j >= A.nm);
                 wy = j + 32 != I.i && !(ti && j + 32 >= A.nm);
+            }
+            if (EXACT) {
+                const int i = min(I.i, A.n - 1), jx = min(j, A.n - 1), jy = min(j + 32, A.n - 1);
+                f64_split2((A.x[jx] - A.x[i]) * xs, (A.x[jy] - A.x[i]) * xs, H[0], L[0]);
+                f64_split2((A.y[jx] - A.y[i]) * xs, (A.y[jy] - A.y[i]) * xs, H[1], L[1]);
+                f64_split2((A.z[jx] - A.z[i]) * xs, (A.z[jy] - A.z[i]) * xs, H[2], L[2]);
+                wx = wx && I.i < A.n && j < A.n;
+                wy = wy && I.i < A.n && j + 32 < A.n;
             } else {
                 ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I.h[0], I.m[0], I.l[0], H[0], L[0]);
                 ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I.h[1], I.m[1], I.l[1], H[1], L[1]);
                 ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I.h[2], I.m[2], I.l[2], H[2], L[2]);
             }
             ff_r2(H, L, s2, tail);
-            if (GEN) {
+            if (GEN) {                             // (NaN times zero would be NaN)
                 s2 = f2_select(wx, wy, s2, one);
                 tail = f2_select(wx, wy, tail, 0ull);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    H[c] = f2_select(wx, wy, H[c], 0ull);
+                    L[c] = f2_select(wx, wy, L[c], 0ull);
+                }
             }
             ff_inv_r3(s2, tail, w, wl);
             const float2 S = f2_get(s2);
-            const bool nx = S.x < fmaxf(I.tn, tj.x), ny = S.y < fmaxf(I.tn, tj.y);
+            const bool fx = EXACT && S.x > kFfExactFar2, fy = EXACT && S.y > kFfExactFar2;
+            const bool nx = fx || !(S.x >= fmaxf(I.tn, tj.x)), ny = fy || !(S.y >= fmaxf(I.tn, tj.y));
             if (PC ? __any_sync(0xffffffffu, nx || ny) : (nx || ny)) {
                 if (PC) {
                     sym_pc_push(pcbuf, pend, lane, nx && wx && j > I.i, I.i, j);
                     sym_pc_push(pcbuf, pend, lane, ny && wy && j + 32 > I.i, I.i, j + 32);
                     if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
                 }
-                const bool bx = S.x < fmaxf(I.thr, q5.z), by = S.y < fmaxf(I.thr, q5.w);
+                const bool bx = fx || !(S.x >= fmaxf(I.thr, q5.z)), by = fy || !(S.y >= fmaxf(I.thr, q5.w));
                 if (bx || by) {
                     const float2 ci = A.ircf[I.i], Tl = f2_get(tail);
                     float2 W = f2_get(w), WL = f2_get(wl);
@@ -143,9 +150,9 @@ __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, in
                         const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
                         const float ih = ti ? ci.x : cj.x, il = ti ? ci.y : cj.y;
                         float wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
-                        if ((h ? S.y : S.x) < close2) {
-                            FfClose o;
-                            ff_close(A.x, A.y, A.z, A.ff_header[2], I.i, j + 32 * h, ih, il, o);
+                        if (!((h ? S.y : S.x) >= close2) || (h ? fy : fx)) {
+                            FfOne o;
+                            ff_one(A, I.i, j + 32 * h, ih, il, o);
 #pragma unroll
                             for (int c = 0; c < 3; c++) {
                                 const float2 u = f2_get(H[c]), v = f2_get(L[c]);
@@ -195,23 +202,24 @@ __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, in
 template <bool PC>
 __global__ void __launch_bounds__(kTlRows, 4)
 kick_tile_ff_kernel(SymArgs A) {
-    __shared__ float4 grp[8 * 32];
+    __shared__ float4 grp[7 * 32];
     __shared__ uint2 pcb[PC ? 4 : 1][PC ? kSymPcBuf : 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, a = blockIdx.x;
     const TlRange R = tl_range(A);
-    const bool wide = (A.ff_header[0] & kFfWide) != 0;
-    const float close2 = reinterpret_cast<const float *>(A.ff_header)[3];
+    const bool exact = ff_exact_pairs(A.ff_header, A.n);
+    const float close2 = exact ? kFfExactClose2 : kFfClose2;
     int pend = 0;
     TlRow I;
-    tl_load_row<PC>(A, a, threadIdx.x, I);
+    tl_load_row<PC>(A, a, threadIdx.x, close2, I);
     double acc[3] = {0.0, 0.0, 0.0};
     for (int g = R.g0; g < R.g1; g++) {
         __syncthreads();
         tl_stage(A, g, grp);
         __syncthreads();
         const double mm = A.tmass[g >> 1];
-        const bool gen = wide || (g >> 1) == a || ((a + 1) * kSymT > A.nm && (g + 1) * 64 > A.nm);
-        if (gen) tl_group<PC, kFfGeneral>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
+        const bool gen = (g >> 1) == a || ((a + 1) * kSymT > A.nm && (g + 1) * 64 > A.nm);
+        if (exact) tl_group<PC, kFfExact>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
+        else if (gen) tl_group<PC, kFfGeneral>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
         else if (mm > 0.0) tl_group<PC, kFfUniform>(A, grp, g, R.k0, R.k1, I, close2, mm, acc, pcb[PC ? w : 0], pend, lane);
         else tl_group<PC, kFfPlain>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
     }
@@ -242,7 +250,8 @@ __device__ __forceinline__ void tl_near_flush(const SymArgs &A, TlNear &B, int &
             const double dx = A.x[j] - A.x[i], dy = A.y[j] - A.y[i], dz = A.z[j] - A.z[i];
             const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
             const double y = rsqrt(r2);
-            const double c = A.m[j] * (changeover_fast(r2 * y, inv_rc(fmax(A.rc[i], A.rc[j]))) * (y * y * y));
+            const double K = r2 < 1e300 ? changeover_fast(r2 * y, inv_rc(fmax(A.rc[i], A.rc[j]))) : 1.0;
+            const double c = A.m[j] * (K * (y * y * y));
             tx = c * dx; ty = c * dy; tz = c * dz;
         }
         B.t[0][lane] = tx; B.t[1][lane] = ty; B.t[2][lane] = tz;
@@ -261,21 +270,28 @@ __device__ __forceinline__ void tl_near_flush(const SymArgs &A, TlNear &B, int &
 
 // FP64: the steps [k0, k1) of row I against the 64 bodies of group g.  acc: sums of (m_j) r^-3 d
 // in the packed units, near: those of the buffered pairs in the caller's units.
+// kFfExact: the displacement from the positions, xyz those of the group in the packed units.
 template <bool PC, int MODE>
-__device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, const float *mtail, int g, int k0, int k1, const TlRow &I,
+__device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, const double (*xyz)[64], int g, int k0, int k1, const TlRow &I,
                                            double (&acc)[3], double *near, TlNear &nb, int &npend,
                                            uint2 *pcbuf, int &pend, int lane) {
-    constexpr bool GEN = MODE == kFfGeneral;
+    constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
+    double xi[3];
+    if (EXACT) {
+        const double xs = scalbn(1.0, -A.ff_header[2]);
+        const int i = min(I.i, A.n - 1);
+        xi[0] = A.x[i] * xs; xi[1] = A.y[i] * xs; xi[2] = A.z[i] * xs;
+    }
     const f2 c15 = f2_dup(1.5f), c1875 = f2_dup(1.875f);
     // r^-3 (L + T): 2^-24 of the terms, so that two floats per sum do for a group
     f2 sh[3], sl[3];
 #pragma unroll
     for (int c = 0; c < 3; c++) sh[c] = sl[c] = 0ull;
-#pragma unroll (kTlUnroll64)
+#pragma unroll (EXACT ? 1 : kTlUnroll64)
     for (int k = k0; k < k1; k++) {
         const float4 q0 = grp[k], q1 = grp[32 + k], q2 = grp[64 + k], q3 = grp[96 + k], q4 = grp[128 + k],
                      q5 = grp[160 + k];
-        const float2 tj = PC ? *reinterpret_cast<const float2 *>(&grp[224 + k].z) : make_float2(q5.z, q5.w);
+        const float2 tj = PC ? *reinterpret_cast<const float2 *>(&grp[192 + k].z) : make_float2(q5.z, q5.w);
         const int j = g * 64 + k;
         bool wx = true, wy = true;
         if (GEN) {
@@ -284,9 +300,22 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
             wy = j + 32 != I.i && I.i < A.n && j + 32 < A.n && !(ti && j + 32 >= A.nm);
         }
         f2 H[3], L[3], T[3];
-        ff_disp3(f2_lo(q0), f2_lo(q2), f2_lo(q4), I.h[0], I.m[0], I.l[0], H[0], L[0], T[0]);
-        ff_disp3(f2_hi(q0), f2_hi(q2), f2_hi(q4), I.h[1], I.m[1], I.l[1], H[1], L[1], T[1]);
-        ff_disp3(f2_lo(q1), f2_lo(q3), f2_lo(q5), I.h[2], I.m[2], I.l[2], H[2], L[2], T[2]);
+        double ex[3], ey[3];                   // kFfExact: the two displacements
+        if (EXACT) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                float hx, lx, tx, hy, ly, ty;
+                ex[c] = xyz[c][k] - xi[c];
+                ey[c] = xyz[c][k + 32] - xi[c];
+                f64_split3(ex[c], hx, lx, tx);
+                f64_split3(ey[c], hy, ly, ty);
+                H[c] = f2_make(hx, hy); L[c] = f2_make(lx, ly); T[c] = f2_make(tx, ty);
+            }
+        } else {
+            ff_disp3(f2_lo(q0), f2_lo(q2), f2_lo(q4), I.h[0], I.m[0], I.l[0], H[0], L[0], T[0]);
+            ff_disp3(f2_hi(q0), f2_hi(q2), f2_hi(q4), I.h[1], I.m[1], I.l[1], H[1], L[1], T[1]);
+            ff_disp3(f2_lo(q1), f2_lo(q3), f2_lo(q5), I.h[2], I.m[2], I.l[2], H[2], L[2], T[2]);
+        }
         const f2 s = f2_fma(H[2], H[2], f2_fma(H[1], H[1], f2_mul(H[0], H[0])));
         const f2 y = f2_rsqrt(s);
         f2 eh, el;
@@ -309,7 +338,7 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
             ff_units_add(f, sc, tu, lo);
             ff_units_add(small, sc, tu, lo);
         } else {
-            const f2 mh = f2_hi(q1), ml = f2_hi(q3), mt = f2_make(mtail[k], mtail[32 + k]);
+            const f2 mh = f2_hi(q1), ml = f2_hi(q3), mt = *reinterpret_cast<const f2 *>(&grp[192 + k]);
             base = f2_mul(wh, mh);
             const float2 B = f2_get(base);
             sc = f2_make(ff_ulp_scale(B.x), ff_ulp_scale(B.y));
@@ -324,10 +353,11 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
         }
         const float2 B = f2_get(base), TU = f2_get(tu), LO = f2_get(ff_units_end(lo));
         // times 2^896, to go with the components' 2^-896
-        double dx = ff_add_units<896>(B.x, TU.x, LO.x), dy = ff_add_units<896>(B.y, TU.y, LO.y);
+        constexpr int UP = EXACT ? 0 : 896;
+        double dx = ff_add_units<UP>(B.x, TU.x, LO.x), dy = ff_add_units<UP>(B.y, TU.y, LO.y);
         // near pairs; PC: the bounds tn include the changeover's
         const float2 S = f2_get(s);
-        const bool px = S.x < fmaxf(I.tn, tj.x), py = S.y < fmaxf(I.tn, tj.y);
+        const bool px = !(S.x >= fmaxf(I.tn, tj.x)), py = !(S.y >= fmaxf(I.tn, tj.y));
         // next to a power of two the bits change scale: 1.5 e, |e| < 5.6e-7, and the products'
         // low parts are at most 17 last places (2^-24 of the base, below the power)
         const bool ux = ff_near_binade<24>(B.x) || !(S.x < 1e36f && B.x > 6e-23f);
@@ -339,7 +369,7 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
                 sym_pc_push(pcbuf, pend, lane, py && wy && j + 32 > I.i, I.i, j + 32);
                 if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
             }
-            const bool bx = ux || S.x < fmaxf(I.thr, q5.z), by = uy || S.y < fmaxf(I.thr, q5.w);
+            const bool bx = ux || !(S.x >= fmaxf(I.thr, q5.z)), by = uy || !(S.y >= fmaxf(I.thr, q5.w));
             // (a massless j's ux, uy hold: nothing to add, unless NaN or infinite)
             sym_pc_push(nb.q, npend, lane, bx && wx && (B.x != 0.0f || !(S.x < 1e36f)), lane, j);
             sym_pc_push(nb.q, npend, lane, by && wy && (B.y != 0.0f || !(S.y < 1e36f)), lane, j + 32);
@@ -355,6 +385,17 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
             for (int c = 0; c < 3; c++) L[c] = f2_select(ox, oy, 0ull, L[c]);
 #pragma unroll
             for (int c = 0; c < 3; c++) T[c] = f2_select(ox, oy, 0ull, T[c]);
+            if (EXACT)
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    if (ox) ex[c] = 0.0;
+                    if (oy) ey[c] = 0.0;
+                }
+        }
+        if (EXACT) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) acc[c] = fma(dy, ey[c], fma(dx, ex[c], acc[c]));
+            continue;
         }
         if (MODE != kFfUniform) {
             const f2 h0 = ch, l0 = cl;
@@ -370,66 +411,32 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
             f2_acc(sh[c], sl[c], th, te);
         }
     }
+    if constexpr (!EXACT) {
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
-        const float2 a = f2_get(sh[c]), b = f2_get(sl[c]);
-        float s, x;
-        ff_two_sum(a.x, a.y, s, x);
-        acc[c] += f64_of_f32_any(s) + f64_of_f32_any(x + (b.x + b.y));
-    }
-}
-
-// FP64, coordinates that three floats do not hold: every pair in FP64, CUDA's double
-// rsqrt, lengths and masses scaled as the packed ones.
-template <bool PC>
-__device__ __noinline__ void tl_group_wide(const SymArgs &A, const float4 *grp, int g, int k0, int k1, float thr, float tn,
-                                           int i, double (&acc)[3], uint2 *pcbuf, int &pend, int lane) {
-    const double xs = scalbn(1.0, -A.ff_header[2]), us = scalbn(1.0, A.ff_header[2]),
-                 ms = scalbn(1.0, -A.ff_header[1]);
-    const bool vi = i < A.n, ti = i >= A.nm;
-    const double xi = vi ? A.x[i] * xs : 0.0, yi = vi ? A.y[i] * xs : 0.0, zi = vi ? A.z[i] * xs : 0.0;
-    const double rci = vi ? A.rc[i] : 0.0;
-    for (int k = 0; k < 64; k++) {
-        const int j = g * 64 + k;
-        if ((k & 31) < k0 || (k & 31) >= k1 || j >= A.n) continue;
-        const float4 *e = grp + (k & 31);
-        const float tj = k & 32 ? e[160].w : e[160].z, tp = PC ? (k & 32 ? e[224].w : e[224].z) : 0.0f;
-        const double dx = A.x[j] * xs - xi, dy = A.y[j] * xs - yi, dz = A.z[j] * xs - zi;
-        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const float r2f = (float)r2;
-        const bool want = vi && j != i && !(ti && j >= A.nm);
-        if (PC) {
-            const bool maybe = want && j > i && r2f < fmaxf(tn, tp);
-            if (__any_sync(0xffffffffu, maybe)) {
-                sym_pc_push(pcbuf, pend, lane, maybe, i, j);
-                if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
-            }
+        for (int c = 0; c < 3; c++) {
+            const float2 a = f2_get(sh[c]), b = f2_get(sl[c]);
+            float s, x;
+            ff_two_sum(a.x, a.y, s, x);
+            acc[c] += f64_of_f32_any(s) + f64_of_f32_any(x + (b.x + b.y));
         }
-        const double y = rsqrt(r2);
-        double c = (A.m[j] * ms * y) * (y * y);
-        if (r2f < fmaxf(thr, tj)) c *= changeover_fast(r2 * y, us * inv_rc(fmax(rci, A.rc[j])));
-        if (!want) continue;
-        acc[0] = fma(c, dx, acc[0]);
-        acc[1] = fma(c, dy, acc[1]);
-        acc[2] = fma(c, dz, acc[2]);
     }
 }
 
 template <bool PC>
 __global__ void __launch_bounds__(kTlRows, kTlBlocks64)
 kick_tile_f64_kernel(SymArgs A) {
-    __shared__ float4 grp[8 * 32];
-    __shared__ float mtail[64];
+    __shared__ float4 grp[7 * 32];
+    __shared__ double xyz[3][64];              // kFfExact: the group's positions
     __shared__ TlNear nb[4];
     __shared__ uint2 pcb[PC ? 4 : 1][PC ? kSymPcBuf : 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, a = blockIdx.x;
     const TlRange R = tl_range(A);
-    const bool wide = (A.ff_header[0] & kFfWide) != 0;
-    const double mscale = scalbn(1.0, -A.ff_header[1]);
+    const bool exact = ff_exact_pairs(A.ff_header, A.n);
+    const double back = scalbn(1.0, 2 * A.ff_header[2] - A.ff_header[1]);     // the near pairs' sums in the packed units
     const bool pads = A.n % kSymT != 0;
     int pend = 0, npend = 0;
     TlRow I;
-    tl_load_row<PC>(A, a, threadIdx.x, I);
+    tl_load_row<PC>(A, a, threadIdx.x, exact ? kFfExactClose2 : kFfClose2, I);
     // sums kept out of the registers: of the near pairs; of up to 4 groups; of all
     // before them (TwoSum) with its compensation
     __shared__ double sums[12][kTlRows];
@@ -439,28 +446,32 @@ kick_tile_f64_kernel(SymArgs A) {
     for (int g = R.g0; g < R.g1; g++) {
         __syncthreads();
         tl_stage(A, g, grp);
-        if (threadIdx.x < 64) {
-            const int j = g * 64 + threadIdx.x;
-            const double m = j < A.n ? A.m[j] * mscale : 0.0, r = m - (double)__double2float_rn(m);
-            mtail[threadIdx.x] = __double2float_rn(r - (double)__double2float_rn(r));
+        if (exact && threadIdx.x < 64) {
+            const double xs = scalbn(1.0, -A.ff_header[2]);
+            const int j = min(g * 64 + (int)threadIdx.x, A.n - 1);
+            xyz[0][threadIdx.x] = A.x[j] * xs; xyz[1][threadIdx.x] = A.y[j] * xs; xyz[2][threadIdx.x] = A.z[j] * xs;
         }
         __syncthreads();
         const double mm = A.tmass[g >> 1];
         const bool gen = (g >> 1) == a || ((a + 1) * kSymT > A.nm && (g + 1) * 64 > A.nm) ||
                          (pads && (a == A.nT - 1 || (g >> 1) == A.nT - 1));
         double acc[3] = {0.0, 0.0, 0.0};
-        if (wide) tl_group_wide<PC>(A, grp, g, R.k0, R.k1, I.thr, I.tn, I.i, acc, pcb[PC ? w : 0], pend, lane);
-        else if (gen) tl_group64<PC, kFfGeneral>(A, grp, mtail, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        if (exact) tl_group64<PC, kFfExact>(A, grp, xyz, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        else if (gen) tl_group64<PC, kFfGeneral>(A, grp, xyz, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
         else if (mm > 0.0)
-            tl_group64<PC, kFfUniform>(A, grp, mtail, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
-        else tl_group64<PC, kFfPlain>(A, grp, mtail, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
-        const double f = !wide && !gen && mm > 0.0 ? mm : 1.0;
+            tl_group64<PC, kFfUniform>(A, grp, xyz, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        else tl_group64<PC, kFfPlain>(A, grp, xyz, g, R.k0, R.k1, I, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        const double f = !exact && !gen && mm > 0.0 ? mm : 1.0;
         const bool fold = ((g - R.g0) & 3) == 3 && g + 1 < R.g1;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             double t = fma(f, acc[c], T[c * kTlRows]);
             if (fold) {
                 double e;
+                if (near[c * kTlRows] != 0.0) {                  // (a body whose pairs are all taken in FP64)
+                    t = fma(back, near[c * kTlRows], t);
+                    near[c * kTlRows] = 0.0;
+                }
                 two_sum_ordered(S[c * kTlRows], t, t, e);
                 S[c * kTlRows] = t;
                 C[c * kTlRows] += e;
@@ -472,13 +483,11 @@ kick_tile_f64_kernel(SymArgs A) {
     tl_near_flush(A, nb[w], npend, I.i - lane, near, lane);
     if (PC) sym_pc_flush(A, pcb[w], pend, lane);
     if (I.i < A.n) {
-        // the near pairs' sums in the packed units
-        const double f = scalbn(1.0, 2 * A.ff_header[2] - A.ff_header[1]);
         double *p = A.part + (size_t)blockIdx.y * 3 * A.n + I.i;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             double t = T[c * kTlRows];
-            if (near[c * kTlRows] != 0.0) t = fma(f, near[c * kTlRows], t);
+            if (near[c * kTlRows] != 0.0) t = fma(back, near[c * kTlRows], t);
             if (R.g1 - R.g0 > 4) t = S[c * kTlRows] + (C[c * kTlRows] + t);
             p[(size_t)c * A.n] = t;
         }

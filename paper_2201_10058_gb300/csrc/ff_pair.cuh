@@ -8,6 +8,13 @@
 
 namespace genga {
 
+// A sum of terms as a double: f64_of_f32_any, but NaN for an infinite or NaN sum (whose
+// bits as they stand would read as 2^128 and 1.5 2^128).
+__device__ __forceinline__ double ff_sum_f64(float v) {
+    const double d = f64_of_f32_any(v);
+    return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u ? __hiloint2double(0x7ff80000, 0) : d;
+}
+
 // One coordinate's displacement as two floats.
 __device__ __forceinline__ void ff_disp(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 nli, f2 &H, f2 &L) {
     f2 e;

@@ -65,7 +65,7 @@ struct IBody {                                 // a lane's row, in both halves: 
 // sum += h + l, in the uniform instance times m_i m_j.
 template <int MODE>
 __device__ __forceinline__ void ff_flush(double &sum, double mm, float h, float l) {
-    const double v = f64_of_f32_any(h) + f64_of_f32_any(l);
+    const double v = ff_sum_f64(h) + f64_of_f32_any(l);
     sum = MODE == kFfUniform ? fma(mm, v, sum) : sum + v;
 }
 

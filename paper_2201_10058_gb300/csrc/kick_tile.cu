@@ -193,7 +193,7 @@ __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, in
             const float2 a = f2_get(sh[c]), b = f2_get(sl[c]);
             float s, x;
             ff_two_sum(a.x, a.y, s, x);
-            const double v = f64_of_f32_any(s) + f64_of_f32_any(x + (b.x + b.y));
+            const double v = ff_sum_f64(s) + f64_of_f32_any(x + (b.x + b.y));
             acc[c] = MODE == kFfUniform ? fma(mm, v, acc[c]) : acc[c] + v;
         }
     }

@@ -21,24 +21,30 @@ __device__ __forceinline__ void ff_disp(f2 hj, f2 mj, f2 lj, f2 nhi, f2 nmi, f2 
     f2_fast_two_sum(f2_add(hj, nhi), f2_add(mj, nmi), H, e);
     L = f2_add(e, f2_add(lj, nli));
 }
-// An FP64 displacement as three floats by integer operations: h truncated, l and t (|l| <
-// 2^-23 |v|) the other bits.  |v| < 2^-74: l = t = 0, |v| < 2^-126 also h = 0; |v| >=
-// 2^100, infinite or NaN: h = NaN.
-__device__ __forceinline__ void f64_split3(double v, float &h, float &l, float &t) {
+// An FP64 displacement times 2^-es as three floats by integer operations: h truncated, l
+// and t (|l| < 2^-23 |v|) the other bits.  With v scaled: |v| < 2^-74: l = t = 0, |v| <
+// 2^-126 also h = 0; |v| >= 2^100, infinite or NaN: h = NaN.
+__device__ __forceinline__ void f64_split3(double v, int es, float &h, float &l, float &t) {
     const unsigned hw = (unsigned)__double2hiint(v), lw = (unsigned)__double2loint(v);
-    const unsigned mag = hw & 0x7fffffffu, sgn = hw & 0x80000000u, E = mag >> 20;
-    h = __uint_as_float(mag >= 0x46300000u ? 0x7fc00000u : mag >= 0x38100000u ? (sgn | ((mag - 0x38000000u) << 3) | (lw >> 29)) : sgn);
-    const unsigned unit = E >= 949u ? sgn | ((E - 948u) << 23) : 0u;       // 2^(E - 1075), the last place
-    const unsigned unit14 = E >= 949u ? sgn | ((E - 934u) << 23) : 0u;
+    const unsigned mag = hw & 0x7fffffffu, sgn = hw & 0x80000000u;
+    const int e = mag < 0x00100000u ? 0 : (int)(mag >> 20) - es;           // exponent field of the scaled value
+    const unsigned top = ((mag - ((unsigned)es << 20) - 0x38000000u) << 3) | (lw >> 29);
+    h = __uint_as_float(e >= 1123 ? 0x7fc00000u : e >= 897 ? sgn | top : sgn);
+    const unsigned unit = e >= 949 ? sgn | ((unsigned)(e - 948) << 23) : 0u;       // 2^(e - 1075), the last place
+    const unsigned unit14 = e >= 949 ? sgn | ((unsigned)(e - 934) << 23) : 0u;
     l = (__uint_as_float(0x4b000000u | (lw >> 14 & 0x7fffu)) - 8388608.0f) * __uint_as_float(unit14);
     t = (__uint_as_float(0x4b000000u | (lw & 0x3fffu)) - 8388608.0f) * __uint_as_float(unit);
 }
-// The same for a component of two pairs, two floats each, the first rounded.
-__device__ __forceinline__ void f64_split2(double vx, double vy, f2 &H, f2 &L) {
-    float hx, lx, tx, hy, ly, ty;
-    f64_split3(vx, hx, lx, tx);
-    f64_split3(vy, hy, ly, ty);
-    f2_fast_two_sum(f2_make(hx, hy), f2_add(f2_make(lx, ly), f2_make(tx, ty)), H, L);
+// The displacements from body i to bodies jx and jy, two floats per component.
+__device__ __forceinline__ void ff_disp_f64(const SymArgs &A, int i, int jx, int jy, int es, f2 (&H)[3], f2 (&L)[3]) {
+    const double *P[3] = {A.x, A.y, A.z};
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        float hx, lx, tx, hy, ly, ty;
+        f64_split3(P[c][jx] - P[c][i], es, hx, lx, tx);
+        f64_split3(P[c][jy] - P[c][i], es, hy, ly, ty);
+        f2_fast_two_sum(f2_make(hx, hy), f2_add(f2_make(lx, ly), f2_make(tx, ty)), H[c], L[c]);
+    }
 }
 
 // g w as two floats (g = gh + gl, w + wl)

@@ -28,7 +28,8 @@
 // What the packing kernel finds takes the instance of the pair loop that unusual
 // inputs need:
 //   * coordinates that three floats do not hold, because they are far smaller than
-//     the largest on their axis (2^-25: 3e-8).  A few: NaN in their place, which
+//     the largest on their axis (2^-25: 3e-8), or larger (S leaves out a few bodies
+//     far outside the others).  A few: NaN in their place, which
 //     takes these bodies' pairs to FP64 one by one (ff_one); many: kFfExact, every
 //     displacement by FP64 subtraction, 3 FP64 instructions per pair;
 //   * kFfTwoMass: a massless body, or one 2^-40 of the heaviest: m_j r^-3 d and
@@ -81,7 +82,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
     constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
     f2 ih[kFfR][3], il[kFfR][3], jh[3], jl[3];
     const f2 one = f2_dup(1.0f);
-    const double xs = EXACT ? scalbn(1.0, -A.ff_header[2]) : 1.0;
+    const int es = EXACT ? A.ff_header[2] : 0;
     const float4 *group = tile + (jb >> 1);
 #pragma unroll 1
     for (int tb = 0; tb < 32; tb += kFfFlush) {
@@ -117,10 +118,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                     want[r][1] = want[r][1] && !(i >= A.nm && j + 32 >= A.nm);
                 }
                 if (EXACT) {
-                    const int i = min(I[r].i, A.n - 1), jx = min(jglob + k, A.n - 1), jy = min(jglob + k + 32, A.n - 1);
-                    f64_split2((A.x[jx] - A.x[i]) * xs, (A.x[jy] - A.x[i]) * xs, H[r][0], L[r][0]);
-                    f64_split2((A.y[jx] - A.y[i]) * xs, (A.y[jy] - A.y[i]) * xs, H[r][1], L[r][1]);
-                    f64_split2((A.z[jx] - A.z[i]) * xs, (A.z[jy] - A.z[i]) * xs, H[r][2], L[r][2]);
+                    ff_disp_f64(A, min(I[r].i, A.n - 1), min(jglob + k, A.n - 1), min(jglob + k + 32, A.n - 1), es, H[r], L[r]);
                     want[r][0] = want[r][0] && I[r].i < A.n && jglob + k < A.n;
                     want[r][1] = want[r][1] && I[r].i < A.n && jglob + k + 32 < A.n;
                 } else {
@@ -375,6 +373,11 @@ kick_sym_ff_kernel(SymArgs A)
     if (PC) sym_pc_flush(A, pcb[w], pend, lane);
 }
 
+// Powers of two that a coordinate may lie above those of nearly all bodies without being
+// left out: a body beyond costs ~10 to 50 ordinary pairs for each of its own, a factor of
+// two in S one bit of the smallest components that are held.
+constexpr int kFfMargin = 4;
+
 // The exponent field of a finite double (0: zero or denormal, -1: infinite or NaN).
 __device__ __forceinline__ int f64_field(double v) {
     const int f = (__double2hiint(v) >> 20) & 0x7ff;
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(256) ff_bounds_kernel(int n, const double *pos
         for (int k = 0; k < 8; k++) m = max(m, sh[threadIdx.x][k]);
         reinterpret_cast<int *>(bounds + 2 * blockIdx.x)[threadIdx.x] = m;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) header[3] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) header[3] = header[5] = 0;
 }
 
 // (Scaled) x = h + m + l: h a multiple of 2^-23 S, m of 2^-47 S (S = 2^e), l the rest
@@ -421,25 +424,43 @@ __device__ __forceinline__ void ff_split(double x, double mag1, double mag2, flo
 // header: the work is FP64 instructions, ~60 per body, and four SMs do a tile in
 // two thirds of the time of one (N = 2,048: 5.1 us against 6.9).
 __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
-    __shared__ int sh[5][kSymT / 32];
+    __shared__ int sh[5];
     __shared__ double tm;
-    int v[5] = {0, 0, 0, 0, 0};
-    for (int k = threadIdx.x; k < nbounds; k += kSymT) {
-        const int4 o = A.bounds[2 * k];
-        v[0] = max(v[0], o.x); v[1] = max(v[1], o.y); v[2] = max(v[2], o.z); v[3] = max(v[3], o.w);
-        v[4] = max(v[4], A.bounds[2 * k + 1].x);
-    }
+    {
+        // warp c, axis c: the largest field of the blocks, but at most kFfMargin above what an
+        // eighth of them exceeds -- bodies far outside the others (ejected ones) would
+        // otherwise set a grid too coarse for all; warp 3: masses
+        const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        int f[(kFfBoundBlocks + 31) / 32], m = 0, small = 0;
 #pragma unroll
-    for (int c = 0; c < 5; c++) {
-        v[c] = __reduce_max_sync(0xffffffffu, v[c]);
-        if ((threadIdx.x & 31) == 0) sh[c][threadIdx.x >> 5] = v[c];
+        for (int k = 0; k < (kFfBoundBlocks + 31) / 32; k++) {
+            const int b = 32 * k + lane;
+            f[k] = b < nbounds ? reinterpret_cast<const int *>(A.bounds + 2 * b)[c] : 0;
+            m = max(m, f[k]);
+            if (c == 3 && b < nbounds) small = max(small, A.bounds[2 * b + 1].x);
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        small = __reduce_max_sync(0xffffffffu, small);
+        if (c < 3 && nbounds >= 8) {
+            int q = 0;                         // largest field that more than an eighth reach
+            for (int s = 1024; s; s >>= 1) {
+                int above = 0;
+#pragma unroll
+                for (int k = 0; k < (kFfBoundBlocks + 31) / 32; k++) above += f[k] >= q + s;
+                if (8 * __reduce_add_sync(0xffffffffu, above) > nbounds) q += s;
+            }
+            m = min(m, q + kFfMargin);
+        }
+        if (lane == 0) {
+            sh[c] = m;
+            if (c == 3) sh[4] = small;
+        }
     }
     __syncthreads();
+    int v[5];
 #pragma unroll
-    for (int c = 0; c < 5; c++)
-#pragma unroll
-        for (int k = 0; k < kSymT / 32; k++) v[c] = max(v[c], sh[c][k]);
-    // S = 2^ex > every |coordinate|; lengths are scaled by 2^-es, which puts S at 2^kFfScale,
+    for (int c = 0; c < 5; c++) v[c] = sh[c];
+    // S = 2^ex > every |coordinate| that is held; lengths are scaled by 2^-es, which puts S at 2^kFfScale,
     // masses by 2^-em, so that the floats' range does not depend on the caller's units
     const int ex = min(max(max(v[0], max(v[1], v[2])) - 1022, -200), 400);
     const int es = ex - kFfScale, em = min(max(v[3] - 1023, -200), 400);
@@ -476,6 +497,11 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
         if (A.ctr) *A.ctr = 0u;
         if (A.cand_count) *A.cand_count = 0ull;
     }
+    int field = 0x7ff;
+    if (i < A.n)
+        field = max(f64_field(A.pos[i]), max(f64_field(A.pos[(size_t)A.n + i]), f64_field(A.pos[2 * (size_t)A.n + i])));
+    const int inner = __syncthreads_count(field - 1022 <= ex - kFfInner);
+    if (inner && threadIdx.x == 0) atomicAdd(&A.header[5], inner);
     // the common (scaled) mass of a full tile of equal masses, else 0
     const double ms = i < A.n ? A.m[i] * scalbn(1.0, -em) : 0.0;
     if (threadIdx.x == 0) tm = ms;

@@ -102,7 +102,12 @@ constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2, kFfExact = 3;      /
 // the FP64 kick (N = 16,384: 3.3 ms against 2.0; 5.4 for the FP64 symmetric form), 3.1
 // times in the mixed one (65,540: 28.8 ms against 9.2; 34.9 with displacement and sums in
 // FP64), while a pair taken by itself costs ~10 to 50 of them.
-__device__ __forceinline__ bool ff_exact_pairs(const int *header, int n) { return 128ll * header[3] > n; }
+// So they do where a quarter of the bodies are within 2^-kFfInner of the largest coordinate
+// from the star: their pairs would be near ones (r < 2^-20 S), taken one by one.
+constexpr int kFfInner = 15;
+__device__ __forceinline__ bool ff_exact_pairs(const int *header, int n) {
+    return 128ll * header[3] > n || 4ll * header[5] > n;
+}
 // Bounds of r^2: below, the parts give no displacement in proper order (2^-20 S) or r^-3
 // nears the end of the floats' range (kFfExact); above (kFfExact), the same.
 constexpr float kFfClose2 = 0x1p-28f, kFfExactClose2 = 0x1p-64f, kFfExactFar2 = 0x1p60f;
@@ -130,7 +135,7 @@ struct FfPack {
     float2 *ircf;
     double *tmass;                    // per tile
     int *header;                      // flags, exponents masses and lengths are scaled by, coordinates not held,
-                                      // kFfClose2 (float); 8 ints
+                                      // kFfClose2 (float), inner bodies; 8 ints
     unsigned *ctr;                    // NULL: left alone
     unsigned long long *cand_count;   // NULL: left alone
 };

@@ -88,7 +88,7 @@ __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, in
                                          double mm, double (&acc)[3], uint2 *pcbuf, int &pend, int lane) {
     constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
     const f2 one = f2_dup(1.0f);
-    const double xs = EXACT ? scalbn(1.0, -A.ff_header[2]) : 1.0;
+    const int es = EXACT ? A.ff_header[2] : 0;
 #pragma unroll 1
     for (int tb = k0; tb < k1; tb += kTlFlush) {
         f2 sh[3], sl[3];
@@ -108,10 +108,7 @@ __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, in
                 wy = j + 32 != I.i && !(ti && j + 32 >= A.nm);
             }
             if (EXACT) {
-                const int i = min(I.i, A.n - 1), jx = min(j, A.n - 1), jy = min(j + 32, A.n - 1);
-                f64_split2((A.x[jx] - A.x[i]) * xs, (A.x[jy] - A.x[i]) * xs, H[0], L[0]);
-                f64_split2((A.y[jx] - A.y[i]) * xs, (A.y[jy] - A.y[i]) * xs, H[1], L[1]);
-                f64_split2((A.z[jx] - A.z[i]) * xs, (A.z[jy] - A.z[i]) * xs, H[2], L[2]);
+                ff_disp_f64(A, min(I.i, A.n - 1), min(j, A.n - 1), min(j + 32, A.n - 1), es, H, L);
                 wx = wx && I.i < A.n && j < A.n;
                 wy = wy && I.i < A.n && j + 32 < A.n;
             } else {
@@ -254,6 +251,18 @@ __device__ __forceinline__ void tl_near_flush(const SymArgs &A, TlNear &B, int &
             const double c = A.m[j] * (K * (y * y * y));
             tx = c * dx; ty = c * dy; tz = c * dz;
         }
+        const unsigned row = B.q[t0].x;
+        if (__all_sync(0xffffffffu, lane >= m || B.q[t0 + lane].x == row)) {
+            // one row's (a body that is not held): a butterfly, 15 FP64 instructions instead of 96
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                tx += __shfl_xor_sync(0xffffffffu, tx, o);
+                ty += __shfl_xor_sync(0xffffffffu, ty, o);
+                tz += __shfl_xor_sync(0xffffffffu, tz, o);
+            }
+            if (lane == (int)row) { sum[0] += tx; sum[kTlRows] += ty; sum[2 * kTlRows] += tz; }
+            continue;
+        }
         B.t[0][lane] = tx; B.t[1][lane] = ty; B.t[2][lane] = tz;
         __syncwarp();
         unsigned mine = 0u;
@@ -307,8 +316,8 @@ __device__ __forceinline__ void tl_group64(const SymArgs &A, const float4 *grp, 
                 float hx, lx, tx, hy, ly, ty;
                 ex[c] = xyz[c][k] - xi[c];
                 ey[c] = xyz[c][k + 32] - xi[c];
-                f64_split3(ex[c], hx, lx, tx);
-                f64_split3(ey[c], hy, ly, ty);
+                f64_split3(ex[c], 0, hx, lx, tx);
+                f64_split3(ey[c], 0, hy, ly, ty);
                 H[c] = f2_make(hx, hy); L[c] = f2_make(lx, ly); T[c] = f2_make(tx, ty);
             }
         } else {

@@ -17,7 +17,7 @@
 // order (deterministic).  The rare pairs inside rc_ij are found by an FP32 test on
 // r^2 against a conservative threshold; only those evaluate the changeover function.
 //   * kick_kernel: the tiled form without packed bodies, for the allocation-free
-//     entry point where its scratch does not hold them (N > 139,000).
+//     entry point where its scratch does not hold them (N > 190,282).
 //
 // kick_kernel, MIXED: FP64 displacement; r^2 formed as an unevaluated sum of two floats
 // from an exact integer split of the displacement (no FP64 work); FP32 rsqrt seed
@@ -50,7 +50,7 @@ constexpr int kTile = 256;
 
 struct KickArgs {
     const double *x, *y, *z, *m;
-    const double *rc, *rc2, *pc2;
+    const double *rc, *pc2;
     const float *thr_rc;        // FP32 upper bound of rc^2
     int n;
     int nm;                     // bodies i >= nm are test particles (nm = n: none)
@@ -691,12 +691,10 @@ cudaError_t launch_fold(const FoldArgs &A, bool comp, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-__global__ void raw_thresholds_kernel(int n, const double *rc, double *rc2, float *thr) {
+__global__ void raw_thresholds_kernel(int n, const double *rc, float *thr) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double r2 = __dmul_rn(rc[i], rc[i]);
-    rc2[i] = r2;
-    thr[i] = fmaxf(__double2float_ru(r2) * 1.0000153f, 1.17549435e-38f);
+    thr[i] = fmaxf(__double2float_ru(__dmul_rn(rc[i], rc[i])) * 1.0000153f, 1.17549435e-38f);
 }
 
 void kick_geometry(int n, int num_sms, int *chunk, int *nchunk) {
@@ -716,11 +714,11 @@ void kick_geometry(int n, int num_sms, int *chunk, int *nchunk) {
 
 }  // namespace
 
-static KickArgs make_args(genga_system *s, bool precheck) {
+static KickArgs make_args(genga_system *s) {
     KickArgs A;
     const int64_t n = s->n;
     A.x = s->pos; A.y = s->pos + n; A.z = s->pos + 2 * n; A.m = s->mass;
-    A.rc = s->rcl[0].rc; A.rc2 = s->rcl[0].rc2; A.pc2 = s->rcl[0].pc2;
+    A.rc = s->rcl[0].rc; A.pc2 = s->rcl[0].pc2;
     A.thr_rc = s->rcl[0].thr_rc;
     A.n = (int)n;
     A.nm = tp_bound(s);
@@ -936,7 +934,7 @@ cudaError_t launch_precheck_only(genga_system *s) {
     const int n = (int)s->n;
     if (!s->kick_part) return cudaErrorInvalidValue;
     if (s->kick_chunk == 0) kick_geometry(n, s->num_sms, &s->kick_chunk, &s->kick_nchunk);
-    KickArgs A = make_args(s, true);
+    KickArgs A = make_args(s);
     // (i-tile x j-chunk) grid like the kick; blocks wholly below the diagonal return at once
     dim3 grid((n + kPcThreads * kPcI - 1) / (kPcThreads * kPcI), s->kick_nchunk);
     GENGA_CUDA_TRY(cudaMemsetAsync(&s->ctr->cand_count, 0, sizeof(unsigned long long), s->stream));
@@ -982,8 +980,8 @@ cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, cudaStream_t stream) 
         chunk = tiles_per_chunk * kTile;
         nchunk = (k.n + chunk - 1) / chunk;
     }
-    float *thr = (float *)(k.scratch + N);
-    raw_thresholds_kernel<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(k.n, k.rc, k.scratch, thr);
+    float *thr = (float *)k.scratch;
+    raw_thresholds_kernel<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(k.n, k.rc, thr);
     GENGA_CUDA_TRY(cudaGetLastError());
     KickArgs A = {};
     A.x = k.pos; A.y = k.pos + k.n; A.z = k.pos + 2 * N; A.m = k.mass;

@@ -10,8 +10,8 @@
 // long as the library is loaded (every GPU that loads the library holds it).
 //
 // Scratch layout (launch_kick_raw): the packed bodies and the tiled kick's partial
-// sums where they fit, else (doubles) rc^2 [n], FP32 thresholds [n floats] and the
-// per-chunk partial sums [nchunk][6][n], nchunk reduced as needed to fit.
+// sums where they fit (n <= 190,282), else FP32 thresholds [n floats] and, from 1.5 n
+// doubles on, the per-chunk partial sums [nchunk][6][n], nchunk reduced as needed to fit.
 #include <cuda.h>
 #include <mutex>
 

@@ -312,13 +312,15 @@ int genga_remove_merged(genga_system_t *sys, int64_t *n_new, int64_t *old_index)
  *   bs_group_seconds  one group's in-block Bulirsch-Stoer integration over a
  *                     (sub-)step (groups of up to 32 members); default 10 s;
  *   barrier_seconds   one grid-barrier wait of the persistent Bulirsch-Stoer
- *                     kernel (groups of more than 32 members); default 2 s.
+ *                     kernel (groups of more than 32 members); default 2 s;
+ *                     bs_group_seconds more for the first one where smaller
+ *                     groups are integrated beside it.
  * A negative value restores the default; 0 makes the first check run out.
  * When a limit is reached the call returns GENGA_ETIMEOUT with a message, the
  * integration of that step stops (the state is left partly advanced), and
  * the system stays usable.  barrier_absent_blocks is a test hook: with n > 0
  * every grid barrier waits for n blocks that do not exist, so every wait
- * runs out after barrier_seconds (0 in normal use).  Errors: EINVAL.        */
+ * runs out after its limit (0 in normal use).  Errors: EINVAL.              */
 int genga_set_wait_limits(genga_system_t *sys, double bs_group_seconds, double barrier_seconds,
                           int32_t barrier_absent_blocks);
 

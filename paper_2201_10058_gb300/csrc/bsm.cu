@@ -57,7 +57,7 @@ constexpr int kPairMembers = 400;
 
 struct GridBarrier {
     unsigned long long count;   // arrivals since the launch; top bit: a wait ran out
-    unsigned err;               // the same, for the host
+    unsigned err;               // the same, for the host: 1, 2 for the first wait
     unsigned running;           // groups still integrating
 };
 
@@ -147,7 +147,8 @@ __device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsign
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (target == 0ull) limit_ns += first_ns;
+        const bool first = target == 0ull;
+        if (first) limit_ns += first_ns;
         target += gridDim.x + absent;
         asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&b->count) : "memory");
         unsigned long long t0 = 0ull, v;
@@ -159,7 +160,7 @@ __device__ bool grid_barrier(GridBarrier *b, unsigned long long limit_ns, unsign
                 if (t0 == 0ull) t0 = now;
                 if (now - t0 >= limit_ns) {
                     atomicOr(&b->count, kBarrierErr);
-                    atomicExch(&b->err, 1u);
+                    atomicCAS(&b->err, 0u, first ? 2u : 1u);
                     v = kBarrierErr;
                     break;
                 }
@@ -1079,7 +1080,7 @@ int bsm_run(genga_system *s, int level, double dt, const std::vector<int2> &grou
     if (hb.err) {
         snprintf(s->err, sizeof(s->err),
                  "persistent Bulirsch-Stoer: a grid-barrier wait exceeded its limit of %.3g s",
-                 1e-9 * (double)s->barrier_limit_ns);
+                 1e-9 * (double)(A.barrier_ns + (hb.err == 2u ? A.first_ns : 0ull)));
         return GENGA_ETIMEOUT;
     }
     scatter(st, mbody, A.Y);

@@ -249,7 +249,8 @@ __device__ void ens_kick(const EnsArgs &A, EnsShared &S, double dt_half, bool pr
 //
 // The FP64 pipe bounds this part (two thirds of the kernel), so what the
 // iterations share -- everything that depends on the position alone -- is formed
-// once, and an iteration is 73 FP64 instructions per body:
+// once, and an iteration is 73 FP64 instructions per body and 6 for the sum of the
+// star's torques:
 //   acc = A e + B u + Q x e,  A = a0 + a1 rdot + a2 rdot^2 + a3 u^2,  B = b0 + b1 rdot,
 //   Q = q_i W + q_s W_star (e = x / r, rdot = e.u), and with T(W) = r W - (x.W) e - e x u
 //   dW = c_w T(W), the star's torque sum c_s T(W_star).
@@ -604,11 +605,13 @@ __device__ void ens_bs_fast(const EnsArgs &A, EnsShared &S, int nm, double dt, u
         F.irc[q - 1] = rc > 1e-30 ? rcp_newton(rc) : rc > 0.0 ? 1.0 / rc : __longlong_as_double(0x7ff0000000000000ll);
         F.ircf[q - 1] = __double2float_rz(F.irc[q - 1]);
     }
-    // lanes without a member stand far off, each its own place
+    // lanes without a member stand a thousand times farther out than member 0, each its own
+    // place (near the star they would end in NaN, which their zero masses do not stop)
+    const double out = 1e3 * (fabs(S.x0[0][b]) + fabs(S.x0[1][b]) + fabs(S.x0[2][b])) * (s + 2);
     double Y[6], f0[6], zm[6], T[8], f[6];
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-        Y[c] = member ? S.x0[c][b] : 1e3 * fabs(S.x0[0][b]) * (s + 2) + (c == 0 ? 1.0 : 0.0);
+        Y[c] = member ? S.x0[c][b] : out;
         Y[3 + c] = member ? S.v0[c][b] : 0.0;
     }
     const int nk = 2 * (col + 1), comp = col < 6 ? col : 0;

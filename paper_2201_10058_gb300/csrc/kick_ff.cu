@@ -46,7 +46,9 @@ constexpr int kFfThreads = 64;                 // two warps: 64 rows each of the
 
 // Chosen by measurement at N = 65,540 (ms per kick): rows per lane 2 (9.5; 1:
 // 10.3 -- the j data and shuffles serve two rows), 2 steps unrolled (1: 9.45, 4:
-// 9.9), 6 blocks per SM by registers (4: 10.2, 7: 9.7).
+// 9.9).  Blocks per SM that the registers must allow: 5, which gives the compiler the 166
+// to 168 it then takes, so that 6 are resident (8.96; bound at 6, 148 registers: 9.17,
+// at 7: 9.16, at 4: 9.69).
 constexpr int kFfR = 2;
 constexpr int kFfUnroll = 2;
 constexpr int kFfMinBlocks = 5;

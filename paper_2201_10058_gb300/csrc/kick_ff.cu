@@ -83,7 +83,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                                         double mm, uint2 *pcbuf, int &pend, int lane) {
     constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
     f2 ih[kFfR][3], il[kFfR][3], jh[3], jl[3];
-    const f2 one = f2_dup(1.0f);
+    const f2 away = f2_dup(kFfMasked2);
     const int es = EXACT ? A.ff_header[2] : 0;
     const float4 *group = tile + (jb >> 1);
 #pragma unroll 1
@@ -131,7 +131,7 @@ __device__ __forceinline__ void ff_rows(const SymArgs &A, const float4 *tile, do
                 f2 s2, tail;
                 ff_r2(H[r], L[r], s2, tail);
                 if (GEN) {                         // (NaN times zero would be NaN)
-                    s2 = f2_select(want[r][0], want[r][1], s2, one);
+                    s2 = f2_select(want[r][0], want[r][1], s2, away);
                     tail = f2_select(want[r][0], want[r][1], tail, 0ull);
 #pragma unroll
                     for (int c = 0; c < 3; c++) {

@@ -87,7 +87,7 @@ template <bool PC, int MODE>
 __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, int g, int k0, int k1, const TlRow &I, float close2,
                                          double mm, double (&acc)[3], uint2 *pcbuf, int &pend, int lane) {
     constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
-    const f2 one = f2_dup(1.0f);
+    const f2 away = f2_dup(kFfMasked2);
     const int es = EXACT ? A.ff_header[2] : 0;
 #pragma unroll 1
     for (int tb = k0; tb < k1; tb += kTlFlush) {
@@ -118,7 +118,7 @@ __device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, in
             }
             ff_r2(H, L, s2, tail);
             if (GEN) {                             // (NaN times zero would be NaN)
-                s2 = f2_select(wx, wy, s2, one);
+                s2 = f2_select(wx, wy, s2, away);
                 tail = f2_select(wx, wy, tail, 0ull);
 #pragma unroll
                 for (int c = 0; c < 3; c++) {

@@ -51,7 +51,7 @@ OPS_PER_CLK_PER_SM = {"mixed": 128, "fp64": 2}
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the mixed
 # symmetric kick kernel at N = 65,540 (P = 4, 129 partial slots: the traffic is
 # the partial sums); None when the kernel has changed since the capture
-KICK_MIXED_DRAM_BYTES = 150205440
+KICK_MIXED_DRAM_BYTES = 149304832
 
 
 def parse():

@@ -9,7 +9,7 @@
 //     of the bodies, 3 FP64 instructions per pair (FP64) or none (mixed);
 //   * symmetric: each unordered pair once, its force to both bodies (Newton's
 //     third law).  The mixed form (kick_ff.cu) is faster than the tiled one from
-//     N ~ 6,000 on (12,000: 0.43 ms against 0.55; 4,096: 0.111 against 0.092) and
+//     N ~ 6,000 on (12,000: 0.41 ms against 0.58; 4,096: 0.111 against 0.089) and
 //     taken where predicted so; the FP64 form (kick_sym_kernel, below), 21 FP64
 //     instructions per unordered pair, only on request (20,011: 7.9 ms against
 //     2.9 tiled; 128: 0.106 against 0.028).

@@ -24,10 +24,10 @@
 //           the displacement is an FP64 subtraction, which the FMAs then take whole: 6
 //           FP64 instructions.
 // Measured (whole kick, us; before: kick_kernel, or FP64 symmetric from 16,384 on):
-//   FP64   N = 1,000: 40 (189), 2,048: 68 (193), 20,011: 2,916 (7,915); error against
+//   FP64   N = 1,000: 39 (189), 2,048: 67 (193), 20,011: 2,867 (7,915); error against
 //          64 bits 1.6e-16 of the norm at 20,011 (2.1e-16)
-//   mixed  N = 1,000: 27 (101), 3,001: 61 (136), 4,096: 89 (246)
-// Bound: FP64 pipe 78 % and FP32 pipe 70 % busy at N = 8,192 (both, in turns, by the
+//   mixed  N = 1,000: 27 (101), 3,001: 59 (136), 4,096: 88 (246)
+// Bound: FP64 pipe 75 % and FP32 pipe 72 % busy at N = 8,192 (both, in turns, by the
 // few warps that 96 registers leave); below N ~ 2,000 the latency of one block.
 #include <algorithm>
 #include <cmath>

@@ -241,6 +241,7 @@ cudaError_t launch_energy(genga_system *s, double *E_host, double *L_host) {
         GENGA_CUDA_TRY(cudaMalloc((void **)&s->en_part, sizeof(double) * (kEnRows * 2 * kEnBlocks + kEnRows)));
     FfPack ff = ff_pack_args(s);
     ff.window = kFfWindowNone;
+    ff.margin = kFfMargin64;
     GENGA_CUDA_TRY(launch_ff_pack(ff, s->stream, &s->launches));
     EnergyArgs A;
     A.x = s->pos; A.y = s->pos + n; A.z = s->pos + 2 * (size_t)n; A.m = s->mass;

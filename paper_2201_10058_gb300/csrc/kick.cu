@@ -959,6 +959,7 @@ cudaError_t launch_kick_raw(const KickRaw &k, int num_sms, cudaStream_t stream) 
         ff.pos = k.pos; ff.m = k.mass; ff.rc = k.rc; ff.pc2 = nullptr; ff.n = k.n; ff.nT = (k.n + kSymT - 1) / kSymT;
         ff_place(ff, k.scratch, ff.nT);
         ff.ctr = nullptr; ff.cand_count = nullptr; ff.window = k.mixed ? kFfWindowMixed : kFfWindow64;
+        ff.margin = k.mixed ? kFfMarginMixed : kFfMargin64;
         SymArgs S = {};
         S.x = k.pos; S.y = k.pos + N; S.z = k.pos + 2 * N; S.m = k.mass; S.rc = k.rc;
         S.n = S.nm = k.n; S.nT = ff.nT; S.part = k.scratch + packed;

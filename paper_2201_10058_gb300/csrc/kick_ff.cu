@@ -375,11 +375,6 @@ kick_sym_ff_kernel(SymArgs A)
     if (PC) sym_pc_flush(A, pcb[w], pend, lane);
 }
 
-// Powers of two that a coordinate may lie above those of nearly all bodies without being
-// left out: a body beyond costs ~10 to 50 ordinary pairs for each of its own, a factor of
-// two in S one bit of the smallest components that are held.
-constexpr int kFfMargin = 4;
-
 // The exponent field of a finite double (0: zero or denormal, -1: infinite or NaN).
 __device__ __forceinline__ int f64_field(double v) {
     const int f = (__double2hiint(v) >> 20) & 0x7ff;
@@ -429,9 +424,9 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
     __shared__ int sh[5];
     __shared__ double tm;
     {
-        // warp c, axis c: the largest field of the blocks, but at most kFfMargin above what an
-        // eighth of them exceeds -- bodies far outside the others (ejected ones) would
-        // otherwise set a grid too coarse for all; warp 3: masses
+        // warp c, axis c: the largest field of the blocks, without those of more than
+        // A.margin above what an eighth of them reach -- bodies far outside the others
+        // (ejected ones) would otherwise set a grid too coarse for all; warp 3: masses
         const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
         int f[(kFfBoundBlocks + 31) / 32], m = 0, small = 0;
 #pragma unroll
@@ -451,7 +446,10 @@ __global__ void __launch_bounds__(kSymT) ff_pack_kernel(FfPack A, int nbounds) {
                 for (int k = 0; k < (kFfBoundBlocks + 31) / 32; k++) above += f[k] >= q + s;
                 if (8 * __reduce_add_sync(0xffffffffu, above) > nbounds) q += s;
             }
-            m = min(m, q + kFfMargin);
+            m = 0;
+#pragma unroll
+            for (int k = 0; k < (kFfBoundBlocks + 31) / 32; k++) m = max(m, f[k] <= q + A.margin ? f[k] : 0);
+            m = __reduce_max_sync(0xffffffffu, m);
         }
         if (lane == 0) {
             sh[c] = m;
@@ -579,6 +577,7 @@ FfPack ff_pack_args(const genga_system *s) {
     k.nT = (int)((s->n + kSymT - 1) / kSymT);
     ff_place(k, s->ff, s->ff_tiles);
     k.window = s->p.precision == GENGA_MIXED ? kFfWindowMixed : kFfWindow64;
+    k.margin = s->p.precision == GENGA_MIXED ? kFfMarginMixed : kFfMargin64;
     k.ctr = nullptr;
     k.cand_count = nullptr;
     return k;

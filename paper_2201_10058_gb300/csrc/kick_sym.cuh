@@ -97,11 +97,12 @@ constexpr int kFfScale = 6;
 constexpr int kFfTwoMass = 1;                  // flag of the packed bodies, see kick_ff.cu
 constexpr int kFfPlain = 0, kFfUniform = 1, kFfGeneral = 2, kFfExact = 3;      // instances of the pair loops
 // A body whose coordinates the three floats do not hold has NaN in their place.  Its pairs
-// take FP64 one by one, and with more than one such coordinate per 128 bodies every pair
-// takes the instance of FP64 displacements (kFfExact): 1.6 times the time of the others in
-// the FP64 kick (N = 16,384: 3.3 ms against 2.0; 5.4 for the FP64 symmetric form), 3.1
-// times in the mixed one (65,540: 28.8 ms against 9.2; 34.9 with displacement and sums in
-// FP64), while a pair taken by itself costs ~10 to 50 of them.
+// take FP64 -- buffered, 32 at a time, in the tiled kick (mixed, one such body in 4,096: 108
+// us against 93; in its own lane: 316), one by one in the symmetric one (16,384: 881
+// against 667) --, and with more than one such coordinate per 128 bodies every pair
+// takes the instance of FP64 displacements (kFfExact): FP64 kick of 16,384 3.2 ms against
+// 2.0 (5.4 for the FP64 symmetric form), mixed kick of 65,540 20.0 against 9.0 (34.9 with
+// displacement and sums in FP64).
 // So they do where a quarter of the bodies are within 2^-kFfInner of the largest coordinate
 // from the star: their pairs would be near ones (r < 2^-20 S), taken one by one.
 constexpr int kFfInner = 15;
@@ -128,12 +129,16 @@ int sym_ff_blocks_per_sm(int P);
 constexpr int kFfBoundBlocks = 152;
 // Coordinates below 2^-window of their axis' S are not held: their last bits lie below
 // the parts.  18: every bit is held (FP64 kick), 25: to 2^-47 (mixed), none: to 2^-72 S,
-// enough for a distance (energy).
+// enough for a distance (energy).  And how many powers of two S may lie above what nearly
+// all bodies reach before a body beyond it is left out: it takes as many from the window.
+// (Mixed kick of 16,384 bodies with |z| < 4e-4 and four planets at 0.03: 669 us with 8, 887
+// with 4, which leaves the planets out.)
 constexpr int kFfWindow64 = 18, kFfWindowMixed = 25, kFfWindowNone = 4096;
+constexpr int kFfMargin64 = 4, kFfMarginMixed = 8;
 struct FfPack {
     const double *pos, *m, *rc, *pc2;
     int n, nT;
-    int window;
+    int window, margin;
     int4 *bounds;                     // scratch, 2 kFfBoundBlocks entries
     float4 *body;                     // whole tiles
     float2 *ircf;

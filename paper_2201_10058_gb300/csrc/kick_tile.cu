@@ -6,7 +6,8 @@
 //
 //   mixed   the pair arithmetic of kick_ff.cu (displacement, r^-3, K and the term
 //           m_j r^-3 d as two floats each, sums in two floats handed to FP64 after
-//           16 steps): ~105 FP32 operations per ordered pair.
+//           16 steps): ~105 FP32 operations per ordered pair.  Pairs of bodies whose
+//           coordinates three floats do not hold go to a buffer, as below.
 //   FP64    results of full double precision with 3 FP64 FMAs per ordered pair.
 //           FP64 issues once in 64 cycles per sub-partition, so everything else is
 //           on the FP32 pipe: displacement H + L + T, exactly (kick_ff.cu), the residual
@@ -82,155 +83,8 @@ __device__ __forceinline__ void tl_stage(const SymArgs &A, int g, float4 *grp) {
     for (int k = threadIdx.x; k < 7 * 32; k += kTlRows) grp[k] = src[(k >> 5) * kFfRow + (k & 31)];
 }
 
-// Mixed: the steps [k0, k1) of row I against the 64 bodies of group g.
-template <bool PC, int MODE>
-__device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, int g, int k0, int k1, const TlRow &I, float close2,
-                                         double mm, double (&acc)[3], uint2 *pcbuf, int &pend, int lane) {
-    constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
-    const f2 away = f2_dup(kFfMasked2);
-    const int es = EXACT ? A.ff_header[2] : 0;
-#pragma unroll 1
-    for (int tb = k0; tb < k1; tb += kTlFlush) {
-        f2 sh[3], sl[3];
-#pragma unroll
-        for (int c = 0; c < 3; c++) sh[c] = sl[c] = 0ull;
-#pragma unroll (EXACT ? 1 : 2)
-        for (int k = tb; k < min(tb + kTlFlush, k1); k++) {
-            const float4 q0 = grp[k], q1 = grp[32 + k], q2 = grp[64 + k], q3 = grp[96 + k], q4 = grp[128 + k],
-                         q5 = grp[160 + k];
-            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&grp[192 + k].z) : make_float2(q5.z, q5.w);
-            const int j = g * 64 + k;
-            f2 H[3], L[3], s2, tail, w, wl;
-            bool wx = true, wy = true;
-            if (GEN) {
-                const bool ti = I.i >= A.nm;
-                wx = j != I.i && !(ti && j >= A.nm);
-                wy = j + 32 != I.i && !(ti && j + 32 >= A.nm);
-            }
-            if (EXACT) {
-                ff_disp_f64(A, min(I.i, A.n - 1), min(j, A.n - 1), min(j + 32, A.n - 1), es, H, L);
-                wx = wx && I.i < A.n && j < A.n;
-                wy = wy && I.i < A.n && j + 32 < A.n;
-            } else {
-                ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I.h[0], I.m[0], I.l[0], H[0], L[0]);
-                ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I.h[1], I.m[1], I.l[1], H[1], L[1]);
-                ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I.h[2], I.m[2], I.l[2], H[2], L[2]);
-            }
-            ff_r2(H, L, s2, tail);
-            if (GEN) {                             // (NaN times zero would be NaN)
-                s2 = f2_select(wx, wy, s2, away);
-                tail = f2_select(wx, wy, tail, 0ull);
-#pragma unroll
-                for (int c = 0; c < 3; c++) {
-                    H[c] = f2_select(wx, wy, H[c], 0ull);
-                    L[c] = f2_select(wx, wy, L[c], 0ull);
-                }
-            }
-            ff_inv_r3(s2, tail, w, wl);
-            const float2 S = f2_get(s2);
-            const bool fx = EXACT && S.x > kFfExactFar2, fy = EXACT && S.y > kFfExactFar2;
-            const bool nx = fx || !(S.x >= fmaxf(I.tn, tj.x)), ny = fy || !(S.y >= fmaxf(I.tn, tj.y));
-            if (PC ? __any_sync(0xffffffffu, nx || ny) : (nx || ny)) {
-                if (PC) {
-                    sym_pc_push(pcbuf, pend, lane, nx && wx && j > I.i, I.i, j);
-                    sym_pc_push(pcbuf, pend, lane, ny && wy && j + 32 > I.i, I.i, j + 32);
-                    if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
-                }
-                const bool bx = fx || !(S.x >= fmaxf(I.thr, q5.z)), by = fy || !(S.y >= fmaxf(I.thr, q5.w));
-                if (bx || by) {
-                    const float2 ci = A.ircf[I.i], Tl = f2_get(tail);
-                    float2 W = f2_get(w), WL = f2_get(wl);
-#pragma unroll 1
-                    for (int h = 0; h < 2; h++) {
-                        if (!(h ? by : bx)) continue;
-                        const float2 cj = A.ircf[j + 32 * h];
-                        const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
-                        const float ih = ti ? ci.x : cj.x, il = ti ? ci.y : cj.y;
-                        float wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x;
-                        if (!((h ? S.y : S.x) >= close2) || (h ? fy : fx)) {
-                            FfOne o;
-                            ff_one(A, I.i, j + 32 * h, ih, il, o);
-#pragma unroll
-                            for (int c = 0; c < 3; c++) {
-                                const float2 u = f2_get(H[c]), v = f2_get(L[c]);
-                                H[c] = f2_make(h ? u.x : o.H[c], h ? o.H[c] : u.y);
-                                L[c] = f2_make(h ? v.x : o.L[c], h ? o.L[c] : v.y);
-                            }
-                            wh = o.w;
-                            wlo = o.wl;
-                        } else {
-                            float Kh, Kl;
-                            ff_changeover(h ? S.y : S.x, h ? Tl.y : Tl.x, ih, il, Kh, Kl);
-                            ff_mul(wh, wlo, Kh, Kl);
-                            if (Kh == 0.0f) wh = wlo = 0.0f;         // also where r^-3 overflows
-                        }
-                        if (h) { W.y = wh; WL.y = wlo; }
-                        else { W.x = wh; WL.x = wlo; }
-                    }
-                    w = f2_make(W.x, W.y);
-                    wl = f2_make(WL.x, WL.y);
-                }
-            }
-            if (GEN) {
-                w = f2_select(wx, wy, w, 0ull);
-                wl = f2_select(wx, wy, wl, 0ull);
-            }
-            f2 ch = w, cl = wl, th[3], te[3];
-            if (MODE != kFfUniform) ff_coeff(f2_hi(q1), f2_hi(q3), w, wl, ch, cl);
-            ff_term(ch, cl, H, L, th, te);
-#pragma unroll
-            for (int c = 0; c < 3; c++) f2_acc(sh[c], sl[c], th[c], te[c]);
-            if (k & 1) {                       // the low parts back below the last place of the high ones
-#pragma unroll
-                for (int c = 0; c < 3; c++) f2_fast_two_sum(sh[c], sl[c], sh[c], sl[c]);
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const float2 a = f2_get(sh[c]), b = f2_get(sl[c]);
-            float s, x;
-            ff_two_sum(a.x, a.y, s, x);
-            const double v = ff_sum_f64(s) + f64_of_f32_any(x + (b.x + b.y));
-            acc[c] = MODE == kFfUniform ? fma(mm, v, acc[c]) : acc[c] + v;
-        }
-    }
-}
-
-template <bool PC>
-__global__ void __launch_bounds__(kTlRows, 4)
-kick_tile_ff_kernel(SymArgs A) {
-    __shared__ float4 grp[7 * 32];
-    __shared__ uint2 pcb[PC ? 4 : 1][PC ? kSymPcBuf : 1];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, a = blockIdx.x;
-    const TlRange R = tl_range(A);
-    const bool exact = ff_exact_pairs(A.ff_header, A.n);
-    const float close2 = exact ? kFfExactClose2 : kFfClose2;
-    int pend = 0;
-    TlRow I;
-    tl_load_row<PC>(A, a, threadIdx.x, close2, I);
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int g = R.g0; g < R.g1; g++) {
-        __syncthreads();
-        tl_stage(A, g, grp);
-        __syncthreads();
-        const double mm = A.tmass[g >> 1];
-        const bool gen = (g >> 1) == a || ((a + 1) * kSymT > A.nm && (g + 1) * 64 > A.nm);
-        if (exact) tl_group<PC, kFfExact>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
-        else if (gen) tl_group<PC, kFfGeneral>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
-        else if (mm > 0.0) tl_group<PC, kFfUniform>(A, grp, g, R.k0, R.k1, I, close2, mm, acc, pcb[PC ? w : 0], pend, lane);
-        else tl_group<PC, kFfPlain>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, pcb[PC ? w : 0], pend, lane);
-    }
-    if (PC) sym_pc_flush(A, pcb[w], pend, lane);
-    if (I.i < A.n) {
-        double *p = A.part + (size_t)blockIdx.y * 3 * A.n + I.i;
-#pragma unroll
-        for (int c = 0; c < 3; c++) p[(size_t)c * A.n] = acc[c];
-    }
-}
-
-// ---------------------------------------------------------------- FP64
-
-// FP64: the warp's buffered near pairs (row lane, body j), 32 at a time: every lane
+// The warp's buffered pairs (row lane, body j) -- FP64: near ones; mixed: those that the
+// packed coordinates do not give --, 32 at a time: every lane
 // forms one pair's term m_j K r^-3 d in FP64 from the positions, then adds the
 // terms of its own row in buffer order.
 struct TlNear {
@@ -276,6 +130,165 @@ __device__ __forceinline__ void tl_near_flush(const SymArgs &A, TlNear &B, int &
     __syncwarp();
     cnt = 0;
 }
+
+// Mixed: the steps [k0, k1) of row I against the 64 bodies of group g; near: sums of the
+// buffered pairs in the caller's units.
+template <bool PC, int MODE>
+__device__ __forceinline__ void tl_group(const SymArgs &A, const float4 *grp, int g, int k0, int k1, const TlRow &I, float close2,
+                                         double mm, double (&acc)[3], double *near, TlNear &nb, int &npend, uint2 *pcbuf,
+                                         int &pend, int lane) {
+    constexpr bool EXACT = MODE == kFfExact, GEN = MODE == kFfGeneral || EXACT;
+    const f2 away = f2_dup(kFfMasked2);
+    const int es = EXACT ? A.ff_header[2] : 0;
+#pragma unroll 1
+    for (int tb = k0; tb < k1; tb += kTlFlush) {
+        f2 sh[3], sl[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++) sh[c] = sl[c] = 0ull;
+#pragma unroll (EXACT ? 1 : 2)
+        for (int k = tb; k < min(tb + kTlFlush, k1); k++) {
+            const float4 q0 = grp[k], q1 = grp[32 + k], q2 = grp[64 + k], q3 = grp[96 + k], q4 = grp[128 + k],
+                         q5 = grp[160 + k];
+            const float2 tj = PC ? *reinterpret_cast<const float2 *>(&grp[192 + k].z) : make_float2(q5.z, q5.w);
+            const int j = g * 64 + k;
+            f2 H[3], L[3], s2, tail, w, wl;
+            bool wx = true, wy = true;
+            if (GEN) {
+                const bool ti = I.i >= A.nm;
+                wx = j != I.i && !(ti && j >= A.nm);
+                wy = j + 32 != I.i && !(ti && j + 32 >= A.nm);
+            }
+            if (EXACT) {
+                ff_disp_f64(A, min(I.i, A.n - 1), min(j, A.n - 1), min(j + 32, A.n - 1), es, H, L);
+                wx = wx && I.i < A.n && j < A.n;
+                wy = wy && I.i < A.n && j + 32 < A.n;
+            } else {
+                ff_disp(f2_lo(q0), f2_lo(q2), f2_lo(q4), I.h[0], I.m[0], I.l[0], H[0], L[0]);
+                ff_disp(f2_hi(q0), f2_hi(q2), f2_hi(q4), I.h[1], I.m[1], I.l[1], H[1], L[1]);
+                ff_disp(f2_lo(q1), f2_lo(q3), f2_lo(q5), I.h[2], I.m[2], I.l[2], H[2], L[2]);
+            }
+            ff_r2(H, L, s2, tail);
+            if (GEN) {                             // (NaN times zero would be NaN)
+                s2 = f2_select(wx, wy, s2, away);
+                tail = f2_select(wx, wy, tail, 0ull);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    H[c] = f2_select(wx, wy, H[c], 0ull);
+                    L[c] = f2_select(wx, wy, L[c], 0ull);
+                }
+            }
+            ff_inv_r3(s2, tail, w, wl);
+            const float2 S = f2_get(s2);
+            const bool fx = EXACT && S.x > kFfExactFar2, fy = EXACT && S.y > kFfExactFar2;
+            const bool nx = fx || !(S.x >= fmaxf(I.tn, tj.x)), ny = fy || !(S.y >= fmaxf(I.tn, tj.y));
+            if (__any_sync(0xffffffffu, nx || ny)) {
+                if (PC) {
+                    sym_pc_push(pcbuf, pend, lane, nx && wx && j > I.i, I.i, j);
+                    sym_pc_push(pcbuf, pend, lane, ny && wy && j + 32 > I.i, I.i, j + 32);
+                    if (pend > kSymPcFlush) sym_pc_flush(A, pcbuf, pend, lane);
+                }
+                // pairs that the packed coordinates do not give (a body that is not held, or
+                // closer than they tell): to the FP64 buffer, no term here
+                const bool ox = fx || !(S.x >= close2), oy = fy || !(S.y >= close2);
+                if (__any_sync(0xffffffffu, ox || oy)) {
+                    const bool vi = I.i < A.n;                   // not a padding body
+                    sym_pc_push(nb.q, npend, lane, ox && wx && vi && j < A.n, lane, j);
+                    sym_pc_push(nb.q, npend, lane, oy && wy && vi && j + 32 < A.n, lane, j + 32);
+                    if (npend > kTlNear - 64) tl_near_flush(A, nb, npend, I.i - lane, near, lane);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        H[c] = f2_select(ox, oy, 0ull, H[c]);
+                        L[c] = f2_select(ox, oy, 0ull, L[c]);
+                    }
+                    w = f2_select(ox, oy, 0ull, w);
+                    wl = f2_select(ox, oy, 0ull, wl);
+                }
+                // changeover band: K in float-float, 1/rc_ij = min(1/rc_i, 1/rc_j) (as float
+                // pairs: rounding is monotone), r^-3 scaled by K
+                const bool bx = !ox && S.x < fmaxf(I.thr, q5.z), by = !oy && S.y < fmaxf(I.thr, q5.w);
+                if (bx || by) {
+                    const float2 ci = A.ircf[I.i], Tl = f2_get(tail);
+                    float2 W = f2_get(w), WL = f2_get(wl);
+#pragma unroll 1
+                    for (int h = 0; h < 2; h++) {
+                        if (!(h ? by : bx)) continue;
+                        const float2 cj = A.ircf[j + 32 * h];
+                        const bool ti = ci.x < cj.x || (ci.x == cj.x && ci.y <= cj.y);
+                        float wh = h ? W.y : W.x, wlo = h ? WL.y : WL.x, Kh, Kl;
+                        ff_changeover(h ? S.y : S.x, h ? Tl.y : Tl.x, ti ? ci.x : cj.x, ti ? ci.y : cj.y, Kh, Kl);
+                        ff_mul(wh, wlo, Kh, Kl);
+                        if (Kh == 0.0f) wh = wlo = 0.0f;         // also where r^-3 overflows
+                        if (h) { W.y = wh; WL.y = wlo; }
+                        else { W.x = wh; WL.x = wlo; }
+                    }
+                    w = f2_make(W.x, W.y);
+                    wl = f2_make(WL.x, WL.y);
+                }
+            }
+            if (GEN) {
+                w = f2_select(wx, wy, w, 0ull);
+                wl = f2_select(wx, wy, wl, 0ull);
+            }
+            f2 ch = w, cl = wl, th[3], te[3];
+            if (MODE != kFfUniform) ff_coeff(f2_hi(q1), f2_hi(q3), w, wl, ch, cl);
+            ff_term(ch, cl, H, L, th, te);
+#pragma unroll
+            for (int c = 0; c < 3; c++) f2_acc(sh[c], sl[c], th[c], te[c]);
+            if (k & 1) {                       // the low parts back below the last place of the high ones
+#pragma unroll
+                for (int c = 0; c < 3; c++) f2_fast_two_sum(sh[c], sl[c], sh[c], sl[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const float2 a = f2_get(sh[c]), b = f2_get(sl[c]);
+            float s, x;
+            ff_two_sum(a.x, a.y, s, x);
+            const double v = ff_sum_f64(s) + f64_of_f32_any(x + (b.x + b.y));
+            acc[c] = MODE == kFfUniform ? fma(mm, v, acc[c]) : acc[c] + v;
+        }
+    }
+}
+
+template <bool PC>
+__global__ void __launch_bounds__(kTlRows, 4)
+kick_tile_ff_kernel(SymArgs A) {
+    __shared__ float4 grp[7 * 32];
+    __shared__ TlNear nb[4];
+    __shared__ double nsum[3][kTlRows];
+    __shared__ uint2 pcb[PC ? 4 : 1][PC ? kSymPcBuf : 1];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, a = blockIdx.x;
+    const TlRange R = tl_range(A);
+    const bool exact = ff_exact_pairs(A.ff_header, A.n);
+    const float close2 = exact ? kFfExactClose2 : kFfClose2;
+    int pend = 0, npend = 0;
+    TlRow I;
+    tl_load_row<PC>(A, a, threadIdx.x, close2, I);
+    double acc[3] = {0.0, 0.0, 0.0}, *near = &nsum[0][threadIdx.x];
+#pragma unroll
+    for (int c = 0; c < 3; c++) near[c * kTlRows] = 0.0;
+    for (int g = R.g0; g < R.g1; g++) {
+        __syncthreads();
+        tl_stage(A, g, grp);
+        __syncthreads();
+        const double mm = A.tmass[g >> 1];
+        const bool gen = (g >> 1) == a || ((a + 1) * kSymT > A.nm && (g + 1) * 64 > A.nm);
+        if (exact) tl_group<PC, kFfExact>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        else if (gen) tl_group<PC, kFfGeneral>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        else if (mm > 0.0) tl_group<PC, kFfUniform>(A, grp, g, R.k0, R.k1, I, close2, mm, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+        else tl_group<PC, kFfPlain>(A, grp, g, R.k0, R.k1, I, close2, 0.0, acc, near, nb[w], npend, pcb[PC ? w : 0], pend, lane);
+    }
+    tl_near_flush(A, nb[w], npend, I.i - lane, near, lane);
+    if (PC) sym_pc_flush(A, pcb[w], pend, lane);
+    if (I.i < A.n) {
+        const double back = scalbn(1.0, 2 * A.ff_header[2] - A.ff_header[1]);     // to the packed units
+        double *p = A.part + (size_t)blockIdx.y * 3 * A.n + I.i;
+#pragma unroll
+        for (int c = 0; c < 3; c++) p[(size_t)c * A.n] = near[c * kTlRows] != 0.0 ? fma(back, near[c * kTlRows], acc[c]) : acc[c];
+    }
+}
+
+// ---------------------------------------------------------------- FP64
 
 // FP64: the steps [k0, k1) of row I against the 64 bodies of group g.  acc: sums of (m_j) r^-3 d
 // in the packed units, near: those of the buffered pairs in the caller's units.

@@ -556,11 +556,21 @@ struct EnsFast {
     double mp[3], irc[3], gm;                  // G m and 1/rc_ij of the partners s ^ q, q = 1 2 3; G m_star
     float ircf[3];
 };
+// rsqrt_newton where its FP32 seed holds x, CUDA's root elsewhere: a coarse column may pass
+// a partner at 1e-19 or fling a member to 1e19 before its step is rejected.
+__device__ __forceinline__ bool ens_in_f32(double x) { return ((unsigned)__double2hiint(x) >> 20) - 898u < 250u; }
+__device__ __forceinline__ double ens_rsqrt(double x) { return ens_in_f32(x) ? rsqrt_newton(x) : rsqrt(x); }
+// The side of the changeover band (changeover_side_f32) for any d2 = d^2, id = 1/d.
+__device__ __forceinline__ int ens_side(double d2, double id, double irc, float ircf) {
+    if (ens_in_f32(d2)) return changeover_side_f32(f32_of_f64_trunc(d2) * f32_of_f64_trunc(id), ircf);
+    const double q = d2 * id * irc;
+    return q < 0.09999 ? -1 : q > 1.0001 ? 1 : 0;
+}
 __device__ __forceinline__ void ens_fast_deriv(const EnsArgs &A, const EnsShared &S, const EnsFast &F, int nm,
                                                double (&f)[6]) {
     const double x = F.z[0], y = F.z[1], z = F.z[2];
     const double r2 = fma(z, z, fma(y, y, x * x));
-    const double ir = rsqrt_newton(r2);
+    const double ir = ens_rsqrt(r2);
     double c = -F.gm * (ir * ir * ir);
     double fac = 1.0;
     if (A.gr == 2) {
@@ -575,10 +585,10 @@ __device__ __forceinline__ void ens_fast_deriv(const EnsArgs &A, const EnsShared
         const double dx = __shfl_xor_sync(0xffffffffu, x, q) - x, dy = __shfl_xor_sync(0xffffffffu, y, q) - y,
                      dz = __shfl_xor_sync(0xffffffffu, z, q) - z;
         const double d2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const double id = rsqrt_newton(d2);
+        const double id = ens_rsqrt(d2);
         double w = F.mp[q - 1] * (id * id * id);
         // 1 - K: 1 below 0.1 rc, 0 above rc
-        const int side = changeover_side_f32(f32_of_f64_trunc(d2) * f32_of_f64_trunc(id), F.ircf[q - 1]);
+        const int side = ens_side(d2, id, F.irc[q - 1], F.ircf[q - 1]);
         if (side == 0) w *= changeover_rest(d2 * id, F.irc[q - 1]);
         if (F.mp[q - 1] == 0.0 || side > 0) w = 0.0;     // no partner (or itself a lane without a member)
         ax = fma(w, dx, ax);
@@ -680,7 +690,7 @@ __device__ void ens_bs_fast(const EnsArgs &A, EnsShared &S, int nm, double dt, u
                     v = nxt;
                 }
             }
-            const bool off = member && col < 6 && fabs(v - last) > lim;
+            const bool off = member && col < 6 && !(fabs(v - last) <= lim);      // (a NaN is not convergence)
             if (k >= 1 && !__any_sync(0xffffffffu, off)) {
                 kconv = k;
 #pragma unroll

@@ -30,7 +30,7 @@ def _inputs(case, n):
     return x, v, m, rc, sorted({*which[:3], *range(0, n, max(1, n // 150))})
 
 
-def _reference(x, m, rc, rows):
+def _reference(x, m, rc, rows, nm):
     X, M, R = (np.asarray(a, dtype=LD) for a in (x, m, rc))
     acc, mag = np.zeros((len(rows), 3), LD), np.zeros((len(rows), 3), LD)
     for k, i in enumerate(rows):
@@ -41,6 +41,8 @@ def _reference(x, m, rc, rows):
         y = np.clip((r / np.maximum(R, R[i]) - LD("0.1")) / LD("0.9"), 0, 1)
         w = LD(G_GAUSS) * M * (y * y / (2 * y * y - 2 * y + 1)) / (r2 * r)
         w[i] = 0
+        if i >= nm:
+            w[nm:] = 0
         t = w[:, None] * d
         acc[k], mag[k] = t.sum(axis=0), abs(t).sum(axis=0)
     return acc, mag
@@ -56,7 +58,7 @@ def test_far_bodies_match_long_double(cuda_lib, case, n):
     import torch
     g = cuda_lib
     x, v, m, rc, rows = _inputs(case, n)
-    ref, mag = _reference(x, m, rc, rows)
+    ref, mag = _reference(x, m, rc, rows, n)
     dev = torch.device("cuda:0")
     T = lambda a: torch.tensor(np.ascontiguousarray(a), device=dev)
     pos, mass, acc = T(x.T), T(m), torch.zeros((3, n), dtype=torch.float64, device=dev)
@@ -79,3 +81,33 @@ def test_far_bodies_match_long_double(cuda_lib, case, n):
         check(precision, (precision, layout))
         assert g.kick_static(pos, mass, T(rc), G_GAUSS, 0.0, precision, None, acc) == 0
         check(precision, "static")
+
+
+@pytest.mark.parametrize("kind", ["test particles", "massless", "very light"])
+@pytest.mark.parametrize("case", [("one", 1e5), ("half", 1e5), ("three", 1e9)], ids=lambda c: "%s %g" % c)
+@pytest.mark.parametrize("n", [700, 2500])
+def test_far_bodies_with_masked_pairs_and_light_masses(cuda_lib, n, case, kind):
+    import torch
+    g = cuda_lib
+    x, v, m, rc, rows = _inputs(case, n)
+    nm = n
+    if kind == "test particles":
+        nm = n // 3
+        m[nm:] *= 1e-4
+    else:
+        m[1::3] *= 0.0 if kind == "massless" else 2.0 ** -45
+    ref, mag = _reference(x, m, rc, rows, nm)
+    dev = torch.device("cuda:0")
+    T = lambda a: torch.tensor(np.ascontiguousarray(a), device=dev)
+    out = torch.zeros((3, n), dtype=torch.float64, device=dev)
+    for precision, layout in ((0, g.GENGA_KICK_TILED), (1, g.GENGA_KICK_TILED), (1, g.GENGA_KICK_SYMMETRIC)):
+        p = g.default_params(G=G_GAUSS, precision=precision, f_pc=1.5)
+        if nm < n:
+            p.tp_mode, p.n_massive = 2, nm
+        s = g.System(T(x.T), T(v.T), T(m), p)
+        s.set_kick_layout(layout)
+        s.set_rcrit(rc)
+        s.kick(0.0, precheck=True, acc_out=out)
+        err = np.abs(out.cpu().numpy().T[rows] - ref)
+        assert np.all(err <= BOUND[precision] * mag + 1e-300), (precision, layout, (err / np.maximum(mag, 1e-300)).max(axis=0))
+        np.testing.assert_array_equal(s.candidates(), O.precheck(x, rc, 1.5, n_massive=nm))
